@@ -1,0 +1,258 @@
+"""The work that performance is measured on: decode steps and prompt chunks through the library's entry points.
+
+A case is one layer stack of a model with a latent (or, for layers that the compression schedule skips, ordinary) KV
+cache.  One pass is what a serving program does for it: per layer the cache write of the new tokens (lorc_append), then
+their attention over the cache (lorc_decode_attn, or lorc_prefill_attn for several tokens per sequence), in that order,
+layer after layer.  Writing the same tokens again leaves the cache as it was, so a pass can be repeated.
+
+Keys of a case:
+  kind      "decode" (one token per sequence), "host" (the same from pinned host buffers), "prefill" (T tokens)
+  D, heads, kv_heads, d_head   model geometry
+  rope      "half", "interleaved" or "none"
+  mode      "latent", or "full" for uncompressed layers
+  layers, r_first, r_last, quantum   ranks fall linearly from the first layer to the last, in steps of `quantum`
+  batch, len_min, len_max   cached tokens per sequence, the new ones included, drawn uniformly from the range
+  page      tokens per page of a paged cache in random page order; 0: contiguous
+  T         new tokens per sequence
+  q_scale   standard deviation of the query elements (1: nearly uniform attention, 64: peaked)
+"""
+import math
+
+import torch
+
+import paper_2410_03111_b200 as lorc
+
+# head geometries: query heads, KV heads, head dimension, model dimension, RoPE base
+GEOMETRY = {
+    "8b": dict(D=4096, heads=32, kv_heads=8, d_head=128, theta=500000.0),
+    "70b": dict(D=8192, heads=64, kv_heads=8, d_head=128, theta=500000.0),
+    "tiny": dict(D=256, heads=4, kv_heads=2, d_head=64, theta=10000.0),
+}
+
+
+def _case(kind, geometry, layers, r_first, r_last, batch, len_min, len_max, T=1, page=0, rope="half", mode="latent",
+          quantum=32, q_scale=8.0):
+    return dict(GEOMETRY[geometry], kind=kind, layers=layers, r_first=r_first, r_last=r_last, quantum=quantum,
+                batch=batch, len_min=len_min, len_max=len_max, T=T, page=page, rope=rope, mode=mode, q_scale=q_scale)
+
+
+def listed():
+    c = {}
+    # the smallest call: a single layer with 64-wide heads, 128 cached tokens and a new one; launches and latency only
+    c["tiny_step"] = _case("decode", "tiny", 1, 32, 32, 1, 129, 129)
+    # one user's chat on an 8B-shaped model: four layers of the progressive rank schedule, a context of odd length
+    c["single_user"] = _case("decode", "8b", 4, 928, 416, 1, 1037, 1037)
+    # the step a serving host makes: hidden states and queries from pinned memory, results back, a small batch
+    c["host_step"] = _case("host", "8b", 4, 928, 416, 16, 1025, 1025)
+    # the headline workload, a quarter of its layers: 8B shape, progressive ranks, batch 16, 4096 tokens and some decoded
+    c["batch_progressive"] = _case("decode", "8b", 8, 928, 416, 16, 4129, 4129)
+    # long context at a low uniform rank
+    c["long_context"] = _case("decode", "8b", 2, 256, 256, 4, 32777, 32777)
+    # 70B shape (eight query heads per KV head), early, middle and late layer of its schedule
+    c["large_model"] = _case("decode", "70b", 3, 864, 352, 8, 8201, 8201)
+    # ragged serving batch over a paged cache
+    c["ragged_paged"] = _case("decode", "8b", 1, 384, 384, 64, 512, 16384, page=64)
+    # layers that the schedule leaves uncompressed
+    c["uncompressed"] = _case("decode", "8b", 2, 1024, 1024, 16, 4129, 4129, mode="full")
+    # a model without rotary embedding: absorbed scores
+    c["no_rotation"] = _case("decode", "8b", 2, 672, 672, 16, 4129, 4129, rope="none")
+    # the other pairing convention of rotary embeddings
+    c["interleaved"] = _case("decode", "8b", 1, 512, 512, 4, 2049, 2049, rope="interleaved")
+    # a whole prompt of one user
+    c["prompt"] = _case("prefill", "8b", 2, 928, 416, 1, 777, 777, T=777)
+    # chunked prompt processing of a batch: the last chunk of 4096-token prompts, paged
+    c["prompt_chunk"] = _case("prefill", "8b", 1, 672, 672, 16, 4096, 4096, T=1024, page=64)
+    return [dict(v, name=k) for k, v in c.items()]
+
+
+def _log_int(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    most = [max(work(c)[k] for c in listed()) for k in ("bytes", "flops")]
+    while True:
+        c = _draw(rng)
+        w = work(c)
+        if w["bytes"] <= most[0] and w["flops"] <= most[1]:
+            return c
+
+
+def _draw(rng):
+    what = rng.choice(["tiny", "single", "batch", "batch", "long", "ragged", "full", "none", "interleaved", "host",
+                       "prompt", "chunk"])
+    geometry = rng.choice(["8b", "8b", "70b"])
+    q_scale = rng.choice([1.0, 8.0, 8.0, 64.0])
+    page = rng.choice([0, 0, 16, 64, 128])
+    hi = 8 * rng.randint(8, 116)                       # ranks 64 .. 928, every multiple of eight
+    lo = max(64, hi - 8 * rng.randint(0, 64))
+    more = dict(q_scale=q_scale, quantum=8)
+    if what == "tiny":
+        n = _log_int(rng, 17, 2000)
+        r = 8 * rng.randint(2, 12)
+        return _case("decode", "tiny", rng.randint(1, 2), r, r, rng.randint(1, 6), max(1, n // 2), n, **more)
+    if what == "single":
+        n = _log_int(rng, 100, 8000)
+        return _case("decode", geometry, rng.randint(1, 4), hi, lo, rng.randint(1, 2), n, n, page=page, **more)
+    if what == "batch":
+        b, n = rng.randint(3, 32), _log_int(rng, 300, 8200)
+        return _case("decode", geometry, rng.randint(1, 4), hi, lo, b, n, n, page=page, **more)
+    if what == "long":
+        b, n = rng.randint(1, 4), _log_int(rng, 16000, 65000)
+        return _case("decode", geometry, 1, hi, lo, b, n, n, page=page, **more)
+    if what == "ragged":
+        b, n = rng.randint(8, 64), _log_int(rng, 2000, 16384)
+        return _case("decode", geometry, 1, hi, lo, b, max(1, n // 32), n, page=rng.choice([16, 32, 64, 128]), **more)
+    if what == "full":
+        b, n = rng.randint(1, 32), _log_int(rng, 200, 8200)
+        return _case("decode", geometry, rng.randint(1, 2), 1024, 1024, b, max(1, n // rng.choice([1, 8])), n, page=page,
+                     mode="full", **more)
+    if what == "none":
+        b, n = rng.randint(1, 32), _log_int(rng, 200, 8200)
+        return _case("decode", geometry, rng.randint(1, 2), hi, lo, b, n, n, page=page, rope="none", **more)
+    if what == "interleaved":
+        b, n = rng.randint(1, 4), _log_int(rng, 100, 2100)
+        return _case("decode", geometry, 1, hi, lo, b, n, n, page=page, rope="interleaved", **more)
+    if what == "host":
+        b, n = rng.randint(1, 32), _log_int(rng, 100, 4200)
+        return _case("host", geometry, rng.randint(1, 4), hi, lo, b, n, n, page=page, **more)
+    if what == "prompt":
+        n = _log_int(rng, 40, 4096)
+        return _case("prefill", geometry, rng.randint(1, 2), hi, lo, rng.randint(1, 2), n, n, T=n, page=page, **more)
+    T = _log_int(rng, 64, 1024)
+    n = T + _log_int(rng, 64, 4096)
+    return _case("prefill", geometry, 1, hi, lo, rng.randint(1, 8), n, n, T=T, page=page, **more)
+
+
+def _ranks(case):
+    n, q = case["kv_heads"] * case["d_head"], case["quantum"]
+    if case["mode"] == "full":
+        return [n] * case["layers"]
+    span = max(1, case["layers"] - 1)
+    r = [case["r_first"] + (case["r_last"] - case["r_first"]) * l / span for l in range(case["layers"])]
+    return [min(n, max(8, q * round(x / q))) for x in r]
+
+
+class State:
+    """What a serving program keeps: the context with its factors and workspace, the caches, the step's inputs."""
+
+    def __init__(self, case, seed):
+        self.case = case
+        L = self.L = lorc.load()
+        dev = "cuda"
+        g = torch.Generator(device=dev)
+        g.manual_seed(seed)
+        D, H, hkv, dh = case["D"], case["heads"], case["kv_heads"], case["d_head"]
+        n, b, T, ps = hkv * dh, case["batch"], case["T"], case["page"]
+        full = case["mode"] == "full"
+        bf16 = torch.bfloat16
+
+        def randn(*shape):
+            return torch.randn(*shape, generator=g, device=dev, dtype=bf16)
+
+        lens = torch.randint(case["len_min"], case["len_max"] + 1, (b,), generator=g, device=dev, dtype=torch.int32)
+        self.lens = torch.clamp(lens, min=T)
+        n_max = case["len_max"]
+        style = {"half": L.LORC_ROPE_HALF_SPLIT, "interleaved": L.LORC_ROPE_INTERLEAVED, "none": L.LORC_ROPE_NONE}
+        self.ctx = L.lorc_create(case["layers"], D, H, hkv, dh, case["theta"], rope_style=style[case["rope"]],
+                                 max_pos=n_max + 64)
+        if ps:
+            per = (n_max + ps - 1) // ps
+            n_pages = b * per
+            self.table = torch.randperm(n_pages, generator=g, device=dev).to(torch.int32).view(b, per)
+        self.k, self.v, self.caches = [], [], []
+        for l, r in enumerate(_ranks(case)):
+            # spectrum sigma_i = i^-0.8, orthonormal factors (a Gaussian matrix with many rows is one, nearly); the
+            # cached coordinates of Gaussian hidden states are then N(0, sigma_i^2)
+            sigma = torch.arange(1, r + 1, device=dev, dtype=torch.float32) ** -0.8
+            if full:
+                w = [(randn(D, n).float() * sigma / math.sqrt(D)) @ (randn(n, n).float() / math.sqrt(n)) for _ in "kv"]
+                w = [m.to(bf16) for m in w]
+                L.lorc_load_factors(self.ctx, l, L.LORC_MODE_FULL, 0, 0, w[0], None, w[1], None)
+                scale = torch.full((n,), float(sigma.square().sum()) ** 0.5 / math.sqrt(n), device=dev).to(bf16)
+            else:
+                a = [(randn(D, r).float() * sigma / math.sqrt(D)).to(bf16) for _ in "kv"]
+                f = [(randn(r, n).float() / math.sqrt(n)).to(bf16) for _ in "kv"]
+                L.lorc_load_factors(self.ctx, l, L.LORC_MODE_LATENT, r, r, a[0], f[0], a[1], f[1])
+                scale = sigma.to(bf16)
+            rows = (n_pages, ps, r) if ps else (b, n_max, r)
+            k, v = randn(*rows).mul_(scale), randn(*rows).mul_(scale)
+            self.k.append(k)
+            self.v.append(v)
+            if ps:
+                c = L.make_cache(k, v, self.lens, b, n_max, page_table=self.table, page_size=ps, max_pages_per_seq=per,
+                                 n_pages=n_pages)
+            else:
+                c = L.make_cache(k, v, self.lens, b, n_max, seq_stride=n_max)
+            self.caches.append(c)
+        need = L.lorc_workspace_bytes(self.ctx, b, n_max)
+        if case["kind"] == "prefill":
+            need = max(need, L.lorc_prefill_workspace_bytes(self.ctx, b, n_max, T))
+        self.ws = torch.zeros(need, dtype=torch.uint8, device=dev)
+        L.lorc_set_workspace(self.ctx, self.ws)
+        self.x = randn(case["layers"], b, T, D)
+        self.q = randn(case["layers"], b, T, H, dh) * case["q_scale"]
+        self.out = torch.zeros_like(self.q)
+        if case["kind"] == "host":
+            self.x, self.q, self.out = (t.cpu().pin_memory() for t in (self.x, self.q, self.out))
+        # per-layer views, as a layer's forward pass holds them
+        self.steps = [(l, c, self.x[l], self.q[l], self.out[l]) for l, c in enumerate(self.caches)]
+
+    def __del__(self):
+        if getattr(self, "ctx", None) is not None:
+            torch.cuda.synchronize()
+            self.L.lorc_destroy(self.ctx)
+            self.ctx = None
+
+
+def prepare(case, seed):
+    return State(case, seed)
+
+
+def run(state):
+    L, ctx, kind, T = state.L, state.ctx, state.case["kind"], state.case["T"]
+    if kind == "host":
+        for layer, cache, x, q, out in state.steps:
+            L.lorc_decode_step_host(ctx, layer, cache, x, q, out)
+        torch.cuda.current_stream().synchronize()      # the host reads the results
+    elif kind == "prefill":
+        for layer, cache, x, q, out in state.steps:
+            L.lorc_append(ctx, layer, cache, x, T)
+            L.lorc_prefill_attn(ctx, layer, cache, q, out, T)
+    else:
+        for layer, cache, x, q, out in state.steps:
+            L.lorc_append(ctx, layer, cache, x)
+            L.lorc_decode_attn(ctx, layer, cache, q, out)
+    return {"out": state.out, "k": state.k, "v": state.v}
+
+
+def work(case):
+    """Latents (or keys and values) and factors read once, new rows, queries and results; the dense contractions."""
+    D, H, dh, b, T = case["D"], case["heads"], case["d_head"], case["batch"], case["T"]
+    n = case["kv_heads"] * dh
+    length = max(T, (case["len_min"] + case["len_max"]) / 2)      # expected cached tokens per sequence
+    pairs = b * T * (length - (T - 1) / 2)                        # (query, key) pairs per head
+    by = fl = 0.0
+    for r in _ranks(case):
+        by += 2 * b * length * 2 * r + 2 * D * 2 * r + 2 * b * T * (D + 2 * r + 2 * H * dh)
+        fl += 2 * b * T * D * 2 * r
+        if case["mode"] == "full":
+            fl += 4 * pairs * H * dh
+            continue
+        by += 2 * 2 * r * n
+        if case["kind"] == "prefill":
+            fl += 2 * b * length * 2 * r * n + 4 * pairs * H * dh
+        elif case["rope"] == "none":
+            fl += 4 * pairs * H * r + 4 * b * H * r * dh
+        else:
+            fl += 2 * b * length * r * n + 2 * pairs * H * (dh + r) + 2 * b * H * r * dh
+    return {"bytes": by, "flops": fl}
+
+
+def tolerance(case):
+    # Against the same computation in fp64 the results of these paths are off by (2-norm, and largest difference over
+    # the larger of the value and the rms): bf16 output alone 1.6e-3 and 0.004, fp16 probabilities (prompts) 1.7e-3 and
+    # 0.010, bf16 probabilities (uncompressed) 2.3e-3 and 0.007, bf16 probabilities and latent output 3.2e-3 and 0.019.
+    # Another correct implementation is off by as much in another direction.
+    latent_step = case["mode"] == "latent" and case["kind"] != "prefill" and case["d_head"] == 128
+    return {"rel": 1e-2, "max": 0.06} if latent_step else {"rel": 7e-3, "max": 0.04}
