@@ -17,6 +17,7 @@ Keys of a case:
   q_scale   standard deviation of the query elements (1: nearly uniform attention, 64: peaked)
 """
 import math
+from types import SimpleNamespace
 
 import torch
 
@@ -133,65 +134,72 @@ def _ranks(case):
     return [min(n, max(8, q * round(x / q))) for x in r]
 
 
+def _inputs(case, seed):
+    """Everything random of a case, on the GPU: lengths, pages, per layer the factors and the cached rows, the step's x and q."""
+    dev = "cuda"
+    g = torch.Generator(device=dev)
+    g.manual_seed(seed)
+    D, H, dh = case["D"], case["heads"], case["d_head"]
+    n, b, T, ps = case["kv_heads"] * dh, case["batch"], case["T"], case["page"]
+    n_max = case["len_max"]
+    bf16 = torch.bfloat16
+
+    def randn(*shape):
+        return torch.randn(*shape, generator=g, device=dev, dtype=bf16)
+
+    lens = torch.randint(case["len_min"], case["len_max"] + 1, (b,), generator=g, device=dev, dtype=torch.int32)
+    i = SimpleNamespace(lens=torch.clamp(lens, min=T), table=None, factors=[], k=[], v=[])
+    if ps:
+        per = (n_max + ps - 1) // ps
+        i.table = torch.randperm(b * per, generator=g, device=dev).to(torch.int32).view(b, per)
+    for r in _ranks(case):
+        # spectrum sigma_i = i^-0.8, orthonormal factors (a Gaussian matrix with many rows is one, nearly); the
+        # cached coordinates of Gaussian hidden states are then N(0, sigma_i^2)
+        sigma = torch.arange(1, r + 1, device=dev, dtype=torch.float32) ** -0.8
+        if case["mode"] == "full":
+            w = [(randn(D, n).float() * sigma / math.sqrt(D)) @ (randn(n, n).float() / math.sqrt(n)) for _ in "kv"]
+            i.factors.append(([m.to(bf16) for m in w], [None, None]))
+            scale = torch.full((n,), float(sigma.square().sum()) ** 0.5 / math.sqrt(n), device=dev).to(bf16)
+        else:
+            a = [(randn(D, r).float() * sigma / math.sqrt(D)).to(bf16) for _ in "kv"]
+            i.factors.append((a, [(randn(r, n).float() / math.sqrt(n)).to(bf16) for _ in "kv"]))
+            scale = sigma.to(bf16)
+        rows = (i.table.numel(), ps, r) if ps else (b, n_max, r)
+        i.k.append(randn(*rows).mul_(scale))
+        i.v.append(randn(*rows).mul_(scale))
+    i.x = randn(case["layers"], b, T, D)
+    i.q = randn(case["layers"], b, T, H, dh) * case["q_scale"]
+    return i
+
+
 class State:
     """What a serving program keeps: the context with its factors and workspace, the caches, the step's inputs."""
 
     def __init__(self, case, seed):
         self.case = case
         L = self.L = lorc.load()
-        dev = "cuda"
-        g = torch.Generator(device=dev)
-        g.manual_seed(seed)
-        D, H, hkv, dh = case["D"], case["heads"], case["kv_heads"], case["d_head"]
-        n, b, T, ps = hkv * dh, case["batch"], case["T"], case["page"]
-        full = case["mode"] == "full"
-        bf16 = torch.bfloat16
-
-        def randn(*shape):
-            return torch.randn(*shape, generator=g, device=dev, dtype=bf16)
-
-        lens = torch.randint(case["len_min"], case["len_max"] + 1, (b,), generator=g, device=dev, dtype=torch.int32)
-        self.lens = torch.clamp(lens, min=T)
-        n_max = case["len_max"]
+        i = _inputs(case, seed)
+        b, T, ps, n_max = case["batch"], case["T"], case["page"], case["len_max"]
+        self.lens, self.table, self.k, self.v, self.x, self.q = i.lens, i.table, i.k, i.v, i.x, i.q
         style = {"half": L.LORC_ROPE_HALF_SPLIT, "interleaved": L.LORC_ROPE_INTERLEAVED, "none": L.LORC_ROPE_NONE}
-        self.ctx = L.lorc_create(case["layers"], D, H, hkv, dh, case["theta"], rope_style=style[case["rope"]],
-                                 max_pos=n_max + 64)
-        if ps:
-            per = (n_max + ps - 1) // ps
-            n_pages = b * per
-            self.table = torch.randperm(n_pages, generator=g, device=dev).to(torch.int32).view(b, per)
-        self.k, self.v, self.caches = [], [], []
-        for l, r in enumerate(_ranks(case)):
-            # spectrum sigma_i = i^-0.8, orthonormal factors (a Gaussian matrix with many rows is one, nearly); the
-            # cached coordinates of Gaussian hidden states are then N(0, sigma_i^2)
-            sigma = torch.arange(1, r + 1, device=dev, dtype=torch.float32) ** -0.8
-            if full:
-                w = [(randn(D, n).float() * sigma / math.sqrt(D)) @ (randn(n, n).float() / math.sqrt(n)) for _ in "kv"]
-                w = [m.to(bf16) for m in w]
-                L.lorc_load_factors(self.ctx, l, L.LORC_MODE_FULL, 0, 0, w[0], None, w[1], None)
-                scale = torch.full((n,), float(sigma.square().sum()) ** 0.5 / math.sqrt(n), device=dev).to(bf16)
-            else:
-                a = [(randn(D, r).float() * sigma / math.sqrt(D)).to(bf16) for _ in "kv"]
-                f = [(randn(r, n).float() / math.sqrt(n)).to(bf16) for _ in "kv"]
-                L.lorc_load_factors(self.ctx, l, L.LORC_MODE_LATENT, r, r, a[0], f[0], a[1], f[1])
-                scale = sigma.to(bf16)
-            rows = (n_pages, ps, r) if ps else (b, n_max, r)
-            k, v = randn(*rows).mul_(scale), randn(*rows).mul_(scale)
-            self.k.append(k)
-            self.v.append(v)
+        self.ctx = L.lorc_create(case["layers"], case["D"], case["heads"], case["kv_heads"], case["d_head"],
+                                 case["theta"], rope_style=style[case["rope"]], max_pos=n_max + 64)
+        mode = L.LORC_MODE_FULL if case["mode"] == "full" else L.LORC_MODE_LATENT
+        self.caches = []
+        for l, (r, (a, f)) in enumerate(zip(_ranks(case), i.factors)):
+            r = 0 if case["mode"] == "full" else r
+            L.lorc_load_factors(self.ctx, l, mode, r, r, a[0], f[0], a[1], f[1])
             if ps:
-                c = L.make_cache(k, v, self.lens, b, n_max, page_table=self.table, page_size=ps, max_pages_per_seq=per,
-                                 n_pages=n_pages)
+                c = L.make_cache(self.k[l], self.v[l], self.lens, b, n_max, page_table=self.table, page_size=ps,
+                                 max_pages_per_seq=self.table.shape[1], n_pages=self.table.numel())
             else:
-                c = L.make_cache(k, v, self.lens, b, n_max, seq_stride=n_max)
+                c = L.make_cache(self.k[l], self.v[l], self.lens, b, n_max, seq_stride=n_max)
             self.caches.append(c)
         need = L.lorc_workspace_bytes(self.ctx, b, n_max)
         if case["kind"] == "prefill":
             need = max(need, L.lorc_prefill_workspace_bytes(self.ctx, b, n_max, T))
-        self.ws = torch.zeros(need, dtype=torch.uint8, device=dev)
+        self.ws = torch.zeros(need, dtype=torch.uint8, device="cuda")
         L.lorc_set_workspace(self.ctx, self.ws)
-        self.x = randn(case["layers"], b, T, D)
-        self.q = randn(case["layers"], b, T, H, dh) * case["q_scale"]
         self.out = torch.zeros_like(self.q)
         if case["kind"] == "host":
             self.x, self.q, self.out = (t.cpu().pin_memory() for t in (self.x, self.q, self.out))
@@ -224,6 +232,60 @@ def run(state):
             L.lorc_append(ctx, layer, cache, x)
             L.lorc_decode_attn(ctx, layer, cache, q, out)
     return {"out": state.out, "k": state.k, "v": state.v}
+
+
+def _rotate(t, pos, case):
+    """t [..., tokens, heads, d_head] rotated at pos [tokens], in the case's pairing convention."""
+    if case["rope"] == "none":
+        return t
+    d = t.shape[-1]
+    j = torch.arange(d // 2, device=t.device, dtype=torch.float64)
+    ang = pos.double()[:, None, None] * case["theta"] ** (-2.0 * j / d)
+    c, s = torch.cos(ang), torch.sin(ang)
+    out = torch.empty_like(t)
+    lo, hi = (slice(0, d // 2), slice(d // 2, d)) if case["rope"] == "half" else (slice(0, d, 2), slice(1, d, 2))
+    a, b = t[..., lo], t[..., hi]
+    out[..., lo], out[..., hi] = a * c - b * s, a * s + b * c
+    return out
+
+
+def exact(case, seed):
+    """run()'s results in fp64 torch: the cache rows before they are rounded, and the attention over the bf16 cache."""
+    i = _inputs(case, seed)
+    b, T, ps, H, dh, hkv = (case[k] for k in ("batch", "T", "page", "heads", "d_head", "kv_heads"))
+    full = case["mode"] == "full"
+    out = torch.zeros(i.q.shape, dtype=torch.float64, device="cuda")
+    lens = i.lens.tolist()
+    caches = {"k": [], "v": []}
+    for l, (a, f) in enumerate(i.factors):
+        kv = [t.double() for t in (i.k[l], i.v[l])]
+        kv = [t.view(-1, t.shape[-1]) for t in kv]
+        for s in range(b):
+            pos = torch.arange(lens[s], device="cuda")
+            rows = (i.table[s, pos // ps].long() * ps + pos % ps) if ps else s * case["len_max"] + pos
+            new = [i.x[l, s].double() @ m.double() for m in a]
+            if full:
+                new[0] = _rotate(new[0].view(T, hkv, dh), pos[-T:], case).reshape(T, -1)
+            for c, y in zip(kv, new):
+                c[rows[-T:]] = y
+            # the attention reads the cache's bf16 rows
+            K, V = (c[rows].bfloat16().double() for c in kv)
+            if not full:
+                K, V = K @ f[0].double(), V @ f[1].double()
+            K, V = K.view(-1, hkv, dh), V.view(-1, hkv, dh)
+            if not full:
+                K = _rotate(K, pos, case)
+            q = _rotate(i.q[l, s].double(), pos[-T:], case)
+            later = pos[None, :] > pos[-T:, None]
+            for h in range(H):
+                kvh = h // (H // hkv)
+                score = (q[:, h] @ K[:, kvh].T / math.sqrt(dh)).masked_fill_(later, -math.inf)
+                out[l, s, :, h] = torch.softmax(score, -1) @ V[:, kvh]
+        caches["k"].append(kv[0].view(i.k[l].shape))
+        caches["v"].append(kv[1].view(i.v[l].shape))
+    if case["kind"] == "host":
+        out = out.cpu()
+    return {"out": out, "k": caches["k"], "v": caches["v"]}
 
 
 def work(case):
