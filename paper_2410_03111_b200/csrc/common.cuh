@@ -26,7 +26,8 @@ struct LorcLayer {
     bf16* A_tiled = nullptr;   // [(r_k+r_v)/8][D/32][32 lanes][8]: A_cat in mma fragment order (fast append), D % 32 == 0
     bf16* B_k = nullptr;       // [r_k, n]   (LATENT)
     bf16* B_v = nullptr;       // [r_v, n]   (LATENT)
-    bf16* B_kT = nullptr;      // [n, r_k]   transposed copy (K-major operand of the key reconstruction)
+    bf16* B_kT = nullptr;      // [n, r_k]   transposed copy (K-major operand of the key reconstruction); with interleaved
+                               //            rotary pairs row head * d_head + j + e * d_head / 2 is feature 2 j + e
     bf16* B_vT = nullptr;      // [n, r_v]   transposed copy (K-major operand of the value up-projection)
 };
 
@@ -118,7 +119,8 @@ static inline size_t lorc_align_up(size_t x, size_t a) { return (x + a - 1) / a 
 // ---- plain fp32 CUDA-core kernels: generic_kernels.cu ------------------------
 cudaError_t lorc_generic_build_rope_table(float2* table, int max_pos, int d_head, double theta,
                                           cudaStream_t st);
-cudaError_t lorc_generic_transpose(const bf16* in, bf16* out, int rows, int cols, cudaStream_t st);
+// out[c][r] = in[r][c]; pair_dh > 0: within every head of pair_dh columns the even columns come first, then the odd ones
+cudaError_t lorc_generic_transpose(const bf16* in, bf16* out, int rows, int cols, int pair_dh, cudaStream_t st);
 cudaError_t lorc_generic_append(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv,
                                 const bf16* x, int T, cudaStream_t st, int* launches);
 // Uncompressed mode, 128-wide heads, bf16 path: streaming decode kernel on mma.sync (full_decode.cu).  Leaves the same

@@ -39,10 +39,11 @@ cudaError_t lorc_generic_build_rope_table(float2* table, int max_pos, int d_head
 }
 
 // ---------------------------------------------------------------------------
-// out[c][r] = in[r][c]
+// out[c'][r] = in[r][c]; c' = c, or (pair_dh > 0) the place of column c when every head of pair_dh columns lists its even
+// columns first, then its odd ones
 // ---------------------------------------------------------------------------
 __global__ void transpose_kernel(const bf16* __restrict__ in, bf16* __restrict__ out, int rows,
-                                 int cols) {
+                                 int cols, int pair_dh) {
     __shared__ bf16 tile[32][33];
     int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
@@ -52,13 +53,15 @@ __global__ void transpose_kernel(const bf16* __restrict__ in, bf16* __restrict__
     __syncthreads();
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
         int c = c0 + i, r = r0 + threadIdx.x;
-        if (r < rows && c < cols) out[(long long)c * rows + r] = tile[threadIdx.x][i];
+        const int w = pair_dh > 0 ? c % pair_dh : 0;
+        const int to = pair_dh > 0 ? c - w + (w >> 1) + (w & 1) * (pair_dh / 2) : c;
+        if (r < rows && c < cols) out[(long long)to * rows + r] = tile[threadIdx.x][i];
     }
 }
 
-cudaError_t lorc_generic_transpose(const bf16* in, bf16* out, int rows, int cols, cudaStream_t st) {
+cudaError_t lorc_generic_transpose(const bf16* in, bf16* out, int rows, int cols, int pair_dh, cudaStream_t st) {
     dim3 grid((cols + 31) / 32, (rows + 31) / 32), block(32, 8);
-    transpose_kernel<<<grid, block, 0, st>>>(in, out, rows, cols);
+    transpose_kernel<<<grid, block, 0, st>>>(in, out, rows, cols, pair_dh);
     return cudaGetLastError();
 }
 

@@ -219,8 +219,9 @@ int lorc_load_factors(lorc_ctx* ctx, int layer, int mode, int r_k, int r_v, cons
         e = cudaMemcpyAsync(L.B_k, B_k, (size_t)r_k * n * sizeof(bf16), cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(L.B_v, B_v, (size_t)r_v * n * sizeof(bf16), cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess) e = lorc_generic_transpose(L.B_k, L.B_kT, r_k, n, st);
-        if (e == cudaSuccess) e = lorc_generic_transpose(L.B_v, L.B_vT, r_v, n, st);
+        if (e == cudaSuccess)
+            e = lorc_generic_transpose(L.B_k, L.B_kT, r_k, n, ctx->pair_style == LORC_ROPE_INTERLEAVED ? ctx->desc.d_head : 0, st);
+        if (e == cudaSuccess) e = lorc_generic_transpose(L.B_v, L.B_vT, r_v, n, 0, st);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
@@ -306,8 +307,12 @@ static int decode_attn_impl(lorc_ctx* ctx, int layer, const lorc_cache* cache, c
     int launches = 0;
     cudaError_t e;
 
-    if (!(ctx->desc.flags & LORC_FLAG_DEBUG_FP32) && lorc_tc_decode_supported(ctx, *L, cv)) {
-        size_t tc = lorc_tc_workspace_bytes(ctx, cv.batch, cv.max_seq_len);
+    const size_t tc = lorc_tc_workspace_bytes(ctx, cv.batch, cv.max_seq_len);
+    bool tensor = !(ctx->desc.flags & LORC_FLAG_DEBUG_FP32) && lorc_tc_decode_supported(ctx, *L, cv);
+    // interleaved pairs: the plain kernels serve what the tensor-core path cannot take (they need less scratch and no
+    // tables of their own).  With 32 heads, b 4, 2049 tokens, r 512 a step takes 37 us here and 3461 us there.
+    if (tensor && lorc_tc_split(ctx)) tensor = tc <= ctx->ws_bytes && lorc_tc_tables_ready(ctx, cv, st);
+    if (tensor) {
         if (tc > ctx->ws_bytes) return fail(ctx, LORC_ERR_WORKSPACE, "decode_attn: workspace too small");
         e = lorc_tc_decode(ctx, layer, *L, cv, (const bf16*)q, (bf16*)out, n_splits, ctx->ws,
                            ctx->ws_bytes, st, &launches, latent_out, pos0, q_pos, ml_out);
@@ -368,7 +373,7 @@ size_t lorc_prefill_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_
     if (!ctx || batch <= 0 || max_seq_len <= 0 || T <= 0) return 0;
     int S = generic_default_splits(max_seq_len);
     size_t gen = ws_layout(ctx, batch * T, S, ctx->n).total;
-    size_t tc = lorc_tc_workspace_bytes(ctx, batch, max_seq_len) ? lorc_tc_prefill_scratch_bytes(ctx, batch, max_seq_len, T) : 0;
+    size_t tc = lorc_tc_prefill_shape_ok(ctx) ? lorc_tc_prefill_scratch_bytes(ctx, batch, max_seq_len, T) : 0;
     return (gen > tc ? gen : tc) + 256;
 }
 

@@ -159,7 +159,7 @@ lorc_score_absorbed_kernel(const __grid_constant__ CUtensorMap mapCK, const __gr
     constexpr int A_STAGES = S::STAGES, NQ = S::NQ;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int nkc = (p.r_k + KC - 1) / KC;
-    const int img_bytes = lorc_tc_image_bytes(HQ);
+    const int img_bytes = lorc_tc_image_bytes(HQ, false);
     constexpr int EPI_WARPS = 4;                         // every lane quarter of the accumulator holds rows in use
 
     if (tid == 0) {
@@ -405,7 +405,7 @@ cudaError_t lorc_tc_score_absorbed_launch(lorc_ctx* ctx, const LorcLayer& L, con
                                           int n_zero, cudaStream_t st, int* launches) {
     const lorc_model_desc& d = ctx->desc;
     const int r_ld = (L.r_k + KC - 1) / KC * KC;
-    const size_t img_bytes = (size_t)lorc_tc_image_bytes(d.n_q_heads);
+    const size_t img_bytes = (size_t)lorc_tc_image_bytes(d.n_q_heads, false);
     for (int s0 = 0; s0 < cv.batch; s0 += LORC_SCORE_MAX_BATCH) {
         const int nb = cv.batch - s0 < LORC_SCORE_MAX_BATCH ? cv.batch - s0 : LORC_SCORE_MAX_BATCH;
         const int parts = d.n_q_heads == 64 ? 2 : 1;

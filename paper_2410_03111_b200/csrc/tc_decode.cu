@@ -64,8 +64,23 @@ void lorc_tc_invalidate_layer(lorc_ctx* ctx, int layer) {
 
 static bool tc_shape_ok(const lorc_ctx* ctx) {
     const lorc_model_desc& d = ctx->desc;
-    return d.d_head == 128 && (d.rope_style == LORC_ROPE_HALF_SPLIT || d.rope_style == LORC_ROPE_NONE) && (d.n_kv_heads % 2) == 0 &&
+    return d.d_head == 128 && (d.n_kv_heads % 2) == 0 &&
            (ctx->group == 4 || ctx->group == 8) && (d.n_q_heads == 32 || d.n_q_heads == 64);
+}
+
+bool lorc_tc_prefill_shape_ok(const lorc_ctx* ctx) {
+    return tc_shape_ok(ctx) && ctx->desc.rope_style != LORC_ROPE_INTERLEAVED;
+}
+
+bool lorc_tc_tables_ready(const lorc_ctx* ctx, const CacheView& cv, cudaStream_t st) {
+    const LorcTcState* T = ctx->tc;
+    if (T && T->attrs_set && T->rope_tile && (size_t)cv.batch * ctx->desc.n_q_heads <= T->rowmax_cap) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cap == cudaStreamCaptureStatusNone;
 }
 
 bool lorc_tc_decode_supported(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv) {
@@ -80,7 +95,7 @@ bool lorc_tc_decode_supported(const lorc_ctx* ctx, const LorcLayer& L, const Cac
 
 static size_t tc_image_area_bytes(const lorc_ctx* ctx, int batch, int max_seq_len) {
     const size_t tiles = (size_t)((max_seq_len + TILE - 1) / TILE);
-    return lorc_align_up((size_t)batch * tiles * lorc_tc_image_bytes(ctx->desc.n_q_heads), 256);
+    return lorc_align_up((size_t)batch * tiles * lorc_tc_image_bytes(ctx->desc.n_q_heads, lorc_tc_split(ctx)), 256);
 }
 
 // the absorbed query of layers without rotation sits between the images and the PV scratch
@@ -214,7 +229,7 @@ cudaError_t lorc_tc_decode(lorc_ctx* ctx, int layer, const LorcLayer& L, const C
 }
 
 bool lorc_tc_prefill_supported(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv) {
-    return lorc_tc_decode_supported(ctx, L, cv);
+    return lorc_tc_prefill_shape_ok(ctx) && lorc_tc_decode_supported(ctx, L, cv);
 }
 
 cudaError_t lorc_tc_prefill(lorc_ctx* ctx, int layer, const LorcLayer& L, const CacheView& cv, const bf16* q, bf16* out,

@@ -26,9 +26,20 @@ bool lorc_tc_append_gemm_supported(const lorc_ctx* ctx, const LorcLayer& L, cons
 cudaError_t lorc_tc_append_gemm(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* x, int T,
                                 cudaStream_t st, int* launches);
 
+// Contexts with interleaved rotary pairs keep fp32-level precision on the tensor-core decode path: softmax numerators and
+// the normalised latent output are carried as two bf16 parts (value rounded, remainder rounded: together 16 significant
+// bits).  The plain kernels, which serve what does not fit this path, keep both in fp32; against fp64 the results are off
+// by 1.6e-3 either way (the bf16 output), with one bf16 part by 2.9e-3.
+inline bool lorc_tc_split(const lorc_ctx* ctx) { return ctx->desc.rope_style == LORC_ROPE_INTERLEAVED; }
+// Whether a call may take that path now: its tables exist, or may be allocated (the stream is not being captured).
+bool lorc_tc_tables_ready(const lorc_ctx* ctx, const CacheView& cv, cudaStream_t st);
+
 // Bytes of one probability tile image (128 tokens of one sequence, all query heads): the bf16 numerators as the PV
-// kernel's swizzled MMA operand, then float m[4][H_q] and float l[4][H_q] (reference and sum per 32-token quarter).
-__host__ __device__ inline int lorc_tc_image_bytes(int n_q_heads) { return 2 * n_q_heads * 64 * 2 + 8 * n_q_heads * 4; }
+// kernel's swizzled MMA operand (split: the rows of the remainders behind those of the rounded values, in every chunk),
+// then float m[4][H_q] and float l[4][H_q] (reference and sum per 32-token quarter).
+__host__ __device__ inline int lorc_tc_image_bytes(int n_q_heads, bool split) {
+    return 2 * n_q_heads * (split ? 2 : 1) * 64 * 2 + 8 * n_q_heads * 4;
+}
 
 // Score kernel (tc_score.cu): key reconstruction, rotation, q.k and the softmax numerators; writes one tile image per
 // 128 tokens into pimg [b, tiles, image] and raises the row maxima (integers, as order-preserving keys).  rope_tile:
@@ -72,6 +83,7 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
 // the latent cache, causal inside the chunk.  Keys and values are reconstructed once into `scratch`
 // (lorc_tc_prefill_scratch_bytes), then a flash-attention kernel runs over them.  mapBKT / mapBVT128: B_K^T, B_V^T
 // [n, r] in swizzled boxes of 64 latent columns x 128 rows.
+bool lorc_tc_prefill_shape_ok(const lorc_ctx* ctx);
 bool lorc_tc_prefill_supported(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv);
 size_t lorc_tc_prefill_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq_len, int T);
 cudaError_t lorc_tc_prefill_set_attrs();

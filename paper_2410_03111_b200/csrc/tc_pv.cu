@@ -25,22 +25,25 @@ namespace {
 constexpr int TILE = 128;
 constexpr int KC = 64;
 // one CTA per SM; 5 stages x 40 KiB with 32 query heads (200 KiB in flight), 4 x 48 KiB with 64
-template <int HQ>
-struct PvStages { static constexpr int value = HQ <= 32 ? 5 : 4; };
+// (NR rows of numerators per tile: the heads, or twice as many where they are carried in two parts)
+template <int NR>
+struct PvStages { static constexpr int value = NR <= 32 ? 5 : NR <= 64 ? 4 : 3; };
 constexpr int P_THREADS = 192;       // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
 
 // ------------------------------------------------------------------------------------------------
 // PV kernel
 // ------------------------------------------------------------------------------------------------
 // Tile image written by the score kernel, fetched with one bulk copy per tile:
-//   [2 chunks of 64 tokens][HQ rows of 128 bytes]   p = bf16(2^(s - m)), 128-byte swizzle (the MMA's B operand)
+//   [2 chunks of 64 tokens][NR rows of 128 bytes]   p = bf16(2^(s - m)), 128-byte swizzle (the MMA's A operand); SPLIT:
+//                                                   rows HQ .. 2 HQ - 1 hold the remainders bf16(2^(s - m) - p)
 //   float m[4][HQ]   integer reference of every 32-token quarter and head (log2 units; -inf: no token)
 //   float l[4][HQ]   sum of the quarter's rounded p
-template <int HQ>
+template <int HQ, bool SPLIT>
 struct Pv2Smem {
-    static constexpr int P_STAGES = PvStages<HQ>::value;
-    static constexpr int IMG = 2 * HQ * KC * 2 + 8 * HQ * 4;
-    // tile images (IMG is a multiple of 1 KiB).  They come first: with 32 heads the MMA's 64-row A operand runs
+    static constexpr int NR = SPLIT ? 2 * HQ : HQ;
+    static constexpr int P_STAGES = PvStages<NR>::value;
+    static constexpr int IMG = 2 * NR * KC * 2 + 8 * HQ * 4;
+    // tile images (IMG is a multiple of 1 KiB).  They come first: with 32 rows the MMA's 64-row A operand runs
     // 4 KiB past a chunk of the image, into the next image or into V, never past the allocation
     uint8_t P[P_STAGES][IMG];
     bf16 V[P_STAGES][2][TILE * KC];       // C_V block: two 64-column halves of [128 tokens][64]; 32 KiB / stage
@@ -56,7 +59,7 @@ struct Pv2Params {
     const uint8_t* pimg;           // [b, tiles, image]
     float* o_part;                 // [b, n_blk, n_csplit, H_q * 128 + H_q]   un-normalised latent output and denominator of every context share
     unsigned* rowmax;              // [b, H_q]   row maxima of the softmax (order-preserving keys of integers)
-    bf16* o_norm;                  // [b, H_q, r_pad]      normalised latent output
+    bf16* o_norm;                  // [b, H_q, r_pad]      normalised latent output; SPLIT: [b, H_q, 2, r_pad], remainders second
     int* done;                     // [b, n_blk]           context shares of a column block that have finished (zero on entry)
     float* ml_out;                 // NULL, or [b, H_q, 2]: reference M (log2 units) and denominator sum_n 2^(s_n - M)
     const int32_t* seq_lens;
@@ -69,12 +72,12 @@ struct Pv2Params {
 // Biased exponent of 2^d for an integer-valued d <= 0 (0, i.e. the number zero, below 2^-126 and for d = -inf).
 __device__ __forceinline__ uint32_t pow2_exponent(float d) { return d >= -126.f ? (uint32_t)(127 + (int)d) : 0u; }
 
-template <int HQ>
+template <int HQ, bool SPLIT>
 __global__ void __launch_bounds__(P_THREADS, 1)
 lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
     extern __shared__ uint8_t raw[];
-    typedef Pv2Smem<HQ> S;
-    constexpr int P_STAGES = PvStages<HQ>::value;
+    typedef Pv2Smem<HQ, SPLIT> S;
+    constexpr int P_STAGES = S::P_STAGES, NR = S::NR;
     S& sm = *reinterpret_cast<S*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     constexpr uint32_t TM_COLS = 128;
     constexpr uint32_t P_BYTES = S::IMG;
@@ -187,7 +190,7 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
         if (ntiles > 0) {
             // O_lat[64 rows (heads; 32 of them unused with 32 heads), 128 rho] += P[heads, 16 tokens] . C_V[16 tokens, 128 rho]:
             // the heads are the M side (a small M costs few cycles per MMA), the latent columns the N side
-            const uint32_t idesc = make_idesc_bf16(64, 128, 0, 1);
+            const uint32_t idesc = make_idesc_bf16(NR <= 64 ? 64 : 128, 128, 0, 1);
             for (int i = 0; i < ntiles && ok; ++i) {
                 const int st = i % P_STAGES;
                 if (!mbar_wait(&sm.fixed[st], (i / P_STAGES) & 1)) { ok = false; break; }
@@ -197,8 +200,8 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
-                        // A: P [heads][128 tokens] (K-major), 64-token chunks of HQ*128 bytes
-                        const uint64_t ad = make_smem_desc_sw128(p0 + (k >> 2) * (HQ * KC * 2) + (k & 3) * 32, 0, 1024);
+                        // A: P [rows][128 tokens] (K-major), 64-token chunks of NR*128 bytes
+                        const uint64_t ad = make_smem_desc_sw128(p0 + (k >> 2) * (NR * KC * 2) + (k & 3) * 32, 0, 1024);
                         // B: C_V block (MN-major: a token's 64 latent columns are contiguous): 16 token rows per step,
                         // the two 64-column halves 16 KiB apart
                         const uint64_t bd = make_smem_desc_sw128(v0 + k * 2048, TILE * KC * 2, 1024);
@@ -228,12 +231,15 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
         asm volatile("bar.sync 2, 128;" ::: "memory");
         // While the tiles stream: every tile image holds p against the integer reference m of its own 32-token
         // quarter; multiplying by 2^(m - M), M the reference of the whole sequence, is exact in bf16 (a change of the
-        // exponent) unless the product is too small to matter.  Thread t owns 2 HQ bytes of the image: with 32 heads
-        // half a row (one head, one quarter), with 64 heads a whole row (one head, both quarters of a chunk).
-        const int frow = (t * 2 * HQ) >> 7;               // row of the image: chunk * HQ + head
-        const int fchunk = frow / HQ, fh = frow % HQ;
-        const int fpiece0 = ((t * 2 * HQ) & 127) >> 4;    // first 16-byte piece (physical) of this thread
-        const int frot = HQ == 32 ? (t >> 1) & 3 : t & 7;  // rotation of the order in which it takes its pieces
+        // exponent) unless the product is too small to matter.  Thread t owns 2 NR bytes of the image: with 32 rows per
+        // chunk half a row (one head, one quarter), with 64 a whole row (one head, both quarters of a chunk), with 128
+        // the same row of both chunks.
+        constexpr int RPT = NR == 128 ? 2 : 1;            // rows per thread
+        constexpr int NP = (NR == 32 ? 64 : 128) / 16;    // 16-byte pieces of a row per thread
+        const int frow0 = NR == 128 ? t : (t * 2 * NR) >> 7;   // (first) row of the image: chunk * NR + row in chunk
+        const int fh = (frow0 % NR) % HQ;
+        const int fpiece0 = NR == 32 ? ((t * 64) & 127) >> 4 : 0;   // first 16-byte piece (physical) of this thread
+        const int frot = NR == 32 ? (t >> 1) & 3 : t & 7;  // rotation of the order in which it takes its pieces
         const float m_mine = sm.m_row[fh];
         const int lh = t % HQ, lpart = t / HQ;            // denominator: head, and which quarters of a tile
         const float m_l = sm.m_row[lh];
@@ -241,37 +247,40 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
         for (int i = 0; i < ntiles && ok; ++i) {
             const int st = i % P_STAGES;
             if (!mbar_wait(&sm.pfull[st], (i / P_STAGES) & 1)) { ok = false; break; }
-            const float* mt = reinterpret_cast<const float*>(sm.P[st] + 2 * HQ * KC * 2);
+            const float* mt = reinterpret_cast<const float*>(sm.P[st] + 2 * NR * KC * 2);
             const float* lt = mt + 4 * HQ;
 #pragma unroll
             for (int qq = 0; qq < 4 / PARTS; ++qq) {
                 const int qrt = lpart * (4 / PARTS) + qq;
                 lacc += lt[qrt * HQ + lh] * __uint_as_float(pow2_exponent(mt[qrt * HQ + lh] - m_l) << 23);
             }
-            // 2^(m - M) of the quarter(s) this thread's pieces belong to, as a bf16 pair (built from the exponent: m and M
-            // are integers).  A piece's quarter is bit 2 of its logical index, physical index xor (head & 7).
-            uint32_t scb[2];
 #pragma unroll
-            for (int hq = 0; hq < 2; ++hq) {
-                const uint32_t e = pow2_exponent(mt[(fchunk * 2 + hq) * HQ + fh] - m_mine) << 7;
-                scb[hq] = e | (e << 16);
-            }
-            uint4* prow = reinterpret_cast<uint4*>(sm.P[st] + frow * 128);
-            constexpr int NP = (2 * HQ) / 16;                 // 16-byte pieces per thread: 4 or 8
-            uint4 v[NP];
-            // (the pieces are taken in an order rotated by the thread index: the threads of a quarter warp, whose
-            // pieces lie 64 or 128 bytes apart, then touch different banks)
+            for (int rr = 0; rr < RPT; ++rr) {
+                const int frow = frow0 + rr * 128, fchunk = frow / NR;
+                // 2^(m - M) of the quarter(s) this thread's pieces belong to, as a bf16 pair (built from the exponent: m and M
+                // are integers).  A piece's quarter is bit 2 of its logical index, physical index xor (row & 7).
+                uint32_t scb[2];
 #pragma unroll
-            for (int j = 0; j < NP; ++j) v[j] = prow[fpiece0 + ((j + frot) & (NP - 1))];
+                for (int hq = 0; hq < 2; ++hq) {
+                    const uint32_t e = pow2_exponent(mt[(fchunk * 2 + hq) * HQ + fh] - m_mine) << 7;
+                    scb[hq] = e | (e << 16);
+                }
+                uint4* prow = reinterpret_cast<uint4*>(sm.P[st] + frow * 128);
+                uint4 v[NP];
+                // (the pieces are taken in an order rotated by the thread index: the threads of a quarter warp, whose
+                // pieces lie 64 or 128 bytes apart, then touch different banks)
 #pragma unroll
-            for (int j = 0; j < NP; ++j) {
-                const int pp = fpiece0 + ((j + frot) & (NP - 1));
-                const uint32_t sb = scb[((pp ^ (fh & 7)) >> 2) & 1];
-                const __nv_bfloat162 sc = *reinterpret_cast<const __nv_bfloat162*>(&sb);
-                __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&v[j]);
+                for (int j = 0; j < NP; ++j) v[j] = prow[fpiece0 + ((j + frot) & (NP - 1))];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) e[k] = __hmul2(e[k], sc);
-                prow[pp] = v[j];
+                for (int j = 0; j < NP; ++j) {
+                    const int pp = fpiece0 + ((j + frot) & (NP - 1));
+                    const uint32_t sb = scb[((pp ^ (fh & 7)) >> 2) & 1];
+                    const __nv_bfloat162 sc = *reinterpret_cast<const __nv_bfloat162*>(&sb);
+                    __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&v[j]);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) e[k] = __hmul2(e[k], sc);
+                    prow[pp] = v[j];
+                }
             }
             fence_proxy_async_smem();      // the MMA reads the image through the asynchronous proxy
             __syncwarp();
@@ -289,9 +298,59 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
         if (ntiles > 0 && ok) {
             if (!mbar_wait(&sm.o_full, 0)) ok = false;
         }
-        // The accumulator holds head 16 q + i (i < 16) in lane i of lane quarter q, 128 latent columns wide.
-        const int hrow = quarter * 16 + lane;             // the head this thread reads (lanes 16..31 of a warp: none)
-        const bool has_row = lane < 16 && hrow < HQ;
+        // A 64-row accumulator holds row 16 q + i (i < 16) in lane i of lane quarter q, a 128-row one row 32 q + i; it is
+        // 128 latent columns wide.  The rows are the heads; SPLIT: quarters 2 and 3 hold the heads' remainders.
+        constexpr int QROWS = NR <= 64 ? 16 : 32;
+        const int hrow = (SPLIT ? quarter & 1 : quarter) * QROWS + lane;     // the head this thread reads
+        const bool has_row = lane < QROWS && hrow < HQ && (!SPLIT || quarter < 2);
+        constexpr int XLD = 132;                          // floats per row of the exchange (16-byte rows, spread over the banks)
+        float* xch = reinterpret_cast<float*>(&sm.V[0][0][0]);
+        if (SPLIT) {
+            // the products of the remainders go to the threads that hold the heads' other part (the C_V stages are free:
+            // every MMA that reads them has completed)
+            if (quarter >= 2) {
+#pragma unroll
+                for (int c0 = 0; c0 < 128; c0 += 32) {
+                    uint32_t r[32];
+                    if (ntiles > 0 && ok) {
+                        tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + c0, r);
+                        tmem_wait_ld();
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) r[i] = 0u;
+                    }
+                    if (lane < QROWS) {
+#pragma unroll
+                        for (int q4 = 0; q4 < 8; ++q4)
+                            *reinterpret_cast<uint4*>(xch + hrow * XLD + c0 + q4 * 4) =
+                                make_uint4(r[q4 * 4], r[q4 * 4 + 1], r[q4 * 4 + 2], r[q4 * 4 + 3]);
+                    }
+                }
+            }
+            __syncwarp();
+            asm volatile("bar.sync 2, 128;" ::: "memory");
+        }
+        // this thread's 32 columns from c0: the accumulator, with the remainders' part added
+        auto take = [&](int c0, uint32_t (&r)[32]) {
+            if (ntiles > 0 && ok) {
+                tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + c0, r);
+                tmem_wait_ld();
+            } else {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) r[i] = 0u;
+            }
+            if (SPLIT && has_row) {
+#pragma unroll
+                for (int i4 = 0; i4 < 8; ++i4) {
+                    const float4 x = *reinterpret_cast<const float4*>(xch + hrow * XLD + c0 + i4 * 4);
+                    r[i4 * 4] = __float_as_uint(__uint_as_float(r[i4 * 4]) + x.x);
+                    r[i4 * 4 + 1] = __float_as_uint(__uint_as_float(r[i4 * 4 + 1]) + x.y);
+                    r[i4 * 4 + 2] = __float_as_uint(__uint_as_float(r[i4 * 4 + 2]) + x.z);
+                    r[i4 * 4 + 3] = __float_as_uint(__uint_as_float(r[i4 * 4 + 3]) + x.w);
+                }
+            }
+        };
+        const int r_ld = SPLIT ? 2 * r_pad : r_pad;       // row of o_norm
         constexpr int SHARE_FLOATS = HQ * 128 + HQ;
         if (p.n_csplit == 1) {
             if (t < HQ) {
@@ -305,28 +364,28 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
             __syncwarp();
             asm volatile("bar.sync 2, 128;" ::: "memory");
             const float li = has_row ? sm.l_inv[hrow] : 0.f;
-            bf16* on = p.o_norm + ((long long)s * p.H_q + (has_row ? hrow : 0)) * r_pad + rho0;
+            bf16* on = p.o_norm + ((long long)s * p.H_q + (has_row ? hrow : 0)) * r_ld + rho0;
 #pragma unroll
             for (int c0 = 0; c0 < 128; c0 += 32) {
                 uint32_t r[32];
-                if (ntiles > 0 && ok) {
-                    tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + c0, r);
-                    tmem_wait_ld();
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) r[i] = 0u;
-                }
+                take(c0, r);
                 if (has_row) {
 #pragma unroll
                     for (int q4 = 0; q4 < 4; ++q4) {
-                        uint32_t w[4];
+                        uint32_t w[4], wl[4];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(r[q4 * 8 + 2 * e]) * li,
-                                                                            __uint_as_float(r[q4 * 8 + 2 * e + 1]) * li);
+                            const float x0 = __uint_as_float(r[q4 * 8 + 2 * e]) * li, x1 = __uint_as_float(r[q4 * 8 + 2 * e + 1]) * li;
+                            const __nv_bfloat162 b2 = __floats2bfloat162_rn(x0, x1);
                             w[e] = *reinterpret_cast<const uint32_t*>(&b2);
+                            if (SPLIT) {
+                                const float2 h2 = __bfloat1622float2(b2);
+                                const __nv_bfloat162 l2 = __floats2bfloat162_rn(x0 - h2.x, x1 - h2.y);
+                                wl[e] = *reinterpret_cast<const uint32_t*>(&l2);
+                            }
                         }
                         *reinterpret_cast<uint4*>(on + c0 + q4 * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+                        if (SPLIT) *reinterpret_cast<uint4*>(on + r_pad + c0 + q4 * 8) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
                     }
                 }
             }
@@ -338,13 +397,7 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
 #pragma unroll
             for (int c0 = 0; c0 < 128; c0 += 32) {
                 uint32_t r[32];
-                if (ntiles > 0 && ok) {
-                    tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + c0, r);
-                    tmem_wait_ld();
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) r[i] = 0u;
-                }
+                take(c0, r);
                 if (has_row) {
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4)
@@ -401,9 +454,14 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                 }
                 __syncwarp();
                 asm volatile("bar.sync 2, 128;" ::: "memory");
-                bf16* on = p.o_norm + (long long)s * p.H_q * r_pad + rho0 + t;
+                bf16* on = p.o_norm + (long long)s * p.H_q * r_ld + rho0 + t;
 #pragma unroll
-                for (int h = 0; h < HQ; ++h) on[(long long)h * r_pad] = __float2bfloat16_rn(acc[h] * sm.l_inv[h]);
+                for (int h = 0; h < HQ; ++h) {
+                    const float x = acc[h] * sm.l_inv[h];
+                    const bf16 hi = __float2bfloat16_rn(x);
+                    on[(long long)h * r_ld] = hi;
+                    if (SPLIT) on[(long long)h * r_ld + r_pad] = __float2bfloat16_rn(x - __bfloat162float(hi));
+                }
             }
         }
         if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
@@ -439,6 +497,7 @@ struct UpParams {
     unsigned* rowmax;              // [b, H_q]   left empty for the next call's score kernel
     int* status;
     int batch, H_q, G, r_v;
+    int parts, r_pad;              // bf16 parts of the latent rows (the second one r_pad columns after the first)
 };
 
 __global__ void __launch_bounds__(U_THREADS, 1)
@@ -448,7 +507,7 @@ lorc_upproj_kernel(const __grid_constant__ CUtensorMap mapON, const __grid_const
     UpSmem& sm = *reinterpret_cast<UpSmem*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int g = blockIdx.x, chunk = blockIdx.y, cq = blockIdx.z;     // KV head, block of 64 rows, column quarter
-    const int nkc = (p.r_v + KC - 1) / KC;
+    const int nslice = (p.r_v + KC - 1) / KC, nkc = nslice * p.parts;    // slices of the rank, of the contraction
     const int seqs_per_cta = U_ROWS / p.G;
     constexpr uint32_t STAGE_BYTES = (U_ROWS + U_NCOL) * KC * 2;
     if (tid == 0) {
@@ -479,7 +538,7 @@ lorc_upproj_kernel(const __grid_constant__ CUtensorMap mapON, const __grid_const
         if (elect_one()) {
             for (int kc = 0; kc < npre; ++kc) {
                 mbar_arrive_expect_tx(&sm.full[kc], STAGE_BYTES);
-                tma_load_2d(sm.B[kc], &mapBVT, &sm.full[kc], kc * KC, g * 128 + cq * U_NCOL);
+                tma_load_2d(sm.B[kc], &mapBVT, &sm.full[kc], (kc % nslice) * KC, g * 128 + cq * U_NCOL);
             }
         }
         __syncwarp();
@@ -491,10 +550,11 @@ lorc_upproj_kernel(const __grid_constant__ CUtensorMap mapON, const __grid_const
             if (elect_one()) {
                 if (kc >= npre) {
                     mbar_arrive_expect_tx(&sm.full[st], STAGE_BYTES);
-                    tma_load_2d(sm.B[st], &mapBVT, &sm.full[st], kc * KC, g * 128 + cq * U_NCOL);
+                    tma_load_2d(sm.B[st], &mapBVT, &sm.full[st], (kc % nslice) * KC, g * 128 + cq * U_NCOL);
                 }
                 // rows (s, i): box of G heads x 128/G sequences (sequences past the batch read as zero)
-                tma_load_3d(sm.A[st], &mapON, &sm.full[st], kc * KC, g * p.G, chunk * seqs_per_cta);
+                tma_load_3d(sm.A[st], &mapON, &sm.full[st], (kc / nslice) * p.r_pad + (kc % nslice) * KC, g * p.G,
+                            chunk * seqs_per_cta);
             }
             __syncwarp();
         }
@@ -561,14 +621,14 @@ lorc_upproj_kernel(const __grid_constant__ CUtensorMap mapON, const __grid_const
 // Result of lorc_decode_attn_latent_out: the normalised latent output without the padding columns, and the row maxima
 // left empty for the next call (what the up-projection kernel does otherwise).
 __global__ void latent_out_kernel(const bf16* __restrict__ o_norm, bf16* __restrict__ o_lat, unsigned* rowmax, int rows,
-                                  int r_v, int r_pad) {
+                                  int r_v, int r_ld) {
     grid_dep_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < rows) rowmax[i] = 0u;
     const int vec = r_v / 8;                              // r_v is a multiple of 8: 16-byte pieces
     if (i < (long long)rows * vec) {
         const long long row = i / vec, c = i % vec;
-        reinterpret_cast<uint4*>(o_lat + row * r_v)[c] = reinterpret_cast<const uint4*>(o_norm + row * r_pad)[c];
+        reinterpret_cast<uint4*>(o_lat + row * r_v)[c] = reinterpret_cast<const uint4*>(o_norm + row * r_ld)[c];
     }
 }
 
@@ -593,10 +653,11 @@ struct PvScratch {
 
 PvScratch pv_scratch_layout(const lorc_ctx* ctx, int batch, int n_csplit, size_t r_pad) {
     PvScratch z;
+    const size_t parts = lorc_tc_split(ctx) ? 2 : 1;
     const size_t hq = (size_t)ctx->desc.n_q_heads;
     // [b][n_blk][n_csplit][H_q * 128 + H_q]
     z.part_bytes = n_csplit > 1 ? lorc_align_up((size_t)batch * (r_pad / 128) * n_csplit * (hq * 128 + hq) * sizeof(float), 256) : 256;
-    z.on_bytes = lorc_align_up((size_t)batch * hq * r_pad * sizeof(bf16), 256);
+    z.on_bytes = lorc_align_up((size_t)batch * hq * parts * r_pad * sizeof(bf16), 256);
     z.done_bytes = lorc_align_up((size_t)batch * (r_pad / 128) * sizeof(int), 256);
     return z;
 }
@@ -628,14 +689,14 @@ size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq_len)
 }
 
 cudaError_t lorc_tc_pv_set_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(lorc_pv2_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(Pv2Smem<32>) + 1024);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lorc_pv2_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(Pv2Smem<64>) + 1024);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lorc_upproj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(UpSmem) + 1024);
+    auto attr = [](const void* kernel, size_t bytes) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes + 1024);
+    };
+    cudaError_t e = attr((const void*)lorc_pv2_kernel<32, false>, sizeof(Pv2Smem<32, false>));
+    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>));
+    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>));
+    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>));
+    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel, sizeof(UpSmem));
     return e;
 }
 
@@ -664,6 +725,8 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
     const lorc_model_desc& d = ctx->desc;
     const int n_blk = plan.n_blk, n_csplit = plan.n_csplit;
     const int r_pad = n_blk * 128;
+    const bool split = lorc_tc_split(ctx);
+    const int r_ld = split ? 2 * r_pad : r_pad;        // row of o_norm
     float* o_part = (float*)scratch;
     bf16* o_norm = (bf16*)((char*)scratch + plan.off_on);
     int* done = (int*)((char*)scratch + plan.off_done);
@@ -677,10 +740,15 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
         p.n_blk = n_blk; p.n_csplit = n_csplit; p.max_pos = d.max_pos;
         p.page_size = cv.page_size; p.max_pages_per_seq = cv.max_pages_per_seq; p.n_pages = cv.n_pages;
         dim3 grid(n_blk, n_csplit, cv.batch);
+        auto launch = [&](auto kernel, size_t bytes) {
+            return lorc_launch_dependent(kernel, grid, dim3(P_THREADS), bytes + 1024, st, mapCV, p);
+        };
         if (d.n_q_heads == 32)
-            e = lorc_launch_dependent(lorc_pv2_kernel<32>, grid, dim3(P_THREADS), sizeof(Pv2Smem<32>) + 1024, st, mapCV, p);
+            e = split ? launch(lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>))
+                      : launch(lorc_pv2_kernel<32, false>, sizeof(Pv2Smem<32, false>));
         else
-            e = lorc_launch_dependent(lorc_pv2_kernel<64>, grid, dim3(P_THREADS), sizeof(Pv2Smem<64>) + 1024, st, mapCV, p);
+            e = split ? launch(lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>))
+                      : launch(lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>));
         *launches += 1;
         if (e != cudaSuccess) return e;
     }
@@ -689,21 +757,22 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
         const int rows = cv.batch * d.n_q_heads;
         const long long work = (long long)rows * (L.r_v / 8);
         e = lorc_launch_dependent(latent_out_kernel, dim3((unsigned)((work + 255) / 256)), dim3(256), 0, st,
-                                  (const bf16*)o_norm, out, rowmax, rows, L.r_v, r_pad);
+                                  (const bf16*)o_norm, out, rowmax, rows, L.r_v, r_ld);
         *launches += 1;
         return e;
     }
-    // o_norm [b, H_q, r_pad] as (rho, head, sequence) with boxes of 64 rho x G heads x 64/G sequences
+    // o_norm [b, H_q, r_ld] as (rho, head, sequence) with boxes of 64 rho x G heads x 64/G sequences
     CUtensorMap mapON;
     {
-        uint64_t dims[3] = {(uint64_t)r_pad, (uint64_t)d.n_q_heads, (uint64_t)cv.batch};
-        uint64_t str[2] = {(uint64_t)r_pad * 2, (uint64_t)d.n_q_heads * r_pad * 2};
+        uint64_t dims[3] = {(uint64_t)r_ld, (uint64_t)d.n_q_heads, (uint64_t)cv.batch};
+        uint64_t str[2] = {(uint64_t)r_ld * 2, (uint64_t)d.n_q_heads * r_ld * 2};
         uint32_t box[3] = {KC, (uint32_t)ctx->group, (uint32_t)(U_ROWS / ctx->group)};
         if (!lorc_make_tmap_bf16(&mapON, o_norm, 3, dims, str, box)) return cudaErrorInvalidValue;
     }
     UpParams u;
     u.out = out; u.rowmax = rowmax; u.status = ctx->status_dev;
     u.batch = cv.batch; u.H_q = d.n_q_heads; u.G = ctx->group; u.r_v = L.r_v;
+    u.parts = split ? 2 : 1; u.r_pad = r_pad;
     dim3 ugrid(d.n_kv_heads, (cv.batch * ctx->group + U_ROWS - 1) / U_ROWS, 128 / U_NCOL);
     e = lorc_launch_dependent(lorc_upproj_kernel, ugrid, dim3(U_THREADS), sizeof(UpSmem) + 1024, st, mapON, mapBVT, u);
     *launches += 1;

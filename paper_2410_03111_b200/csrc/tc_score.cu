@@ -119,7 +119,9 @@ __device__ __forceinline__ int qrot_index(int j, int half, int g) {
     return ((((kk * 2 + half) * (G / 2) + (g >> 1)) * 4 + c) << 2) + ((g & 1) << 1) + e;
 }
 
-template <int G>
+// SPLIT (interleaved rotary pairs): B_K^T lists the first members of a head's pairs, then the second ones, so that the
+// accumulator has the half-split layout; queries are read in pairs; numerators are written as two bf16 parts.
+template <int G, bool SPLIT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Q_THREADS, 1)
 lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_constant__ CUtensorMap mapBKT,
                   const ScoreParams p) {
@@ -129,7 +131,7 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
     const int rank = (int)cluster_ctarank();           // 0 = leader (issues the MMAs, owns the full / acc_empty barriers)
     const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const int nkc = (p.r_k + KC - 1) / KC;
-    const int img_bytes = lorc_tc_image_bytes(p.H_q);
+    const int img_bytes = lorc_tc_image_bytes(p.H_q, SPLIT);
 
     if (tid == 0) {
         for (int i = 0; i < Q_STAGES; ++i) {
@@ -307,8 +309,14 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
             for (int i = 0; i < 2 * G; ++i) {
                 const int h = un.hp * 2 * G + i;
                 const uint32_t* qp = reinterpret_cast<const uint32_t*>(p.q + ((long long)un.s * p.H_q + h) * 128);
-                qa[i] = __ldg(qp + lane);
-                qb[i] = __ldg(qp + 32 + lane);
+                if (SPLIT) {
+                    const uint2 w = __ldg(reinterpret_cast<const uint2*>(qp) + lane);      // a0 b0 a1 b1
+                    qa[i] = __byte_perm(w.x, w.y, 0x5410);
+                    qb[i] = __byte_perm(w.x, w.y, 0x7632);
+                } else {
+                    qa[i] = __ldg(qp + lane);
+                    qb[i] = __ldg(qp + 32 + lane);
+                }
             }
             // the epilogue warps are done with the unit that used this buffer before
             if (!mbar_wait(&sm.q_empty[buf], ((uc >> 1) & 1) ^ 1)) { ok = false; break; }
@@ -439,8 +447,9 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
             if (!un.valid) continue;
             // softmax numerators of this warp's 32 tokens (a quarter of the tile) against their own integer reference
             uint8_t* img = p.pimg + ((long long)un.s * p.tiles + un.tile) * img_bytes;
-            uint8_t* chunk_img = img + (quarter >> 1) * (p.H_q * KC * 2);
-            float* m_out = reinterpret_cast<float*>(img + 2 * p.H_q * KC * 2) + quarter * p.H_q;
+            const int chunk_bytes = p.H_q * KC * 2 * (SPLIT ? 2 : 1);
+            uint8_t* chunk_img = img + (quarter >> 1) * chunk_bytes;
+            float* m_out = reinterpret_cast<float*>(img + 2 * chunk_bytes) + quarter * p.H_q;
             float* l_out = m_out + 4 * p.H_q;
             const int n_first = un.tile * TILE + quarter * 32 + r;
             const int tc0 = (quarter & 1) * 32 + r;
@@ -454,7 +463,7 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
                     if (n_first + 8 * m < un.len) mxv = fmaxf(mxv, tot[m][i]);
                 }
                 // a NaN among the scores means non-finite numbers in the cache, the factors or the query
-                if (ssum != ssum) lorc_set_status(p.status, LORC_ERR_ARG);
+                if (!SPLIT && ssum != ssum) lorc_set_status(p.status, LORC_ERR_ARG);
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) mxv = fmaxf(mxv, __shfl_xor_sync(0xffffffffu, mxv, o));
                 const float mref = ceilf(mxv);                 // -inf: no token of the sequence in this quarter
@@ -463,10 +472,17 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
                 for (int m = 0; m < 4; ++m) {
                     const bool valid = n_first + 8 * m < un.len;
                     // p = 2^(s - m), rounded to bf16 (the same rounded value enters the denominator)
-                    const bf16 pr = __float2bfloat16_rn(valid ? ex2_approx(tot[m][i] - mref) : 0.f);
+                    const float pf = valid ? ex2_approx(tot[m][i] - mref) : 0.f;
+                    const bf16 pr = __float2bfloat16_rn(pf);
                     lsum += __bfloat162float(pr);
                     const int tc = tc0 + 8 * m;
-                    *reinterpret_cast<bf16*>(chunk_img + h * 128 + ((((tc >> 3) ^ (h & 7)) << 4) | ((tc & 7) << 1))) = pr;
+                    bf16* at = reinterpret_cast<bf16*>(chunk_img + h * 128 + ((((tc >> 3) ^ (h & 7)) << 4) | ((tc & 7) << 1)));
+                    *at = pr;
+                    if (SPLIT) {
+                        const bf16 lo = __float2bfloat16_rn(pf - __bfloat162float(pr));
+                        lsum += __bfloat162float(lo);
+                        at[p.H_q * KC] = lo;                  // H_q rows further on (a multiple of 8: the same swizzle)
+                    }
                 }
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
@@ -510,11 +526,11 @@ __global__ void rope_tile_kernel(float2* out, double theta) {
 }  // namespace
 
 cudaError_t lorc_tc_score_set_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(lorc_score_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(ScoreSmem) + 1024);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lorc_score_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(ScoreSmem) + 1024);
+    const int bytes = (int)sizeof(ScoreSmem) + 1024;
+    cudaError_t e = cudaFuncSetAttribute(lorc_score_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(lorc_score_kernel<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(lorc_score_kernel<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(lorc_score_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     return e;
 }
 
@@ -530,7 +546,7 @@ cudaError_t lorc_tc_score_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheV
                                  const float4* rope_tile, int tiles, int* zero, int n_zero, const int32_t* pos0,
                                  const int32_t* q_pos, cudaStream_t st, int* launches) {
     const lorc_model_desc& d = ctx->desc;
-    const size_t img_bytes = (size_t)lorc_tc_image_bytes(d.n_q_heads);
+    const size_t img_bytes = (size_t)lorc_tc_image_bytes(d.n_q_heads, lorc_tc_split(ctx));
     for (int s0 = 0; s0 < cv.batch; s0 += LORC_SCORE_MAX_BATCH) {
         const int nb = cv.batch - s0 < LORC_SCORE_MAX_BATCH ? cv.batch - s0 : LORC_SCORE_MAX_BATCH;
         ScoreParams sp;
@@ -555,11 +571,10 @@ cudaError_t lorc_tc_score_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheV
         if (max_units < n_pairs) n_pairs = (int)max_units;
         if (n_pairs < 1) n_pairs = 1;
         const size_t smem = sizeof(ScoreSmem) + 1024;
-        cudaError_t e;
-        if (ctx->group == 4)
-            e = lorc_launch_dependent(lorc_score_kernel<4>, dim3(2 * n_pairs), dim3(Q_THREADS), smem, st, mapCK, mapBKT, sp);
-        else
-            e = lorc_launch_dependent(lorc_score_kernel<8>, dim3(2 * n_pairs), dim3(Q_THREADS), smem, st, mapCK, mapBKT, sp);
+        const bool split = lorc_tc_split(ctx);
+        auto kernel = ctx->group == 4 ? (split ? lorc_score_kernel<4, true> : lorc_score_kernel<4, false>)
+                                      : (split ? lorc_score_kernel<8, true> : lorc_score_kernel<8, false>);
+        cudaError_t e = lorc_launch_dependent(kernel, dim3(2 * n_pairs), dim3(Q_THREADS), smem, st, mapCK, mapBKT, sp);
         *launches += 1;
         if (e != cudaSuccess) return e;
     }

@@ -1,0 +1,136 @@
+"""Interleaved rotary pairs on the tensor-core decode path: numerators and latent outputs in two bf16 parts.
+
+The path took over from the plain fp32 kernels, so its results carry no more error than theirs: the rounding of the bf16
+output, and beside it 2e-4 of the row rms.  (Two bf16 parts hold 16 significant bits: 2^-17 = 8e-6 relative per numerator
+and per latent output; fp32 sums of up to 1024 products add about 2^-24 sqrt(1024) = 2e-6 per score unit.  An element is a
+sum of many such terms of random sign, the row rms their common scale; 2e-4 leaves a factor of ten.)"""
+import numpy as np
+import pytest
+
+from oracle import lorc_oracle as O
+from workloads import synth
+
+import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+INTERLEAVED = 1
+G8B = dict(D=1024, H_q=32, H_kv=8, d_h=128)
+G70B = dict(D=1024, H_q=64, H_kv=8, d_h=128)
+G_N512 = dict(D=512, H_q=32, H_kv=4, d_h=128)      # eight query heads per KV head on 32 heads
+
+
+def _problem(geom, r_k, r_v, lens, flags=0):
+    prob = H.Problem(r_k=r_k, r_v=r_v, theta=500000.0, layer=31, style=INTERLEAVED, **geom)
+    sess = H.Session(prob, max_pos=max(lens) + 3, batch=len(lens), flags=flags)
+    xs = [synth.hidden_states(n, prob.D, 31, chunk=s).astype(np.float64) for s, n in enumerate(lens)]
+    return prob, sess, *H.oracle_latents(prob, xs)
+
+
+def _close(got, want):
+    rms = np.sqrt(np.mean(want ** 2, axis=-1, keepdims=True))
+    excess = np.abs(got - want) - (0.5 * H.bf16_ulp(want) + 2e-4 * rms)
+    assert np.all(excess <= 0.0), float((excess / rms).max())
+
+
+@pytest.mark.parametrize("geom,r_k,r_v,lens,page,n_splits", [
+    (G8B, 72, 136, [1, 37, 128, 129], 0, 0),        # rank tails, a sequence that ends a tile, one that starts the next
+    (G8B, 512, 512, [700, 2], 0, 1),                # one share per column block
+    (G8B, 264, 64, [513, 300, 5], 16, 0),
+    (G70B, 136, 248, [257, 640], 64, 0),            # 64 heads: 128 rows of numerators, three stages
+    (G70B, 64, 128, [385, 1], 0, 2),
+    (G_N512, 192, 96, [200, 511], 128, 0),
+])
+def test_interleaved_decode(geom, r_k, r_v, lens, page, n_splits):
+    import torch
+    prob, sess, ck, cv = _problem(geom, r_k, r_v, lens)
+    L, b = sess.L, len(lens)
+    if page:
+        held = H.paged_cache(sess, b, lens, page, order_seed=5, k_rows=ck, v_rows=cv)
+    else:
+        held = H.contiguous_cache(sess, b, max(lens) + 3, lens, ck, cv)
+    for q_scale in (1.0, 8.0, 64.0):
+        q = synth.queries(b, prob.H_q, 128, 31, int(q_scale), q_scale).astype(np.float64)
+        out = torch.zeros(b, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
+        L.lorc_decode_attn(sess.ctx, 0, held[0], H.dev_bf16(q), out, n_splits=n_splits)
+        assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+        assert L.lorc_last_path(sess.ctx) == 2, "the tensor-core path was not taken"
+        _close(H.host_f64(out), H.oracle_decode(prob, ck, cv, q))
+    lat = torch.zeros(b, prob.H_q, r_v, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn_latent_out(sess.ctx, 0, held[0], H.dev_bf16(q), lat, n_splits=n_splits)
+    assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+    for s in range(b):
+        _close(H.host_f64(lat[s]), O.decode_attn_latent_out(ck[s], cv[s], prob.B_k, q[s], prob.H_kv, prob.theta, INTERLEAVED))
+    sess.close()
+
+
+def test_interleaved_falls_back_to_plain_kernels():
+    """A workspace that only holds the plain kernels' partial results, and a first call under stream capture (no table may
+    be allocated then), run the plain kernels; the call after it may take the tensor-core path."""
+    import torch
+    lens = [300, 40]
+    prob, sess, ck, cv = _problem(G8B, 96, 96, lens)
+    L, b = sess.L, len(lens)
+    held = H.contiguous_cache(sess, b, max(lens) + 3, lens, ck, cv)
+    q = synth.queries(b, prob.H_q, 128, 31, 1, 8.0).astype(np.float64)
+    qd, want = H.dev_bf16(q), H.oracle_decode(prob, ck, cv, q)
+    out = torch.zeros(b, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        L.lorc_decode_attn(sess.ctx, 0, held[0], qd, out)
+        assert L.lorc_last_path(sess.ctx) == 1
+    graph.replay()
+    assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+    _close(H.host_f64(out), want)
+    for nbytes, path in ((b * prob.H_q * (96 + 2) * 4 + 512, 1), (None, 2)):
+        L.lorc_set_workspace(sess.ctx, sess.ws, nbytes)
+        out.zero_()
+        L.lorc_decode_attn(sess.ctx, 0, held[0], qd, out)
+        assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+        assert L.lorc_last_path(sess.ctx) == path
+        _close(H.host_f64(out), want)
+    with torch.cuda.graph(graph2 := torch.cuda.CUDAGraph()):
+        L.lorc_decode_attn(sess.ctx, 0, held[0], qd, out)
+        assert L.lorc_last_path(sess.ctx) == 2
+    for _ in range(2):
+        out.zero_()
+        graph2.replay()
+        assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+        _close(H.host_f64(out), want)
+    del graph, graph2
+    sess.close()
+
+
+def test_interleaved_context_shards():
+    import torch
+    from paper_2410_03111_b200 import sharded
+    lens, world = [700, 130, 17], 2
+    prob, sess, ck, cv = _problem(G8B, 160, 96, lens)
+    L, b = sess.L, len(lens)
+    q = synth.queries(b, prob.H_q, 128, 31, 2, 8.0).astype(np.float64)
+    qd = H.dev_bf16(q)
+    pos0, cnt = sharded.shard_bounds(lens, world)
+    q_pos = torch.tensor([n - 1 for n in lens], dtype=torch.int32, device="cuda")
+    outs = torch.zeros(world, b, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
+    mls = torch.zeros(world, b, prob.H_q, 2, dtype=torch.float32, device="cuda")
+    for r in range(world):
+        rows = [[c[s][pos0[r][s]:pos0[r][s] + cnt[r][s]] for s in range(b)] for c in (ck, cv)]
+        held = H.contiguous_cache(sess, b, max(lens) + 3, cnt[r], *rows)
+        p0 = torch.tensor(pos0[r], dtype=torch.int32, device="cuda")
+        L.lorc_decode_attn_shard(sess.ctx, 0, held[0], qd, p0, q_pos, outs[r], mls[r])
+        assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+        assert L.lorc_last_path(sess.ctx) == 2
+        for s in range(b):
+            a, n = pos0[r][s], cnt[r][s]
+            if n:
+                pos = np.arange(a, a + n)
+                _close(H.host_f64(outs[r, s]), O.decode_attn_latent(ck[s][a:a + n], cv[s][a:a + n], prob.B_k, prob.B_v, q[s],
+                                                                    prob.H_kv, prob.theta, INTERLEAVED, pos, lens[s] - 1))
+                lse = O.shard_log2_sum_exp(ck[s][a:a + n], prob.B_k, q[s], prob.H_kv, prob.theta, pos, lens[s] - 1, INTERLEAVED)
+                ml = H.host_f64(mls[r, s])
+                assert np.max(np.abs(ml[:, 0] + np.log2(ml[:, 1]) - lse)) <= 2e-4
+    merged = torch.zeros(b, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
+    L.lorc_merge_shards(sess.ctx, world, outs, mls, merged, b)
+    assert L.lorc_sync_status(sess.ctx) == 0
+    H.assert_rows_close(H.host_f64(merged), H.oracle_decode(prob, ck, cv, q), 1e-2)
+    sess.close()
