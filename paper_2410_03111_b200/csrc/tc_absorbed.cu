@@ -216,6 +216,14 @@ lorc_score_absorbed_kernel(const __grid_constant__ CUtensorMap mapCK, const __gr
             int tile;
             locate_tile(sm, f, p.batch, s, tile);
             const int sg = p.seq0 + s, len = sm.lens[s];
+            const int ppt = paged ? TILE / p.page_size : 0;
+            int pages[8];
+            if (paged) {
+                const int mine = lorc_tile_page(p.page_table, sg, tile, lane, len, p.page_size, p.max_pages_per_seq,
+                                                p.n_pages, p.status);
+#pragma unroll
+                for (int pg = 0; pg < 8; ++pg) pages[pg] = __shfl_sync(0xffffffffu, mine, pg);
+            }
             for (int kc = 0; kc < nkc; ++kc) {
                 if (!mbar_wait(&sm.empty[st], par)) { ok = false; break; }
                 if (elect_one()) {
@@ -223,21 +231,11 @@ lorc_score_absorbed_kernel(const __grid_constant__ CUtensorMap mapCK, const __gr
                     if (!paged) {
                         tma_load_3d(sm.C[st], &mapCK, &sm.full[st], kc * KC, tile * TILE, sg);
                     } else {
-                        // one box per page; pages past the end of the sequence (or with a bad table entry) are read
-                        // from page 0: those tokens are masked, but every box must deliver its bytes
-                        const int ppt = TILE / p.page_size;
-                        for (int pg = 0; pg < ppt; ++pg) {
-                            const int lp = tile * ppt + pg;
-                            int page = 0;
-                            if ((long long)lp * p.page_size < len && lp < p.max_pages_per_seq) {
-                                page = p.page_table[(long long)sg * p.max_pages_per_seq + lp];
-                                if (page < 0 || page >= p.n_pages) {
-                                    lorc_set_status(p.status, LORC_ERR_CAPACITY);
-                                    page = 0;
-                                }
-                            }
-                            tma_load_3d(sm.C[st] + pg * p.page_size * KC, &mapCK, &sm.full[st], kc * KC, 0, page);
-                        }
+                        // one box per page
+#pragma unroll
+                        for (int pg = 0; pg < 8; ++pg)
+                            if (pg < ppt)
+                                tma_load_3d(sm.C[st] + pg * p.page_size * KC, &mapCK, &sm.full[st], kc * KC, 0, pages[pg]);
                     }
 #pragma unroll
                     for (int part = 0; part < NQ; ++part)

@@ -122,6 +122,14 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
             int s, tp, hp, len;
             if (!decode(u, s, tp, hp, len)) continue;
             const int tile = 2 * tp + rank;
+            const int ppt = p.page_table ? TILE / p.page_size : 0;
+            int pages[8];
+            if (p.page_table) {
+                const int mine = lorc_tile_page(p.page_table, s, tile, lane, len, p.page_size, p.max_pages_per_seq, p.n_pages,
+                                                p.status);
+#pragma unroll
+                for (int pg = 0; pg < 8; ++pg) pages[pg] = __shfl_sync(0xffffffffu, mine, pg);
+            }
             for (int kc = 0; kc < nkc; ++kc) {
                 if (!mbar_wait_addr(empty0 + st * 8, par)) { ok = false; break; }
                 const uint32_t lead_bar = lead_full0 + st * 8;
@@ -132,20 +140,11 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
                         // (a tile past the buffer's rows reads as zero)
                         tma_load_3d_pair_addr(a_dst, &mapC, lead_bar, kc * KC, tile * TILE, s);
                     } else {
-                        // one box per page; pages past the end of the sequence (or with a bad table entry) come from page 0
-                        const int ppt = TILE / p.page_size;
-                        for (int pg = 0; pg < ppt; ++pg) {
-                            const int lp = tile * ppt + pg;
-                            int page = 0;
-                            if ((long long)lp * p.page_size < len && lp < p.max_pages_per_seq) {
-                                page = p.page_table[(long long)s * p.max_pages_per_seq + lp];
-                                if (page < 0 || page >= p.n_pages) {
-                                    lorc_set_status(p.status, LORC_ERR_CAPACITY);
-                                    page = 0;
-                                }
-                            }
-                            tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, &mapC, lead_bar, kc * KC, 0, page);
-                        }
+                        // one box per page
+#pragma unroll
+                        for (int pg = 0; pg < 8; ++pg)
+                            if (pg < ppt)
+                                tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, &mapC, lead_bar, kc * KC, 0, pages[pg]);
                     }
                     tma_load_2d_pair_addr(b_base + st * (TILE * KC * 2), &mapBT, lead_bar, kc * KC, hp * R_N + rank * 128);
                 }

@@ -124,10 +124,22 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
         // start.  So the first stages' C_V boxes are requested right away, and only the images wait for that kernel
         // to finish.
         {
+            const bool paged = p.page_table != nullptr;
+            const int ppt = paged ? TILE / p.page_size : 0;
+            auto tile_page = [&](int tile) {
+                return lorc_tile_page(p.page_table, s, tile, lane, len, p.page_size, p.max_pages_per_seq, p.n_pages, p.status);
+            };
+            int mine = paged && ntiles > 0 ? tile_page(tile_lo) : 0;
             for (int i = 0; i < ntiles && ok; ++i) {
                 const int tile = tile_lo + i;
                 const int n0 = tile * TILE;
                 const int st = i % P_STAGES;
+                int pages[8];
+                if (paged) {
+#pragma unroll
+                    for (int pg = 0; pg < 8; ++pg) pages[pg] = __shfl_sync(0xffffffffu, mine, pg);
+                    if (i + 1 < ntiles) mine = tile_page(tile + 1);      // on its way while this tile's boxes go out
+                }
                 if (i == P_STAGES) {
                     // images of the stages whose C_V boxes went out before the wait
                     grid_dep_wait();
@@ -152,22 +164,13 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                     tma_load_3d(sm.V[st][0], &mapCV, &sm.vfull[st], rho0, n0, s);
                     tma_load_3d(sm.V[st][1], &mapCV, &sm.vfull[st], rho0 + 64, n0, s);
                 } else {
-                    // One box per page.  Pages past the end of the sequence (or with a bad table entry) are read
-                    // from page 0 instead: their probabilities are zero, but the rows must hold finite numbers,
-                    // which stale shared memory would not guarantee.
-                    const int ppt = TILE / p.page_size;
-                    for (int pg = 0; pg < ppt; ++pg) {
-                        const int lp = n0 / p.page_size + pg;
-                        int page = 0;
-                        if (lp * p.page_size < len && lp < p.max_pages_per_seq) {
-                            page = p.page_table[(long long)s * p.max_pages_per_seq + lp];
-                            if (page < 0 || page >= p.n_pages) {
-                                lorc_set_status(p.status, LORC_ERR_CAPACITY);
-                                page = 0;
-                            }
-                        }
-                        tma_load_3d(sm.V[st][0] + pg * p.page_size * KC, &mapCV, &sm.vfull[st], rho0, 0, page);
-                        tma_load_3d(sm.V[st][1] + pg * p.page_size * KC, &mapCV, &sm.vfull[st], rho0 + 64, 0, page);
+                    // One box per page.  (Pages past the end of the sequence come from page 0: their probabilities are
+                    // zero, but the rows must hold finite numbers, which stale shared memory would not guarantee.)
+#pragma unroll
+                    for (int pg = 0; pg < 8; ++pg) {
+                        if (pg >= ppt) break;
+                        tma_load_3d(sm.V[st][0] + pg * p.page_size * KC, &mapCV, &sm.vfull[st], rho0, 0, pages[pg]);
+                        tma_load_3d(sm.V[st][1] + pg * p.page_size * KC, &mapCV, &sm.vfull[st], rho0 + 64, 0, pages[pg]);
                     }
                 }
                 }

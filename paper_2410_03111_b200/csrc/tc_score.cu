@@ -213,6 +213,14 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
             Unit un;
             decode_unit(sm, w, rank, n_flat, p.batch, un);
             const int row0 = un.tile * TILE, brow = un.hp * 256 + b_row, sg = p.seq0 + un.s;
+            const int ppt = paged ? TILE / p.page_size : 0;
+            int pages[8];
+            if (paged) {
+                const int mine = lorc_tile_page(p.page_table, sg, un.tile, lane, un.len, p.page_size, p.max_pages_per_seq,
+                                                p.n_pages, p.status);
+#pragma unroll
+                for (int pg = 0; pg < 8; ++pg) pages[pg] = __shfl_sync(0xffffffffu, mine, pg);
+            }
             for (int x = 0; x < nkc * KC; x += KC) {
                 if (!mbar_wait_addr(empty0 + st * 8, par)) { ok = false; break; }
                 const uint32_t lead_bar = lead_full0 + st * 8;
@@ -222,21 +230,11 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
                     if (!paged) {
                         tma_load_3d_pair_addr(a_dst, &mapCK, lead_bar, x, row0, sg);
                     } else {
-                        // one box per page; pages past the end of the sequence (or with a bad table entry) are
-                        // read from page 0: those rows are masked, but every box must deliver its bytes
-                        const int ppt = TILE / p.page_size;
-                        for (int pg = 0; pg < ppt; ++pg) {
-                            const int lp = un.tile * ppt + pg;
-                            int page = 0;
-                            if ((long long)lp * p.page_size < un.len && lp < p.max_pages_per_seq) {
-                                page = p.page_table[(long long)sg * p.max_pages_per_seq + lp];
-                                if (page < 0 || page >= p.n_pages) {
-                                    lorc_set_status(p.status, LORC_ERR_CAPACITY);
-                                    page = 0;
-                                }
-                            }
-                            tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, &mapCK, lead_bar, x, 0, page);
-                        }
+                        // one box per page
+#pragma unroll
+                        for (int pg = 0; pg < 8; ++pg)
+                            if (pg < ppt)
+                                tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, &mapCK, lead_bar, x, 0, pages[pg]);
                     }
                     tma_load_2d_pair_addr(b_base + st * (128 * KC * 2), &mapBKT, lead_bar, x, brow);
                 }
