@@ -128,6 +128,12 @@ cudaError_t lorc_generic_append(const lorc_ctx* ctx, const LorcLayer& L, const C
 bool lorc_full_decode_supported(const lorc_ctx* ctx, const LorcLayer& L);
 cudaError_t lorc_full_decode(const lorc_ctx* ctx, const CacheView& cv, const bf16* q, int n_splits, float* part_ml,
                              float* part_o, cudaStream_t st, int* launches);
+// Compressed layers, one query per sequence, bf16 path: the plain computation with mma.sync reconstruction (small_decode.cu).
+// Leaves the same per-split partial results too.
+bool lorc_small_decode_supported(const lorc_ctx* ctx, const LorcLayer& L);
+cudaError_t lorc_small_decode(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* q, int n_splits,
+                              float* part_ml, float* part_o, cudaStream_t st, int* launches, const int32_t* pos0,
+                              const int32_t* q_pos);
 // latent_out: stop before the value up-projection and write the normalised latent output [b, H_q, r_v] to `out`.
 // T > 1: T queries per sequence (q, out [b, T, H_q, d_head]; partial results for b * T units), query t of a sequence
 // at position seq_lens[s] - T + t, attending to the tokens up to its own.
@@ -146,3 +152,19 @@ cudaError_t lorc_generic_combine(const lorc_ctx* ctx, const LorcLayer& L, int ba
 // token granularity of a split in the plain decode kernel
 #define LORC_GENERIC_TILE 32
 #define LORC_MAX_SPLITS 256
+// tokens per step of the small-shape decode kernel
+#define LORC_SMALL_TILE 64
+// Default number of context splits for one layer: about 512 tokens each; where the small-shape kernel runs, as many as give
+// two blocks per SM, down to one step each.
+static inline int lorc_default_splits(int max_seq_len, int sm_count, int batch, int n_kv_heads, bool small) {
+    int s = (max_seq_len + 511) / 512;
+    if (small) {
+        int fill = (2 * sm_count + batch * n_kv_heads - 1) / (batch * n_kv_heads);
+        const int steps = (max_seq_len + LORC_SMALL_TILE - 1) / LORC_SMALL_TILE;
+        if (fill > steps) fill = steps;
+        if (s < fill) s = fill;
+    }
+    if (s < 1) s = 1;
+    if (s > LORC_MAX_SPLITS) s = LORC_MAX_SPLITS;
+    return s;
+}

@@ -30,14 +30,6 @@ void free_layer(LorcLayer& L) {
     L = LorcLayer();
 }
 
-// Default number of context splits of the plain kernels: about 512 tokens each.
-int generic_default_splits(int max_seq_len) {
-    int s = (max_seq_len + 511) / 512;
-    if (s < 1) s = 1;
-    if (s > LORC_MAX_SPLITS) s = LORC_MAX_SPLITS;
-    return s;
-}
-
 struct WsLayout {
     size_t off_ml, off_o, total;
 };
@@ -237,8 +229,13 @@ int lorc_load_factors(lorc_ctx* ctx, int layer, int mode, int r_k, int r_v, cons
 
 size_t lorc_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_len) {
     if (!ctx || batch <= 0 || max_seq_len <= 0) return 0;
-    int S = generic_default_splits(max_seq_len);
+    int S = lorc_default_splits(max_seq_len, ctx->sm_count, batch, ctx->desc.n_kv_heads, false);
     size_t gen = ws_layout(ctx, batch, S, ctx->n).total;
+    if (!lorc_tc_workspace_bytes(ctx, batch, max_seq_len)) {
+        // the small-shape kernel takes more, shorter shares
+        S = lorc_default_splits(max_seq_len, ctx->sm_count, batch, ctx->desc.n_kv_heads, true);
+        gen = ws_layout(ctx, batch, S, ctx->n).total;
+    }
     size_t tc = lorc_align_up(lorc_tc_workspace_bytes(ctx, batch, max_seq_len), 256);
     return (gen > tc ? gen : tc) + staging_bytes(ctx, batch) + 256;
 }
@@ -322,7 +319,9 @@ static int decode_attn_impl(lorc_ctx* ctx, int layer, const lorc_cache* cache, c
         return LORC_OK;
     }
 
-    int S = n_splits > 0 ? n_splits : generic_default_splits(cv.max_seq_len);
+    int S = n_splits > 0 ? n_splits
+                         : lorc_default_splits(cv.max_seq_len, ctx->sm_count, cv.batch, ctx->desc.n_kv_heads,
+                                               lorc_small_decode_supported(ctx, *L));
     int tiles = (cv.max_seq_len + LORC_GENERIC_TILE - 1) / LORC_GENERIC_TILE;
     if (S > tiles) S = tiles;
     if (S > LORC_MAX_SPLITS) S = LORC_MAX_SPLITS;
@@ -371,7 +370,7 @@ int lorc_merge_shards(lorc_ctx* ctx, int n_shards, const void* outs, const float
 
 size_t lorc_prefill_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_len, int T) {
     if (!ctx || batch <= 0 || max_seq_len <= 0 || T <= 0) return 0;
-    int S = generic_default_splits(max_seq_len);
+    int S = lorc_default_splits(max_seq_len, ctx->sm_count, batch, ctx->desc.n_kv_heads, false);
     size_t gen = ws_layout(ctx, batch * T, S, ctx->n).total;
     size_t tc = lorc_tc_prefill_shape_ok(ctx) ? lorc_tc_prefill_scratch_bytes(ctx, batch, max_seq_len, T) : 0;
     return (gen > tc ? gen : tc) + 256;
@@ -405,7 +404,7 @@ int lorc_prefill_attn(lorc_ctx* ctx, int layer, const lorc_cache* cache, const v
     // plain kernels: every (sequence, query) is a decode query over the sequence cut after its own token
     const bool latent = (L->mode == LORC_MODE_LATENT);
     const int W = latent ? L->r_v : ctx->desc.d_head;
-    int S = generic_default_splits(cv.max_seq_len);
+    int S = lorc_default_splits(cv.max_seq_len, ctx->sm_count, cv.batch, ctx->desc.n_kv_heads, false);
     int tiles = (cv.max_seq_len + LORC_GENERIC_TILE - 1) / LORC_GENERIC_TILE;
     if (S > tiles) S = tiles;
     while (S > 1 && ws_layout(ctx, cv.batch * T, S, W).total > ctx->ws_bytes) --S;
