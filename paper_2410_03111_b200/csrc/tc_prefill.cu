@@ -7,9 +7,9 @@
 // kernel runs over that buffer.
 //
 //   reconstruct kernel  K^[tile, head] = RoPE(C_K[tile, :] . B_K[:, head]),  V[tile, head] = C_V[tile, :] . B_V[:, head]
-//                       persistent CTA pairs over (two 128-token tiles, pair of KV heads): TMA-staged 64-wide slices,
-//                       tcgen05 cta_group::2 (M = 256 tokens, N = 256), rotation in the epilogue (thread = token row)
-//                       under the next unit's MMAs, 16-bit rows to the buffer: keys as
+//                       persistent CTA pairs over (keys or values, two 128-token tiles, pair of KV heads): TMA-staged
+//                       64-wide slices, tcgen05 cta_group::2 (M = 256 tokens, N = 256), rotation in the epilogue under the
+//                       next unit's MMAs, fp16 boxes to the buffer by TMA: keys as
 //                       fp16 (the scores are then exact to 2^-11 of |q| |k|, four times closer than with bf16 keys),
 //                       values as fp16 too (a reconstructed element must stay below 65504 in magnitude)
 //   attention kernel    one CTA per two blocks of 128 query rows (128 / G positions x G heads of one KV head each); the
@@ -38,46 +38,52 @@ constexpr float LOG2E = 1.4426950408889634f;
 // ------------------------------------------------------------------------------------------------
 // reconstruction of keys (rotated) or values into [b, n_rows, n] fp16
 // ------------------------------------------------------------------------------------------------
-// Persistent CTA PAIRS (clusters of two, cta_group::2 MMAs) walk units (sequence, pair of 128-token tiles, pair of KV
-// heads), the head pair running fastest (the pairs that work on the same latent rows at the same time share them in
-// L2).  Per unit  acc[256 tokens, 256 features] = C[tiles, :] . B[:, 2 heads]  in 64-wide slices: each CTA stages its
+// Persistent CTA PAIRS (clusters of two, cta_group::2 MMAs) walk units (keys or values, sequence, pair of 128-token tiles,
+// pair of KV heads), the head pair running fastest (the pairs that work on the same latent rows at the same time share them
+// in L2).  Per unit  acc[256 tokens, 256 features] = C[tiles, :] . B[:, 2 heads]  in 64-wide slices: each CTA stages its
 // own 128 tokens and HALF of the factor slice (what a CTA can take in through TMA, not the MMA rate, bounds a
-// single CTA with the whole slice); the accumulator is double-buffered in tensor memory, so the epilogue of one unit
-// (rotation, rounding, 512-byte row stores of the CTA's own tokens) runs under the MMAs of the next.
-constexpr int R_STAGES = 6;
-constexpr int R_THREADS = 192;       // warp 0 TMA, warp 1 MMA (leader CTA issues), warps 2..5 epilogue
+// single CTA with the whole slice); the accumulator is double-buffered in tensor memory, so the epilogue of one unit runs
+// under the MMAs of the next.  The epilogue has eight warps, four per head; a lane holds four tokens x two adjacent rotary
+// pairs per step (16-lane x 256-bit loads), so rotation operands come in 64-byte runs, two fp16 go to shared memory as one
+// conflict-free word, and the finished 128 x 64 boxes leave by TMA.  (With four warps, thread = token row, the row-wise
+// 16-byte stores and table reads touched 32 lines per access and the epilogue took three times as long as the MMAs:
+// 284 us for the keys and values of 16 x 4096 tokens at rank 672, 162 us now.)
+constexpr int R_STAGES = 5;
+constexpr int R_THREADS = 384;       // warp 0 TMA, warp 1 MMA (leader CTA issues), warps 4..11 epilogue
 constexpr int R_N = 256;             // features per unit: two KV heads
 
 struct RecSmem {
     bf16 A[R_STAGES][TILE * KC];          // latent slice of this CTA's tile [128 tokens][64]
     bf16 B[R_STAGES][TILE * KC];          // this CTA's half of the factor slice [128 features][64]
+    uint8_t O[2][2][TILE * 128];          // finished boxes: [head][half of the head][128 tokens][64 fp16], 128-byte swizzle
     uint64_t full[R_STAGES], empty[R_STAGES], acc_full[2], acc_empty[2];
     uint32_t tmem_base;
 };
 
 struct RecParams {
-    bf16* out;                     // [b, n_rows, n]
     const int32_t* seq_lens;
     const int32_t* page_table;
     const float2* rope_table;      // [max_pos][64]
     int* status;
-    int r, n, n_rows, max_pos, batch, tile_pairs, n_hp;
+    int r_k, r_v, n_rows, max_pos, batch, tile_pairs, n_hp;
     int page_size, max_pages_per_seq, n_pages;
 };
 
-template <bool ROPE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(R_THREADS, 1)
-lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_constant__ CUtensorMap mapBT, const RecParams p) {
+lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_constant__ CUtensorMap mapCV,
+                        const __grid_constant__ CUtensorMap mapBKT, const __grid_constant__ CUtensorMap mapBVT,
+                        const __grid_constant__ CUtensorMap mapKO, const __grid_constant__ CUtensorMap mapVO, const RecParams p) {
     extern __shared__ uint8_t raw[];
     RecSmem& sm = *reinterpret_cast<RecSmem*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int rank = (int)cluster_ctarank();           // 0 = leader (issues the MMAs, owns the full / acc_empty barriers)
     const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-    const int nkc = (p.r + KC - 1) / KC;
-    const int total = p.batch * p.tile_pairs * p.n_hp;
-    // unit -> (sequence, tile pair, head pair); a unit whose first tile lies past the sequence's cached tokens is
+    const int per_kind = p.batch * p.tile_pairs * p.n_hp, total = 2 * per_kind;
+    // unit -> (values?, sequence, tile pair, head pair); a unit whose first tile lies past the sequence's cached tokens is
     // skipped by both CTAs and every role alike (sequences beyond the buffer are reported by the attention kernel)
-    auto decode = [&](int u, int& s, int& tp, int& hp, int& len) -> bool {
+    auto decode = [&](int u, bool& val, int& s, int& tp, int& hp, int& len) -> bool {
+        val = u >= per_kind;
+        if (val) u -= per_kind;
         hp = u % p.n_hp;
         const int st = u / p.n_hp;
         tp = st % p.tile_pairs;
@@ -94,12 +100,15 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sm.acc_full[i], 1);
-            mbar_init(&sm.acc_empty[i], 2 * 4);             // one arrival per epilogue warp, both CTAs
+            mbar_init(&sm.acc_empty[i], 2 * 8);             // one arrival per epilogue warp, both CTAs
         }
         fence_barrier_init();
-        prefetch_tensormap(&mapC);
-        prefetch_tensormap(&mapBT);
+        prefetch_tensormap(&mapCK);
+        prefetch_tensormap(&mapCV);
+        prefetch_tensormap(&mapBKT);
+        prefetch_tensormap(&mapBVT);
     }
+    grid_dep_wait();                                     // the latent rows may come from the kernel before this one
     if (warp == 1) {
         tmem_alloc_pair(&sm.tmem_base, 512);
         tmem_relinquish_pair();
@@ -109,6 +118,7 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
     cluster_arrive_release();                            // the peer's barriers are initialised before anyone signals them
     cluster_wait_acquire();
     tc_fence_after_sync();
+    grid_dep_launch();
     const uint32_t tmem = sm.tmem_base;
     bool ok = true;
 
@@ -119,9 +129,12 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
         const uint32_t lead_full0 = mapa_shared(full0, 0);   // all bytes of a stage are counted on the leader's barrier
         uint32_t st = 0, par = 1;
         for (int u = pair_id; u < total && ok; u += n_pairs) {
+            bool val;
             int s, tp, hp, len;
-            if (!decode(u, s, tp, hp, len)) continue;
-            const int tile = 2 * tp + rank;
+            if (!decode(u, val, s, tp, hp, len)) continue;
+            const int tile = 2 * tp + rank, nkc = ((val ? p.r_v : p.r_k) + KC - 1) / KC;
+            const CUtensorMap* mapC = val ? &mapCV : &mapCK;
+            const CUtensorMap* mapBT = val ? &mapBVT : &mapBKT;
             const int ppt = p.page_table ? TILE / p.page_size : 0;
             int pages[8];
             if (p.page_table) {
@@ -138,15 +151,15 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
                     if (rank == 0) mbar_arrive_expect_tx_addr(full0 + st * 8, 2 * 2 * TILE * KC * 2);
                     if (p.page_table == nullptr) {
                         // (a tile past the buffer's rows reads as zero)
-                        tma_load_3d_pair_addr(a_dst, &mapC, lead_bar, kc * KC, tile * TILE, s);
+                        tma_load_3d_pair_addr(a_dst, mapC, lead_bar, kc * KC, tile * TILE, s);
                     } else {
                         // one box per page
 #pragma unroll
                         for (int pg = 0; pg < 8; ++pg)
                             if (pg < ppt)
-                                tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, &mapC, lead_bar, kc * KC, 0, pages[pg]);
+                                tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, mapC, lead_bar, kc * KC, 0, pages[pg]);
                     }
-                    tma_load_2d_pair_addr(b_base + st * (TILE * KC * 2), &mapBT, lead_bar, kc * KC, hp * R_N + rank * 128);
+                    tma_load_2d_pair_addr(b_base + st * (TILE * KC * 2), mapBT, lead_bar, kc * KC, hp * R_N + rank * 128);
                 }
                 __syncwarp();
                 if (++st == R_STAGES) { st = 0; par ^= 1; }
@@ -157,7 +170,6 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
         if (rank == 0) {
             const uint32_t idesc = make_idesc_bf16(256, R_N, 0, 0);
-            const int nk_last = (p.r - (nkc - 1) * KC + 15) >> 4;     // 16-column steps the last stage really holds
             const uint64_t da0 = make_smem_desc_sw128(smem_u32(sm.A[0]), 0, 1024);
             const uint64_t db0 = make_smem_desc_sw128(smem_u32(sm.B[0]), 0, 1024);
             const uint32_t a_lo0 = (uint32_t)da0, a_hi = (uint32_t)(da0 >> 32);
@@ -165,8 +177,11 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
             const uint32_t empty0 = smem_u32(&sm.empty[0]), full0 = smem_u32(&sm.full[0]);
             uint32_t st = 0, par = 0, uc = 0;
             for (int u = pair_id; u < total && ok; u += n_pairs) {
+                bool val;
                 int s, tp, hp, len;
-                if (!decode(u, s, tp, hp, len)) continue;
+                if (!decode(u, val, s, tp, hp, len)) continue;
+                const int r = val ? p.r_v : p.r_k, nkc = (r + KC - 1) / KC;
+                const int nk_last = (r - (nkc - 1) * KC + 15) >> 4;     // 16-column steps the last stage really holds
                 const int buf = uc & 1;
                 if (!mbar_wait(&sm.acc_empty[buf], ((uc >> 1) & 1) ^ 1)) { ok = false; break; }
                 tc_fence_after_sync();
@@ -196,63 +211,86 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_c
             }
             if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
         }
-    } else {
+    } else if (warp >= 4) {
         // ------------------------------------------------------------------ epilogue (both CTAs): this CTA's 128 tokens
-        const int quarter = warp % 4;
-        const int row = quarter * 32 + lane;                         // token of the tile = TMEM lane
+        const int hd = (warp - 4) >> 2, quarter = warp % 4;          // head of the pair, TMEM lane quarter
+        const int r = lane >> 2, c = lane & 3;                       // tokens 32 quarter + r + 8 m, rotary pairs 8 kk + 2 c, + 1
+        const bool issuer = tid == 128 + hd * 128;                   // the thread that stores this head's boxes
         const uint32_t lead_acc_empty[2] = {mapa_shared(smem_u32(&sm.acc_empty[0]), 0),
                                             mapa_shared(smem_u32(&sm.acc_empty[1]), 0)};
+        // the lane's word of row 32 quarter + r (+ 8 m: 1 KiB further on), 16-byte piece kk, in both boxes
+        uint8_t* o0 = sm.O[hd][0] + (quarter * 32 + r) * 128 + c * 4;
+        uint8_t* o1 = sm.O[hd][1] + (quarter * 32 + r) * 128 + c * 4;
+        auto head_sync = [&]() {                                     // the four warps of a head
+            __syncwarp();
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + hd) : "memory");
+        };
         uint32_t uc = 0;
-        for (int u = pair_id; u < total && ok; u += n_pairs) {
+        for (int u = pair_id; u < total; u += n_pairs) {
+            bool val;
             int s, tp, hp, len;
-            if (!decode(u, s, tp, hp, len)) continue;
-            const int buf = uc & 1;
-            if (!mbar_wait(&sm.acc_full[buf], (uc >> 1) & 1)) { ok = false; break; }
+            if (!decode(u, val, s, tp, hp, len)) continue;
+            const int buf = uc & 1, tile = 2 * tp + rank;
+            if (issuer) bulk_wait_read();                            // the boxes of the unit before have left
+            head_sync();
+            // (after a wait that ran out the warp stays in the loop's barriers: every warp of the head takes the same ones)
+            if (ok && !mbar_wait(&sm.acc_full[buf], (uc >> 1) & 1)) ok = false;
             tc_fence_after_sync();
-            const int pos = (2 * tp + rank) * TILE + row;
-            const float2* cs = p.rope_table + (long long)min(pos, p.max_pos - 1) * 64;
-#pragma unroll 1
-            for (int hd = 0; hd < 2; ++hd) {
-                bf16* dst = p.out + ((long long)s * p.n_rows + pos) * p.n + (hp * 2 + hd) * 128;
-                const uint32_t tcol = tmem + ((uint32_t)(quarter * 32) << 16) + buf * R_N + hd * 128;
+            const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + buf * R_N + hd * 128;
+            const int pos0 = tile * TILE + quarter * 32 + r;
+            const float4* cs[4];
 #pragma unroll
-                for (int c0 = 0; c0 < 64; c0 += 32) {
-                    uint32_t ra[32], rb[32];
-                    tmem_ld32(tcol + c0, ra);          // elements c0 .. c0 + 31 of the head
-                    tmem_ld32(tcol + 64 + c0, rb);     // their partners in the second half
-                    tmem_wait_ld();
-                    if (pos < p.n_rows) {
-                        uint32_t wa[16], wb[16];
+            for (int m = 0; m < 4; ++m)
+                cs[m] = reinterpret_cast<const float4*>(p.rope_table + (long long)min(pos0 + 8 * m, p.max_pos - 1) * 64) + c;
+            auto step = [&](int kk, bool rot) {
+                uint32_t ra[2][4], rb[2][4];
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            float a0 = __uint_as_float(ra[2 * i]), a1 = __uint_as_float(ra[2 * i + 1]);
-                            float b0 = __uint_as_float(rb[2 * i]), b1 = __uint_as_float(rb[2 * i + 1]);
-                            if (ROPE) {
-                                const float4 t = __ldg(reinterpret_cast<const float4*>(cs + c0 + 2 * i));   // (cos, sin) x 2
-                                const float x0 = a0 * t.x - b0 * t.y, y0 = a0 * t.y + b0 * t.x;
-                                const float x1 = a1 * t.z - b1 * t.w, y1 = a1 * t.w + b1 * t.z;
-                                a0 = x0; b0 = y0; a1 = x1; b1 = y1;
-                            }
-                            {                    // keys and values alike: fp16
-                                const __half2 pa = __floats2half2_rn(a0, a1), pb = __floats2half2_rn(b0, b1);
-                                wa[i] = *reinterpret_cast<const uint32_t*>(&pa);
-                                wb[i] = *reinterpret_cast<const uint32_t*>(&pb);
-                            }
-                        }
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            reinterpret_cast<uint4*>(dst + c0)[v] = make_uint4(wa[4 * v], wa[4 * v + 1], wa[4 * v + 2], wa[4 * v + 3]);
-                            reinterpret_cast<uint4*>(dst + 64 + c0)[v] = make_uint4(wb[4 * v], wb[4 * v + 1], wb[4 * v + 2], wb[4 * v + 3]);
-                        }
-                    }
+                for (int hf = 0; hf < 2; ++hf) {
+                    tmem_ld16x256_x1(tbase + ((uint32_t)(hf * 16) << 16) + kk * 8, ra[hf]);
+                    tmem_ld16x256_x1(tbase + ((uint32_t)(hf * 16) << 16) + 64 + kk * 8, rb[hf]);
                 }
+                float4 t[4];
+                if (rot) {
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) t[m] = __ldg(cs[m] + 4 * kk);       // (cos, sin) x 2
+                }
+                tmem_wait_ld();
+                const int piece = (kk ^ r) << 4;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    float a0 = __uint_as_float(ra[m >> 1][2 * (m & 1)]), a1 = __uint_as_float(ra[m >> 1][2 * (m & 1) + 1]);
+                    float b0 = __uint_as_float(rb[m >> 1][2 * (m & 1)]), b1 = __uint_as_float(rb[m >> 1][2 * (m & 1) + 1]);
+                    if (rot) {
+                        const float x0 = a0 * t[m].x - b0 * t[m].y, y0 = a0 * t[m].y + b0 * t[m].x;
+                        const float x1 = a1 * t[m].z - b1 * t[m].w, y1 = a1 * t[m].w + b1 * t[m].z;
+                        a0 = x0; b0 = y0; a1 = x1; b1 = y1;
+                    }
+                    *reinterpret_cast<__half2*>(o0 + m * 1024 + piece) = __floats2half2_rn(a0, a1);
+                    *reinterpret_cast<__half2*>(o1 + m * 1024 + piece) = __floats2half2_rn(b0, b1);
+                }
+            };
+            if (val) {
+#pragma unroll 4
+                for (int kk = 0; kk < 8; ++kk) step(kk, false);
+            } else {
+#pragma unroll 4
+                for (int kk = 0; kk < 8; ++kk) step(kk, true);
             }
             // this warp has read its part of the accumulator
             tc_fence_before_sync();
+            fence_proxy_async_smem();      // the stores read the boxes through the asynchronous proxy
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(lead_acc_empty[buf]);
+            head_sync();
+            if (issuer && ok && tile * TILE < p.n_rows) {
+                const CUtensorMap* mapO = val ? &mapVO : &mapKO;
+                tma_store_3d(mapO, sm.O[hd][0], (hp * 2 + hd) * 128, tile * TILE, s);
+                tma_store_3d(mapO, sm.O[hd][1], (hp * 2 + hd) * 128 + 64, tile * TILE, s);
+                bulk_commit();
+            }
             ++uc;
         }
+        if (issuer) bulk_wait_all();
         if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
     }
     // both CTAs are done with tensor memory and with each other's barriers before either lets go
@@ -323,18 +361,6 @@ lorc_prefill_attn_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_
     const int qp = TILE / p.G;                                // query positions per block of 128 rows
     // the CTAs with the latest positions see the most keys: they go first
     const int t0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * 2 * qp;   // first position (inside the chunk) of this CTA
-    int len = p.seq_lens[s];
-    if (len > p.max_pos || len > p.n_rows) {
-        if (tid == 0) lorc_set_status(p.status, LORC_ERR_CAPACITY);
-        len = 0;
-    }
-    if (len < p.T) {                                          // the chunk is not in the cache: nothing to attend
-        if (tid == 0 && len > 0) lorc_set_status(p.status, LORC_ERR_ARG);
-        len = 0;
-    }
-    const int t_last = min(p.T, t0 + 2 * qp) - 1;             // last query position of the CTA
-    const int n_tiles = len > 0 ? (len - p.T + t_last) / TILE + 1 : 0;
-
     if (tid == 0) {
         mbar_init(&sm.q_full, 1);
         mbar_init(&sm.q_ready, 8);
@@ -355,6 +381,19 @@ lorc_prefill_attn_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_
         prefetch_tensormap(&mapK);
         prefetch_tensormap(&mapV);
     }
+    grid_dep_wait();
+    int len = p.seq_lens[s];
+    if (len > p.max_pos || len > p.n_rows) {
+        if (tid == 0) lorc_set_status(p.status, LORC_ERR_CAPACITY);
+        len = 0;
+    }
+    if (len < p.T) {                                          // the chunk is not in the cache: nothing to attend
+        if (tid == 0 && len > 0) lorc_set_status(p.status, LORC_ERR_ARG);
+        len = 0;
+    }
+    const int t_last = min(p.T, t0 + 2 * qp) - 1;             // last query position of the CTA
+    const int n_tiles = len > 0 ? (len - p.T + t_last) / TILE + 1 : 0;
+
     if (warp == 1) {
         tmem_alloc(&sm.tmem_base, 512);
         tmem_relinquish();
@@ -362,6 +401,7 @@ lorc_prefill_attn_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    grid_dep_launch();
     const uint32_t tmem = sm.tmem_base;
     bool ok = true;
 
@@ -633,11 +673,8 @@ size_t lorc_tc_prefill_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq
 }
 
 cudaError_t lorc_tc_prefill_set_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(lorc_reconstruct_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(lorc_reconstruct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(RecSmem) + 1024);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lorc_reconstruct_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(RecSmem) + 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(lorc_prefill_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(FaSmem) + 1024);
@@ -655,23 +692,6 @@ cudaError_t lorc_tc_prefill_launch(lorc_ctx* ctx, const LorcLayer& L, const Cach
     const int tiles = (int)(rows / TILE);
     cudaError_t e;
 
-    RecParams rp;
-    rp.seq_lens = cv.seq_lens; rp.page_table = cv.page_table; rp.rope_table = ctx->rope_table; rp.status = ctx->status_dev;
-    rp.n = ctx->n; rp.n_rows = (int)rows; rp.max_pos = d.max_pos;
-    rp.page_size = cv.page_size; rp.max_pages_per_seq = cv.max_pages_per_seq; rp.n_pages = cv.n_pages;
-    rp.batch = cv.batch; rp.tile_pairs = (tiles + 1) / 2; rp.n_hp = d.n_kv_heads / 2;
-    const int units = cv.batch * rp.tile_pairs * rp.n_hp;
-    const int pairs = units < ctx->sm_count / 2 ? units : ctx->sm_count / 2;
-    dim3 rgrid(2 * pairs);
-    rp.out = khat; rp.r = L.r_k;
-    lorc_reconstruct_kernel<true><<<rgrid, R_THREADS, sizeof(RecSmem) + 1024, st>>>(mapCK, mapBKT, rp);
-    *launches += 1;
-    rp.out = vbuf; rp.r = L.r_v;
-    lorc_reconstruct_kernel<false><<<rgrid, R_THREADS, sizeof(RecSmem) + 1024, st>>>(mapCV, mapBVT128, rp);
-    *launches += 1;
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-
     CUtensorMap mapQ, mapK, mapV;
     {
         // q [b, T, H_q, 128]: box = 64 elements x G heads x 128 / G positions
@@ -685,12 +705,24 @@ cudaError_t lorc_tc_prefill_launch(lorc_ctx* ctx, const LorcLayer& L, const Cach
         if (!lorc_make_tmap_bf16(&mapK, khat, 3, kd, ks, kb)) return cudaErrorInvalidValue;
         if (!lorc_make_tmap_bf16(&mapV, vbuf, 3, kd, ks, kb)) return cudaErrorInvalidValue;
     }
+
+    RecParams rp;
+    rp.seq_lens = cv.seq_lens; rp.page_table = cv.page_table; rp.rope_table = ctx->rope_table; rp.status = ctx->status_dev;
+    rp.r_k = L.r_k; rp.r_v = L.r_v; rp.n_rows = (int)rows; rp.max_pos = d.max_pos;
+    rp.page_size = cv.page_size; rp.max_pages_per_seq = cv.max_pages_per_seq; rp.n_pages = cv.n_pages;
+    rp.batch = cv.batch; rp.tile_pairs = (tiles + 1) / 2; rp.n_hp = d.n_kv_heads / 2;
+    const int units = 2 * cv.batch * rp.tile_pairs * rp.n_hp;
+    const int pairs = units < ctx->sm_count / 2 ? units : ctx->sm_count / 2;
+    e = lorc_launch_dependent(lorc_reconstruct_kernel, dim3(2 * pairs), dim3(R_THREADS), sizeof(RecSmem) + 1024, st, mapCK, mapCV,
+                              mapBKT, mapBVT128, mapK, mapV, rp);
+    *launches += 1;
+    if (e != cudaSuccess) return e;
+
     FaParams fp;
     fp.out = out; fp.seq_lens = cv.seq_lens; fp.rope_table = ctx->rope_table; fp.status = ctx->status_dev;
     fp.T = T; fp.H_q = d.n_q_heads; fp.G = ctx->group; fp.n_rows = (int)rows; fp.max_pos = d.max_pos;
     const int qp = 2 * TILE / ctx->group;                      // query positions per CTA (two blocks of 128 rows)
     dim3 fgrid((T + qp - 1) / qp, d.n_kv_heads, cv.batch);
-    lorc_prefill_attn_kernel<<<fgrid, F_THREADS, sizeof(FaSmem) + 1024, st>>>(mapQ, mapK, mapV, fp);
     *launches += 1;
-    return cudaGetLastError();
+    return lorc_launch_dependent(lorc_prefill_attn_kernel, fgrid, dim3(F_THREADS), sizeof(FaSmem) + 1024, st, mapQ, mapK, mapV, fp);
 }
