@@ -126,6 +126,7 @@ cudaError_t lorc_generic_append(const lorc_ctx* ctx, const LorcLayer& L, const C
 // Uncompressed mode, 128-wide heads, bf16 path: streaming decode kernel on mma.sync (full_decode.cu).  Leaves the same
 // per-split partial results as the plain kernel, for lorc_generic_combine.
 bool lorc_full_decode_supported(const lorc_ctx* ctx, const LorcLayer& L);
+int lorc_full_decode_splits(const lorc_ctx* ctx, int batch, int max_seq_len);
 cudaError_t lorc_full_decode(const lorc_ctx* ctx, const CacheView& cv, const bf16* q, int n_splits, float* part_ml,
                              float* part_o, cudaStream_t st, int* launches);
 // Compressed layers, one query per sequence, bf16 path: the plain computation with mma.sync reconstruction (small_decode.cu).
@@ -154,17 +155,5 @@ cudaError_t lorc_generic_combine(const lorc_ctx* ctx, const LorcLayer& L, int ba
 #define LORC_MAX_SPLITS 256
 // tokens per step of the small-shape decode kernel
 #define LORC_SMALL_TILE 64
-// Default number of context splits for one layer: about 512 tokens each; where the small-shape kernel runs, as many as give
-// two blocks per SM, down to one step each.
-static inline int lorc_default_splits(int max_seq_len, int sm_count, int batch, int n_kv_heads, bool small) {
-    int s = (max_seq_len + 511) / 512;
-    if (small) {
-        int fill = (2 * sm_count + batch * n_kv_heads - 1) / (batch * n_kv_heads);
-        const int steps = (max_seq_len + LORC_SMALL_TILE - 1) / LORC_SMALL_TILE;
-        if (fill > steps) fill = steps;
-        if (s < fill) s = fill;
-    }
-    if (s < 1) s = 1;
-    if (s > LORC_MAX_SPLITS) s = LORC_MAX_SPLITS;
-    return s;
-}
+// Default number of context splits of a call on this layer (before it is lowered to what the scratch holds).
+int lorc_default_splits(const lorc_ctx* ctx, const LorcLayer& L, int batch, int max_seq_len);

@@ -15,6 +15,9 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "sm100_ptx.cuh"
+
+using namespace sm100;
 
 namespace {
 
@@ -85,6 +88,8 @@ full_decode_mma_kernel(const bf16* __restrict__ q, CacheView cv, int G, int n_sp
     const int g = lane >> 2, t = lane & 3;            // fragment row / column group of this lane
     const int split = blockIdx.x, kvh = blockIdx.y, s = blockIdx.z;
     const int H_q = G * (int)gridDim.y;
+    grid_dep_wait();
+    grid_dep_launch();
     int len = cv.seq_lens[s];
     if (len > max_pos) {
         if (tid == 0) lorc_set_status(status, LORC_ERR_CAPACITY);
@@ -281,6 +286,15 @@ bool lorc_full_decode_supported(const lorc_ctx* ctx, const LorcLayer& L) {
            !(ctx->desc.flags & LORC_FLAG_DEBUG_FP32);
 }
 
+// Context shares: as many as are resident at once (three blocks per SM), so that every block streams from the start to the
+// end of the launch; down to one 64-token step each.  (With 512 tokens per share, b 16 x 8 KV heads x 4129 tokens were 1152
+// blocks in 2.6 rounds, each with its own ramp: 64 us, 55 us now.)
+int lorc_full_decode_splits(const lorc_ctx* ctx, int batch, int max_seq_len) {
+    const long long units = (long long)batch * ctx->desc.n_kv_heads;
+    const long long fill = 3ll * ctx->sm_count / units, steps = (max_seq_len + FD_TILE - 1) / FD_TILE;
+    return (int)(fill < 1 ? 1 : fill < steps ? fill : steps);
+}
+
 cudaError_t lorc_full_decode(const lorc_ctx* ctx, const CacheView& cv, const bf16* q, int n_splits, float* part_ml,
                              float* part_o, cudaStream_t st, int* launches) {
     const lorc_model_desc& d = ctx->desc;
@@ -295,8 +309,7 @@ cudaError_t lorc_full_decode(const lorc_ctx* ctx, const CacheView& cv, const bf1
         if (e != cudaSuccess) return e;
         if (known) attr[ctx->device] = true;
     }
-    full_decode_mma_kernel<<<grid, 128, sizeof(FdSmem), st>>>(q, cv, ctx->group, n_splits, ctx->pair_style, ctx->rope_table, d.max_pos,
-                                                 part_ml, part_o, ctx->status_dev);
     *launches += 1;
-    return cudaGetLastError();
+    return lorc_launch_dependent(full_decode_mma_kernel, grid, dim3(128), sizeof(FdSmem), st, q, cv, ctx->group, n_splits,
+                                 ctx->pair_style, (const float2*)ctx->rope_table, d.max_pos, part_ml, part_o, ctx->status_dev);
 }

@@ -30,6 +30,19 @@ void free_layer(LorcLayer& L) {
     L = LorcLayer();
 }
 
+int clamp_splits(long long s) { return s < 1 ? 1 : s > LORC_MAX_SPLITS ? LORC_MAX_SPLITS : (int)s; }
+
+// The scalar kernels' default: about 512 tokens per split.
+int plain_splits(int max_seq_len) { return clamp_splits((max_seq_len + 511) / 512); }
+
+// Where the small-shape kernel runs: as many as give two blocks per SM, down to one step each.
+int small_splits(const lorc_ctx* ctx, int batch, int max_seq_len) {
+    const long long units = (long long)batch * ctx->desc.n_kv_heads;
+    const long long fill = (2 * ctx->sm_count + units - 1) / units, steps = (max_seq_len + LORC_SMALL_TILE - 1) / LORC_SMALL_TILE;
+    const int s = clamp_splits(fill < steps ? fill : steps), p = plain_splits(max_seq_len);
+    return s > p ? s : p;
+}
+
 struct WsLayout {
     size_t off_ml, off_o, total;
 };
@@ -102,6 +115,12 @@ int get_layer(lorc_ctx* ctx, int layer, LorcLayer** L) {
 }
 
 }  // namespace
+
+int lorc_default_splits(const lorc_ctx* ctx, const LorcLayer& L, int batch, int max_seq_len) {
+    if (lorc_full_decode_supported(ctx, L)) return clamp_splits(lorc_full_decode_splits(ctx, batch, max_seq_len));
+    if (lorc_small_decode_supported(ctx, L)) return small_splits(ctx, batch, max_seq_len);
+    return plain_splits(max_seq_len);
+}
 
 extern "C" {
 
@@ -229,13 +248,9 @@ int lorc_load_factors(lorc_ctx* ctx, int layer, int mode, int r_k, int r_v, cons
 
 size_t lorc_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_len) {
     if (!ctx || batch <= 0 || max_seq_len <= 0) return 0;
-    int S = lorc_default_splits(max_seq_len, ctx->sm_count, batch, ctx->desc.n_kv_heads, false);
-    size_t gen = ws_layout(ctx, batch, S, ctx->n).total;
-    if (!lorc_tc_workspace_bytes(ctx, batch, max_seq_len)) {
-        // the small-shape kernel takes more, shorter shares
-        S = lorc_default_splits(max_seq_len, ctx->sm_count, batch, ctx->desc.n_kv_heads, true);
-        gen = ws_layout(ctx, batch, S, ctx->n).total;
-    }
+    // (no tcgen05 kernels for this geometry: the small-shape kernel takes more, shorter shares than the plain ones)
+    const bool small = !lorc_tc_workspace_bytes(ctx, batch, max_seq_len);
+    size_t gen = ws_layout(ctx, batch, small ? small_splits(ctx, batch, max_seq_len) : plain_splits(max_seq_len), ctx->n).total;
     size_t tc = lorc_align_up(lorc_tc_workspace_bytes(ctx, batch, max_seq_len), 256);
     return (gen > tc ? gen : tc) + staging_bytes(ctx, batch) + 256;
 }
@@ -319,9 +334,7 @@ static int decode_attn_impl(lorc_ctx* ctx, int layer, const lorc_cache* cache, c
         return LORC_OK;
     }
 
-    int S = n_splits > 0 ? n_splits
-                         : lorc_default_splits(cv.max_seq_len, ctx->sm_count, cv.batch, ctx->desc.n_kv_heads,
-                                               lorc_small_decode_supported(ctx, *L));
+    int S = n_splits > 0 ? n_splits : lorc_default_splits(ctx, *L, cv.batch, cv.max_seq_len);
     int tiles = (cv.max_seq_len + LORC_GENERIC_TILE - 1) / LORC_GENERIC_TILE;
     if (S > tiles) S = tiles;
     if (S > LORC_MAX_SPLITS) S = LORC_MAX_SPLITS;
@@ -370,7 +383,7 @@ int lorc_merge_shards(lorc_ctx* ctx, int n_shards, const void* outs, const float
 
 size_t lorc_prefill_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_len, int T) {
     if (!ctx || batch <= 0 || max_seq_len <= 0 || T <= 0) return 0;
-    int S = lorc_default_splits(max_seq_len, ctx->sm_count, batch, ctx->desc.n_kv_heads, false);
+    int S = plain_splits(max_seq_len);
     size_t gen = ws_layout(ctx, batch * T, S, ctx->n).total;
     size_t tc = lorc_tc_prefill_shape_ok(ctx) ? lorc_tc_prefill_scratch_bytes(ctx, batch, max_seq_len, T) : 0;
     return (gen > tc ? gen : tc) + 256;
@@ -404,7 +417,7 @@ int lorc_prefill_attn(lorc_ctx* ctx, int layer, const lorc_cache* cache, const v
     // plain kernels: every (sequence, query) is a decode query over the sequence cut after its own token
     const bool latent = (L->mode == LORC_MODE_LATENT);
     const int W = latent ? L->r_v : ctx->desc.d_head;
-    int S = lorc_default_splits(cv.max_seq_len, ctx->sm_count, cv.batch, ctx->desc.n_kv_heads, false);
+    int S = plain_splits(cv.max_seq_len);
     int tiles = (cv.max_seq_len + LORC_GENERIC_TILE - 1) / LORC_GENERIC_TILE;
     if (S > tiles) S = tiles;
     while (S > 1 && ws_layout(ctx, cv.batch * T, S, W).total > ctx->ws_bytes) --S;

@@ -76,9 +76,7 @@ extern "C" int lorc_decode_attn_static(lorc_ctx* ctx, int layer, const lorc_cach
 
     const bool latent = (L.mode == LORC_MODE_LATENT);
     const int W = latent ? L.r_v : ctx->desc.d_head;
-    int S = n_splits > 0 ? n_splits
-                         : lorc_default_splits(c->max_seq_len, ctx->sm_count, c->batch, ctx->desc.n_kv_heads,
-                                               lorc_small_decode_supported(ctx, L));
+    int S = n_splits > 0 ? n_splits : lorc_default_splits(ctx, L, c->batch, c->max_seq_len);
     int tiles = (c->max_seq_len + LORC_GENERIC_TILE - 1) / LORC_GENERIC_TILE;
     if (S > tiles) S = tiles;
     if (S > LORC_MAX_SPLITS) S = LORC_MAX_SPLITS;
