@@ -127,8 +127,8 @@ cudaError_t lorc_generic_append(const lorc_ctx* ctx, const LorcLayer& L, const C
 // per-split partial results as the plain kernel, for lorc_generic_combine.
 bool lorc_full_decode_supported(const lorc_ctx* ctx, const LorcLayer& L);
 int lorc_full_decode_splits(const lorc_ctx* ctx, int batch, int max_seq_len);
-cudaError_t lorc_full_decode(const lorc_ctx* ctx, const CacheView& cv, const bf16* q, int n_splits, float* part_ml,
-                             float* part_o, cudaStream_t st, int* launches);
+cudaError_t lorc_full_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* q, int n_splits,
+                             float* part_ml, float* part_o, cudaStream_t st, int* launches);
 // Compressed layers, one query per sequence, bf16 path: the plain computation with mma.sync reconstruction (small_decode.cu).
 // Leaves the same per-split partial results too.
 bool lorc_small_decode_supported(const lorc_ctx* ctx, const LorcLayer& L);
@@ -138,7 +138,7 @@ cudaError_t lorc_small_decode(const lorc_ctx* ctx, const LorcLayer& L, const Cac
 // latent_out: stop before the value up-projection and write the normalised latent output [b, H_q, r_v] to `out`.
 // T > 1: T queries per sequence (q, out [b, T, H_q, d_head]; partial results for b * T units), query t of a sequence
 // at position seq_lens[s] - T + t, attending to the tokens up to its own.
-cudaError_t lorc_generic_decode(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv,
+cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv,
                                 const bf16* q, bf16* out, int n_splits, float* part_ml,
                                 float* part_o, cudaStream_t st, int* launches, bool latent_out = false, int T = 1,
                                 const int32_t* pos0 = nullptr, const int32_t* q_pos = nullptr, float* ml_out = nullptr);

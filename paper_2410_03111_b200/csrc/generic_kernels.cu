@@ -481,7 +481,7 @@ cudaError_t lorc_generic_combine(const lorc_ctx* ctx, const LorcLayer& L, int ba
                                  out, W, ctx->n, up ? d.d_head : W, ctx->group, n_splits, ctx->status_dev, ml_out);
 }
 
-cudaError_t lorc_generic_decode(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv,
+cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv,
                                 const bf16* q, bf16* out, int n_splits, float* part_ml,
                                 float* part_o, cudaStream_t st, int* launches, bool latent_out, int T,
                                 const int32_t* pos0, const int32_t* q_pos, float* ml_out) {
@@ -493,7 +493,7 @@ cudaError_t lorc_generic_decode(const lorc_ctx* ctx, const LorcLayer& L, const C
         // uncompressed mode with 128-wide heads: the streaming kernel on the warp-level tensor cores
         {
             LorcStageTimer timer(ctx, LORC_STAGE_SCORE, st);
-            cudaError_t e = lorc_full_decode(ctx, cv, q, n_splits, part_ml, part_o, st, launches);
+            cudaError_t e = lorc_full_decode(ctx, L, cv, q, n_splits, part_ml, part_o, st, launches);
             if (e != cudaSuccess) return e;
         }
         return lorc_generic_combine(ctx, L, cv.batch, n_splits, part_ml, part_o, out, st, launches, false, nullptr);

@@ -109,8 +109,8 @@ size_t lorc_tc_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_len) 
            lorc_tc_pv_scratch_bytes(ctx, batch, max_seq_len);
 }
 
-static bool build_cache_maps(LorcTcLayer& T, const LorcLayer& L, const CacheView& cv) {
-    long long key[6] = {cv.page_table ? 1 : 0, cv.seq_stride, cv.batch, cv.page_size, cv.n_pages, L.r_k * 4096LL + L.r_v};
+static bool build_cache_maps(LorcTcLayer& T, const LorcLayer& L, const CacheView& cv, int box_rows) {
+    long long key[6] = {(cv.page_table ? 1 : 0) + 2 * box_rows, cv.seq_stride, cv.batch, cv.page_size, cv.n_pages, L.r_k * 4096LL + L.r_v};
     bool same = T.k_ptr == cv.k && T.v_ptr == cv.v;
     for (int i = 0; i < 6; ++i) same = same && key[i] == T.key_dims[i];
     if (same) return true;
@@ -122,17 +122,25 @@ static bool build_cache_maps(LorcTcLayer& T, const LorcLayer& L, const CacheView
         if (cv.page_table == nullptr) {
             dims[0] = r; dims[1] = (uint64_t)cv.seq_stride; dims[2] = cv.batch;
             str[0] = (uint64_t)r * 2; str[1] = (uint64_t)cv.seq_stride * r * 2;
-            box[0] = KC; box[1] = TILE; box[2] = 1;
+            box[0] = KC; box[1] = box_rows; box[2] = 1;
         } else {
             dims[0] = r; dims[1] = cv.page_size; dims[2] = cv.n_pages;
             str[0] = (uint64_t)r * 2; str[1] = (uint64_t)cv.page_size * r * 2;
-            box[0] = KC; box[1] = cv.page_size; box[2] = 1;
+            box[0] = KC; box[1] = box_rows; box[2] = 1;
         }
         if (!lorc_make_tmap_bf16(which ? &T.mapCV : &T.mapCK, base, 3, dims, str, box)) return false;
     }
     T.k_ptr = cv.k;
     T.v_ptr = cv.v;
     for (int i = 0; i < 6; ++i) T.key_dims[i] = key[i];
+    return true;
+}
+
+bool lorc_tc_full_maps(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int box_rows, CUtensorMap** mapK, CUtensorMap** mapV) {
+    LorcTcLayer& T = tc_state(ctx)->layers[&L - ctx->layers.data()];
+    if (!build_cache_maps(T, L, cv, box_rows)) return false;
+    *mapK = &T.mapCK;
+    *mapV = &T.mapCV;
     return true;
 }
 
@@ -165,7 +173,7 @@ static cudaError_t tc_prepare(lorc_ctx* ctx, LorcTcState* T, LorcTcLayer& TL, co
         if (!lorc_make_tmap_bf16(&TL.mapBVT128, L.B_vT, 2, d2, s2, b3)) return cudaErrorInvalidValue;
         TL.has_bkt = true;
     }
-    if (!build_cache_maps(TL, L, cv)) return cudaErrorInvalidValue;
+    if (!build_cache_maps(TL, L, cv, cv.page_table ? cv.page_size : TILE)) return cudaErrorInvalidValue;
 
     return cudaSuccess;
 }

@@ -99,6 +99,10 @@ cudaError_t lorc_tc_prefill(lorc_ctx* ctx, int layer, const LorcLayer& L, const 
 cudaError_t lorc_fast_retile_factor(const bf16* A_cat, bf16* A_tiled, int D, int R, int pair_cols, int d_head,
                                     cudaStream_t st);
 
+// Tensor maps of an uncompressed layer's cache: boxes of 64 columns x box_rows tokens, 128-byte swizzle.  They are kept with
+// the layer and encoded again when the cache's pointers or geometry change.
+bool lorc_tc_full_maps(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int box_rows, CUtensorMap** mapK, CUtensorMap** mapV);
+
 // Drop cached per-layer state (tensor maps) when factors are reloaded / the context dies.
 void lorc_tc_invalidate_layer(lorc_ctx* ctx, int layer);
 void lorc_tc_release(lorc_ctx* ctx);

@@ -1,0 +1,73 @@
+"""Streaming decode kernel of uncompressed layers: edges of steps and shares, page sizes that cut a step into boxes, head
+counts, and cache rows past the sequence that hold NaN.
+
+Probabilities are rounded to bf16 (2^-9 relative each, of random sign) and the output once more: the observed row error is
+2.3e-3, the bound the repository's bf16 tolerance of 1e-2."""
+import numpy as np
+import pytest
+
+from oracle import lorc_oracle as O
+from workloads import synth
+
+import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H_q,H_kv,lens,style,page,n_splits", [
+    (8, 1, [1, 15, 16, 17, 63, 64, 65], 0, 0, 0),
+    (8, 8, [129, 700], 1, 48, 3),                  # one head per KV head; four boxes of 16 rows, pages no power of two
+    (12, 4, [200, 64], 0, 32, 0),                  # three heads per KV head, boxes of 32
+    (32, 8, [1000, 1], 1, 64, 1),                  # one share: every stage is reused
+    (64, 8, [333, 448], 2, 128, 40),               # eight heads per KV head, more shares than steps
+    (6, 3, [97], 0, 16, 2),
+])
+def test_full_decode(H_q, H_kv, lens, style, page, n_splits):
+    import torch
+    L = H.lib()
+    rng = np.random.default_rng(H_q + len(lens))
+    n, b, n_max = H_kv * 128, len(lens), max(lens) + 70
+    ctx = L.lorc_create(1, 256, H_q, H_kv, 128, 10000.0, rope_style=style, max_pos=n_max)
+    w = torch.zeros(256, n, dtype=torch.bfloat16, device="cuda")
+    L.lorc_load_factors(ctx, 0, L.LORC_MODE_FULL, 0, 0, w, None, w, None)
+    ws = torch.zeros(L.lorc_workspace_bytes(ctx, b, n_max), dtype=torch.uint8, device="cuda")
+    L.lorc_set_workspace(ctx, ws)
+    rows = [[synth.to_bf16_exact(rng.standard_normal((m, n))) for m in lens] for _ in "kv"]
+    sl = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    if page:
+        per = (n_max + page - 1) // page
+        table = rng.permutation(b * per + 1)[:b * per].reshape(b, per).astype(np.int32)
+        kv = []
+        for which in rows:
+            c = torch.full((b * per + 1, page, n), float("nan"), dtype=torch.bfloat16, device="cuda")
+            for s, r in enumerate(which):
+                for i in range(0, lens[s], page):
+                    part = H.dev_bf16(r[i:i + page])
+                    c[int(table[s, i // page]), :part.shape[0]] = part
+            kv.append(c)
+        tab = torch.from_numpy(table).cuda()
+        cache = L.make_cache(*kv, sl, b, max(lens), page_table=tab, page_size=page, max_pages_per_seq=per, n_pages=b * per + 1)
+    else:
+        kv = []
+        for which in rows:
+            c = torch.full((b, n_max, n), float("nan"), dtype=torch.bfloat16, device="cuda")
+            for s, r in enumerate(which):
+                c[s, :lens[s]] = H.dev_bf16(r)
+            kv.append(c)
+        cache = L.make_cache(*kv, sl, b, max(lens), seq_stride=n_max)
+    for q_scale in (1.0, 8.0):
+        q = synth.queries(b, H_q, 128, 35, int(q_scale), q_scale).astype(np.float64)
+        for entry in (L.lorc_decode_attn, L.lorc_decode_attn_static):
+            out = torch.full((b, H_q, 128), 3.0, dtype=torch.bfloat16, device="cuda")
+            entry(ctx, 0, cache, H.dev_bf16(q), out, n_splits=n_splits)
+            assert L.lorc_sync_status(ctx) == 0, L.lorc_last_error(ctx)
+            assert L.lorc_last_path(ctx) == 3
+            for s, m in enumerate(lens):
+                k, v = (which[s].astype(np.float64).reshape(m, H_kv, 128) for which in rows)
+                qs = q[s]
+                if style == H.ROPE_NONE:
+                    want = O.attention_one_query(qs, k, v)
+                else:
+                    want = O.decode_attn_cached_kv(k, v, qs, 10000.0, style)
+                H.assert_rows_close(H.host_f64(out[s]), want, 1e-2, (lens, s))
+    L.lorc_destroy(ctx)
