@@ -113,10 +113,25 @@ def _ptr(t):
     return t.data_ptr()
 
 
+_current_stream = None     # () -> handle of the current device's current stream; set by the first call that needs it
+
+
+def _find_current_stream():
+    """torch.cuda.current_stream().cuda_stream without the stream object (3.3 us a call; the raw getters 0.4 us)."""
+    global _current_stream
+    import torch
+    handle = torch.cuda.current_stream().cuda_stream      # initialises CUDA
+    get, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if get is None or device is None:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+    else:
+        _current_stream = lambda: get(device())
+    return handle
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream() if _current_stream is not None else _find_current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
