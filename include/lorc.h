@@ -263,7 +263,8 @@ int lorc_decode_attn_static(lorc_ctx* ctx, int layer, const lorc_cache* cache, c
  * q_host [batch, n_q_heads, d_head] to staging at the end of the workspace, runs
  * lorc_append (T = 1) and lorc_decode_attn, and copies the result to out_host
  * [batch, n_q_heads, d_head]; all on `stream`, asynchronously when the host
- * buffers are pinned.  The caller synchronises the stream before reading
+ * buffers are pinned.  (Pinned, mapped and 16-byte aligned buffers are read and
+ * written by the kernels themselves, others by copies.)  The caller synchronises the stream before reading
  * out_host.  The cache stays on the device. */
 int lorc_decode_step_host(lorc_ctx* ctx, int layer, const lorc_cache* cache, const void* x_host,
                           const void* q_host, void* out_host, int n_splits, void* stream);
