@@ -61,6 +61,7 @@ struct lorc_ctx {
     size_t ws_bytes = 0;
     std::string err;
     int last_path = 0;
+    bool host_out = false;         // the call in progress writes its result to mapped host memory
     int64_t launches = 0;
     LorcTcState* tc = nullptr;
     LorcProfile* prof = nullptr;   // event bookkeeping, created on first use

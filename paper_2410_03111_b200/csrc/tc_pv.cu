@@ -488,9 +488,13 @@ constexpr int U_THREADS = 192;
 constexpr int U_NCOL = 32;           // output columns per CTA (a quarter of a head)
 constexpr int U_ROWS = 64;           // output rows (sequence, head of the KV head) per CTA: the M of the MMA
 
+constexpr int U_LD = 80;             // bytes per row of the transposition buffer (64 and padding)
+
+template <bool HOST>
 struct UpSmem {
     bf16 A[U_STAGES][U_ROWS * KC];        // o_norm rows [64 rows (s, i)][64 rho]
     bf16 B[U_STAGES][U_NCOL * KC];        // B_V^T slice [32 columns j][64 rho]
+    uint8_t O[HOST ? 4 : 0][16 * U_LD];   // HOST: per epilogue warp: 16 finished rows of 64 bytes
     uint64_t full[U_STAGES], empty[U_STAGES], d_full;
     uint32_t tmem_base;
 };
@@ -503,11 +507,14 @@ struct UpParams {
     int parts, r_pad;              // bf16 parts of the latent rows (the second one r_pad columns after the first)
 };
 
+// HOST: `out` is mapped host memory
+template <bool HOST>
 __global__ void __launch_bounds__(U_THREADS, 1)
 lorc_upproj_kernel(const __grid_constant__ CUtensorMap mapON, const __grid_constant__ CUtensorMap mapBVT,
                    const UpParams p) {
     extern __shared__ uint8_t raw[];
-    UpSmem& sm = *reinterpret_cast<UpSmem*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+    typedef UpSmem<HOST> S;
+    S& sm = *reinterpret_cast<S*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int g = blockIdx.x, chunk = blockIdx.y, cq = blockIdx.z;     // KV head, block of 64 rows, column quarter
     const int nslice = (p.r_v + KC - 1) / KC, nkc = nslice * p.parts;    // slices of the rank, of the contraction
@@ -589,28 +596,39 @@ lorc_upproj_kernel(const __grid_constant__ CUtensorMap mapON, const __grid_const
         if (!mbar_wait(&sm.d_full, 0)) ok = false;
         if (ok) {
             tc_fence_after_sync();
-            // A 64-row accumulator keeps row 16 q + i (i < 16) in lane i of lane quarter q; row = s_local * G + i
+            // A 64-row accumulator keeps row 16 q + i (i < 16) in lane i of lane quarter q; row = s_local * G + i.  A lane stores
+            // its row's 64 bytes, unless `out` lies in host memory, where a store of 16 bytes is a bus transaction of
+            // its own (20 us for 131 KB): there the rows go through shared memory and leave with four lanes per row (12 us).
             const int quarter = warp % 4;
-            const int row = quarter * 16 + (lane & 15);
-            const bool has_row = lane < 16;
-            const int s = chunk * seqs_per_cta + row / p.G, h = g * p.G + row % p.G;
-            {
-                uint32_t r[32];
-                tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16), r);
-                tmem_wait_ld();
-                if (has_row && s < p.batch) {
-                    uint4* dst = reinterpret_cast<uint4*>(p.out + ((long long)s * p.H_q + h) * 128 + cq * U_NCOL);
+            uint32_t r[32];
+            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16), r);
+            tmem_wait_ld();
+            auto row_of = [&](int row) -> uint4* {
+                const int s = chunk * seqs_per_cta + row / p.G, h = g * p.G + row % p.G;
+                return s < p.batch ? reinterpret_cast<uint4*>(p.out + ((long long)s * p.H_q + h) * 128 + cq * U_NCOL) : nullptr;
+            };
+            uint4* dst = row_of(quarter * 16 + (lane & 15));
+            if constexpr (HOST) dst = reinterpret_cast<uint4*>(sm.O[warp - 2] + lane * U_LD);
+            if (lane < 16 && dst) {
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        uint32_t w[4];
+                for (int q4 = 0; q4 < 4; ++q4) {
+                    uint32_t w[4];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(r[q4 * 8 + 2 * e]),
-                                                                     __uint_as_float(r[q4 * 8 + 2 * e + 1]));
-                            w[e] = *reinterpret_cast<uint32_t*>(&b);
-                        }
-                        dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
+                    for (int e = 0; e < 4; ++e) {
+                        __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(r[q4 * 8 + 2 * e]),
+                                                                 __uint_as_float(r[q4 * 8 + 2 * e + 1]));
+                        w[e] = *reinterpret_cast<uint32_t*>(&b);
                     }
+                    dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+            if constexpr (HOST) {
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int lr = i * 8 + (lane >> 2);
+                    uint4* to = row_of(quarter * 16 + lr);
+                    if (to) to[lane & 3] = *reinterpret_cast<const uint4*>(sm.O[warp - 2] + lr * U_LD + (lane & 3) * 16);
                 }
             }
         }
@@ -699,7 +717,8 @@ cudaError_t lorc_tc_pv_set_attrs() {
     if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>));
     if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>));
     if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>));
-    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel, sizeof(UpSmem));
+    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel<false>, sizeof(UpSmem<false>));
+    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel<true>, sizeof(UpSmem<true>));
     return e;
 }
 
@@ -777,7 +796,8 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
     u.batch = cv.batch; u.H_q = d.n_q_heads; u.G = ctx->group; u.r_v = L.r_v;
     u.parts = split ? 2 : 1; u.r_pad = r_pad;
     dim3 ugrid(d.n_kv_heads, (cv.batch * ctx->group + U_ROWS - 1) / U_ROWS, 128 / U_NCOL);
-    e = lorc_launch_dependent(lorc_upproj_kernel, ugrid, dim3(U_THREADS), sizeof(UpSmem) + 1024, st, mapON, mapBVT, u);
+    e = ctx->host_out ? lorc_launch_dependent(lorc_upproj_kernel<true>, ugrid, dim3(U_THREADS), sizeof(UpSmem<true>) + 1024, st, mapON, mapBVT, u)
+                      : lorc_launch_dependent(lorc_upproj_kernel<false>, ugrid, dim3(U_THREADS), sizeof(UpSmem<false>) + 1024, st, mapON, mapBVT, u);
     *launches += 1;
     return e;
 }
