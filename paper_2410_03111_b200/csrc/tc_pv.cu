@@ -653,19 +653,31 @@ __global__ void latent_out_kernel(const bf16* __restrict__ o_norm, bf16* __restr
     }
 }
 
-// Column blocks and context shares of one PV launch: one CTA per SM, and as few context shares as fill the SMs once
-// (a CTA with four stages in flight pulls its share of the HBM bandwidth alone; fewer shares mean longer streams per
-// CTA and, at one share, no share reduction at all).
+// Column blocks and context shares of one PV launch: one CTA per SM at most, and the number of shares whose chain is shortest.
+// In units of one tile (about 0.45 us of a CTA's stream): the tiles of a share, and with more than one share 8 for publishing
+// it and taking turns at the counter and 0.8 per share for the addition by the last one.  So up to 16 tiles are best left to one
+// CTA, and more than about sqrt(tiles / 0.8) shares never pay.  (As many shares as fill the SMs, which was the rule before,
+// cost 2 to 3 us a call up to 16 tiles and most at long contexts of one user: 8B shape, one layer with its cache write, 8200
+// tokens, rank 256: 64 shares 41 us, 9 shares 26 us; 1037 tokens, rank 928: 9 shares 27.0 us, one 24.8 us.)
 void pv_plan(const lorc_ctx* ctx, const LorcLayer& L, int batch, int max_seq_len, int n_splits_hint, int* n_blk,
              int* n_csplit) {
     const int tiles = (max_seq_len + TILE - 1) / TILE;
     *n_blk = (L.r_v + 127) / 128;
-    const int slots = ctx->sm_count;
-    int cs = n_splits_hint > 0 ? n_splits_hint : slots / (batch * *n_blk);
-    if (cs > tiles) cs = tiles;
-    if (cs > 64) cs = 64;
-    if (cs < 1) cs = 1;
-    *n_csplit = cs;
+    int most = n_splits_hint > 0 ? n_splits_hint : ctx->sm_count / (batch * *n_blk);
+    if (most > tiles) most = tiles;
+    if (most > 64) most = 64;
+    if (most < 1) most = 1;
+    *n_csplit = most;
+    if (n_splits_hint > 0) return;
+    int best = 5 * tiles;                                     // five times the cost, in tiles
+    *n_csplit = 1;
+    for (int cs = 2; cs <= most; ++cs) {
+        const int cost = 5 * ((tiles + cs - 1) / cs + 8) + 4 * cs;
+        if (cost < best) {
+            best = cost;
+            *n_csplit = cs;
+        }
+    }
 }
 
 struct PvScratch {
