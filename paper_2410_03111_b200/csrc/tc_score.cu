@@ -31,7 +31,14 @@ constexpr int KC = 64;               // latent columns per pipeline stage
 constexpr float LOG2E = 1.4426950408889634f;
 
 constexpr int Q_STAGES = 6;
-constexpr int Q_THREADS = 352;       // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue, warp 10 query
+// warp 0 TMA, warp 1 MMA, warps 2..9 epilogue, warp 10 query.  Every scheduler has two epilogue warps that keep it busy, so
+// a single-warp role runs slowly: one producer warp takes 370 to 520 cycles per stage, with page lookups 830, against 512 of
+// MMAs, and where the rank is low the epilogue (about 3900 cycles per unit at G = 4, a part of it locating the unit and
+// waiting) is the longest role of all.  The LONG form, for launches of many rounds at such ranks, has a second producer warp
+// for the factor slices, looks pages up a unit ahead and lets the query warp locate each unit for the epilogue; it starts
+// 0.1 us later, so short launches keep the other form (see lorc_tc_score_launch).
+template <bool LONG>
+struct ScoreThreads { static constexpr int value = LONG ? 384 : 352; };
 constexpr int Q_EPI_WARPS = 8;
 
 struct ScoreSmem {
@@ -40,6 +47,7 @@ struct ScoreSmem {
     float4 trig[33][32];                  // in-tile rotation table, see rope_tile_kernel                     16.5 KiB
     float qrot[2][2][1024];               // [buffer][head of pair][rotated, scaled query; see qrot_index]    16 KiB
     uint64_t full[Q_STAGES], empty[Q_STAGES], acc_full[2], acc_empty[2], q_full[2], q_empty[2], trig_full;
+    int4 unit[2];                         // LONG: of the query buffer: sequence, tile, length, head pair (-1: nothing to write)
     uint32_t tmem_base;
     int32_t tile_start[LORC_SCORE_MAX_BATCH + 1];   // first flat tile of every sequence
     int32_t lens[LORC_SCORE_MAX_BATCH];             // checked sequence lengths (0: nothing to do)
@@ -121,12 +129,13 @@ __device__ __forceinline__ int qrot_index(int j, int half, int g) {
 
 // SPLIT (interleaved rotary pairs): B_K^T lists the first members of a head's pairs, then the second ones, so that the
 // accumulator has the half-split layout; queries are read in pairs; numerators are written as two bf16 parts.
-template <int G, bool SPLIT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Q_THREADS, 1)
+template <int G, bool SPLIT, bool LONG>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ScoreThreads<LONG>::value, 1)
 lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_constant__ CUtensorMap mapBKT,
                   const ScoreParams p) {
     extern __shared__ uint8_t raw[];
     ScoreSmem& sm = *reinterpret_cast<ScoreSmem*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+    constexpr int Q_THREADS = ScoreThreads<LONG>::value;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int rank = (int)cluster_ctarank();           // 0 = leader (issues the MMAs, owns the full / acc_empty barriers)
     const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
@@ -209,35 +218,98 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
         const int b_row = rank * 128;
         uint32_t st = 0, par = 1;                            // stage and the parity its empty barrier is waited with
         bool ok = true;
-        for (Walk w(pair_id, n_pairs, p.n_hp); w.u < total_units && ok; w.next()) {
-            Unit un;
-            decode_unit(sm, w, rank, n_flat, p.batch, un);
-            const int row0 = un.tile * TILE, brow = un.hp * 256 + b_row, sg = p.seq0 + un.s;
+        if constexpr (LONG) {
+            // the latent slices only; the next unit is located behind this one's first boxes
             const int ppt = paged ? TILE / p.page_size : 0;
-            int pages[8];
-            if (paged) {
-                const int mine = lorc_tile_page(p.page_table, sg, un.tile, lane, un.len, p.page_size, p.max_pages_per_seq,
-                                                p.n_pages, p.status);
+            Walk w(pair_id, n_pairs, p.n_hp);
+            Unit un;
+            int mine = 0;                                    // this lane's page of the unit's tile
+            auto locate = [&]() {
+                decode_unit(sm, w, rank, n_flat, p.batch, un);
+                if (paged)
+                    mine = lorc_tile_page(p.page_table, p.seq0 + un.s, un.tile, lane, un.len, p.page_size, p.max_pages_per_seq,
+                                          p.n_pages, p.status);
+            };
+            if (w.u < total_units) locate();
+            while (w.u < total_units && ok) {
+                const int row0 = un.tile * TILE, sg = p.seq0 + un.s;
+                int pages[8];
+                if (paged) {
 #pragma unroll
-                for (int pg = 0; pg < 8; ++pg) pages[pg] = __shfl_sync(0xffffffffu, mine, pg);
+                    for (int pg = 0; pg < 8; ++pg) pages[pg] = __shfl_sync(0xffffffffu, mine, pg);
+                }
+                for (int x = 0; x < nkc * KC; x += KC) {
+                    if (!mbar_wait_addr(empty0 + st * 8, par)) { ok = false; break; }
+                    const uint32_t lead_bar = lead_full0 + st * 8;
+                    const uint32_t a_dst = a_base + st * (TILE * KC * 2);
+                    if (elect_one()) {
+                        if (rank == 0) mbar_arrive_expect_tx_addr(full0 + st * 8, 2 * 2 * TILE * KC * 2);
+                        if (!paged) {
+                            tma_load_3d_pair_addr(a_dst, &mapCK, lead_bar, x, row0, sg);
+                        } else {
+                            // one box per page
+#pragma unroll
+                            for (int pg = 0; pg < 8; ++pg) {
+                                if (pg >= ppt) break;
+                                tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, &mapCK, lead_bar, x, 0, pages[pg]);
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    if (++st == Q_STAGES) { st = 0; par ^= 1; }
+                    if (x == 0) {
+                        w.next();
+                        if (w.u < total_units) locate();
+                    }
+                }
             }
+        } else {
+            for (Walk w(pair_id, n_pairs, p.n_hp); w.u < total_units && ok; w.next()) {
+                Unit un;
+                decode_unit(sm, w, rank, n_flat, p.batch, un);
+                const int row0 = un.tile * TILE, brow = un.hp * 256 + b_row, sg = p.seq0 + un.s;
+                const int ppt = paged ? TILE / p.page_size : 0;
+                int pages[8];
+                if (paged) {
+                    const int mine = lorc_tile_page(p.page_table, sg, un.tile, lane, un.len, p.page_size, p.max_pages_per_seq,
+                                                    p.n_pages, p.status);
+#pragma unroll
+                    for (int pg = 0; pg < 8; ++pg) pages[pg] = __shfl_sync(0xffffffffu, mine, pg);
+                }
+                for (int x = 0; x < nkc * KC; x += KC) {
+                    if (!mbar_wait_addr(empty0 + st * 8, par)) { ok = false; break; }
+                    const uint32_t lead_bar = lead_full0 + st * 8;
+                    const uint32_t a_dst = a_base + st * (TILE * KC * 2);
+                    if (elect_one()) {
+                        if (rank == 0) mbar_arrive_expect_tx_addr(full0 + st * 8, 2 * 2 * TILE * KC * 2);
+                        if (!paged) {
+                            tma_load_3d_pair_addr(a_dst, &mapCK, lead_bar, x, row0, sg);
+                        } else {
+                            // one box per page
+#pragma unroll
+                            for (int pg = 0; pg < 8; ++pg)
+                                if (pg < ppt)
+                                    tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, &mapCK, lead_bar, x, 0, pages[pg]);
+                        }
+                        tma_load_2d_pair_addr(b_base + st * (128 * KC * 2), &mapBKT, lead_bar, x, brow);
+                    }
+                    __syncwarp();
+                    if (++st == Q_STAGES) { st = 0; par ^= 1; }
+                }
+            }
+        }
+        if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
+    } else if (LONG && warp == 11) {
+        // ------------------------------------------------------------------ TMA of this CTA's half of the factor slices
+        const uint32_t b_base = smem_u32(sm.B[0]), empty0 = smem_u32(&sm.empty[0]);
+        const uint32_t lead_full0 = mapa_shared(smem_u32(&sm.full[0]), 0);
+        uint32_t st = 0, par = 1;
+        bool ok = true;
+        for (int u = pair_id; u < total_units && ok; u += n_pairs) {
+            const int brow = (u % p.n_hp) * 256 + rank * 128;
             for (int x = 0; x < nkc * KC; x += KC) {
                 if (!mbar_wait_addr(empty0 + st * 8, par)) { ok = false; break; }
-                const uint32_t lead_bar = lead_full0 + st * 8;
-                const uint32_t a_dst = a_base + st * (TILE * KC * 2);
-                if (elect_one()) {
-                    if (rank == 0) mbar_arrive_expect_tx_addr(full0 + st * 8, 2 * 2 * TILE * KC * 2);
-                    if (!paged) {
-                        tma_load_3d_pair_addr(a_dst, &mapCK, lead_bar, x, row0, sg);
-                    } else {
-                        // one box per page
-#pragma unroll
-                        for (int pg = 0; pg < 8; ++pg)
-                            if (pg < ppt)
-                                tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, &mapCK, lead_bar, x, 0, pages[pg]);
-                    }
-                    tma_load_2d_pair_addr(b_base + st * (128 * KC * 2), &mapBKT, lead_bar, x, brow);
-                }
+                if (elect_one()) tma_load_2d_pair_addr(b_base + st * (128 * KC * 2), &mapBKT, lead_full0 + st * 8, x, brow);
                 __syncwarp();
                 if (++st == Q_STAGES) { st = 0; par ^= 1; }
             }
@@ -330,6 +402,7 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
                 *reinterpret_cast<float2*>(dst + qrot_index<G>(2 * lane, 1, g)) =
                     make_float2((a0 * cs.y + b0 * cs.x) * scale, (a1 * cs.w + b1 * cs.z) * scale);
             }
+            if (LONG && lane == 0) sm.unit[buf] = make_int4(un.s, un.tile, un.len, un.valid ? un.hp : -1);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.q_full[buf]);
         }
@@ -350,9 +423,13 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
         const uint64_t minus1 = f2_pack(-1.f, -1.f);
         for (Walk w(pair_id, n_pairs, p.n_hp); w.u < total_units && ok; w.next(), ++uc) {
             Unit un;
-            decode_unit(sm, w, rank, n_flat, p.batch, un);
+            if (!LONG) decode_unit(sm, w, rank, n_flat, p.batch, un);
             const int buf = uc & 1;
             if (!mbar_wait(&sm.q_full[buf], (uc >> 1) & 1)) { ok = false; break; }
+            if (LONG) {
+                const int4 v = sm.unit[buf];
+                un.s = v.x; un.tile = v.y; un.len = v.z; un.hp = v.w; un.valid = v.w >= 0;
+            }
             if (!mbar_wait(&sm.acc_full[buf], (uc >> 1) & 1)) { ok = false; break; }
             tc_fence_after_sync();
             // Packed fp32: every operation below acts on the thread's two adjacent rotary pairs (columns 2c, 2c + 1
@@ -524,12 +601,15 @@ __global__ void rope_tile_kernel(float2* out, double theta) {
 }  // namespace
 
 cudaError_t lorc_tc_score_set_attrs() {
-    const int bytes = (int)sizeof(ScoreSmem) + 1024;
-    cudaError_t e = cudaFuncSetAttribute(lorc_score_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(lorc_score_kernel<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(lorc_score_kernel<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(lorc_score_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    return e;
+    const void* kernels[] = {(const void*)lorc_score_kernel<4, false, false>, (const void*)lorc_score_kernel<4, false, true>,
+                             (const void*)lorc_score_kernel<4, true, false>,  (const void*)lorc_score_kernel<4, true, true>,
+                             (const void*)lorc_score_kernel<8, false, false>, (const void*)lorc_score_kernel<8, false, true>,
+                             (const void*)lorc_score_kernel<8, true, false>,  (const void*)lorc_score_kernel<8, true, true>};
+    for (const void* k : kernels) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ScoreSmem) + 1024);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t lorc_tc_rope_tile_fill(float2* table, double theta, cudaStream_t st) {
@@ -570,9 +650,23 @@ cudaError_t lorc_tc_score_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheV
         if (n_pairs < 1) n_pairs = 1;
         const size_t smem = sizeof(ScoreSmem) + 1024;
         const bool split = lorc_tc_split(ctx);
-        auto kernel = ctx->group == 4 ? (split ? lorc_score_kernel<4, true> : lorc_score_kernel<4, false>)
-                                      : (split ? lorc_score_kernel<8, true> : lorc_score_kernel<8, false>);
-        cudaError_t e = lorc_launch_dependent(kernel, dim3(2 * n_pairs), dim3(Q_THREADS), smem, st, mapCK, mapBKT, sp);
+        // LONG: from eight rounds of units at ranks where the epilogue, not the MMAs, sets the pace: 64 ragged sequences up to
+        // 16384 tokens, r 384, pages of 64: 560 -> 551 us a step; b 4, 32777 tokens, r 256, two layers: 222 -> 219; one round
+        // (b 1, 1037 tokens) is 0.6 % slower in it, 15 rounds at r 928 as fast.
+        auto launch = [&](auto kernel, int threads) {
+            return lorc_launch_dependent(kernel, dim3(2 * n_pairs), dim3(threads), smem, st, mapCK, mapBKT, sp);
+        };
+        auto pick = [&](auto short_form, auto long_form) {
+            return max_units >= 8ll * n_pairs && L.r_k <= 640 ? launch(long_form, ScoreThreads<true>::value)
+                                                              : launch(short_form, ScoreThreads<false>::value);
+        };
+        cudaError_t e;
+        if (ctx->group == 4)
+            e = split ? pick(lorc_score_kernel<4, true, false>, lorc_score_kernel<4, true, true>)
+                      : pick(lorc_score_kernel<4, false, false>, lorc_score_kernel<4, false, true>);
+        else
+            e = split ? pick(lorc_score_kernel<8, true, false>, lorc_score_kernel<8, true, true>)
+                      : pick(lorc_score_kernel<8, false, false>, lorc_score_kernel<8, false, true>);
         *launches += 1;
         if (e != cudaSuccess) return e;
     }
