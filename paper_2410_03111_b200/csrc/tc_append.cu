@@ -2,7 +2,7 @@
 //
 // C_K, C_V[new tokens] = bf16(x . [A_K | A_V])  (Sec. 3.1: the cache keeps X times the Sigma-carrying factor), one GEMM
 // with M = tokens, N = r_k + r_v, K = D.  At decode (a token per sequence) the call is bound by the factor stream and
-// runs on the warp-level kernel; from 128 tokens per launch on it is a dense contraction and runs here.
+// runs on the warp-level kernel; with more tokens it is a dense contraction and runs here.
 //
 // Persistent CTA pairs (clusters of two, cta_group::2 MMAs) walk units of 256 tokens x up to NB columns of [A_K | A_V].
 // K = D in 64-wide TMA stages; x rows are the K-major A operand (128 tokens per CTA), the factor rows (D index) with their
@@ -244,9 +244,17 @@ lorc_append_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
 
 }  // namespace
 
+// Whether a launch runs here.  The warp-level kernel takes one block per 8 columns and 16 tokens, two at a time on an SM, and its
+// time goes with the rounds of them; this one takes a time of its own up to 256 tokens (about 18 us at D 4096).  They cross at
+// three rounds, whatever the rank and D.  Cache write and attention of one prompt, warp-level against here: 8B shape, r 928,
+// 48 tokens 34.1 / 34.9 us, 64 tokens 38.9 / 35.9, 127 tokens 51.6 / 36.1; r 416, 127 tokens 33.2 / 33.4; r 128, 127 tokens
+// 22.8 / 31.7; D 8192, r 928, 64 tokens 50.8 / 46.3.  Where the warp-level kernel does not run (D not a multiple of 256), from
+// 128 tokens on.
 bool lorc_tc_append_gemm_supported(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int T) {
-    return L.mode == LORC_MODE_LATENT && (long long)cv.batch * T >= TILE && ctx->desc.d_model % KC == 0 &&
-           L.r_k % 8 == 0 && L.r_v % 8 == 0 && lorc_get_tmap_encode() != nullptr;
+    if (L.mode != LORC_MODE_LATENT || ctx->desc.d_model % KC || L.r_k % 8 || L.r_v % 8 || !lorc_get_tmap_encode()) return false;
+    const long long n_tok = (long long)cv.batch * T;
+    if (!lorc_tc_append_supported(ctx, L, cv, T)) return n_tok >= TILE;
+    return (L.r_k + L.r_v) / 8 * ((n_tok + 15) / 16) > 6ll * ctx->sm_count;
 }
 
 cudaError_t lorc_tc_append_gemm(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* x, int T,

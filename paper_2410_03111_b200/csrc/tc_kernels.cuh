@@ -21,7 +21,7 @@ cudaError_t lorc_tc_decode(lorc_ctx* ctx, int layer, const LorcLayer& L, const C
                            const int32_t* q_pos = nullptr, float* ml_out = nullptr);
 cudaError_t lorc_tc_append(lorc_ctx* ctx, int layer, const LorcLayer& L, const CacheView& cv,
                            const bf16* x, int T, cudaStream_t st, int* launches);
-// Cache write of compressed layers as a tcgen05 GEMM (tc_append.cu), for launches of at least 128 tokens.
+// Cache write of compressed layers as a tcgen05 GEMM (tc_append.cu), for prompt-sized launches.
 bool lorc_tc_append_gemm_supported(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int T);
 cudaError_t lorc_tc_append_gemm(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* x, int T,
                                 cudaStream_t st, int* launches);

@@ -11,11 +11,13 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("r_k,r_v,b,T,page", [
-    (8, 8, 1, 128, 0),            # 16 columns: one unit of 32, half a block per CTA
-    (96, 72, 2, 77, 16),          # 168 columns: a last block of 40, rounded up to 64; tokens of two sequences in a tile
+    (8, 8, 16, 447, 0),           # 16 columns: units of 32, half a block per CTA
+    (96, 72, 2, 357, 16),         # 168 columns: a last block of 40, rounded up to 64; tokens of two sequences in a tile
     (264, 256, 1, 257, 0),        # a third token block of one row
     (512, 512, 5, 333, 64),       # full-width units
     (928, 416, 1, 129, 128),
+    (928, 928, 1, 49, 0),         # fewer tokens than a CTA's half of a unit
+    (160, 128, 1, 200, 0),        # the warp-level kernel: fewer than three rounds of its blocks
     (1024, 1000, 16, 520, 0),     # more units than pairs: several rounds, both accumulators
 ])
 def test_prompt_sized_append(r_k, r_v, b, T, page):
