@@ -5,6 +5,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "host_range.cuh"
 #include "sm100_ptx.cuh"
 #include "tc_kernels.cuh"
 
@@ -449,20 +450,24 @@ stage_in_kernel(const uint4* __restrict__ x, uint4* __restrict__ x_d, int nx, co
         q_d[i - nx] = q[i - nx];
 }
 
-// Device address of a 16-byte aligned host buffer that kernels may access (pinned or registered as a whole, and mapped), or
-// null.
+// Device address of a host buffer that kernels may access (see lorc_mapped_address), or null.
 static void* mapped_host(const void* host, size_t bytes) {
-    if ((uintptr_t)host & 15) return nullptr;
-    cudaPointerAttributes first, last;
-    if (cudaPointerGetAttributes(&first, host) != cudaSuccess ||
-        cudaPointerGetAttributes(&last, (const char*)host + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer ||
-        (char*)last.devicePointer - (char*)first.devicePointer != (ptrdiff_t)bytes - 1 || ((uintptr_t)first.devicePointer & 15))
-        return nullptr;
-    return first.devicePointer;
+    typedef CUresult (*attributes_fn)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const attributes_fn attributes = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &p, cudaEnableDefault, &q) != cudaSuccess) cudaGetLastError();
+        return p && q == cudaDriverEntryPointSuccess ? (attributes_fn)p : (attributes_fn) nullptr;
+    }();
+    if (!attributes) return nullptr;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    LorcHostRange r = {};
+    size_t size = 0;
+    void* to[] = {&r.type, &r.managed, &r.device, &r.start, &size};
+    if (attributes(5, what, to, (CUdeviceptr)host) != CUDA_SUCCESS) return nullptr;
+    r.size = size;
+    return (void*)lorc_mapped_address(r, (uint64_t)host, bytes);
 }
 
 int lorc_decode_step_host(lorc_ctx* ctx, int layer, const lorc_cache* cache, const void* x_host,

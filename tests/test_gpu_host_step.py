@@ -53,3 +53,23 @@ def test_step_from_host_buffers(geom, kind):
     for a, c in zip(*results):
         assert torch.equal(a, c)
     sess.close()
+
+
+def test_pinned_buffers_need_one_staging_launch():
+    """A slice of a pinned allocation is staged by a kernel (one launch more than the copies need), a pageable buffer is not."""
+    import torch
+    prob = H.Problem(264, 4, 2, 64, 32, 24, layer=34)
+    sess = H.Session(prob, max_pos=64, batch=2)
+    L = sess.L
+    held = H.contiguous_cache(sess, 2, 64, [9, 40])
+    launches = []
+    for pinned in (True, False):
+        buf = torch.zeros(4096, dtype=torch.bfloat16)
+        buf = buf.pin_memory() if pinned else buf
+        x, q, out = buf[8:8 + 528].view(2, 264), buf[1024:1536].view(2, 4, 64), buf[2048:2560].view(2, 4, 64)
+        before = L.lorc_launch_count(sess.ctx)
+        L.lorc_decode_step_host(sess.ctx, 0, held[0], x, q, out)
+        assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+        launches.append(L.lorc_launch_count(sess.ctx) - before)
+    assert launches[0] == launches[1] + 1
+    sess.close()
