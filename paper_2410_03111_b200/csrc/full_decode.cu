@@ -79,6 +79,7 @@ struct FdSmem {
     float qs[8][FD_DH];                              // rotated, scaled queries of the G heads (rows G..7 zero)
     float m[4][8], l[4][8];
     uint64_t full[FD_STAGES], empty[FD_STAGES];
+    uint32_t dead[FD_STAGES];                        // boxes of the stage whose page lies outside the pool, one bit each
 };
 
 struct FdParams {
@@ -112,11 +113,11 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
     grid_dep_wait();
     grid_dep_launch();
     int len = cv.seq_lens[s];
-    if (len > p.max_pos || len > cv.capacity) {
-        if (tid == 0) lorc_set_status(p.status, LORC_ERR_CAPACITY);
-        len = 0;
-    }
-    if (len < 0) len = 0;
+    if ((len > p.max_pos || len > cv.capacity) && tid == 0) lorc_set_status(p.status, LORC_ERR_CAPACITY);
+    if (len < 0 || len > p.max_pos) len = 0;
+    const int q_pos = len - 1;
+    // tokens past the capacity, and those whose page lies outside the pool, are left out of the attention
+    if (len > cv.capacity) len = (int)cv.capacity;
     // this CTA's share of the context, in whole 64-token tiles
     const int tiles = (len + FD_TILE - 1) / FD_TILE;
     const int tps = (tiles + p.n_splits - 1) / p.n_splits;
@@ -129,14 +130,15 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
     if (warp == 4) {
         // ------------------------------------------------------------------ producer (one elected lane issues)
         const int nbox = FD_TILE / p.box_rows;        // boxes per tile and half: 1, or up to 4 on small pages
-        // lane i < nbox: the page of the tile's i-th box (a table entry outside the pool: page 0, and the error is reported)
+        // lane i < nbox: the page of the tile's i-th box, -1 for a table entry outside the pool (reported).  Such a box, and one
+        // past the end of the sequence, is fetched from behind the pool, where it reads as zero.
         auto lookup = [&](int t0) {
-            int page = 0;
+            int page = cv.page_table ? cv.n_pages : 0;
             if (cv.page_table != nullptr && lane < nbox && t0 + lane * p.box_rows < len) {
                 page = cv.page_table[(long long)s * cv.max_pages_per_seq + (t0 + lane * p.box_rows) / cv.page_size];
                 if (page < 0 || page >= cv.n_pages) {
                     lorc_set_status(p.status, LORC_ERR_CAPACITY);
-                    page = 0;
+                    page = -1;
                 }
             }
             return page;
@@ -145,11 +147,14 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
         for (int i = 0; i < n_steps; ++i) {
             const int st = i % FD_STAGES, t0 = t_begin + i * FD_TILE;
             int pages[4];
+            const uint32_t dead = __ballot_sync(0xffffffffu, mine < 0);
+            if (mine < 0) mine = cv.n_pages;
 #pragma unroll
             for (int j = 0; j < 4; ++j) pages[j] = __shfl_sync(0xffffffffu, mine, j);
             if (i + 1 < n_steps) mine = lookup(t0 + FD_TILE);
             if (!mbar_wait(&sm.empty[st], ((i / FD_STAGES) & 1) ^ 1)) { ok = false; break; }
             if (elect_one()) {
+                sm.dead[st] = dead;
                 mbar_arrive_expect_tx(&sm.full[st], 2 * 2 * FD_TILE * 64 * 2);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -177,7 +182,7 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
             if (h < G && len > 0) {
                 const bf16* qp = p.q + ((long long)s * H_q + kvh * G + h) * FD_DH;
                 const float a = __bfloat162float(qp[ia]), b = __bfloat162float(qp[ib]);
-                const float2 cs = p.rope_table[(long long)(len - 1) * (FD_DH / 2) + jj];
+                const float2 cs = p.rope_table[(long long)q_pos * (FD_DH / 2) + jj];
                 const float scale = rsqrtf((float)FD_DH);
                 ra = (a * cs.x - b * cs.y) * scale;
                 rb = (a * cs.y + b * cs.x) * scale;
@@ -208,10 +213,12 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
         // mi = lane / 8 addresses a row of matrix mi: keys (tokens 0..7 | 8..15) x (dims 0..7), then (dims 8..15); values
         // (dims 0..7 | 8..15) x (tokens 0..7), then (tokens 8..15)
         const int mi = lane >> 3, lr = lane & 7;
+        const int box = warp * 16 / p.box_rows;          // the box of a stage that holds this warp's tokens
         const uint32_t k_row = (uint32_t)(warp * 16 + (mi & 1) * 8 + lr) * 128, v_row = (uint32_t)(warp * 16 + (mi >> 1) * 8 + lr) * 128;
         for (int i = 0; i < n_steps; ++i) {
             const int st = i % FD_STAGES, tw = t_begin + i * FD_TILE + warp * 16;     // first token of this warp
             if (!mbar_wait(&sm.full[st], (i / FD_STAGES) & 1)) { ok = false; break; }
+            const int t_live = (sm.dead[st] >> box) & 1 ? 0 : t_end;
             const uint32_t k0 = smem_u32(sm.u.kv[st][0][0]), v0 = smem_u32(sm.u.kv[st][1][0]);
             // scores of tokens g, g + 8 against heads 2 t, 2 t + 1; four short chains
             float sc[4][4];
@@ -229,7 +236,7 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 x[j] = (sc[0][j] + sc[1][j]) + (sc[2][j] + sc[3][j]);
-                if (tw + g + (j >> 1) * 8 >= t_end) x[j] = -INFINITY;
+                if (tw + g + (j >> 1) * 8 >= t_live) x[j] = -INFINITY;
             }
             // running softmax over this warp's tokens
             float m_new[2];

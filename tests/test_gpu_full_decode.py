@@ -71,3 +71,78 @@ def test_full_decode(H_q, H_kv, lens, style, page, n_splits):
                     want = O.decode_attn_cached_kv(k, v, qs, 10000.0, style)
                 H.assert_rows_close(H.host_f64(out[s]), want, 1e-2, (lens, s))
     L.lorc_destroy(ctx)
+
+
+@pytest.mark.parametrize("page,n_splits", [(16, 1), (32, 0), (64, 3), (96, 1)])
+def test_pages_outside_the_pool_are_left_out(page, n_splits):
+    """Tokens whose page-table entry lies outside the pool take no part, whatever the pool's first page holds; the status word
+    reports them."""
+    import torch
+    L = H.lib()
+    rng = np.random.default_rng(page)
+    H_q, H_kv, lens = 8, 2, [400, 70]
+    n, b, per = H_kv * 128, len(lens), (max(lens) + page - 1) // page
+    ctx = L.lorc_create(1, 256, H_q, H_kv, 128, 10000.0, max_pos=512)
+    w = torch.zeros(256, n, dtype=torch.bfloat16, device="cuda")
+    L.lorc_load_factors(ctx, 0, L.LORC_MODE_FULL, 0, 0, w, None, w, None)
+    ws = torch.zeros(L.lorc_workspace_bytes(ctx, b, 512), dtype=torch.uint8, device="cuda")
+    L.lorc_set_workspace(ctx, ws)
+    rows = [[synth.to_bf16_exact(rng.standard_normal((m, n))) for m in lens] for _ in "kv"]
+    kv = [torch.full((b * per + 1, page, n), 50.0, dtype=torch.bfloat16, device="cuda") for _ in "kv"]     # page 0 is not in use
+    table = np.arange(1, b * per + 1, dtype=np.int32).reshape(b, per)
+    for c, which in zip(kv, rows):
+        for s, r in enumerate(which):
+            for i in range(0, lens[s], page):
+                part = H.dev_bf16(r[i:i + page])
+                c[int(table[s, i // page]), :part.shape[0]] = part
+    live = [np.ones(m, dtype=bool) for m in lens]
+    for s, i, entry in ((0, 0, -1), (0, 2, b * per + 1), (0, (lens[0] - 1) // page, 10 ** 6)):
+        table[s, i] = entry
+        live[s][i * page:(i + 1) * page] = False
+    sl, tab = torch.tensor(lens, dtype=torch.int32, device="cuda"), torch.from_numpy(table).cuda()
+    cache = L.make_cache(*kv, sl, b, max(lens), page_table=tab, page_size=page, max_pages_per_seq=per, n_pages=b * per + 1)
+    q = synth.queries(b, H_q, 128, 36, 1, 8.0).astype(np.float64)
+    out = torch.full((b, H_q, 128), 3.0, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn(ctx, 0, cache, H.dev_bf16(q), out, n_splits=n_splits)
+    assert L.lorc_sync_status(ctx) == L.LORC_ERR_CAPACITY
+    assert L.lorc_last_path(ctx) == 3
+    for s, m in enumerate(lens):
+        k, v = (which[s].astype(np.float64).reshape(m, H_kv, 128)[live[s]] for which in rows)
+        want = O.decode_attn_cached_kv(k, v, q[s], 10000.0, q_position=m - 1)
+        H.assert_rows_close(H.host_f64(out[s]), want, 1e-2, (page, s))
+    L.lorc_destroy(ctx)
+
+
+@pytest.mark.parametrize("page", [0, 16, 48])
+def test_length_beyond_the_capacity(page):
+    """A length beyond the rows that exist: the query sits at the end of that length, the rows that exist are attended, and
+    the status word reports it."""
+    import torch
+    L = H.lib()
+    rng = np.random.default_rng(7)
+    H_q, H_kv, rows_max = 4, 1, 96 if page else 101
+    n, lens = H_kv * 128, [rows_max + 9, 50]
+    ctx = L.lorc_create(1, 256, H_q, H_kv, 128, 10000.0, max_pos=128)
+    w = torch.zeros(256, n, dtype=torch.bfloat16, device="cuda")
+    L.lorc_load_factors(ctx, 0, L.LORC_MODE_FULL, 0, 0, w, None, w, None)
+    ws = torch.zeros(L.lorc_workspace_bytes(ctx, 2, 128), dtype=torch.uint8, device="cuda")
+    L.lorc_set_workspace(ctx, ws)
+    rows = [[synth.to_bf16_exact(rng.standard_normal((rows_max, n))) for _ in lens] for _ in "kv"]
+    sl = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    kv = [torch.stack([H.dev_bf16(r) for r in which]) for which in rows]
+    if page:
+        per = rows_max // page
+        tab = torch.arange(2 * per, dtype=torch.int32, device="cuda").view(2, per)
+        cache = L.make_cache(*[c.view(2 * per, page, n) for c in kv], sl, 2, rows_max, page_table=tab, page_size=page,
+                             max_pages_per_seq=per, n_pages=2 * per)
+    else:
+        cache = L.make_cache(*kv, sl, 2, rows_max, seq_stride=rows_max)
+    q = synth.queries(2, H_q, 128, 36, 2, 8.0).astype(np.float64)
+    out = torch.full((2, H_q, 128), 3.0, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn(ctx, 0, cache, H.dev_bf16(q), out)
+    assert L.lorc_sync_status(ctx) == L.LORC_ERR_CAPACITY
+    for s, m in enumerate(lens):
+        k, v = (which[s].astype(np.float64).reshape(-1, H_kv, 128)[:m] for which in rows)
+        want = O.decode_attn_cached_kv(k, v, q[s], 10000.0, q_position=m - 1)
+        H.assert_rows_close(H.host_f64(out[s]), want, 1e-2, (page, s))
+    L.lorc_destroy(ctx)
