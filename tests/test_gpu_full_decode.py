@@ -1,8 +1,8 @@
 """Streaming decode kernel of uncompressed layers: edges of steps and shares, page sizes that cut a step into boxes, head
 counts, and cache rows past the sequence that hold NaN.
 
-Probabilities are rounded to bf16 (2^-9 relative each, of random sign) and the output once more: the observed row error is
-2.3e-3, the bound the repository's bf16 tolerance of 1e-2."""
+Probabilities are carried in two bf16 parts and the output is rounded to bf16: the observed row error is 1.7e-3, the bound the
+repository's bf16 tolerance of 1e-2; test_error_beside_the_output_rounding holds what lies beside the rounding closer."""
 import numpy as np
 import pytest
 
@@ -145,4 +145,37 @@ def test_length_beyond_the_capacity(page):
         k, v = (which[s].astype(np.float64).reshape(-1, H_kv, 128)[:m] for which in rows)
         want = O.decode_attn_cached_kv(k, v, q[s], 10000.0, q_position=m - 1)
         H.assert_rows_close(H.host_f64(out[s]), want, 1e-2, (page, s))
+    L.lorc_destroy(ctx)
+
+
+@pytest.mark.parametrize("n_splits", [0, 1, 9])
+@pytest.mark.parametrize("q_scale", [1.0, 8.0])
+def test_error_beside_the_output_rounding(q_scale, n_splits):
+    """Half an ulp of the bf16 output, and beside it 2e-4 of the row rms: two bf16 parts leave 2^-17 = 8e-6 in a probability
+    and 2^-18 in a query element (about 8 * 2^-18 = 3e-5 in a score of standard deviation 8), random in sign over the
+    tokens.  (One bf16 part leaves 2e-3.)"""
+    import torch
+    L = H.lib()
+    rng = np.random.default_rng(11)
+    H_q, H_kv, lens = 32, 8, [2100, 600]
+    n, b = H_kv * 128, len(lens)
+    ctx = L.lorc_create(1, 256, H_q, H_kv, 128, 10000.0, max_pos=2112)
+    w = torch.zeros(256, n, dtype=torch.bfloat16, device="cuda")
+    L.lorc_load_factors(ctx, 0, L.LORC_MODE_FULL, 0, 0, w, None, w, None)
+    ws = torch.zeros(L.lorc_workspace_bytes(ctx, b, 2112), dtype=torch.uint8, device="cuda")
+    L.lorc_set_workspace(ctx, ws)
+    rows = [[synth.to_bf16_exact(rng.standard_normal((2112, n))) for _ in lens] for _ in "kv"]
+    kv = [torch.stack([H.dev_bf16(r) for r in which]) for which in rows]
+    sl = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    cache = L.make_cache(*kv, sl, b, max(lens), seq_stride=2112)
+    q = synth.queries(b, H_q, 128, 36, 3, q_scale).astype(np.float64)
+    out = torch.zeros(b, H_q, 128, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn(ctx, 0, cache, H.dev_bf16(q), out, n_splits=n_splits)
+    assert L.lorc_sync_status(ctx) == 0, L.lorc_last_error(ctx)
+    for s, m in enumerate(lens):
+        k, v = (which[s].astype(np.float64).reshape(-1, H_kv, 128)[:m] for which in rows)
+        want = O.decode_attn_cached_kv(k, v, q[s], 10000.0)
+        rms = np.sqrt(np.mean(want ** 2, axis=-1, keepdims=True))
+        excess = np.abs(H.host_f64(out[s]) - want) - (0.5 * H.bf16_ulp(want) + 2e-4 * rms)
+        assert np.all(excess <= 0.0), float((excess / rms).max())
     L.lorc_destroy(ctx)
