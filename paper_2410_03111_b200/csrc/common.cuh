@@ -128,8 +128,9 @@ cudaError_t lorc_generic_append(const lorc_ctx* ctx, const LorcLayer& L, const C
 // per-split partial results as the plain kernel, for lorc_generic_combine.
 bool lorc_full_decode_supported(const lorc_ctx* ctx, const LorcLayer& L);
 int lorc_full_decode_splits(const lorc_ctx* ctx, int batch, int max_seq_len);
+// by_length: a sequence takes as many of the n_splits shares as its length calls for, else all of them.
 cudaError_t lorc_full_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* q, int n_splits,
-                             float* part_ml, float* part_o, cudaStream_t st, int* launches);
+                             bool by_length, float* part_ml, float* part_o, cudaStream_t st, int* launches);
 // Compressed layers, one query per sequence, bf16 path: the plain computation with mma.sync reconstruction (small_decode.cu).
 // Leaves the same per-split partial results too.
 bool lorc_small_decode_supported(const lorc_ctx* ctx, const LorcLayer& L);
@@ -142,7 +143,8 @@ cudaError_t lorc_small_decode(const lorc_ctx* ctx, const LorcLayer& L, const Cac
 cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv,
                                 const bf16* q, bf16* out, int n_splits, float* part_ml,
                                 float* part_o, cudaStream_t st, int* launches, bool latent_out = false, int T = 1,
-                                const int32_t* pos0 = nullptr, const int32_t* q_pos = nullptr, float* ml_out = nullptr);
+                                const int32_t* pos0 = nullptr, const int32_t* q_pos = nullptr, float* ml_out = nullptr,
+                                bool by_length = false);
 // Merge of the results of context shards (lorc_merge_shards).
 cudaError_t lorc_generic_merge_shards(const lorc_ctx* ctx, int n_shards, const bf16* outs, const float* mls, bf16* out,
                                       int batch, cudaStream_t st, int* launches);

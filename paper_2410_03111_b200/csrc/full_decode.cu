@@ -1,6 +1,6 @@
 // Decode attention of the uncompressed reference mode (ordinary KV cache: keys stored rotated, values as they are)
 // on the warp-level tensor cores.  The work is one pass over 2 n bf16 numbers per token and is bound by HBM, so the
-// kernel is shaped for streaming: a CTA owns one (sequence, KV head, context share); a producer warp keeps three 64-token
+// kernel is shaped for streaming: a CTA owns one (sequence, KV head, context share) (see lorc_full_decode_splits); a producer warp keeps three 64-token
 // stages of keys and values in flight by TMA; each of four consumer warps owns 16 of a stage's tokens with its own running
 // softmax (no block-wide synchronisation inside the loop).  The tokens (scores) and the dimensions (output) are the M side of
 // the m16n8k16 tiles, the G <= 8 query heads the N side, so no row of a tile is padding:
@@ -14,7 +14,7 @@
 // with the length of a share, because a higher reference moves p to other places between powers of two.  The second part
 // costs 0.5 % where HBM sets the pace and 3 to 4 % where a single block's stream does.
 //
-// b 16, 8 KV heads of 128, 4129 tokens (271 MB): 44 us, 6.2 TB/s, 0.94 of the measured copy rate.  (With per-lane
+// b 16, 8 KV heads of 128, 4129 tokens (271 MB): 45 us, 6.0 TB/s, 0.93 of the measured copy rate.  (With per-lane
 // asynchronous copies and the heads on the M side, half of them padding, a warp issued seven times the instructions per tile
 // and the issue slots, not HBM, set the pace: 55 us.)
 // Each CTA leaves (m, l, un-normalised O) per query head for the merge kernel of the plain family.
@@ -93,8 +93,50 @@ struct FdParams {
     float* part_ml;
     float* part_o;
     int* status;
-    int G, n_splits, rope_style, max_pos, box_rows;
+    int G, n_kv, n_splits, rope_style, max_pos, box_rows;
+    int slots;                     // 0: every sequence has n_splits shares; else at most as many, and `slots` together
 };
+
+// Shares of a sequence of `tiles` steps when all of them have `total` (with `slots`): in proportion to its length, so that
+// the blocks of a launch are resident at once and equally long whatever the lengths are.  The sum over the batch is at most
+// slots + batch.  (Steps are counted up to 2^15 a sequence, which keeps the sums of any batch in 32 bits.)
+__device__ __forceinline__ int fd_weight(const FdParams& p, int len) {
+    return len <= 0 || len > p.max_pos ? 0 : min((len - 1) / FD_TILE + 1, 1 << 15);
+}
+__device__ __forceinline__ int fd_shares(const FdParams& p, int weight, int total) {
+    return max(1, min(p.n_splits, weight * p.slots / max(total, 1)));
+}
+
+// Block `f` of a KV head -> sequence (-1: none), its length, share, number of shares; executed by whole warps.  (The result
+// comes from warp reductions: those leave it in uniform registers, where loop bounds and TMA coordinates want it.)
+__device__ __forceinline__ int4 fd_locate(const FdParams& p, int f, int lane) {
+    const CacheView& cv = p.cv;
+    if (p.slots == 0) return make_int4(f / p.n_splits, cv.seq_lens[f / p.n_splits], f % p.n_splits, p.n_splits);
+    const int len0 = lane < cv.batch ? cv.seq_lens[lane] : 0;
+    int sum = fd_weight(p, len0);
+    for (int i = lane + 32; i < cv.batch; i += 32) sum += fd_weight(p, cv.seq_lens[i]);
+    const int total = __reduce_add_sync(0xffffffffu, sum);
+    int first = 0;
+    for (int i0 = 0; i0 < cv.batch; i0 += 32) {
+        const int i = i0 + lane, len = i0 == 0 ? len0 : i < cv.batch ? cv.seq_lens[i] : 0;
+        const int n = i < cv.batch ? fd_shares(p, fd_weight(p, len), total) : 0;
+        int end = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += x;
+        }
+        const unsigned hit = __ballot_sync(0xffffffffu, f < first + end);
+        if (hit) {
+            const bool mine = lane == __ffs(hit) - 1;
+            return make_int4(i0 + __ffs(hit) - 1, __reduce_add_sync(0xffffffffu, mine ? len : 0),
+                             __reduce_add_sync(0xffffffffu, mine ? f - first - (end - n) : 0),
+                             __reduce_add_sync(0xffffffffu, mine ? n : 0));
+        }
+        first += __shfl_sync(0xffffffffu, end, 31);
+    }
+    return make_int4(-1, 0, 0, 1);
+}
 
 __global__ void __launch_bounds__(FD_THREADS, FD_BLOCKS_PER_SM)
 full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV, const FdParams p) {
@@ -102,9 +144,9 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
     FdSmem& sm = *reinterpret_cast<FdSmem*>((reinterpret_cast<uintptr_t>(fd_raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t = lane & 3;            // fragment row / column group of this lane
-    const int split = blockIdx.x, kvh = blockIdx.y, s = blockIdx.z;
+    const int kvh = (int)blockIdx.x % p.n_kv;
     const CacheView& cv = p.cv;
-    const int G = p.G, H_q = G * (int)gridDim.y;
+    const int G = p.G, H_q = G * p.n_kv;
     if (tid == 0) {
         for (int i = 0; i < FD_STAGES; ++i) {
             mbar_init(&sm.full[i], 1);
@@ -116,7 +158,17 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
     }
     grid_dep_wait();
     grid_dep_launch();
-    int len = cv.seq_lens[s];
+    const int4 share = fd_locate(p, (int)blockIdx.x / p.n_kv, lane);
+    const int s = share.x, split = share.z, n_shares = share.w;
+    int len = share.y;
+    if (s < 0) return;
+    // the slots of the shares that this sequence does not have
+    if (split == 0)
+        for (int i = tid; i < G * (p.n_splits - n_shares); i += FD_THREADS) {
+            const int h = i / (p.n_splits - n_shares), c = n_shares + i % (p.n_splits - n_shares);
+            *reinterpret_cast<float2*>(p.part_ml + (((long long)s * H_q + kvh * G + h) * p.n_splits + c) * 2) =
+                make_float2(-INFINITY, 0.f);
+        }
     if ((len > p.max_pos || len > cv.capacity) && tid == 0) lorc_set_status(p.status, LORC_ERR_CAPACITY);
     if (len < 0 || len > p.max_pos) len = 0;
     const int q_pos = len - 1;
@@ -124,7 +176,7 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
     if (len > cv.capacity) len = (int)cv.capacity;
     // this CTA's share of the context, in whole 64-token tiles
     const int tiles = (len + FD_TILE - 1) / FD_TILE;
-    const int tps = (tiles + p.n_splits - 1) / p.n_splits;
+    const int tps = (tiles + n_shares - 1) / n_shares;
     const int t_begin = min(len, split * tps * FD_TILE), t_end = min(len, (split + 1) * tps * FD_TILE);
     const int n_steps = (t_end - t_begin + FD_TILE - 1) / FD_TILE;
     const int col0 = kvh * FD_DH;
@@ -349,19 +401,25 @@ bool lorc_full_decode_supported(const lorc_ctx* ctx, const LorcLayer& L) {
            !(ctx->desc.flags & LORC_FLAG_DEBUG_FP32);
 }
 
-// Context shares: as many as are resident at once, so that every block streams from the start to the end of the launch;
-// down to one 64-token step each.  (512 tokens per share made 1152 blocks in 2.6 rounds at b 16, 8 KV heads, 4129 tokens,
-// each round with its own ramp: 64 us instead of 55.)
+// Blocks of a KV head that are resident at once.
+static int fd_slots(const lorc_ctx* ctx) { return FD_BLOCKS_PER_SM * ctx->sm_count / ctx->desc.n_kv_heads; }
+
+// Most context shares of a sequence: an equal part of the resident blocks, so that every block streams from the start to the
+// end of the launch (down to one 64-token step each).  Where that makes shares of more than 1024 tokens, which take a block
+// longer than 17 us, there is room for shares of 512 tokens and the kernel deals the resident blocks out by length.  (With
+// equal parts alone one sequence of 8200 tokens among 23 of 256, 8 KV heads, is streamed by 8 blocks: 74 us, dealt out 19.
+// Shares of 512 tokens for all make 1152 blocks in 3.9 rounds at b 16, 8 KV heads, 4129 tokens: 56 us against 49.  Dealing
+// costs 0.5 to 1 us where all lengths are equal.)
 int lorc_full_decode_splits(const lorc_ctx* ctx, int batch, int max_seq_len) {
-    const long long units = (long long)batch * ctx->desc.n_kv_heads;
-    const long long fill = (long long)FD_BLOCKS_PER_SM * ctx->sm_count / units, steps = (max_seq_len + FD_TILE - 1) / FD_TILE;
-    return (int)(fill < 1 ? 1 : fill < steps ? fill : steps);
+    const int slots = fd_slots(ctx), steps = (max_seq_len - 1) / FD_TILE + 1, room = (max_seq_len - 1) / 512 + 1;
+    int n = slots / batch > 1 ? slots / batch : 1;
+    if (max_seq_len > 1024ll * n && n < room) n = room < slots ? room : slots;
+    return n < 1 ? 1 : n < steps ? n : steps;
 }
 
-cudaError_t lorc_full_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* q, int n_splits, float* part_ml,
-                             float* part_o, cudaStream_t st, int* launches) {
+cudaError_t lorc_full_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* q, int n_splits, bool by_length,
+                             float* part_ml, float* part_o, cudaStream_t st, int* launches) {
     const lorc_model_desc& d = ctx->desc;
-    dim3 grid(n_splits, d.n_kv_heads, cv.batch);
     const size_t smem = sizeof(FdSmem) + 1024;
     // the attribute belongs to a device's copy of the kernel: one flag per device (devices beyond the table set it
     // on every call, which is only slower)
@@ -372,13 +430,17 @@ cudaError_t lorc_full_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView&
         if (e != cudaSuccess) return e;
         if (known) attr[ctx->device] = true;
     }
+    // nothing to deal where an equal part of the resident blocks is as many shares as a sequence has room for
+    const int slots = by_length && n_splits > fd_slots(ctx) / cv.batch && n_splits > 1 ? fd_slots(ctx) : 0;
     // a box never leaves its page: page sizes are multiples of 16
     FdParams p;
     p.box_rows = !cv.page_table || cv.page_size % 64 == 0 ? 64 : cv.page_size % 32 == 0 ? 32 : 16;
     CUtensorMap *mapK, *mapV;
     if (!lorc_tc_full_maps(ctx, L, cv, p.box_rows, &mapK, &mapV)) return cudaErrorInvalidValue;
     p.q = q; p.cv = cv; p.rope_table = ctx->rope_table; p.part_ml = part_ml; p.part_o = part_o; p.status = ctx->status_dev;
-    p.G = ctx->group; p.n_splits = n_splits; p.rope_style = ctx->pair_style; p.max_pos = d.max_pos;
+    p.G = ctx->group; p.n_kv = d.n_kv_heads; p.n_splits = n_splits; p.slots = slots; p.rope_style = ctx->pair_style; p.max_pos = d.max_pos;
+    const long long even = (long long)cv.batch * n_splits, most = (long long)slots + cv.batch;
+    const dim3 grid((unsigned)(d.n_kv_heads * (slots > 0 && most < even ? most : even)));
     *launches += 1;
     return lorc_launch_dependent(full_decode_mma_kernel, grid, dim3(FD_THREADS), smem, st, *mapK, *mapV, p);
 }

@@ -401,6 +401,7 @@ combine_generic_kernel(const float* __restrict__ part_ml, const float* __restric
     __shared__ float w_s[LORC_MAX_SPLITS];
     __shared__ float red[256];
     __shared__ float L_s;
+    __shared__ int used_s;
     const int h = blockIdx.x, s = blockIdx.y, H_q = gridDim.x, tid = threadIdx.x, nt = blockDim.x;
     const long long unit0 = ((long long)s * H_q + h) * n_splits;
     sm100::grid_dep_wait();
@@ -414,16 +415,20 @@ combine_generic_kernel(const float* __restrict__ part_ml, const float* __restric
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
         double L = 0.0;
+        int used = 0;                    // shares up to the last one that saw a token
         for (int c = tid; c < n_splits; c += 32) {
             const float2 ml = *reinterpret_cast<const float2*>(part_ml + (unit0 + c) * 2);
             const float w = (ml.y > 0.f) ? expf(ml.x - M) : 0.f;
             w_s[c] = w;
+            if (ml.y != 0.f) used = c + 1;
             L += (double)w * (double)ml.y;
         }
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+        used = __reduce_max_sync(0xffffffffu, used);
         if (tid == 0) {
             L_s = (float)L;
+            used_s = used;
             if (ml_out) {
                 // reference in log2 units and the denominator relative to it (a shard of a context may be empty)
                 ml_out[((long long)s * H_q + h) * 2] = L > 0.0 ? M * 1.4426950408889634f : 0.f;
@@ -435,12 +440,14 @@ combine_generic_kernel(const float* __restrict__ part_ml, const float* __restric
     }
     __syncthreads();
     const float L = L_s;
+    const int used = __reduce_max_sync(0xffffffffu, used_s);      // in a uniform register
     const float inv = (L > 0.f) ? 1.f / L : 0.f;
     for (int col = tid; col < W; col += nt) {
+        const float* po = part_o + unit0 * W + col;
         float a = 0.f;
 #pragma unroll 4
-        for (int c = 0; c < n_splits; ++c) {
-            const float w = w_s[c], x = part_o[(unit0 + c) * W + col];
+        for (int c = 0; c < used; ++c) {
+            const float w = w_s[c], x = po[c * W];
             if (w != 0.f) a = fmaf(w, x, a);
         }
         o_lat[col] = a * inv;
@@ -484,7 +491,7 @@ cudaError_t lorc_generic_combine(const lorc_ctx* ctx, const LorcLayer& L, int ba
 cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv,
                                 const bf16* q, bf16* out, int n_splits, float* part_ml,
                                 float* part_o, cudaStream_t st, int* launches, bool latent_out, int T,
-                                const int32_t* pos0, const int32_t* q_pos, float* ml_out) {
+                                const int32_t* pos0, const int32_t* q_pos, float* ml_out, bool by_length) {
     const lorc_model_desc& d = ctx->desc;
     const int G = ctx->group;
     const bool latent = (L.mode == LORC_MODE_LATENT);
@@ -493,7 +500,7 @@ cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheVi
         // uncompressed mode with 128-wide heads: the streaming kernel on the warp-level tensor cores
         {
             LorcStageTimer timer(ctx, LORC_STAGE_SCORE, st);
-            cudaError_t e = lorc_full_decode(ctx, L, cv, q, n_splits, part_ml, part_o, st, launches);
+            cudaError_t e = lorc_full_decode(ctx, L, cv, q, n_splits, by_length, part_ml, part_o, st, launches);
             if (e != cudaSuccess) return e;
         }
         return lorc_generic_combine(ctx, L, cv.batch, n_splits, part_ml, part_o, out, st, launches, false, nullptr);

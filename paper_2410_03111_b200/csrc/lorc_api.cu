@@ -346,7 +346,7 @@ static int decode_attn_impl(lorc_ctx* ctx, int layer, const lorc_cache* cache, c
     float* part_ml = (float*)((char*)ctx->ws + w.off_ml);
     float* part_o = (float*)((char*)ctx->ws + w.off_o);
     e = lorc_generic_decode(ctx, *L, cv, (const bf16*)q, (bf16*)out, S, part_ml, part_o, st, &launches, latent_out, 1,
-                            pos0, q_pos, ml_out);
+                            pos0, q_pos, ml_out, n_splits == 0);
     ctx->launches += launches;
     ctx->last_path = lorc_full_decode_supported(ctx, *L) ? 3 : 1;
     if (e != cudaSuccess) return fail_cuda(ctx, e, "lorc_decode_attn");

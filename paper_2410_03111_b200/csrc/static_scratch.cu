@@ -111,7 +111,7 @@ extern "C" int lorc_decode_attn_static(lorc_ctx* ctx, int layer, const lorc_cach
     float* part_o = (float*)((char*)g_scratch_addr[dev] + lorc_align_up(units * 2 * sizeof(float), 256));
     int launches = 0;
     e = lorc_generic_decode(ctx, L, cv, (const bf16*)q, (bf16*)out, S, part_ml, part_o, (cudaStream_t)stream,
-                            &launches);
+                            &launches, false, 1, nullptr, nullptr, nullptr, n_splits == 0);
     ctx->launches += launches;
     ctx->last_path = lorc_full_decode_supported(ctx, L) ? 3 : 1;
     if (e != cudaSuccess) {

@@ -179,3 +179,53 @@ def test_error_beside_the_output_rounding(q_scale, n_splits):
         excess = np.abs(H.host_f64(out[s]) - want) - (0.5 * H.bf16_ulp(want) + 2e-4 * rms)
         assert np.all(excess <= 0.0), float((excess / rms).max())
     L.lorc_destroy(ctx)
+
+
+@pytest.mark.parametrize("lens,H_q,H_kv", [
+    ([3000] + [64, 0, 1, 65] * 8, 16, 8),            # 33 sequences: the second group of 32 is searched too
+    ([130, 9000] * 20, 8, 1),                        # more resident blocks than sequences
+    ([130, 2000] * 35, 8, 1),                        # equal parts of them are short enough
+    ([100] * 40 + [2500], 64, 8),                    # fewer; the long one comes last
+    ([64], 4, 4),
+])
+def test_shares_by_length(lens, H_q, H_kv):
+    """Sequences of very unequal length in one call: the blocks that are resident at once are dealt out by length."""
+    import torch
+    L = H.lib()
+    n, b, n_max = H_kv * 128, len(lens), max(lens)
+    ctx = L.lorc_create(1, 256, H_q, H_kv, 128, 10000.0, max_pos=n_max)
+    w = torch.zeros(256, n, dtype=torch.bfloat16, device="cuda")
+    L.lorc_load_factors(ctx, 0, L.LORC_MODE_FULL, 0, 0, w, None, w, None)
+    ws = torch.full((L.lorc_workspace_bytes(ctx, b, n_max),), 255, dtype=torch.uint8, device="cuda")     # NaN everywhere
+    L.lorc_set_workspace(ctx, ws)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    kv = [torch.randn(b, n_max, n, generator=g, device="cuda", dtype=torch.bfloat16) for _ in "kv"]
+    sl = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    cache = L.make_cache(*kv, sl, b, n_max, seq_stride=n_max)
+    q = synth.queries(b, H_q, 128, 36, 4, 8.0).astype(np.float64)
+    out = torch.full((b, H_q, 128), 3.0, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn(ctx, 0, cache, H.dev_bf16(q), out)
+    assert L.lorc_sync_status(ctx) == (L.LORC_ERR_EMPTY if 0 in lens else 0)
+    # share results sit at the front of the workspace: [sequence][head][room for shares] of (reference, denominator)
+    slots = 2 * torch.cuda.get_device_properties(0).multi_processor_count // H_kv
+    equal = max(1, slots // b)
+    room = min((n_max + 63) // 64, max(equal, min((n_max + 511) // 512, slots)) if n_max > 1024 * equal else equal)
+    ml = ws[:b * H_q * room * 8].view(torch.float32).view(b, H_q, room, 2).cpu().numpy()
+    steps = np.array([(m + 63) // 64 for m in lens])
+    if room > equal:
+        want_shares = np.clip(steps * slots // max(1, steps.sum()), 1, room)
+    else:
+        want_shares = np.full(b, room)                   # equal parts
+    for s, m in enumerate(lens):
+        per = -(-steps[s] // want_shares[s])
+        assert np.all((ml[s, :, :, 1] > 0).sum(axis=1) == (-(-steps[s] // per) if m else 0)), s
+        if m == 0:
+            assert float(out[s].abs().max()) == 0.0
+            continue
+        k, v = (c[s, :m].double().cpu().numpy().reshape(m, H_kv, 128) for c in kv)
+        H.assert_rows_close(H.host_f64(out[s]), O.decode_attn_cached_kv(k, v, q[s], 10000.0), 1e-2, s)
+    again = torch.zeros_like(out)
+    L.lorc_decode_attn(ctx, 0, cache, H.dev_bf16(q), again)
+    L.lorc_sync_status(ctx)
+    assert torch.equal(out, again)
+    L.lorc_destroy(ctx)
