@@ -1,9 +1,9 @@
 // Decode attention of the uncompressed reference mode (ordinary KV cache: keys stored rotated, values as they are)
 // on the warp-level tensor cores.  The work is one pass over 2 n bf16 numbers per token and is bound by HBM, so the
-// kernel is shaped for streaming: a CTA owns one (sequence, KV head, context share) (see lorc_full_decode_splits); a producer warp keeps three 64-token
-// stages of keys and values in flight by TMA; each of four consumer warps owns 16 of a stage's tokens with its own running
-// softmax (no block-wide synchronisation inside the loop).  The tokens (scores) and the dimensions (output) are the M side of
-// the m16n8k16 tiles, the G <= 8 query heads the N side, so no row of a tile is padding:
+// kernel is shaped for streaming: a CTA owns one (sequence, KV head, context share), see lorc_full_decode_splits; a producer
+// warp keeps three 64-token stages of keys and values in flight by TMA; each of four consumer warps owns 16 of a stage's tokens
+// with its own running softmax (no block-wide synchronisation inside the loop).  The tokens (scores) and the dimensions (output)
+// are the M side of the m16n8k16 tiles, the G <= 8 query heads the N side, so no row of a tile is padding:
 //
 //   S^T[16 tok x 8]   = K[16 tok x 128] . Q^^T            q^ = RoPE(q, N-1)/sqrt(d_h) split into bf16 hi + lo parts,
 //                                                          so the scores keep fp32-level accuracy
@@ -200,7 +200,8 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
             return page;
         };
         int mine = n_steps > 0 ? lookup(t_begin) : 0;
-        for (int i = 0; i < n_steps; ++i) {
+        int i = 0;
+        for (; i < n_steps; ++i) {
             const int st = i % FD_STAGES, t0 = t_begin + i * FD_TILE;
             int pages[4];
             const uint32_t dead = __ballot_sync(0xffffffffu, mine < 0);
@@ -226,6 +227,10 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
             }
             __syncwarp();
         }
+        // The block stays until the copies into its shared memory have landed (or the limit has passed once more), also when a
+        // wait has run out.  Otherwise the consumers wait for all of them anyhow.
+        for (int j = max(i - FD_STAGES, 0); j < i; ++j)
+            if (!mbar_wait(&sm.full[j % FD_STAGES], (j / FD_STAGES) & 1)) ok = false;
         if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
     } else {
         // ------------------------------------------------------------------ consumers
