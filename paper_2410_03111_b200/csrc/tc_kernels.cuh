@@ -111,16 +111,17 @@ void lorc_tc_release(lorc_ctx* ctx);
 // with one round trip per tile and shuffles them to the lane that issues the boxes.  (Looked up box by box inside the loop
 // over the slices of the rank, a table access stood before every copy: a step of 64 ragged sequences of up to 16384
 // tokens, r 384, 64-token pages took 659 us and takes 596 us.)  Pages past the end of the sequence, or with a bad table entry, are read from
-// page 0: their rows are masked, but every box must deliver its bytes.
+// page `none`: 0 (their rows are masked, but every box must deliver its bytes), or n_pages, which lies behind the pool and
+// reads as zero.
 __device__ __forceinline__ int lorc_tile_page(const int32_t* table, long long seq, int tile, int lane, int len, int page_size,
-                                              int max_pages, int n_pages, int* status) {
+                                              int max_pages, int n_pages, int* status, int none = 0) {
     const int ppt = 128 / page_size, lp = tile * ppt + lane;
-    int page = 0;
+    int page = none;
     if (lane < ppt && (long long)lp * page_size < len && lp < max_pages) {
         page = table[seq * max_pages + lp];
         if (page < 0 || page >= n_pages) {
             lorc_set_status(status, LORC_ERR_CAPACITY);
-            page = 0;
+            page = none;
         }
     }
     return page;

@@ -127,7 +127,8 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
             const bool paged = p.page_table != nullptr;
             const int ppt = paged ? TILE / p.page_size : 0;
             auto tile_page = [&](int tile) {
-                return lorc_tile_page(p.page_table, s, tile, lane, len, p.page_size, p.max_pages_per_seq, p.n_pages, p.status);
+                return lorc_tile_page(p.page_table, s, tile, lane, len, p.page_size, p.max_pages_per_seq, p.n_pages, p.status,
+                                      SPLIT ? p.n_pages : 0);
             };
             int mine = paged && ntiles > 0 ? tile_page(tile_lo) : 0;
             for (int i = 0; i < ntiles && ok; ++i) {
@@ -164,8 +165,9 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                     tma_load_3d(sm.V[st][0], &mapCV, &sm.vfull[st], rho0, n0, s);
                     tma_load_3d(sm.V[st][1], &mapCV, &sm.vfull[st], rho0 + 64, n0, s);
                 } else {
-                    // One box per page.  (Pages past the end of the sequence come from page 0: their probabilities are
-                    // zero, but the rows must hold finite numbers, which stale shared memory would not guarantee.)
+                    // One box per page.  (Pages past the end of the sequence come from page 0, SPLIT: from behind the pool: their
+                    // probabilities are zero, but the rows must hold finite numbers, which stale shared memory would not
+                    // guarantee.)
 #pragma unroll
                     for (int pg = 0; pg < 8; ++pg) {
                         if (pg >= ppt) break;
@@ -283,6 +285,16 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) e[k] = __hmul2(e[k], sc);
                     prow[pp] = v[j];
+                }
+            }
+            if (SPLIT && (tile_lo + i + 1) * TILE > len) {
+                // The rows of C_V past the end of the sequence may hold anything, as for the plain kernels, whose place this
+                // path takes: their probabilities are zero, and zero the rows.  (Thread = row; the last tile of a sequence only.)
+                if (!mbar_wait(&sm.vfull[st], (i / P_STAGES) & 1)) { ok = false; break; }
+                if ((tile_lo + i) * TILE + t >= len) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        *reinterpret_cast<uint4*>(&sm.V[st][j >> 3][t * KC + (j & 7) * 8]) = make_uint4(0u, 0u, 0u, 0u);
                 }
             }
             fence_proxy_async_smem();      // the MMA reads the image through the asynchronous proxy

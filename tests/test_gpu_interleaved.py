@@ -134,3 +134,41 @@ def test_interleaved_context_shards():
     assert L.lorc_sync_status(sess.ctx) == 0
     H.assert_rows_close(H.host_f64(merged), H.oracle_decode(prob, ck, cv, q), 1e-2)
     sess.close()
+
+
+@pytest.mark.parametrize("geom,page,n_splits", [(G8B, 0, 1), (G8B, 16, 2), (G70B, 64, 0), (G70B, 0, 3)])
+def test_interleaved_rows_past_the_end_may_hold_anything(geom, page, n_splits):
+    """Cache rows past a sequence's end, and pages that no sequence uses (the pool's first among them), hold NaN."""
+    import torch
+    lens = [385, 128, 17, 250]
+    prob, sess, ck, cv = _problem(geom, 72, 200, lens)
+    L, b = sess.L, len(lens)
+    n_max, nan = max(lens) + 3, float("nan")
+    q = synth.queries(b, prob.H_q, 128, 31, 5, 8.0).astype(np.float64)
+    sl = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    kv = []
+    if page:
+        per = (n_max + page - 1) // page
+        table = 1 + np.random.default_rng(3).permutation(b * per).reshape(b, per).astype(np.int32)
+        for rows, r in ((ck, 72), (cv, 200)):
+            c = torch.full((b * per + 1, page, r), nan, dtype=torch.bfloat16, device="cuda")
+            for s in range(b):
+                for i in range(0, lens[s], page):
+                    part = H.dev_bf16(rows[s][i:i + page])
+                    c[int(table[s, i // page]), :part.shape[0]] = part
+            kv.append(c)
+        tab = torch.from_numpy(table).cuda()
+        cache = L.make_cache(*kv, sl, b, max(lens), page_table=tab, page_size=page, max_pages_per_seq=per, n_pages=b * per + 1)
+    else:
+        for rows, r in ((ck, 72), (cv, 200)):
+            c = torch.full((b, n_max, r), nan, dtype=torch.bfloat16, device="cuda")
+            for s in range(b):
+                c[s, :lens[s]] = H.dev_bf16(rows[s])
+            kv.append(c)
+        cache = L.make_cache(*kv, sl, b, max(lens), seq_stride=n_max)
+    out = torch.zeros(b, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn(sess.ctx, 0, cache, H.dev_bf16(q), out, n_splits=n_splits)
+    assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+    assert L.lorc_last_path(sess.ctx) == 2
+    _close(H.host_f64(out), H.oracle_decode(prob, ck, cv, q))
+    sess.close()
