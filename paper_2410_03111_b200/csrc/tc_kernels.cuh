@@ -31,6 +31,9 @@ cudaError_t lorc_tc_append_gemm(lorc_ctx* ctx, const LorcLayer& L, const CacheVi
 // bits).  The plain kernels, which serve what does not fit this path, keep both in fp32; against fp64 the results are off
 // by 1.6e-3 either way (the bf16 output), with one bf16 part by 2.9e-3.
 inline bool lorc_tc_split(const lorc_ctx* ctx) { return ctx->desc.rope_style == LORC_ROPE_INTERLEAVED; }
+// Rows of a sequence that exist: such contexts leave tokens past the capacity, and those whose page lies outside the pool, out
+// of the attention (and report them), as the plain kernels do.
+inline int lorc_tc_max_rows(const CacheView& cv) { return cv.capacity < INT32_MAX ? (int)cv.capacity : INT32_MAX; }
 // Whether a call may take that path now: its tables exist, or may be allocated (the stream is not being captured).
 bool lorc_tc_tables_ready(const lorc_ctx* ctx, const CacheView& cv, cudaStream_t st);
 

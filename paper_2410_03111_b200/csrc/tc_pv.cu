@@ -66,6 +66,7 @@ struct Pv2Params {
     const int32_t* page_table;
     int* status;
     int batch, H_q, n_kv, r_v, tiles, n_blk, n_csplit, max_pos;
+    int max_rows;                  // SPLIT: rows of a sequence that exist
     int page_size, max_pages_per_seq, n_pages;
 };
 
@@ -85,7 +86,9 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
     const int blk = blockIdx.x, cs = blockIdx.y, s = blockIdx.z;
 
     int len = p.seq_lens[s];
-    if (len > p.max_pos || len > p.tiles * TILE) len = 0;     // the score kernel reports the capacity error
+    if (len > p.max_pos) len = 0;                             // the score kernel reports the capacity errors
+    if (SPLIT) len = min(len, p.max_rows);
+    if (len > p.tiles * TILE) len = 0;
     if (len < 0) len = 0;
     // this CTA's share of the context: whole 128-token tiles, dealt evenly over the context shares
     const int tiles_s = (len + TILE - 1) / TILE;
@@ -783,7 +786,7 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
         p.pimg = pimg; p.o_part = o_part; p.rowmax = rowmax; p.o_norm = o_norm; p.done = done; p.ml_out = ml_out;
         p.seq_lens = cv.seq_lens; p.page_table = cv.page_table; p.status = ctx->status_dev;
         p.batch = cv.batch; p.H_q = d.n_q_heads; p.n_kv = d.n_kv_heads; p.r_v = L.r_v; p.tiles = tiles;
-        p.n_blk = n_blk; p.n_csplit = n_csplit; p.max_pos = d.max_pos;
+        p.n_blk = n_blk; p.n_csplit = n_csplit; p.max_pos = d.max_pos; p.max_rows = lorc_tc_max_rows(cv);
         p.page_size = cv.page_size; p.max_pages_per_seq = cv.max_pages_per_seq; p.n_pages = cv.n_pages;
         dim3 grid(n_blk, n_csplit, cv.batch);
         auto launch = [&](auto kernel, size_t bytes) {

@@ -67,6 +67,7 @@ struct ScoreParams {
     int* zero;                     // words the first block clears for the kernels that follow
     int* status;
     int batch, seq0, H_q, n_hp, r_k, tiles, n_zero, max_pos;
+    int max_rows;                  // SPLIT: rows of a sequence that exist
     int page_size, max_pages_per_seq, n_pages;
 };
 
@@ -168,7 +169,7 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
         for (int i = tid; i < p.n_zero; i += Q_THREADS) p.zero[i] = 0;
     for (int i = tid; i < p.batch; i += Q_THREADS) {
         int len = p.seq_lens[i];
-        if (len > p.max_pos || len > p.tiles * TILE) {   // beyond what the tables or the scratch were sized for
+        if (len > p.max_pos || (!SPLIT && len > p.tiles * TILE)) {   // beyond what the tables or the scratch were sized for
             lorc_set_status(p.status, LORC_ERR_CAPACITY);
             len = 0;
         }
@@ -177,6 +178,10 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
             // the query may not precede a cached key, nor leave the tables
             lorc_set_status(p.status, LORC_ERR_CAPACITY);
             len = 0;
+        }
+        if (SPLIT && len > min(p.max_rows, p.tiles * TILE)) {    // rows that do not exist are left out, as by the plain kernels
+            lorc_set_status(p.status, LORC_ERR_CAPACITY);
+            len = p.max_rows <= p.tiles * TILE ? p.max_rows : 0;
         }
         sm.lens[i] = len > 0 ? len : 0;
         sm.qrel[i] = qr;
@@ -430,6 +435,18 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
                 const int4 v = sm.unit[buf];
                 un.s = v.x; un.tile = v.y; un.len = v.z; un.hp = v.w; un.valid = v.w >= 0;
             }
+            // SPLIT: whether the page of the warp's first and of its second sixteen tokens lies in the pool
+            bool page_ok[2] = {true, true};
+            if (SPLIT && p.page_table != nullptr) {
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    const int n = un.tile * TILE + quarter * 32 + hf * 16;
+                    if (n < un.len) {
+                        const int page = p.page_table[(long long)(p.seq0 + un.s) * p.max_pages_per_seq + n / p.page_size];
+                        page_ok[hf] = page >= 0 && page < p.n_pages;
+                    }
+                }
+            }
             if (!mbar_wait(&sm.acc_full[buf], (uc >> 1) & 1)) { ok = false; break; }
             tc_fence_after_sync();
             // Packed fp32: every operation below acts on the thread's two adjacent rotary pairs (columns 2c, 2c + 1
@@ -528,6 +545,7 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
             float* l_out = m_out + 4 * p.H_q;
             const int n_first = un.tile * TILE + quarter * 32 + r;
             const int tc0 = (quarter & 1) * 32 + r;
+            auto live = [&](int m) { return n_first + 8 * m < un.len && page_ok[m >> 1]; };    // token r + 8 m takes part
 #pragma unroll
             for (int i = 0; i < G / 4; ++i) {
                 const int h = (un.hp * 2 + grp) * G + 4 * i + c;
@@ -535,7 +553,7 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
                     ssum += tot[m][i];
-                    if (n_first + 8 * m < un.len) mxv = fmaxf(mxv, tot[m][i]);
+                    if (live(m)) mxv = fmaxf(mxv, tot[m][i]);
                 }
                 // a NaN among the scores means non-finite numbers in the cache, the factors or the query
                 if (!SPLIT && ssum != ssum) lorc_set_status(p.status, LORC_ERR_ARG);
@@ -545,9 +563,8 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
                 float lsum = 0.f;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    const bool valid = n_first + 8 * m < un.len;
                     // p = 2^(s - m), rounded to bf16 (the same rounded value enters the denominator)
-                    const float pf = valid ? ex2_approx(tot[m][i] - mref) : 0.f;
+                    const float pf = live(m) ? ex2_approx(tot[m][i] - mref) : 0.f;
                     const bf16 pr = __float2bfloat16_rn(pf);
                     lsum += __bfloat162float(pr);
                     const int tc = tc0 + 8 * m;
@@ -641,7 +658,7 @@ cudaError_t lorc_tc_score_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheV
         sp.n_zero = s0 == 0 ? n_zero : 0;
         sp.status = ctx->status_dev;
         sp.batch = nb; sp.seq0 = s0; sp.H_q = d.n_q_heads; sp.n_hp = d.n_kv_heads / 2; sp.r_k = L.r_k;
-        sp.tiles = tiles; sp.max_pos = d.max_pos;
+        sp.tiles = tiles; sp.max_pos = d.max_pos; sp.max_rows = lorc_tc_max_rows(cv);
         sp.page_size = cv.page_size; sp.max_pages_per_seq = cv.max_pages_per_seq; sp.n_pages = cv.n_pages;
         // units if every sequence were full: an upper bound that only caps the grid
         const long long max_units = ((long long)nb * tiles + 1) / 2 * sp.n_hp;

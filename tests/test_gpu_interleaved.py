@@ -172,3 +172,50 @@ def test_interleaved_rows_past_the_end_may_hold_anything(geom, page, n_splits):
     assert L.lorc_last_path(sess.ctx) == 2
     _close(H.host_f64(out), H.oracle_decode(prob, ck, cv, q))
     sess.close()
+
+
+@pytest.mark.parametrize("geom,page,n_splits", [(G8B, 16, 1), (G8B, 64, 0), (G70B, 32, 2), (G_N512, 128, 0)])
+def test_interleaved_pages_outside_the_pool_are_left_out(geom, page, n_splits):
+    import torch
+    lens = [500, 300, 20]
+    prob, sess, ck, cv = _problem(geom, 96, 136, lens)
+    L, b = sess.L, len(lens)
+    held = H.paged_cache(sess, b, lens, page, order_seed=6, k_rows=ck, v_rows=cv)
+    cache, k, v, sl, ptd, pt = held
+    live = [np.ones(n, dtype=bool) for n in lens]
+    for s, i, entry in ((0, 0, -1), (0, (lens[0] - 1) // page, 10 ** 6), (1, 1, cache.n_pages)):
+        ptd[s, i] = entry
+        live[s][i * page:(i + 1) * page] = False
+    q = synth.queries(b, prob.H_q, 128, 31, 6, 8.0).astype(np.float64)
+    out = torch.zeros(b, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn(sess.ctx, 0, cache, H.dev_bf16(q), out, n_splits=n_splits)
+    assert L.lorc_sync_status(sess.ctx) == L.LORC_ERR_CAPACITY
+    assert L.lorc_last_path(sess.ctx) == 2
+    for s in range(b):
+        pos = np.flatnonzero(live[s])
+        _close(H.host_f64(out[s]), O.decode_attn_latent(ck[s][pos], cv[s][pos], prob.B_k, prob.B_v, q[s], prob.H_kv, prob.theta,
+                                                        INTERLEAVED, pos, lens[s] - 1))
+    sess.close()
+
+
+@pytest.mark.parametrize("page", [0, 16])
+def test_interleaved_length_beyond_the_capacity(page):
+    """The rows that exist are attended, by a query at the end of the length given; the status word reports it."""
+    import torch
+    rows = 208 if page else 203
+    prob, sess, ck, cv = _problem(G8B, 96, 64, [rows, rows])
+    L, lens = sess.L, [rows + 2, 90]
+    if page:
+        held = H.paged_cache(sess, 2, [rows, rows], page, order_seed=6, k_rows=ck, v_rows=cv)
+    else:
+        held = H.contiguous_cache(sess, 2, rows, [rows, rows], ck, cv)
+    held[3][:] = torch.tensor(lens, dtype=torch.int32)
+    q = synth.queries(2, prob.H_q, 128, 31, 7, 8.0).astype(np.float64)
+    out = torch.zeros(2, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn(sess.ctx, 0, held[0], H.dev_bf16(q), out)
+    assert L.lorc_sync_status(sess.ctx) == L.LORC_ERR_CAPACITY
+    assert L.lorc_last_path(sess.ctx) == 2
+    for s, n in enumerate((rows, 90)):
+        _close(H.host_f64(out[s]), O.decode_attn_latent(ck[s][:n], cv[s][:n], prob.B_k, prob.B_v, q[s], prob.H_kv, prob.theta,
+                                                        INTERLEAVED, np.arange(n), lens[s] - 1))
+    sess.close()
