@@ -552,11 +552,12 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
                 float mxv = -INFINITY, ssum = 0.f;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    ssum += tot[m][i];
+                    if (!SPLIT || live(m)) ssum += tot[m][i];
                     if (live(m)) mxv = fmaxf(mxv, tot[m][i]);
                 }
-                // a NaN among the scores means non-finite numbers in the cache, the factors or the query
-                if (!SPLIT && ssum != ssum) lorc_set_status(p.status, LORC_ERR_ARG);
+                // a NaN among the scores means non-finite numbers in the cache, the factors or the query (SPLIT: in rows that
+                // take part)
+                if (ssum != ssum) lorc_set_status(p.status, LORC_ERR_ARG);
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) mxv = fmaxf(mxv, __shfl_xor_sync(0xffffffffu, mxv, o));
                 const float mref = ceilf(mxv);                 // -inf: no token of the sequence in this quarter

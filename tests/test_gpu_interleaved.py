@@ -219,3 +219,23 @@ def test_interleaved_length_beyond_the_capacity(page):
         _close(H.host_f64(out[s]), O.decode_attn_latent(ck[s][:n], cv[s][:n], prob.B_k, prob.B_v, q[s], prob.H_kv, prob.theta,
                                                         INTERLEAVED, np.arange(n), lens[s] - 1))
     sess.close()
+
+
+@pytest.mark.parametrize("style", [0, INTERLEAVED])
+def test_nan_in_a_cached_row_is_an_argument_error_for_both_pairings(style):
+    import torch
+    prob = H.Problem(r_k=64, r_v=64, theta=500000.0, layer=31, style=style, **G8B)
+    sess = H.Session(prob, max_pos=300, batch=2)
+    L, lens = sess.L, [290, 40]
+    rng = np.random.default_rng(1)
+    rows = [[synth.to_bf16_exact(rng.standard_normal((n, 64))) for n in lens] for _ in "kv"]
+    cache, k, v, sl = H.contiguous_cache(sess, 2, 300, lens, *rows)
+    q = H.dev_bf16(synth.queries(2, prob.H_q, 128, 31, 8, 8.0))
+    out = torch.zeros(2, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
+    L.lorc_decode_attn(sess.ctx, 0, cache, q, out)
+    assert L.lorc_sync_status(sess.ctx) == 0
+    k[0, 133, 5] = float("nan")
+    L.lorc_decode_attn(sess.ctx, 0, cache, q, out)
+    assert L.lorc_sync_status(sess.ctx) == L.LORC_ERR_ARG
+    assert L.lorc_last_path(sess.ctx) == 2
+    sess.close()
