@@ -230,8 +230,9 @@ cudaError_t lorc_tc_decode(lorc_ctx* ctx, int layer, const LorcLayer& L, const C
                                      q_pos, st, launches);
         if (e != cudaSuccess) return e;
     }
+    if (d.rope_style == LORC_ROPE_NONE) pos0 = q_pos = nullptr;       // positions play no part
     const cudaError_t e2 = lorc_tc_pv_launch(ctx, L, cv, TL.mapCV, TL.mapBVT, pimg, T->rowmax, tiles, plan, pv_scratch,
-                                             out, latent_out, ml_out, st, launches);
+                                             out, latent_out, pos0, q_pos, ml_out, st, launches);
     if (e2 == cudaSuccess) T->rowmax_dirty = false;
     return e2;
 }

@@ -79,8 +79,8 @@ void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& c
                      LorcPvPlan* plan);
 cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCV,
                               const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, int tiles,
-                              const LorcPvPlan& plan, void* scratch, bf16* out, bool latent_out, float* ml_out,
-                              cudaStream_t st, int* launches);
+                              const LorcPvPlan& plan, void* scratch, bf16* out, bool latent_out, const int32_t* pos0,
+                              const int32_t* q_pos, float* ml_out, cudaStream_t st, int* launches);
 
 // Prompt processing (tc_prefill.cu): attention of the T newest tokens of every sequence (q, out [b, T, H_q, 128]) over
 // the latent cache, causal inside the chunk.  Keys and values are reconstructed once into `scratch`
@@ -128,6 +128,12 @@ __device__ __forceinline__ int lorc_tile_page(const int32_t* table, long long se
         }
     }
     return page;
+}
+
+// Whether the query of a non-empty sequence (a shard, where pos0 and q_pos are given) neither precedes a cached key nor leaves
+// the tables; otherwise the sequence is treated as empty.
+__device__ __forceinline__ bool lorc_query_ok(const int32_t* pos0, const int32_t* q_pos, int s, int len, int max_pos) {
+    return !q_pos || (pos0[s] >= 0 && q_pos[s] < max_pos && q_pos[s] - pos0[s] >= len - 1);
 }
 
 // Order-preserving map from finite floats (and infinities) to unsigned integers: a < b  <=>  key(a) < key(b).  No float

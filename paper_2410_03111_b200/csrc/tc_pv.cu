@@ -67,6 +67,8 @@ struct Pv2Params {
     int* status;
     int batch, H_q, n_kv, r_v, tiles, n_blk, n_csplit, max_pos;
     int max_rows;                  // SPLIT: rows of a sequence that exist
+    const int32_t* pos0;           // as in the score kernel
+    const int32_t* q_pos;
     int page_size, max_pages_per_seq, n_pages;
 };
 
@@ -88,7 +90,7 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
     int len = p.seq_lens[s];
     if (len > p.max_pos) len = 0;                             // the score kernel reports the capacity errors
     if (SPLIT) len = min(len, p.max_rows);
-    if (len > p.tiles * TILE) len = 0;
+    if (len > p.tiles * TILE || (len > 0 && !lorc_query_ok(p.pos0, p.q_pos, s, p.seq_lens[s], p.max_pos))) len = 0;
     if (len < 0) len = 0;
     // this CTA's share of the context: whole 128-token tiles, dealt evenly over the context shares
     const int tiles_s = (len + TILE - 1) / TILE;
@@ -769,8 +771,8 @@ void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& c
 // score kernel clears it).
 cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCV,
                               const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, int tiles,
-                              const LorcPvPlan& plan, void* scratch, bf16* out, bool latent_out, float* ml_out,
-                              cudaStream_t st, int* launches) {
+                              const LorcPvPlan& plan, void* scratch, bf16* out, bool latent_out, const int32_t* pos0,
+                              const int32_t* q_pos, float* ml_out, cudaStream_t st, int* launches) {
     const lorc_model_desc& d = ctx->desc;
     const int n_blk = plan.n_blk, n_csplit = plan.n_csplit;
     const int r_pad = n_blk * 128;
@@ -787,6 +789,7 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
         p.seq_lens = cv.seq_lens; p.page_table = cv.page_table; p.status = ctx->status_dev;
         p.batch = cv.batch; p.H_q = d.n_q_heads; p.n_kv = d.n_kv_heads; p.r_v = L.r_v; p.tiles = tiles;
         p.n_blk = n_blk; p.n_csplit = n_csplit; p.max_pos = d.max_pos; p.max_rows = lorc_tc_max_rows(cv);
+        p.pos0 = pos0; p.q_pos = q_pos;
         p.page_size = cv.page_size; p.max_pages_per_seq = cv.max_pages_per_seq; p.n_pages = cv.n_pages;
         dim3 grid(n_blk, n_csplit, cv.batch);
         auto launch = [&](auto kernel, size_t bytes) {

@@ -174,8 +174,7 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
             len = 0;
         }
         int qr = p.q_pos ? p.q_pos[i] - p.pos0[i] : len - 1;
-        if (qr < len - 1 || qr >= p.max_pos || (p.q_pos && (p.pos0[i] < 0 || p.q_pos[i] >= p.max_pos))) {
-            // the query may not precede a cached key, nor leave the tables
+        if (len > 0 && !lorc_query_ok(p.pos0, p.q_pos, i, len, p.max_pos)) {
             lorc_set_status(p.status, LORC_ERR_CAPACITY);
             len = 0;
         }

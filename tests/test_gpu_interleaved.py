@@ -239,3 +239,38 @@ def test_nan_in_a_cached_row_is_an_argument_error_for_both_pairings(style):
     assert L.lorc_sync_status(sess.ctx) == L.LORC_ERR_ARG
     assert L.lorc_last_path(sess.ctx) == 2
     sess.close()
+
+
+@pytest.mark.parametrize("style", [0, INTERLEAVED])
+def test_shards_that_are_empty_or_end_behind_the_query(style):
+    """An empty shard is no error wherever it starts; a shard whose last token lies behind the query is treated as empty and
+    reported, whatever the workspace holds."""
+    import torch
+    prob = H.Problem(r_k=64, r_v=64, theta=500000.0, layer=31, style=style, **G8B)
+    sess = H.Session(prob, max_pos=400, batch=2)
+    L = sess.L
+    rng = np.random.default_rng(1)
+    rows = [[synth.to_bf16_exact(rng.standard_normal((200, 64))) for _ in range(2)] for _ in "kv"]
+    cache, k, v, sl = H.contiguous_cache(sess, 2, 200, [200, 200], *rows)
+    q = H.dev_bf16(synth.queries(2, prob.H_q, 128, 31, 9, 8.0))
+
+    def shard(lens, pos0, q_pos):
+        sl[:] = torch.tensor(lens, dtype=torch.int32)
+        out = torch.full((2, prob.H_q, 128), 3.0, dtype=torch.bfloat16, device="cuda")
+        ml = torch.full((2, prob.H_q, 2), 3.0, dtype=torch.float32, device="cuda")
+        at = [torch.tensor(p, dtype=torch.int32, device="cuda") for p in (pos0, q_pos)]
+        sess.ws.fill_(255)                                       # NaN in every stale tile image
+        L.lorc_decode_attn_shard(sess.ctx, 0, cache, q, *at, out, ml)
+        status = L.lorc_sync_status(sess.ctx)
+        assert L.lorc_last_path(sess.ctx) == 2
+        return status, H.host_f64(out), H.host_f64(ml)
+
+    status, ref, _ = shard([0, 150], [0, 100], [99, 260])
+    assert status == 0 and np.all(ref[0] == 0.0)
+    status, out, ml = shard([0, 150], [256, 100], [99, 260])     # the empty shard starts behind the query
+    assert status == 0, L.lorc_last_error(sess.ctx)
+    assert np.all(out[0] == 0.0) and np.all(ml[0, :, 1] == 0.0) and np.array_equal(out[1], ref[1])
+    status, out, ml = shard([200, 150], [100, 100], [298, 260])  # the first shard's last token sits at 299
+    assert status == L.LORC_ERR_CAPACITY
+    assert np.all(out[0] == 0.0) and np.all(ml[0, :, 1] == 0.0) and np.array_equal(out[1], ref[1])
+    sess.close()
