@@ -127,9 +127,9 @@ def test_tc_decode_matches_plain_kernels_and_split_counts():
 
 
 def test_tc_decode_many_context_shares_with_64_query_heads():
-    """Eight query heads per KV head, one sequence, one column block: the context is dealt over as many shares as it
-    has tiles, more than one bulk-copy batch of the share reduction holds (four shares of 32 KiB), so the last share
-    adds them up over several batches; forced share counts around the batch size as well."""
+    """Eight query heads per KV head, one sequence, one column block: forced share counts up to one per tile, around and
+    above what one bulk-copy batch of the share reduction holds (four shares of 32 KiB), so that the last share adds
+    them up over several batches.  (The default plan takes one share at these 12 tiles.)"""
     import torch
     prob = H.Problem(GEOM["D"], 64, GEOM["H_kv"], GEOM["d_h"], 128, 128, theta=500000.0, layer=22)
     lens = [1500]
@@ -144,6 +144,33 @@ def test_tc_decode_many_context_shares_with_64_query_heads():
         assert sess.L.lorc_sync_status(sess.ctx) == 0, sess.L.lorc_last_error(sess.ctx)
         assert sess.L.lorc_last_path(sess.ctx) == 2, "the tensor-core path was not taken"
         assert O.rel_l2_rows(H.host_f64(out), want) <= TOL, S
+    sess.close()
+
+
+@pytest.mark.parametrize("H_q,r_v,lens,shares", [
+    (32, 136, [2049], 6),          # 17 tiles: the first length with several shares
+    (32, 72, [2048, 33], 4),       # 16 tiles: four
+    (64, 128, [4200], 7),
+    (32, 128, [1920], 1),          # 15 tiles: one
+])
+def test_tc_decode_default_share_count(H_q, r_v, lens, shares):
+    """Without a share count the plan takes the number of shares whose chain is shortest: to the bit what that number gives
+    when it is asked for, and not what another one gives."""
+    import torch
+    prob = H.Problem(GEOM["D"], H_q, GEOM["H_kv"], GEOM["d_h"], 64, r_v, theta=500000.0, layer=22)
+    b, rng = len(lens), np.random.default_rng(r_v)
+    ck, cv = ([synth.to_bf16_exact(rng.standard_normal((n, r)) * np.arange(1, r + 1) ** -0.8) for n in lens] for r in (64, r_v))
+    q = synth.queries(b, H_q, GEOM["d_h"], 22, 1, 8.0).astype(np.float64)
+    sess = H.Session(prob, max_pos=max(lens), batch=b)
+    held = H.contiguous_cache(sess, b, max(lens), lens, ck, cv)
+    outs = []
+    for S in (0, shares, 2 if shares == 1 else 1):
+        out = torch.zeros(b, H_q, GEOM["d_h"], dtype=torch.bfloat16, device="cuda")
+        sess.L.lorc_decode_attn(sess.ctx, 0, held[0], H.dev_bf16(q), out, n_splits=S)
+        assert sess.L.lorc_sync_status(sess.ctx) == 0, sess.L.lorc_last_error(sess.ctx)
+        H.assert_rows_close(H.host_f64(out), H.oracle_decode(prob, ck, cv, q), TOL, S)
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1]) and not torch.equal(outs[0], outs[2])
     sess.close()
 
 
