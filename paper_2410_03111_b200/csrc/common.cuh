@@ -152,7 +152,8 @@ cudaError_t lorc_generic_merge_shards(const lorc_ctx* ctx, int n_shards, const b
 // part_ml [b, H_q, S, 2] (running max in natural-log units, sum), part_o [b, H_q, S, W].
 cudaError_t lorc_generic_combine(const lorc_ctx* ctx, const LorcLayer& L, int batch, int n_splits,
                                  const float* part_ml, const float* part_o, bf16* out,
-                                 cudaStream_t st, int* launches, bool latent_out = false, float* ml_out = nullptr);
+                                 cudaStream_t st, int* launches, bool latent_out = false, float* ml_out = nullptr,
+                                 bool spare = false);
 // token granularity of a split in the plain decode kernel
 #define LORC_GENERIC_TILE 32
 #define LORC_MAX_SPLITS 256

@@ -97,14 +97,17 @@ struct FdParams {
     int slots;                     // 0: every sequence has n_splits shares; else at most as many, and `slots` together
 };
 
-// Shares of a sequence of `tiles` steps when all of them have `total` (with `slots`): in proportion to its length, so that
-// the blocks of a launch are resident at once and equally long whatever the lengths are.  The sum over the batch is at most
-// slots + batch.  (Steps are counted up to 2^15 a sequence, which keeps the sums of any batch in 32 bits.)
+// Shares of a sequence of `weight` steps when all of them have `total` (with `slots`): in proportion to its length, so that the
+// blocks of a launch are resident at once and about equally long whatever the lengths are.  Its part of `slots`, rounded down,
+// or its part of slots - batch + 1, rounded up (which adds up to at most `slots` too), whichever is more; for equal lengths
+// both are slots / batch.  In all at most slots + batch.  (Steps are counted up to 2^15 a sequence, which keeps the sums of any
+// batch in 32 bits.)
 __device__ __forceinline__ int fd_weight(const FdParams& p, int len) {
     return len <= 0 || len > p.max_pos ? 0 : min((len - 1) / FD_TILE + 1, 1 << 15);
 }
 __device__ __forceinline__ int fd_shares(const FdParams& p, int weight, int total) {
-    return max(1, min(p.n_splits, weight * p.slots / max(total, 1)));
+    const int d = max(total, 1), up = max(p.slots - p.cv.batch + 1, 0);
+    return max(1, min(p.n_splits, max(weight * p.slots / d, (weight * up + d - 1) / d)));
 }
 
 // Block `f` of a KV head -> sequence (-1: none), its length, share, number of shares; executed by whole warps.  (The result

@@ -391,8 +391,9 @@ decode_generic_kernel(const bf16* __restrict__ q, CacheView cv, const bf16* __re
 
 // Merge the splits of one (sequence, head) and apply the value up-projection.  A block is a chain of short steps, each
 // bound by latency: the split weights take one warp (lane = split), the up-projection is split over blockDim / DH slices of
-// the latent columns (3 shares, rank 32: 7.9 -> 5.6 us).
-template <bool LATENT>
+// the latent columns (3 shares, rank 32: 7.9 -> 5.6 us).  SPARE: a sequence may use fewer than n_splits shares; the rows of the
+// others are not read.
+template <bool LATENT, bool SPARE>
 __global__ void __launch_bounds__(256)
 combine_generic_kernel(const float* __restrict__ part_ml, const float* __restrict__ part_o,
                        const bf16* __restrict__ B_v, bf16* __restrict__ out, int W, int n, int DH, int G,
@@ -420,15 +421,15 @@ combine_generic_kernel(const float* __restrict__ part_ml, const float* __restric
             const float2 ml = *reinterpret_cast<const float2*>(part_ml + (unit0 + c) * 2);
             const float w = (ml.y > 0.f) ? expf(ml.x - M) : 0.f;
             w_s[c] = w;
-            if (ml.y != 0.f) used = c + 1;
+            if (SPARE && ml.y != 0.f) used = c + 1;
             L += (double)w * (double)ml.y;
         }
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-        used = __reduce_max_sync(0xffffffffu, used);
+        if (SPARE) used = __reduce_max_sync(0xffffffffu, used);
         if (tid == 0) {
             L_s = (float)L;
-            used_s = used;
+            if (SPARE) used_s = used;
             if (ml_out) {
                 // reference in log2 units and the denominator relative to it (a shard of a context may be empty)
                 ml_out[((long long)s * H_q + h) * 2] = L > 0.0 ? M * 1.4426950408889634f : 0.f;
@@ -440,14 +441,13 @@ combine_generic_kernel(const float* __restrict__ part_ml, const float* __restric
     }
     __syncthreads();
     const float L = L_s;
-    const int used = __reduce_max_sync(0xffffffffu, used_s);      // in a uniform register
+    const int used = SPARE ? __reduce_max_sync(0xffffffffu, used_s) : n_splits;      // (in a uniform register)
     const float inv = (L > 0.f) ? 1.f / L : 0.f;
     for (int col = tid; col < W; col += nt) {
-        const float* po = part_o + unit0 * W + col;
         float a = 0.f;
 #pragma unroll 4
         for (int c = 0; c < used; ++c) {
-            const float w = w_s[c], x = po[c * W];
+            const float w = w_s[c], x = SPARE ? (part_o + unit0 * W + col)[c * W] : part_o[(unit0 + c) * W + col];
             if (w != 0.f) a = fmaf(w, x, a);
         }
         o_lat[col] = a * inv;
@@ -473,7 +473,7 @@ combine_generic_kernel(const float* __restrict__ part_ml, const float* __restric
 
 cudaError_t lorc_generic_combine(const lorc_ctx* ctx, const LorcLayer& L, int batch, int n_splits,
                                  const float* part_ml, const float* part_o, bf16* out,
-                                 cudaStream_t st, int* launches, bool latent_out, float* ml_out) {
+                                 cudaStream_t st, int* launches, bool latent_out, float* ml_out, bool spare) {
     const lorc_model_desc& d = ctx->desc;
     const bool latent = (L.mode == LORC_MODE_LATENT);
     const int W = latent ? L.r_v : d.d_head;
@@ -483,9 +483,10 @@ cudaError_t lorc_generic_combine(const lorc_ctx* ctx, const LorcLayer& L, int ba
     // (not latent, or merge only: the normalised latent output [b, H_q, r_v] is the result, in rows of width W)
     const bool up = latent && !latent_out;
     *launches += 1;
-    return lorc_launch_dependent(up ? combine_generic_kernel<true> : combine_generic_kernel<false>, cgrid,
-                                 dim3(up ? 256 : 128), smem, st, part_ml, part_o, up ? (const bf16*)L.B_v : (const bf16*)nullptr,
-                                 out, W, ctx->n, up ? d.d_head : W, ctx->group, n_splits, ctx->status_dev, ml_out);
+    auto kernel = up ? combine_generic_kernel<true, false>
+                     : spare ? combine_generic_kernel<false, true> : combine_generic_kernel<false, false>;
+    return lorc_launch_dependent(kernel, cgrid, dim3(up ? 256 : 128), smem, st, part_ml, part_o,
+                                 up ? (const bf16*)L.B_v : (const bf16*)nullptr, out, W, ctx->n, up ? d.d_head : W, ctx->group, n_splits, ctx->status_dev, ml_out);
 }
 
 cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv,
@@ -503,7 +504,7 @@ cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheVi
             cudaError_t e = lorc_full_decode(ctx, L, cv, q, n_splits, by_length, part_ml, part_o, st, launches);
             if (e != cudaSuccess) return e;
         }
-        return lorc_generic_combine(ctx, L, cv.batch, n_splits, part_ml, part_o, out, st, launches, false, nullptr);
+        return lorc_generic_combine(ctx, L, cv.batch, n_splits, part_ml, part_o, out, st, launches, false, nullptr, by_length);
     }
     if (T == 1 && lorc_small_decode_supported(ctx, L)) {
         {

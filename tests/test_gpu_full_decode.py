@@ -213,7 +213,8 @@ def test_shares_by_length(lens, H_q, H_kv):
     ml = ws[:b * H_q * room * 8].view(torch.float32).view(b, H_q, room, 2).cpu().numpy()
     steps = np.array([(m + 63) // 64 for m in lens])
     if room > equal:
-        want_shares = np.clip(steps * slots // max(1, steps.sum()), 1, room)
+        up, total = max(slots - b + 1, 0), steps.sum()
+        want_shares = np.clip(np.maximum(steps * slots // total, -(-steps * up // total)), 1, room)
     else:
         want_shares = np.full(b, room)                   # equal parts
     for s, m in enumerate(lens):
