@@ -171,11 +171,11 @@ cudaError_t lorc_generic_append(const lorc_ctx* ctx, const LorcLayer& L, const C
 }
 
 // ---------------------------------------------------------------------------
-// Decode attention, one block per (context split, KV head, sequence).
+// Decode attention, one block per (context split and 1024 columns of the output, KV head, sequence).
 // ---------------------------------------------------------------------------
 #define GEN_TILE LORC_GENERIC_TILE
 #define GEN_GMAX 8          // query heads per KV head supported
-#define GEN_NC 8            // accumulator columns per thread: 8 * 128 = 1024 >= r_v
+#define GEN_NC 8            // accumulator columns per thread: a block covers 8 * 128 = 1024 of the output's
 
 template <int DH, bool LATENT>
 __global__ void __launch_bounds__(128)
@@ -199,9 +199,10 @@ decode_generic_kernel(const bf16* __restrict__ q, CacheView cv, const bf16* __re
     // With T queries per sequence (prompt processing) blockIdx.z runs over (sequence, query): query t of a chunk of T
     // sits at position seq_lens[s] - T + t and sees the tokens up to its own, i.e. it is the decode query of the
     // sequence cut after that token.  sq indexes queries, partial results and outputs; s the cache.
-    const int split = blockIdx.x, g = blockIdx.y, sq = blockIdx.z, s = sq / T;
+    const int split = blockIdx.x % n_splits, g = blockIdx.y, sq = blockIdx.z, s = sq / T;
     const int H_q = G * (int)gridDim.y;
     const int W = LATENT ? r_v : DH;         // width of the output accumulator
+    const int col0 = LATENT ? (int)(blockIdx.x / n_splits) * GEN_NC * 128 : 0;
     int len = cv.seq_lens[s];
     if (T > 1) len = len >= T ? len - (T - 1 - sq % T) : 0;
     // context shards: the cached rows sit at positions p0 .. p0 + len - 1, the query at qpos (not before the last row)
@@ -354,7 +355,7 @@ decode_generic_kernel(const bf16* __restrict__ q, CacheView cv, const bf16* __re
         // O[h][col] = O[h][col]*alpha + sum_t p[h][t] * V[t][col]
 #pragma unroll
         for (int c = 0; c < GEN_NC; ++c) {
-            int col = tid + c * 128;
+            int col = col0 + tid + c * 128;
             if (col >= W) break;
 #pragma unroll
             for (int h = 0; h < GEN_GMAX; ++h)
@@ -377,13 +378,13 @@ decode_generic_kernel(const bf16* __restrict__ q, CacheView cv, const bf16* __re
     for (int h = 0; h < GEN_GMAX; ++h) {
         if (h >= G) break;
         long long unit = ((long long)sq * H_q + g * G + h) * n_splits + split;
-        if (tid == 0) {
+        if (tid == 0 && col0 == 0) {
             part_ml[unit * 2 + 0] = m_s[h];
             part_ml[unit * 2 + 1] = l_s[h];
         }
 #pragma unroll
         for (int c = 0; c < GEN_NC; ++c) {
-            int col = tid + c * 128;
+            int col = col0 + tid + c * 128;
             if (col < W) part_o[unit * W + col] = acc[h][c];
         }
     }
@@ -496,7 +497,8 @@ cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheVi
     const lorc_model_desc& d = ctx->desc;
     const int G = ctx->group;
     const bool latent = (L.mode == LORC_MODE_LATENT);
-    dim3 grid(n_splits, d.n_kv_heads, cv.batch * T);
+    const int col_blocks = latent ? (L.r_v + GEN_NC * 128 - 1) / (GEN_NC * 128) : 1;
+    dim3 grid(n_splits * col_blocks, d.n_kv_heads, cv.batch * T);
     if (T == 1 && lorc_full_decode_supported(ctx, L)) {
         // uncompressed mode with 128-wide heads: the streaming kernel on the warp-level tensor cores
         {

@@ -48,3 +48,33 @@ def test_small_decode(D, H_q, H_kv, d_h, r_k, r_v, lens, style, page, n_splits):
             assert L.lorc_last_path(sess.ctx) == 1
             _close(H.host_f64(out), want)
     sess.close()
+
+
+@pytest.mark.parametrize("entry,flags,r_v", [("lorc_decode_attn", 0, 1032), ("lorc_decode_attn", 1, 1536), ("lorc_decode_attn_static", 0, 1160)])
+def test_value_ranks_above_1024(entry, flags, r_v):
+    """Ranks that only the scalar kernel takes: its blocks cover 1024 columns of the latent output each."""
+    import torch
+    L = H.lib()
+    D, H_q, H_kv, d_h, r_k, lens = 64, 32, 32, 64, 16, [70, 33]
+    n, b, rng = H_kv * d_h, len(lens), np.random.default_rng(r_v)
+    A_k, A_v = (synth.to_bf16_exact(rng.standard_normal((D, r))) for r in (r_k, r_v))
+    B_k, B_v = (synth.to_bf16_exact(rng.standard_normal((r, n)) / np.sqrt(n)) for r in (r_k, r_v))
+    ctx = L.lorc_create(1, D, H_q, H_kv, d_h, 10000.0, max_pos=72, flags=flags)
+    L.lorc_load_factors(ctx, 0, L.LORC_MODE_LATENT, r_k, r_v, *[H.dev_bf16(a) for a in (A_k, B_k, A_v, B_v)])
+    ws = torch.full((L.lorc_workspace_bytes(ctx, b, 72),), 255, dtype=torch.uint8, device="cuda")
+    L.lorc_set_workspace(ctx, ws)
+    ck, cv = ([synth.to_bf16_exact(rng.standard_normal((m, r))) for m in lens] for r in (r_k, r_v))
+    kv = [torch.zeros(b, 72, r, dtype=torch.bfloat16, device="cuda") for r in (r_k, r_v)]
+    for c, rows in zip(kv, (ck, cv)):
+        for s, x in enumerate(rows):
+            c[s, :lens[s]] = H.dev_bf16(x)
+    sl = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    cache = L.make_cache(*kv, sl, b, 72, seq_stride=72)
+    q = synth.queries(b, H_q, d_h, 33, 1, 1.0).astype(np.float64)
+    for n_splits in (0, 2):
+        out = torch.full((b, H_q, d_h), 3.0, dtype=torch.bfloat16, device="cuda")
+        getattr(L, entry)(ctx, 0, cache, H.dev_bf16(q), out, n_splits=n_splits)
+        assert L.lorc_sync_status(ctx) == 0, L.lorc_last_error(ctx)
+        for s in range(b):
+            _close(H.host_f64(out[s]), O.decode_attn_latent(ck[s], cv[s], B_k, B_v, q[s], H_kv, 10000.0))
+    L.lorc_destroy(ctx)
