@@ -18,13 +18,6 @@ namespace {
 // step.  Those 8 values fill the fragment slots of two m16n8k16 steps; x is loaded with the same slot
 // order, so the contraction is unchanged.
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                               uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 
 // FULL (uncompressed mode): the factor is [W_K | W_V] and keys are cached rotated.  The key columns of the tiled
 // factor are permuted (see retile_factor_kernel) so that the two accumulator columns a thread ends up with are the two

@@ -34,13 +34,6 @@ constexpr int FD_STAGES = 3;
 constexpr int FD_THREADS = 160;      // warps 0..3 consumers, warp 4 TMA
 constexpr int FD_BLOCKS_PER_SM = 2;
 
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -293,8 +286,8 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
                 uint32_t a[4];
                 const int piece = 2 * (ks & 3) + (mi >> 1);
                 ldmatrix_x4(a, k0 + (ks >> 2) * (FD_TILE * 128) + k_row + ((piece ^ lr) << 4));
-                mma_16816(sc[ks & 1], a, qhi[ks][0], qhi[ks][1]);
-                mma_16816(sc[2 + (ks & 1)], a, qlo[ks][0], qlo[ks][1]);
+                mma_bf16_16816(sc[ks & 1], a[0], a[1], a[2], a[3], qhi[ks][0], qhi[ks][1]);
+                mma_bf16_16816(sc[2 + (ks & 1)], a[0], a[1], a[2], a[3], qlo[ks][0], qlo[ks][1]);
             }
             float x[4];
 #pragma unroll
@@ -354,8 +347,8 @@ full_decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_co
                 uint32_t a[4];
                 const int piece = 2 * (db & 3) + (mi & 1);
                 ldmatrix_x4_trans(a, v0 + (db >> 2) * (FD_TILE * 128) + v_row + ((piece ^ lr) << 4));
-                mma_16816(o[db], a, b0, b1);
-                mma_16816(o[db], a, c0, c1);
+                mma_bf16_16816(o[db], a[0], a[1], a[2], a[3], b0, b1);
+                mma_bf16_16816(o[db], a[0], a[1], a[2], a[3], c0, c1);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.empty[st]);

@@ -37,14 +37,6 @@ struct SdParams {
     int r_k, r_v, G, n_splits, rope_style, max_pos;
 };
 
-__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                          uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 // GM: query heads per KV head rounded up to 2, 4 or 8 (rows past p.G hold zero queries and are not written)
 template <int DH, int GM>
 __global__ void __launch_bounds__(SD_THREADS)
@@ -139,8 +131,8 @@ small_decode_kernel(const SdParams p) {
                         w[i] = in ? __ldg(reinterpret_cast<const uint4*>(bp + (long long)(n0 + i) * 8 * p.r_k + k0)) : zero;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
-                        mma_16816(k[n0 + i], x.x, y.x, x.y, y.y, w[i].x, w[i].y);
-                        mma_16816(k[n0 + i], x.z, y.z, x.w, y.w, w[i].z, w[i].w);
+                        mma_bf16_16816(k[n0 + i], x.x, y.x, x.y, y.y, w[i].x, w[i].y);
+                        mma_bf16_16816(k[n0 + i], x.z, y.z, x.w, y.w, w[i].z, w[i].w);
                     }
                 }
             }
