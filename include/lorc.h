@@ -106,7 +106,10 @@ typedef struct lorc_model_desc {
  * seq_lens[s] <= max_seq_len (rounded up to a multiple of 128 on the tensor-core
  * path) and seq_lens[s] <= max_pos: a longer sequence is treated as empty and the
  * status word is set to LORC_ERR_CAPACITY; nothing is read or written out of
- * bounds.  Rows at positions >= seq_lens[s] may be read by tile loads; they must
+ * bounds.  (The plain kernels, the streaming kernel of the uncompressed mode and
+ * contexts with interleaved pairs report a sequence that is longer than the
+ * capacity, and pages outside the pool, the same way, but attend to the rows that
+ * exist.)  Rows at positions >= seq_lens[s] may be read by tile loads; they must
  * hold finite numbers (zero the cache once when allocating it). */
 typedef struct lorc_cache {
     void* k;                      /* device */
@@ -172,7 +175,8 @@ int lorc_append(lorc_ctx* ctx, int layer, const lorc_cache* cache, const void* x
  *   k_n = B_K[:, g]^T C_K[n], rotated at n;  q^ = RoPE(q, seq_lens[s]-1);
  *   p = softmax_n(q^ . k_n / sqrt(d_head)),  out = (sum_n p_n C_V[n]) B_V[:, g]
  * over n in [0, seq_lens[s]).  Keys and values are never written to memory.
- * n_splits = 0 lets the library choose how many CTAs share one sequence's context;
+ * n_splits = 0 lets the library choose how many CTAs share one sequence's context
+ * (in the uncompressed mode with 128-wide heads by the lengths of all sequences);
  * a positive value asks for that many shares (context splits of the plain kernels
  * and of the uncompressed mode; context shares per latent column block of the
  * tensor-core path), clamped to what the workspace holds.  Uses the workspace.
@@ -263,8 +267,9 @@ int lorc_decode_attn_static(lorc_ctx* ctx, int layer, const lorc_cache* cache, c
  * q_host [batch, n_q_heads, d_head] to staging at the end of the workspace, runs
  * lorc_append (T = 1) and lorc_decode_attn, and copies the result to out_host
  * [batch, n_q_heads, d_head]; all on `stream`, asynchronously when the host
- * buffers are pinned.  (Pinned, mapped and 16-byte aligned buffers are read and
- * written by the kernels themselves, others by copies.)  The caller synchronises the stream before reading
+ * buffers are pinned.  (Mapped and 16-byte aligned buffers that lie inside one
+ * pinned allocation or registration are read and written by the kernels
+ * themselves, others by copies.)  The caller synchronises the stream before reading
  * out_host.  The cache stays on the device. */
 int lorc_decode_step_host(lorc_ctx* ctx, int layer, const lorc_cache* cache, const void* x_host,
                           const void* q_host, void* out_host, int n_splits, void* stream);

@@ -672,9 +672,9 @@ __global__ void latent_out_kernel(const bf16* __restrict__ o_norm, bf16* __restr
 
 // Column blocks and context shares of one PV launch: one CTA per SM at most, and the number of shares whose chain is shortest.
 // In units of one tile (about 0.45 us of a CTA's stream): the tiles of a share, and with more than one share 8 for publishing
-// it and taking turns at the counter and 0.8 per share for the addition by the last one.  So up to 16 tiles are best left to one
+// it and taking turns at the counter and 0.8 per share for the addition by the last one.  So up to 15 tiles are best left to one
 // CTA, and more than about sqrt(tiles / 0.8) shares never pay.  (As many shares as fill the SMs, which was the rule before,
-// cost 2 to 3 us a call up to 16 tiles and most at long contexts of one user: 8B shape, one layer with its cache write, 8200
+// cost 2 to 3 us a call up to 15 tiles and most at long contexts of one user: 8B shape, one layer with its cache write, 8200
 // tokens, rank 256: 64 shares 41 us, 9 shares 26 us; 1037 tokens, rank 928: 9 shares 27.0 us, one 24.8 us.)
 void pv_plan(const lorc_ctx* ctx, const LorcLayer& L, int batch, int max_seq_len, int n_splits_hint, int* n_blk,
              int* n_csplit) {
