@@ -179,7 +179,7 @@ int lorc_append(lorc_ctx* ctx, int layer, const lorc_cache* cache, const void* x
  * (in the uncompressed mode with 128-wide heads by the lengths of all sequences);
  * a positive value asks for that many shares (context splits of the plain kernels
  * and of the uncompressed mode; context shares per latent column block of the
- * tensor-core path), clamped to what the workspace holds.  Uses the workspace.
+ * tensor-core path, at most 16), clamped to what the workspace holds.  Uses the workspace.
  * A sequence with seq_lens[s] <= 0 gets a row of zeros and sets status EMPTY.
  * The first call on a context, and the first call with a larger batch than any
  * before, sets up small library-owned tables (an in-tile rotation table, one word

@@ -393,19 +393,29 @@ static inline bool lorc_make_tmap_bf16(CUtensorMap* map, const void* base, int r
     return r == CUDA_SUCCESS;
 }
 
-// Launch with the programmatic-serialization attribute (see grid_dep_wait above).
+// Launch with the programmatic-serialization attribute (see grid_dep_wait above); clusters of cluster_y blocks along y where
+// that is more than one.
 template <typename... KArgs>
-static inline cudaError_t lorc_launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                                cudaStream_t stream, KArgs... args) {
+static inline cudaError_t lorc_launch_dependent_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int cluster_y,
+                                                        cudaStream_t stream, KArgs... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = (unsigned)cluster_y;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster_y > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... KArgs>
+static inline cudaError_t lorc_launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                                cudaStream_t stream, KArgs... args) {
+    return lorc_launch_dependent_cluster(kernel, grid, block, smem, 1, stream, args...);
 }

@@ -136,9 +136,8 @@ struct AbsParams {
     unsigned* rowmax;              // [b, H_q]
     const int32_t* seq_lens;
     const int32_t* page_table;
-    int* zero;
     int* status;
-    int batch, seq0, H_q, r_k, tiles, n_zero, max_pos;
+    int batch, seq0, H_q, r_k, tiles, max_pos;
     int page_size, max_pages_per_seq, n_pages;
 };
 
@@ -176,8 +175,6 @@ lorc_score_absorbed_kernel(const __grid_constant__ CUtensorMap mapCK, const __gr
         prefetch_tensormap(&mapQ);
     }
     grid_dep_wait();                                     // q~ comes from the kernel before this one
-    if (blockIdx.x == 0)
-        for (int i = tid; i < p.n_zero; i += A_THREADS) p.zero[i] = 0;
     for (int i = tid; i < p.batch; i += A_THREADS) {
         int len = p.seq_lens[i];
         if (len > p.max_pos || len > p.tiles * TILE) {
@@ -399,8 +396,8 @@ cudaError_t lorc_tc_absorbed_set_attrs() {
 // qabs: scratch of lorc_tc_absorbed_scratch_bytes.  Launches the absorb kernel and the score kernel (one pair per
 // block of LORC_SCORE_MAX_BATCH sequences); outputs as lorc_tc_score_launch.
 cudaError_t lorc_tc_score_absorbed_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCK,
-                                          const bf16* q, bf16* qabs, uint8_t* pimg, unsigned* rowmax, int tiles, int* zero,
-                                          int n_zero, cudaStream_t st, int* launches) {
+                                          const bf16* q, bf16* qabs, uint8_t* pimg, unsigned* rowmax, int tiles,
+                                          cudaStream_t st, int* launches) {
     const lorc_model_desc& d = ctx->desc;
     const int r_ld = (L.r_k + KC - 1) / KC * KC;
     const size_t img_bytes = (size_t)lorc_tc_image_bytes(d.n_q_heads, false);
@@ -425,8 +422,6 @@ cudaError_t lorc_tc_score_absorbed_launch(lorc_ctx* ctx, const LorcLayer& L, con
         ap.rowmax = rowmax + (size_t)s0 * d.n_q_heads;
         ap.seq_lens = cv.seq_lens + s0;
         ap.page_table = cv.page_table;
-        ap.zero = zero;
-        ap.n_zero = s0 == 0 ? n_zero : 0;
         ap.status = ctx->status_dev;
         ap.batch = nb; ap.seq0 = s0; ap.H_q = d.n_q_heads; ap.r_k = L.r_k; ap.tiles = tiles; ap.max_pos = d.max_pos;
         ap.page_size = cv.page_size; ap.max_pages_per_seq = cv.max_pages_per_seq; ap.n_pages = cv.n_pages;

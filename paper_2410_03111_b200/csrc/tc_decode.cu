@@ -106,7 +106,7 @@ static size_t tc_absorbed_bytes(const lorc_ctx* ctx, int batch) {
 size_t lorc_tc_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_len) {
     if (!tc_shape_ok(ctx)) return 0;
     return tc_image_area_bytes(ctx, batch, max_seq_len) + tc_absorbed_bytes(ctx, batch) +
-           lorc_tc_pv_scratch_bytes(ctx, batch, max_seq_len);
+           lorc_tc_pv_scratch_bytes(ctx, batch);
 }
 
 static bool build_cache_maps(LorcTcLayer& T, const LorcLayer& L, const CacheView& cv, int box_rows) {
@@ -218,16 +218,13 @@ cudaError_t lorc_tc_decode(lorc_ctx* ctx, int layer, const LorcLayer& L, const C
     T->rowmax_dirty = true;
     {
         LorcStageTimer timer(ctx, LORC_STAGE_SCORE, st);
-        int* zero = (int*)((char*)pv_scratch + plan.off_done);
         cudaError_t e;
         if (d.rope_style == LORC_ROPE_NONE)
             // no rotation between the key up-projection and the dot product: the up-projection moves to the query
-            e = lorc_tc_score_absorbed_launch(ctx, L, cv, TL.mapCK, q, qabs, pimg, T->rowmax, tiles, zero,
-                                              cv.batch * plan.n_blk, st, launches);
+            e = lorc_tc_score_absorbed_launch(ctx, L, cv, TL.mapCK, q, qabs, pimg, T->rowmax, tiles, st, launches);
         else
             e = lorc_tc_score_launch(ctx, L, cv, TL.mapCK, TL.mapBKT, q, pimg, T->rowmax,
-                                     reinterpret_cast<const float4*>(T->rope_tile), tiles, zero, cv.batch * plan.n_blk, pos0,
-                                     q_pos, st, launches);
+                                     reinterpret_cast<const float4*>(T->rope_tile), tiles, pos0, q_pos, st, launches);
         if (e != cudaSuccess) return e;
     }
     if (d.rope_style == LORC_ROPE_NONE) pos0 = q_pos = nullptr;       // positions play no part

@@ -46,14 +46,14 @@ __host__ __device__ inline int lorc_tc_image_bytes(int n_q_heads, bool split) {
 
 // Score kernel (tc_score.cu): key reconstruction, rotation, q.k and the softmax numerators; writes one tile image per
 // 128 tokens into pimg [b, tiles, image] and raises the row maxima (integers, as order-preserving keys).  rope_tile:
-// the in-tile rotation table (33 x 32 float4, lorc_tc_rope_tile_fill).  Its first block clears zero[0 .. n_zero).
+// the in-tile rotation table (33 x 32 float4, lorc_tc_rope_tile_fill).
 #define LORC_SCORE_MAX_BATCH 64      // sequences per launch (larger batches take several launches)
 cudaError_t lorc_tc_score_set_attrs();
 cudaError_t lorc_tc_rope_tile_fill(float2* table, double theta, cudaStream_t st);
 cudaError_t lorc_tc_score_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCK,
                                  const CUtensorMap& mapBKT, const bf16* q, uint8_t* pimg, unsigned* rowmax,
-                                 const float4* rope_tile, int tiles, int* zero, int n_zero, const int32_t* pos0,
-                                 const int32_t* q_pos, cudaStream_t st, int* launches);
+                                 const float4* rope_tile, int tiles, const int32_t* pos0, const int32_t* q_pos, cudaStream_t st,
+                                 int* launches);
 
 // Score kernel of layers without rotation (tc_absorbed.cu): the key up-projection is absorbed into the query
 // (q~ = B_K q, written to `qabs`, lorc_tc_absorbed_scratch_bytes of scratch), the scores are a skinny GEMM over the
@@ -61,21 +61,19 @@ cudaError_t lorc_tc_score_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheV
 size_t lorc_tc_absorbed_scratch_bytes(const lorc_ctx* ctx, int batch);
 cudaError_t lorc_tc_absorbed_set_attrs();
 cudaError_t lorc_tc_score_absorbed_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCK,
-                                          const bf16* q, bf16* qabs, uint8_t* pimg, unsigned* rowmax, int tiles, int* zero,
-                                          int n_zero, cudaStream_t st, int* launches);
+                                          const bf16* q, bf16* qabs, uint8_t* pimg, unsigned* rowmax, int tiles,
+                                          cudaStream_t st, int* launches);
 
 // P.C_V and value up-projection (tc_pv.cu).  mapCV: C_V cache in 64-column x 128-row (or page-sized) swizzled boxes;
 // mapBVT: B_V^T [n, r_v] in swizzled boxes of 64 latent columns x 32 rows.  The plan says how a launch splits the
-// work and where its pieces of scratch lie; the `done` words (plan.n_blk * batch ints at off_done) must be zero when
-// the PV kernel starts.  The up-projection kernel writes `out` and leaves the row maxima empty again.
+// work: column blocks and context shares of each.  The up-projection kernel writes `out` and leaves the row maxima empty again.
 struct LorcPvPlan {
     int n_blk, n_csplit;
     bool fits;
-    size_t off_on, off_done;
 };
-size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq_len);
+size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch);
 cudaError_t lorc_tc_pv_set_attrs();
-void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
+void lorc_tc_pv_plan(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
                      LorcPvPlan* plan);
 cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCV,
                               const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, int tiles,

@@ -8,13 +8,14 @@
 // epilogue warps multiply it by 2^(m - M), M the reference of the whole sequence (exact: only the exponent changes),
 // and add up the denominator; then
 //       O_lat^T += C_V[tile, block]^T . P^T                    tcgen05, MN-major A
-// and at the end the CTA writes its 128 x H_q piece of the latent output, normalised, as bf16 (with several context
-// shares, the share that finishes last adds the others' pieces and denominators first).
+// and at the end the CTA writes its 128 x H_q piece of the latent output, normalised, as bf16.  Several context shares of a
+// block form a cluster: each leaves its piece in shared memory, and each adds up and writes its part of the heads and columns.
 //
 // Up-projection.  One CTA per (KV head g, 64 output rows = 64 / G sequences, quarter of the head's columns)
 // multiplies those rows by B_V[:, g] (TMA-staged from a transposed copy): out = o . B_V[:, g] in TMEM, then bf16.
 #include <math.h>
 
+#include "sm100_pair.cuh"
 #include "sm100_ptx.cuh"
 #include "tc_kernels.cuh"
 
@@ -50,17 +51,14 @@ struct Pv2Smem {
     float red[128 / HQ][HQ];
     float m_row[HQ];                      // row maximum over the whole sequence
     float l_inv[HQ];
-    uint64_t vfull[P_STAGES], pfull[P_STAGES], fixed[P_STAGES], empty[P_STAGES], o_full, red_full;
+    uint64_t vfull[P_STAGES], pfull[P_STAGES], fixed[P_STAGES], empty[P_STAGES], o_full;
     uint32_t tmem_base;
-    int last;
 };
 
 struct Pv2Params {
     const uint8_t* pimg;           // [b, tiles, image]
-    float* o_part;                 // [b, n_blk, n_csplit, H_q * 128 + H_q]   un-normalised latent output and denominator of every context share
     unsigned* rowmax;              // [b, H_q]   row maxima of the softmax (order-preserving keys of integers)
     bf16* o_norm;                  // [b, H_q, r_pad]      normalised latent output; SPLIT: [b, H_q, 2, r_pad], remainders second
-    int* done;                     // [b, n_blk]           context shares of a column block that have finished (zero on entry)
     float* ml_out;                 // NULL, or [b, H_q, 2]: reference M (log2 units) and denominator sum_n 2^(s_n - M)
     const int32_t* seq_lens;
     const int32_t* page_table;
@@ -107,7 +105,6 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
             mbar_init(&sm.empty[i], 1);
         }
         mbar_init(&sm.o_full, 1);
-        mbar_init(&sm.red_full, 1);
         fence_barrier_init();
         prefetch_tensormap(&mapCV);
     }
@@ -120,6 +117,9 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
     tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
     bool ok = true;
+    constexpr int XLD = 132;                              // floats per row of the exchanges (16-byte rows, spread over the banks)
+    const int r_pad = p.n_blk * 128;
+    const int r_ld = SPLIT ? 2 * r_pad : r_pad;           // row of o_norm
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -229,7 +229,6 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
         // ------------------------------------------------------------------ exponent shift, then epilogue
         const int t = tid - 64;
         const int quarter = warp % 4;
-        const int r_pad = p.n_blk * 128;
         constexpr int PARTS = 128 / HQ;                   // threads per head in the denominator sums
         grid_dep_wait();                                  // images and row maxima come from the kernel before this one
         grid_dep_launch();
@@ -323,7 +322,6 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
         constexpr int QROWS = NR <= 64 ? 16 : 32;
         const int hrow = (SPLIT ? quarter & 1 : quarter) * QROWS + lane;     // the head this thread reads
         const bool has_row = lane < QROWS && hrow < HQ && (!SPLIT || quarter < 2);
-        constexpr int XLD = 132;                          // floats per row of the exchange (16-byte rows, spread over the banks)
         float* xch = reinterpret_cast<float*>(&sm.V[0][0][0]);
         if (SPLIT) {
             // the products of the remainders go to the threads that hold the heads' other part (the C_V stages are free:
@@ -370,8 +368,6 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                 }
             }
         };
-        const int r_ld = SPLIT ? 2 * r_pad : r_pad;       // row of o_norm
-        constexpr int SHARE_FLOATS = HQ * 128 + HQ;
         if (p.n_csplit == 1) {
             if (t < HQ) {
                 sm.l_inv[t] = l_share > 0.f ? 1.f / l_share : 0.f;
@@ -410,10 +406,8 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                 }
             }
         } else {
-            // publish this share (a contiguous block: [H_q][128] outputs, then [H_q] denominators); the share that
-            // arrives last adds them all up (in share order, so the result does not depend on which one that is)
-            float* blk_base = p.o_part + ((long long)s * p.n_blk + blk) * p.n_csplit * SHARE_FLOATS;
-            float* op = blk_base + (long long)cs * SHARE_FLOATS;
+            // this share's piece, for the CTAs of the cluster
+            float* share = xch + (SPLIT ? HQ * XLD : 0);
 #pragma unroll
             for (int c0 = 0; c0 < 128; c0 += 32) {
                 uint32_t r[32];
@@ -421,70 +415,61 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                 if (has_row) {
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4)
-                        *reinterpret_cast<uint4*>(op + hrow * 128 + c0 + q4 * 4) =
+                        *reinterpret_cast<uint4*>(share + hrow * XLD + c0 + q4 * 4) =
                             make_uint4(r[q4 * 4], r[q4 * 4 + 1], r[q4 * 4 + 2], r[q4 * 4 + 3]);
                 }
             }
-            if (t < HQ) op[HQ * 128 + t] = l_share;
-            __threadfence();
-            __syncwarp();   // a named barrier counts a warp once only if the warp arrives converged
-            asm volatile("bar.sync 2, 128;" ::: "memory");
-            if (t == 0) sm.last = atomicAdd(p.done + s * p.n_blk + blk, 1) == p.n_csplit - 1;
-            __syncwarp();   // a named barrier counts a warp once only if the warp arrives converged
-            asm volatile("bar.sync 2, 128;" ::: "memory");
-            if (sm.last != 0) {
-                __threadfence();
-                // The shares come in by bulk copy, a batch at a time, into the C_V stages (every MMA that read them has
-                // completed: o_full): one round trip per batch instead of one per share.  Thread = latent column.
-                constexpr int PER = (P_STAGES * 2 * TILE * KC * 2) / (SHARE_FLOATS * 4);
-                float* stage = reinterpret_cast<float*>(&sm.V[0][0][0]);
-                float acc[HQ];
-#pragma unroll
-                for (int h = 0; h < HQ; ++h) acc[h] = 0.f;
-                l_share = 0.f;
-                uint32_t par = 0;
-                for (int c0 = 0; c0 < p.n_csplit && ok; c0 += PER) {
-                    const int nb = min(PER, p.n_csplit - c0);
-                    if (c0 > 0) {
-                        __syncwarp();
-                        asm volatile("bar.sync 2, 128;" ::: "memory");   // everyone has added the previous batch
-                    }
-                    if (t == 0) {
-                        fence_proxy_async_all();     // the other shares' stores (seen through the counter) before the copies
-                        mbar_arrive_expect_tx(&sm.red_full, (uint32_t)(nb * SHARE_FLOATS * 4));
-                        for (int j = 0; j < nb; ++j)
-                            bulk_load(stage + j * SHARE_FLOATS, blk_base + (long long)(c0 + j) * SHARE_FLOATS,
-                                      SHARE_FLOATS * 4, &sm.red_full);
-                    }
-                    if (!mbar_wait(&sm.red_full, par)) { ok = false; break; }
-                    par ^= 1;
-                    for (int j = 0; j < nb; ++j) {
-#pragma unroll
-                        for (int h = 0; h < HQ; ++h) acc[h] += stage[j * SHARE_FLOATS + h * 128 + t];
-                        if (t < HQ) l_share += stage[j * SHARE_FLOATS + HQ * 128 + t];
-                    }
-                }
-                if (t < HQ) {
-                    sm.l_inv[t] = l_share > 0.f ? 1.f / l_share : 0.f;
-                    if (!(l_share > 0.f) && blk == 0 && !p.ml_out) lorc_set_status(p.status, LORC_ERR_EMPTY);
-                    if (p.ml_out && blk == 0) {
-                        p.ml_out[((long long)s * p.H_q + t) * 2] = sm.m_row[t];
-                        p.ml_out[((long long)s * p.H_q + t) * 2 + 1] = l_share;
-                    }
-                }
-                __syncwarp();
-                asm volatile("bar.sync 2, 128;" ::: "memory");
-                bf16* on = p.o_norm + (long long)s * p.H_q * r_ld + rho0 + t;
-#pragma unroll
-                for (int h = 0; h < HQ; ++h) {
-                    const float x = acc[h] * sm.l_inv[h];
-                    const bf16 hi = __float2bfloat16_rn(x);
-                    on[(long long)h * r_ld] = hi;
-                    if (SPLIT) on[(long long)h * r_ld + r_pad] = __float2bfloat16_rn(x - __bfloat162float(hi));
-                }
-            }
+            if (t < HQ) sm.l_inv[t] = l_share;
         }
         if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
+    }
+    if (p.n_csplit > 1) {
+        // The pieces of all shares are there; each CTA takes every n_csplit-th group of 128 x four columns and adds the shares up in
+        // their order.  (Through memory, with the last share to arrive adding all of them, this took 5 us for two shares and 9 for
+        // eighteen.  Interleaved pairs, b 4, 2049 tokens, six shares: step 33.6 -> 31.1 us; 70B shape, b 8, 8201 tokens, two to five
+        // shares: 364 -> 353 us for three layers; b 4, 32777 tokens, r 256: 216 -> 212 us for two.)
+        __syncwarp();
+        cluster_arrive_release();
+        cluster_wait_acquire();
+        if (warp >= 2) {
+            const uint32_t share0 = smem_u32(&sm.V[0][0][0]) + (SPLIT ? HQ * XLD * 4 : 0), l0 = smem_u32(sm.l_inv);
+            for (int i = cs * 128 + tid - 64; i < HQ * 32; i += p.n_csplit * 128) {
+                const int h = i >> 5, c = (i & 31) * 4;
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                float l = 0.f;
+#pragma unroll 4
+                for (int j = 0; j < p.n_csplit; ++j) {
+                    const float4 v = ld_cluster_f4(mapa_shared(share0 + (h * XLD + c) * 4, j));
+                    l += ld_cluster_f1(mapa_shared(l0 + h * 4, j));
+                    x.x += v.x; x.y += v.y; x.z += v.z; x.w += v.w;
+                }
+                if (blk == 0 && c == 0) {
+                    if (p.ml_out) {
+                        p.ml_out[((long long)s * p.H_q + h) * 2] = sm.m_row[h];
+                        p.ml_out[((long long)s * p.H_q + h) * 2 + 1] = l;
+                    } else if (!(l > 0.f)) {
+                        lorc_set_status(p.status, LORC_ERR_EMPTY);
+                    }
+                }
+                const float li = l > 0.f ? 1.f / l : 0.f;
+                const float y[4] = {x.x * li, x.y * li, x.z * li, x.w * li};
+                bf16* on = p.o_norm + ((long long)s * p.H_q + h) * r_ld + rho0 + c;
+                uint32_t w[2], wl[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(y[2 * e], y[2 * e + 1]);
+                    w[e] = *reinterpret_cast<const uint32_t*>(&b2);
+                    const float2 h2 = __bfloat1622float2(b2);
+                    const __nv_bfloat162 l2 = __floats2bfloat162_rn(y[2 * e] - h2.x, y[2 * e + 1] - h2.y);
+                    wl[e] = *reinterpret_cast<const uint32_t*>(&l2);
+                }
+                *reinterpret_cast<uint2*>(on) = make_uint2(w[0], w[1]);
+                if (SPLIT) *reinterpret_cast<uint2*>(on + r_pad) = make_uint2(wl[0], wl[1]);
+            }
+            __syncwarp();
+        }
+        cluster_arrive_release();                        // no CTA leaves while another may still read its piece
+        cluster_wait_acquire();
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -670,46 +655,50 @@ __global__ void latent_out_kernel(const bf16* __restrict__ o_norm, bf16* __restr
     }
 }
 
-// Column blocks and context shares of one PV launch: one CTA per SM at most, and the number of shares whose chain is shortest.
-// In units of one tile (about 0.45 us of a CTA's stream): the tiles of a share, and with more than one share 8 for publishing
-// it and taking turns at the counter and 0.8 per share for the addition by the last one.  So up to 15 tiles are best left to one
-// CTA, and more than about sqrt(tiles / 0.8) shares never pay.  (As many shares as fill the SMs, which was the rule before,
-// cost 2 to 3 us a call up to 15 tiles and most at long contexts of one user: 8B shape, one layer with its cache write, 8200
-// tokens, rank 256: 64 shares 41 us, 9 shares 26 us; 1037 tokens, rank 928: 9 shares 27.0 us, one 24.8 us.)
-void pv_plan(const lorc_ctx* ctx, const LorcLayer& L, int batch, int max_seq_len, int n_splits_hint, int* n_blk,
-             int* n_csplit) {
-    const int tiles = (max_seq_len + TILE - 1) / TILE;
-    *n_blk = (L.r_v + 127) / 128;
-    int most = n_splits_hint > 0 ? n_splits_hint : ctx->sm_count / (batch * *n_blk);
-    if (most > tiles) most = tiles;
-    if (most > 64) most = 64;
-    if (most < 1) most = 1;
-    *n_csplit = most;
-    if (n_splits_hint > 0) return;
-    int best = 5 * tiles;                                     // five times the cost, in tiles
-    *n_csplit = 1;
-    for (int cs = 2; cs <= most; ++cs) {
-        const int cost = 5 * ((tiles + cs - 1) / cs + 8) + 4 * cs;
-        if (cost < best) {
-            best = cost;
-            *n_csplit = cs;
-        }
-    }
+// Scratch: the normalised latent output [b][H_q][parts][r_pad] of a layer with n_blk column blocks.
+size_t on_bytes(const lorc_ctx* ctx, int batch, int n_blk) {
+    return lorc_align_up((size_t)batch * ctx->desc.n_q_heads * (lorc_tc_split(ctx) ? 2 : 1) * n_blk * 128 * sizeof(bf16), 256);
 }
 
-struct PvScratch {
-    size_t part_bytes, on_bytes, done_bytes;
-};
+template <class Fn>
+cudaError_t with_pv_kernel(const lorc_ctx* ctx, Fn fn) {
+    const bool split = lorc_tc_split(ctx);
+    if (ctx->desc.n_q_heads == 32)
+        return split ? fn(lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>) + 1024)
+                     : fn(lorc_pv2_kernel<32, false>, sizeof(Pv2Smem<32, false>) + 1024);
+    return split ? fn(lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>) + 1024)
+                 : fn(lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>) + 1024);
+}
 
-PvScratch pv_scratch_layout(const lorc_ctx* ctx, int batch, int n_csplit, size_t r_pad) {
-    PvScratch z;
-    const size_t parts = lorc_tc_split(ctx) ? 2 : 1;
-    const size_t hq = (size_t)ctx->desc.n_q_heads;
-    // [b][n_blk][n_csplit][H_q * 128 + H_q]
-    z.part_bytes = n_csplit > 1 ? lorc_align_up((size_t)batch * (r_pad / 128) * n_csplit * (hq * 128 + hq) * sizeof(float), 256) : 256;
-    z.on_bytes = lorc_align_up((size_t)batch * hq * parts * r_pad * sizeof(bf16), 256);
-    z.done_bytes = lorc_align_up((size_t)batch * (r_pad / 128) * sizeof(int), 256);
-    return z;
+constexpr int PV_MAX_SHARES = 16;    // the largest cluster
+
+// Clusters of `shares` blocks that are resident at once (asked for once per context; 0: no such launch).
+int pv_clusters(lorc_ctx* ctx, int shares) {
+    if (shares == 1) return ctx->sm_count;
+    int& known = ctx->pv_clusters[shares];
+    if (known == 0) {
+        int n = 0;
+        const cudaError_t e = with_pv_kernel(ctx, [&](auto kernel, size_t smem) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(1, shares, 1);
+            cfg.blockDim = dim3(P_THREADS);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 1;
+            attr[0].val.clusterDim.y = (unsigned)shares;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+        });
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        known = n > 0 ? n : -1;
+    }
+    return known > 0 ? known : 0;
 }
 
 }  // namespace
@@ -717,58 +706,51 @@ PvScratch pv_scratch_layout(const lorc_ctx* ctx, int batch, int n_csplit, size_t
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq_len) {
-    // the planned number of context shares for the narrowest layer (one column block), which is the largest
-    const int tiles = (max_seq_len + TILE - 1) / TILE;
-    int cs = 2 * ctx->sm_count / batch;
-    if (cs > tiles) cs = tiles;
-    if (cs > 64) cs = 64;
-    if (cs < 1) cs = 1;
-    const size_t r_pad = (size_t)((ctx->n + 127) / 128) * 128;
-    size_t worst = 0;
-    // the share area grows with (column blocks x shares), which the plan keeps near the number of SMs
-    for (int n_blk = 1; n_blk <= (int)(r_pad / 128); ++n_blk) {
-        int c = ctx->sm_count / (batch * n_blk);
-        if (c > cs) c = cs;
-        if (c < 1) c = 1;
-        const PvScratch z = pv_scratch_layout(ctx, batch, c, (size_t)n_blk * 128);
-        if (z.part_bytes > worst) worst = z.part_bytes;
-    }
-    const PvScratch z = pv_scratch_layout(ctx, batch, 1, r_pad);
-    return worst + z.on_bytes + z.done_bytes;
-}
+size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch) { return on_bytes(ctx, batch, (ctx->n + 127) / 128); }
 
 cudaError_t lorc_tc_pv_set_attrs() {
-    auto attr = [](const void* kernel, size_t bytes) {
+    auto attr = [](const void* kernel, size_t bytes, bool wide_clusters) {
+        cudaError_t e = wide_clusters ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
+        if (e != cudaSuccess) return e;
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes + 1024);
     };
-    cudaError_t e = attr((const void*)lorc_pv2_kernel<32, false>, sizeof(Pv2Smem<32, false>));
-    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>));
-    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>));
-    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>));
-    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel<false>, sizeof(UpSmem<false>));
-    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel<true>, sizeof(UpSmem<true>));
+    cudaError_t e = attr((const void*)lorc_pv2_kernel<32, false>, sizeof(Pv2Smem<32, false>), true);
+    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>), true);
+    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>), true);
+    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>), true);
+    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel<false>, sizeof(UpSmem<false>), false);
+    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel<true>, sizeof(UpSmem<true>), false);
     return e;
 }
 
-void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
+// One CTA per SM at most, as many clusters as are resident at once, and the number of shares whose chain is shortest.  In units
+// of one tile (about 0.45 us of a CTA's stream): the tiles of a share, and with more than one share 8 and 0.8 per share.  So up to
+// 15 tiles one CTA takes a block.  (That is what merging through memory cost; the exchange in the cluster takes about 2 us less.
+// But the number of shares decides in which order a block's sums are taken, and calls that leave it to the library keep their
+// results to the bit.)
+void lorc_tc_pv_plan(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
                      LorcPvPlan* plan) {
-    int n_blk, n_csplit;
-    pv_plan(ctx, L, cv.batch, cv.max_seq_len, n_splits_hint, &n_blk, &n_csplit);
-    PvScratch z;
-    for (;; --n_csplit) {
-        z = pv_scratch_layout(ctx, cv.batch, n_csplit, (size_t)n_blk * 128);
-        if (z.part_bytes + z.on_bytes + z.done_bytes <= scratch_bytes || n_csplit == 1) break;
+    const int tiles = (cv.max_seq_len + TILE - 1) / TILE, most = tiles < PV_MAX_SHARES ? tiles : PV_MAX_SHARES;
+    plan->n_blk = (L.r_v + 127) / 128;
+    plan->n_csplit = 1;
+    plan->fits = on_bytes(ctx, cv.batch, plan->n_blk) <= scratch_bytes;
+    const long long blocks = (long long)cv.batch * plan->n_blk;
+    if (n_splits_hint > 0) {
+        plan->n_csplit = n_splits_hint < most ? n_splits_hint : most;
+        while (plan->n_csplit > 1 && pv_clusters(ctx, plan->n_csplit) == 0) --plan->n_csplit;
+        return;
     }
-    plan->n_blk = n_blk;
-    plan->n_csplit = n_csplit;
-    plan->fits = z.part_bytes + z.on_bytes + z.done_bytes <= scratch_bytes;
-    plan->off_on = z.part_bytes;
-    plan->off_done = z.part_bytes + z.on_bytes;
+    int best = 5 * tiles;                                     // five times the cost, in tiles
+    for (int cs = 2; cs <= most && blocks * cs <= ctx->sm_count; ++cs) {
+        const int cost = 5 * ((tiles + cs - 1) / cs + 8) + 4 * cs;
+        if (cost < best && blocks <= pv_clusters(ctx, cs)) {
+            best = cost;
+            plan->n_csplit = cs;
+        }
+    }
 }
 
-// scratch: [o_part | o_norm | done]; `done` (plan.n_blk * batch words) must be zero when the PV kernel starts (the
-// score kernel clears it).
+// scratch: the normalised latent output
 cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCV,
                               const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, int tiles,
                               const LorcPvPlan& plan, void* scratch, bf16* out, bool latent_out, const int32_t* pos0,
@@ -778,29 +760,21 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
     const int r_pad = n_blk * 128;
     const bool split = lorc_tc_split(ctx);
     const int r_ld = split ? 2 * r_pad : r_pad;        // row of o_norm
-    float* o_part = (float*)scratch;
-    bf16* o_norm = (bf16*)((char*)scratch + plan.off_on);
-    int* done = (int*)((char*)scratch + plan.off_done);
+    bf16* o_norm = (bf16*)scratch;
     cudaError_t e;
     {
         LorcStageTimer timer(ctx, LORC_STAGE_PV, st);
         Pv2Params p;
-        p.pimg = pimg; p.o_part = o_part; p.rowmax = rowmax; p.o_norm = o_norm; p.done = done; p.ml_out = ml_out;
+        p.pimg = pimg; p.rowmax = rowmax; p.o_norm = o_norm; p.ml_out = ml_out;
         p.seq_lens = cv.seq_lens; p.page_table = cv.page_table; p.status = ctx->status_dev;
         p.batch = cv.batch; p.H_q = d.n_q_heads; p.n_kv = d.n_kv_heads; p.r_v = L.r_v; p.tiles = tiles;
         p.n_blk = n_blk; p.n_csplit = n_csplit; p.max_pos = d.max_pos; p.max_rows = lorc_tc_max_rows(cv);
         p.pos0 = pos0; p.q_pos = q_pos;
         p.page_size = cv.page_size; p.max_pages_per_seq = cv.max_pages_per_seq; p.n_pages = cv.n_pages;
         dim3 grid(n_blk, n_csplit, cv.batch);
-        auto launch = [&](auto kernel, size_t bytes) {
-            return lorc_launch_dependent(kernel, grid, dim3(P_THREADS), bytes + 1024, st, mapCV, p);
-        };
-        if (d.n_q_heads == 32)
-            e = split ? launch(lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>))
-                      : launch(lorc_pv2_kernel<32, false>, sizeof(Pv2Smem<32, false>));
-        else
-            e = split ? launch(lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>))
-                      : launch(lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>));
+        e = with_pv_kernel(ctx, [&](auto kernel, size_t smem) {
+            return lorc_launch_dependent_cluster(kernel, grid, dim3(P_THREADS), smem, n_csplit, st, mapCV, p);
+        });
         *launches += 1;
         if (e != cudaSuccess) return e;
     }

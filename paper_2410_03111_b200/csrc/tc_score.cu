@@ -64,9 +64,8 @@ struct ScoreParams {
     const int32_t* page_table;     // NULL: contiguous
     const float2* rope_table;      // [max_pos][64]
     const float4* rope_tile;       // [33][32]   in-tile rotation table in its shared-memory layout
-    int* zero;                     // words the first block clears for the kernels that follow
     int* status;
-    int batch, seq0, H_q, n_hp, r_k, tiles, n_zero, max_pos;
+    int batch, seq0, H_q, n_hp, r_k, tiles, max_pos;
     int max_rows;                  // SPLIT: rows of a sequence that exist
     int page_size, max_pages_per_seq, n_pages;
 };
@@ -165,8 +164,6 @@ lorc_score_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_consta
     // Everything above may overlap the tail of the previous kernel in the stream; inputs are read, results written
     // and tensor memory claimed only once that kernel has completed.
     grid_dep_wait();
-    if (blockIdx.x == 0)
-        for (int i = tid; i < p.n_zero; i += Q_THREADS) p.zero[i] = 0;
     for (int i = tid; i < p.batch; i += Q_THREADS) {
         int len = p.seq_lens[i];
         if (len > p.max_pos || (!SPLIT && len > p.tiles * TILE)) {   // beyond what the tables or the scratch were sized for
@@ -635,11 +632,11 @@ cudaError_t lorc_tc_rope_tile_fill(float2* table, double theta, cudaStream_t st)
 }
 
 // One launch per block of LORC_SCORE_MAX_BATCH sequences (the kernel keeps the block's lengths and tile offsets in
-// shared memory).  The first launch clears `zero[0 .. n_zero)` for the kernels that follow it in the stream.
+// shared memory).
 cudaError_t lorc_tc_score_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCK,
                                  const CUtensorMap& mapBKT, const bf16* q, uint8_t* pimg, unsigned* rowmax,
-                                 const float4* rope_tile, int tiles, int* zero, int n_zero, const int32_t* pos0,
-                                 const int32_t* q_pos, cudaStream_t st, int* launches) {
+                                 const float4* rope_tile, int tiles, const int32_t* pos0, const int32_t* q_pos, cudaStream_t st,
+                                 int* launches) {
     const lorc_model_desc& d = ctx->desc;
     const size_t img_bytes = (size_t)lorc_tc_image_bytes(d.n_q_heads, lorc_tc_split(ctx));
     for (int s0 = 0; s0 < cv.batch; s0 += LORC_SCORE_MAX_BATCH) {
@@ -654,8 +651,6 @@ cudaError_t lorc_tc_score_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheV
         sp.page_table = cv.page_table;
         sp.rope_table = ctx->rope_table;
         sp.rope_tile = rope_tile;
-        sp.zero = zero;
-        sp.n_zero = s0 == 0 ? n_zero : 0;
         sp.status = ctx->status_dev;
         sp.batch = nb; sp.seq0 = s0; sp.H_q = d.n_q_heads; sp.n_hp = d.n_kv_heads / 2; sp.r_k = L.r_k;
         sp.tiles = tiles; sp.max_pos = d.max_pos; sp.max_rows = lorc_tc_max_rows(cv);
