@@ -133,11 +133,12 @@ int lorc_full_decode_splits(const lorc_ctx* ctx, int batch, int max_seq_len);
 cudaError_t lorc_full_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* q, int n_splits,
                              bool by_length, float* part_ml, float* part_o, cudaStream_t st, int* launches);
 // Compressed layers, one query per sequence, bf16 path: the plain computation with mma.sync reconstruction (small_decode.cu).
-// Leaves the same per-split partial results too.
+// Leaves the same per-split partial results too, unless it merges them itself (up to eight splits of low ranks): then `out` is
+// complete and *merged set.
 bool lorc_small_decode_supported(const lorc_ctx* ctx, const LorcLayer& L);
 cudaError_t lorc_small_decode(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* q, int n_splits,
-                              float* part_ml, float* part_o, cudaStream_t st, int* launches, const int32_t* pos0,
-                              const int32_t* q_pos);
+                              float* part_ml, float* part_o, bf16* out, bool may_merge, bool* merged, cudaStream_t st,
+                              int* launches, const int32_t* pos0, const int32_t* q_pos);
 // latent_out: stop before the value up-projection and write the normalised latent output [b, H_q, r_v] to `out`.
 // T > 1: T queries per sequence (q, out [b, T, H_q, d_head]; partial results for b * T units), query t of a sequence
 // at position seq_lens[s] - T + t, attending to the tokens up to its own.

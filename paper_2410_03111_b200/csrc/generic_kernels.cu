@@ -509,11 +509,14 @@ cudaError_t lorc_generic_decode(lorc_ctx* ctx, const LorcLayer& L, const CacheVi
         return lorc_generic_combine(ctx, L, cv.batch, n_splits, part_ml, part_o, out, st, launches, false, nullptr, by_length);
     }
     if (T == 1 && lorc_small_decode_supported(ctx, L)) {
+        bool merged = false;
         {
             LorcStageTimer timer(ctx, LORC_STAGE_SCORE, st);
-            cudaError_t e = lorc_small_decode(ctx, L, cv, q, n_splits, part_ml, part_o, st, launches, pos0, q_pos);
+            cudaError_t e = lorc_small_decode(ctx, L, cv, q, n_splits, part_ml, part_o, out, !latent_out && !ml_out, &merged, st,
+                                              launches, pos0, q_pos);
             if (e != cudaSuccess) return e;
         }
+        if (merged) return cudaSuccess;
         return lorc_generic_combine(ctx, L, cv.batch, n_splits, part_ml, part_o, out, st, launches, latent_out, ml_out);
     }
     {

@@ -393,10 +393,10 @@ static inline bool lorc_make_tmap_bf16(CUtensorMap* map, const void* base, int r
     return r == CUDA_SUCCESS;
 }
 
-// Launch with the programmatic-serialization attribute (see grid_dep_wait above); clusters of cluster_y blocks along y where
-// that is more than one.
+// Launch with the programmatic-serialization attribute (see grid_dep_wait above); in clusters where
+// `cluster` is more than one block.
 template <typename... KArgs>
-static inline cudaError_t lorc_launch_dependent_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int cluster_y,
+static inline cudaError_t lorc_launch_dependent_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, dim3 cluster,
                                                         cudaStream_t stream, KArgs... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -407,15 +407,15 @@ static inline cudaError_t lorc_launch_dependent_cluster(void (*kernel)(KArgs...)
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 1;
-    attr[1].val.clusterDim.y = (unsigned)cluster_y;
-    attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.x = cluster.x;
+    attr[1].val.clusterDim.y = cluster.y;
+    attr[1].val.clusterDim.z = cluster.z;
     cfg.attrs = attr;
-    cfg.numAttrs = cluster_y > 1 ? 2 : 1;
+    cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 template <typename... KArgs>
 static inline cudaError_t lorc_launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                                 cudaStream_t stream, KArgs... args) {
-    return lorc_launch_dependent_cluster(kernel, grid, block, smem, 1, stream, args...);
+    return lorc_launch_dependent_cluster(kernel, grid, block, smem, dim3(1), stream, args...);
 }

@@ -9,11 +9,16 @@
 //   rotation and q.k in registers (the accumulator columns of a rotary pair belong to one thread), softmax over the 64
 //   tokens, then O_lat += P . C_V with fp32 FMAs, thread = (8 latent columns, group of tokens).
 // Such calls are small: the kernel is bound by its chain of dependent loads, so shares are short (64 tokens when that
-// fills the chip).  At 129 tokens, rank 32, 4 heads of 64 it takes 11 us where the scalar kernel took 99 us; the step with
-// cache write and merge takes 19 us instead of 72.
+// fills the chip).  Where a call has at most eight shares and the rank is low they form a cluster that merges them through
+// distributed shared memory and up-projects the result: one launch less.  At 129 tokens, rank 32, 4 heads of 64 the kernel takes
+// 11 us where the scalar kernel took 99 us; the step with cache write and merge took 72 us with that one, then 19; one step among
+// many, launched from Python: 11.8 us with the merge kernel, 9.5 with the merge inside.
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
+#include "sm100_pair.cuh"
 #include "sm100_ptx.cuh"
 #include "tc_kernels.cuh"
 
@@ -23,6 +28,9 @@ namespace {
 
 constexpr int SD_THREADS = 128;
 constexpr int SD_TILE = LORC_SMALL_TILE;             // tokens per step: 16 per warp
+// Merge inside: as many shares as every GPU takes in a cluster, and r_v * d_h at most this, so that a thread holds its 64 or
+// fewer elements of B_V in registers before the shares meet.  (Larger ranks: a block per head of the merge kernel is faster.)
+constexpr int SD_MERGE_SHARES = 8, SD_MERGE_WORK = 64 * SD_THREADS;
 
 struct SdParams {
     const bf16* q;
@@ -33,12 +41,15 @@ struct SdParams {
     const int32_t* q_pos;
     float* part_ml;
     float* part_o;
+    bf16* out;                     // MERGE: [b, H_q, DH]
+    const bf16* B_v;               // MERGE: [r_v, n]
     int* status;
-    int r_k, r_v, G, n_splits, rope_style, max_pos;
+    int r_k, r_v, G, n_splits, rope_style, max_pos, n;
 };
 
 // GM: query heads per KV head rounded up to 2, 4 or 8 (rows past p.G hold zero queries and are not written)
-template <int DH, int GM>
+// MERGE: the shares of a (sequence, KV head) form a cluster
+template <int DH, int GM, bool MERGE>
 __global__ void __launch_bounds__(SD_THREADS)
 small_decode_kernel(const SdParams p) {
     constexpr int HALF = DH / 2, NT = DH / 8;
@@ -235,16 +246,97 @@ small_decode_kernel(const SdParams p) {
             for (int e = 0; e < 8; ++e) red[(h * ntg + tg) * p.r_v + cg * 8 + e] = acc[h][e];
     }
     __syncthreads();
+    __shared__ float part[MERGE ? GM * (SD_MERGE_WORK / DH) : 1];        // MERGE: [G][r_v]
     for (int i = tid; i < p.G * p.r_v; i += SD_THREADS) {
         const int h = i / p.r_v, col = i - h * p.r_v;
         float a = 0.f;
         for (int x = 0; x < ntg; ++x) a += red[(h * ntg + x) * p.r_v + col];
-        p.part_o[(((long long)s * H_q + g * p.G + h) * p.n_splits + split) * p.r_v + col] = a;
+        if (MERGE)
+            part[i] = a;
+        else
+            p.part_o[(((long long)s * H_q + g * p.G + h) * p.n_splits + split) * p.r_v + col] = a;
     }
-    if (tid < p.G) {
-        const long long unit = ((long long)s * H_q + g * p.G + tid) * p.n_splits + split;
-        p.part_ml[unit * 2] = m_s[it & 1][tid];
-        p.part_ml[unit * 2 + 1] = l_s[tid];
+    if constexpr (!MERGE) {
+        if (tid < p.G) {
+            const long long unit = ((long long)s * H_q + g * p.G + tid) * p.n_splits + split;
+            p.part_ml[unit * 2] = m_s[it & 1][tid];
+            p.part_ml[unit * 2 + 1] = l_s[tid];
+        }
+    } else {
+        // The arithmetic and the order of the sums are those of the merge kernel.  A share's CTA takes every n_splits-th head;
+        // thread = (output column j, slices sl and sl + SL of the rank), its elements of B_V on their way while the shares meet.
+        constexpr int SL = SD_THREADS / DH, SLICES = 256 / DH, NW = 64 / 2;
+        __shared__ float ml[GM][2];
+        __shared__ float o_lat[SD_MERGE_WORK / DH], sums[SLICES][DH];
+        if (tid < GM) {
+            ml[tid][0] = m_s[it & 1][tid];
+            ml[tid][1] = l_s[tid];
+        }
+        const int j = tid % DH, sl = tid / DH;
+        bf16 w[2][NW];
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                const int k = i * SLICES + sl + x * SL;
+                w[x][i] = k < p.r_v ? p.B_v[(long long)k * p.n + g * DH + j] : __float2bfloat16_rn(0.f);
+            }
+        __syncwarp();
+        cluster_arrive_release();
+        cluster_wait_acquire();
+        const uint32_t part0 = smem_u32(part), ml0 = smem_u32(&ml[0][0]);
+        for (int h = split; h < p.G; h += p.n_splits) {
+            float m[SD_MERGE_SHARES], l[SD_MERGE_SHARES], M = -INFINITY;
+#pragma unroll
+            for (int c = 0; c < SD_MERGE_SHARES; ++c) {
+                m[c] = -INFINITY;
+                l[c] = 0.f;
+                if (c < p.n_splits) {
+                    m[c] = ld_cluster_f1(mapa_shared(ml0 + h * 8, c));
+                    l[c] = ld_cluster_f1(mapa_shared(ml0 + h * 8 + 4, c));
+                }
+                if (l[c] > 0.f) M = fmaxf(M, m[c]);
+            }
+            double L = 0.0;
+#pragma unroll
+            for (int c = 0; c < SD_MERGE_SHARES; ++c) {
+                m[c] = l[c] > 0.f ? expf(m[c] - M) : 0.f;                // the share's weight
+                L += (double)m[c] * (double)l[c];
+            }
+            const float Lf = (float)L, inv = Lf > 0.f ? 1.f / Lf : 0.f;
+            if (tid == 0 && !(L > 0.0)) lorc_set_status(p.status, LORC_ERR_EMPTY);
+            for (int col = tid; col < p.r_v; col += SD_THREADS) {
+                float x[SD_MERGE_SHARES], a = 0.f;
+#pragma unroll
+                for (int c = 0; c < SD_MERGE_SHARES; ++c)
+                    x[c] = c < p.n_splits ? ld_cluster_f1(mapa_shared(part0 + (h * p.r_v + col) * 4, c)) : 0.f;
+#pragma unroll
+                for (int c = 0; c < SD_MERGE_SHARES; ++c)
+                    if (m[c] != 0.f) a = fmaf(m[c], x[c], a);
+                o_lat[col] = a * inv;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                float a = 0.f;
+#pragma unroll
+                for (int i = 0; i < NW; ++i) {
+                    const int k = i * SLICES + sl + x * SL;
+                    if (k < p.r_v) a = fmaf(o_lat[k], __bfloat162float(w[x][i]), a);
+                }
+                sums[sl + x * SL][j] = a;
+            }
+            __syncthreads();
+            if (tid < DH) {
+                float a = sums[0][tid];
+#pragma unroll
+                for (int x = 1; x < SLICES; ++x) a += sums[x][tid];
+                p.out[((long long)s * H_q + g * p.G + h) * DH + tid] = __float2bfloat16_rn(a);
+            }
+        }
+        __syncwarp();
+        cluster_arrive_release();                        // no CTA leaves while another may still read its part
+        cluster_wait_acquire();
     }
 }
 
@@ -256,18 +348,24 @@ bool lorc_small_decode_supported(const lorc_ctx* ctx, const LorcLayer& L) {
 }
 
 cudaError_t lorc_small_decode(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const bf16* q, int n_splits,
-                              float* part_ml, float* part_o, cudaStream_t st, int* launches, const int32_t* pos0,
-                              const int32_t* q_pos) {
+                              float* part_ml, float* part_o, bf16* out, bool may_merge, bool* merged, cudaStream_t st,
+                              int* launches, const int32_t* pos0, const int32_t* q_pos) {
     const lorc_model_desc& d = ctx->desc;
     SdParams p;
     p.q = q; p.cv = cv; p.B_kT = L.B_kT; p.rope_table = ctx->rope_table; p.pos0 = pos0; p.q_pos = q_pos;
     p.part_ml = part_ml; p.part_o = part_o; p.status = ctx->status_dev;
     p.r_k = L.r_k; p.r_v = L.r_v; p.G = ctx->group; p.n_splits = n_splits; p.rope_style = ctx->pair_style;
-    p.max_pos = d.max_pos;
+    p.max_pos = d.max_pos; p.out = out; p.B_v = L.B_v; p.n = ctx->n;
     const bool wide = d.d_head == 128;
-    auto kernel = ctx->group <= 2 ? (wide ? small_decode_kernel<128, 2> : small_decode_kernel<64, 2>)
-                  : ctx->group <= 4 ? (wide ? small_decode_kernel<128, 4> : small_decode_kernel<64, 4>)
-                                    : (wide ? small_decode_kernel<128, 8> : small_decode_kernel<64, 8>);
+    *merged = may_merge && n_splits <= SD_MERGE_SHARES && L.r_v * d.d_head <= SD_MERGE_WORK;
+    auto pick = [&](auto merge) {
+        constexpr bool M = decltype(merge)::value;
+        return ctx->group <= 2 ? (wide ? small_decode_kernel<128, 2, M> : small_decode_kernel<64, 2, M>)
+               : ctx->group <= 4 ? (wide ? small_decode_kernel<128, 4, M> : small_decode_kernel<64, 4, M>)
+                                 : (wide ? small_decode_kernel<128, 8, M> : small_decode_kernel<64, 8, M>);
+    };
     *launches += 1;
-    return lorc_launch_dependent(kernel, dim3(n_splits, d.n_kv_heads, cv.batch), dim3(SD_THREADS), 0, st, p);
+    const dim3 grid(n_splits, d.n_kv_heads, cv.batch), block(SD_THREADS);
+    return *merged ? lorc_launch_dependent_cluster(pick(std::true_type()), grid, block, 0, dim3(n_splits), st, p)
+                   : lorc_launch_dependent(pick(std::false_type()), grid, block, 0, st, p);
 }

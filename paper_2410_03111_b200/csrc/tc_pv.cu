@@ -773,7 +773,7 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
         p.page_size = cv.page_size; p.max_pages_per_seq = cv.max_pages_per_seq; p.n_pages = cv.n_pages;
         dim3 grid(n_blk, n_csplit, cv.batch);
         e = with_pv_kernel(ctx, [&](auto kernel, size_t smem) {
-            return lorc_launch_dependent_cluster(kernel, grid, dim3(P_THREADS), smem, n_csplit, st, mapCV, p);
+            return lorc_launch_dependent_cluster(kernel, grid, dim3(P_THREADS), smem, dim3(1, n_csplit, 1), st, mapCV, p);
         });
         *launches += 1;
         if (e != cudaSuccess) return e;
