@@ -27,7 +27,8 @@ namespace {
 constexpr int TILE = 128;
 constexpr int KC = 64;
 constexpr float LOG2E = 1.4426950408889634f;
-constexpr int A_THREADS = 192;       // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
+constexpr int A_EPI_WARPS = 8;
+constexpr int A_THREADS = 64 + 32 * A_EPI_WARPS;      // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
 constexpr int A_ROWS = 64;           // rows of the query operand (heads; rows beyond H_q are padding)
 
 // q~ in memory, r_ld = r_k rounded up to 64:
@@ -118,14 +119,15 @@ absorb_query_kernel(const bf16* __restrict__ q, const bf16* __restrict__ B_kT, b
 
 // 64 heads: a stage holds the latent slice and two query operands (high parts, remainders), two MMAs per k-step add
 // them in the accumulator.  32 heads: one query operand carries both (rows 0..31 high parts, rows 32..63 remainders),
-// one MMA per k-step, and the warps that hold the remainder rows hand their values to the warps of the high-part rows.
+// one MMA per k-step, and the warps that hold high parts and remainders of the same heads swap halves of them, so that each ends
+// with the scores of 32 tokens.
 template <int HQ>
 struct AbsSmem {
     static constexpr int NQ = HQ == 64 ? 2 : 1;          // query operands per stage
     static constexpr int STAGES = HQ == 64 ? 6 : 8;
     bf16 C[STAGES][TILE * KC];            // latent slice [128 tokens][64]                16 KiB
     bf16 Q[STAGES][NQ][A_ROWS * KC];      // q~ operand(s) [64 rows][64]                   8 KiB each
-    float4 xch[2][16][32];                // remainder-row scores on their way to the high-part rows (32 heads)
+    float4 xch[2][2][2][2][4][32];        // 32 heads: scores swapped, [tile parity][half of the tile][heads 16..31][remainders][8-token group]
     uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2];
     uint32_t tmem_base;
     int32_t tile_start[LORC_SCORE_MAX_BATCH + 1];
@@ -160,7 +162,6 @@ lorc_score_absorbed_kernel(const __grid_constant__ CUtensorMap mapCK, const __gr
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int nkc = (p.r_k + KC - 1) / KC;
     const int img_bytes = lorc_tc_image_bytes(HQ, false);
-    constexpr int EPI_WARPS = 4;                         // every lane quarter of the accumulator holds rows in use
 
     if (tid == 0) {
         for (int i = 0; i < A_STAGES; ++i) {
@@ -169,7 +170,7 @@ lorc_score_absorbed_kernel(const __grid_constant__ CUtensorMap mapCK, const __gr
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sm.acc_full[i], 1);
-            mbar_init(&sm.acc_empty[i], EPI_WARPS);
+            mbar_init(&sm.acc_empty[i], A_EPI_WARPS);
         }
         fence_barrier_init();
         prefetch_tensormap(&mapCK);
@@ -278,99 +279,114 @@ lorc_score_absorbed_kernel(const __grid_constant__ CUtensorMap mapCK, const __gr
         if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
     } else {
         // ------------------------------------------------------------------ epilogue: softmax numerators
-        // A 64-row accumulator keeps head 16 q + i (i < 16) in lane i of lane quarter q.  With 16-lane x 256-bit loads
-        // lane (r = lane / 4, c = lane % 4) holds, per 8-token group k, the heads 16 q + r and 16 q + r + 8 and the tokens
-        // 8 k + 2 c, 8 k + 2 c + 1: all 32 lanes work, and the four lanes of equal r share a head.
-        const int quarter = warp % 4;
-        {
-            const int r = lane >> 2, c = lane & 3;
-            uint32_t uc = 0;
-            int s = 0;
-            for (int f = blockIdx.x; f < n_flat && ok; f += gridDim.x, ++uc) {
-                int tile;
-                locate_tile(sm, f, p.batch, s, tile);
-                const int len = sm.lens[s], buf = uc & 1;
-                if (!mbar_wait(&sm.acc_full[buf], (uc >> 1) & 1)) { ok = false; break; }
-                tc_fence_after_sync();
-                const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + buf * 128;
-                uint32_t v[16][4];                                // [8-token group][head r: tokens 2c, 2c+1 | head r+8: same]
+        // A 64-row accumulator keeps row 16 q + i (i < 16) in lane i of lane quarter q.  Two warps per quarter, one per half of
+        // the tile.  With 16-lane x 256-bit loads lane (r = lane / 4, c = lane % 4) holds, per 8-token group k, the rows
+        // 16 q + r and 16 q + r + 8 and the tokens 8 k + 2 c, 8 k + 2 c + 1: all 32 lanes work, and the four lanes of equal r
+        // share a head.  (With one warp per quarter, and 32 heads' work left to two of them, a tile took them 6 us, twice what
+        // its loads take: two layers of r 672, b 16, 4129 tokens 119.8 us, now 112.8.)
+        const int quarter = warp % 4, half = (warp - 2) >> 2;
+        const int part = HQ == 32 ? quarter >> 1 : 0;            // 32 heads: lane quarters 2 and 3 hold the remainders
+        const int h0 = (HQ == 32 ? quarter & 1 : quarter) * 16;
+        const int r = lane >> 2, c = lane & 3;
+        constexpr int NQT = HQ == 32 ? 1 : 2;                    // 32-token quarters of the tile that a warp finishes
+        uint32_t uc = 0;
+        int s = 0;
+        // (after a wait that ran out the warp stays in the loop's barriers: both warps of a swap take the same ones)
+        for (int f = blockIdx.x; f < n_flat; f += gridDim.x, ++uc) {
+            int tile;
+            locate_tile(sm, f, p.batch, s, tile);
+            const int len = sm.lens[s], buf = uc & 1;
+            if (ok && !mbar_wait(&sm.acc_full[buf], (uc >> 1) & 1)) ok = false;
+            tc_fence_after_sync();
+            const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + buf * 128 + half * 64;
+            uint32_t v[8][4];                                    // [8-token group][row r: tokens 2c, 2c+1 | row r+8: same]
 #pragma unroll
-                for (int k = 0; k < 16; ++k) tmem_ld16x256_x1(tbase + k * 8, v[k]);
-                tmem_wait_ld();
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm.acc_empty[buf]);
-                if (HQ == 32) {
-                    // lane quarters 2 and 3 hold the remainder rows of the heads of quarters 0 and 1, in the same layout
-                    if (quarter >= 2) {
+            for (int k = 0; k < 8; ++k) tmem_ld16x256_x1(tbase + k * 8, v[k]);
+            tmem_wait_ld();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.acc_empty[buf]);
+            float sc[NQT][4][4];
+            if constexpr (HQ == 32) {
+                // the warp of the high parts keeps the first 32 tokens and gives the others, the warp of the remainders the
+                // other way round (two buffers: the next swap's barrier comes before this one's is written again)
+                float4(*give)[32] = sm.xch[buf][half][quarter & 1][part];
+                const float4(*take)[32] = sm.xch[buf][half][quarter & 1][part ^ 1];
 #pragma unroll
-                        for (int k = 0; k < 16; ++k)
-                            sm.xch[quarter - 2][k][lane] = make_float4(__uint_as_float(v[k][0]), __uint_as_float(v[k][1]),
-                                                                       __uint_as_float(v[k][2]), __uint_as_float(v[k][3]));
+                for (int k = 0; k < 4; ++k) {
+                    uint32_t g[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        g[e] = part ? v[k][e] : v[4 + k][e];
+                        sc[0][k][e] = __uint_as_float(part ? v[4 + k][e] : v[k][e]);
                     }
-                    __syncwarp();   // a named barrier counts a warp once only if the warp arrives converged
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                    if (quarter < 2) {
-#pragma unroll
-                        for (int k = 0; k < 16; ++k) {
-                            const float4 x = sm.xch[quarter][k][lane];
-                            v[k][0] = __float_as_uint(__uint_as_float(v[k][0]) + x.x);
-                            v[k][1] = __float_as_uint(__uint_as_float(v[k][1]) + x.y);
-                            v[k][2] = __float_as_uint(__uint_as_float(v[k][2]) + x.z);
-                            v[k][3] = __float_as_uint(__uint_as_float(v[k][3]) + x.w);
-                        }
-                    }
-                    __syncwarp();
-                    asm volatile("bar.sync 2, 128;" ::: "memory");   // the values have been taken: the next tile may overwrite them
-                    if (quarter >= 2) continue;
+                    give[k][lane] = make_float4(__uint_as_float(g[0]), __uint_as_float(g[1]), __uint_as_float(g[2]), __uint_as_float(g[3]));
                 }
-                uint8_t* img = p.pimg + ((long long)s * p.tiles + tile) * img_bytes;
-                float* m_out = reinterpret_cast<float*>(img + 2 * HQ * KC * 2);
-                float* l_out = m_out + 4 * HQ;
+                __syncwarp();   // a named barrier counts a warp once only if the warp arrives converged
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + half * 2 + (quarter & 1)) : "memory");
 #pragma unroll
-                for (int qt = 0; qt < 4; ++qt) {                  // 32-token quarter of the tile
-                    uint8_t* chunk_img = img + (qt >> 1) * (HQ * KC * 2);
+                for (int k = 0; k < 4; ++k) {
+                    const float4 x = take[k][lane];
+                    sc[0][k][0] += x.x;
+                    sc[0][k][1] += x.y;
+                    sc[0][k][2] += x.z;
+                    sc[0][k][3] += x.w;
+                }
+            } else {
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        const int h = quarter * 16 + r + 8 * hh;
-                        float sc[4][2];
-                        float mxv = -INFINITY, ssum = 0.f;
+                for (int qq = 0; qq < NQT; ++qq)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
+                    for (int k = 0; k < 4; ++k)
 #pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                sc[k][e] = __uint_as_float(v[qt * 4 + k][2 * hh + e]);
-                                ssum += sc[k][e];
-                                if (tile * TILE + qt * 32 + 8 * k + 2 * c + e < len) mxv = fmaxf(mxv, sc[k][e]);
-                            }
-                        // a NaN among the scores means non-finite numbers in the cache, the factors or the query
-                        if (ssum != ssum) lorc_set_status(p.status, LORC_ERR_ARG);
-                        mxv = fmaxf(mxv, __shfl_xor_sync(0xffffffffu, mxv, 1));
-                        mxv = fmaxf(mxv, __shfl_xor_sync(0xffffffffu, mxv, 2));
-                        const float mref = ceilf(mxv);            // -inf: no token of the sequence in this quarter
-                        float lsum = 0.f;
+                        for (int e = 0; e < 4; ++e) sc[qq][k][e] = __uint_as_float(v[qq * 4 + k][e]);
+            }
+            if (!ok) continue;
+            uint8_t* img = p.pimg + ((long long)s * p.tiles + tile) * img_bytes;
+            float* m_out = reinterpret_cast<float*>(img + 2 * HQ * KC * 2);
+            float* l_out = m_out + 4 * HQ;
+            uint8_t* chunk_img = img + half * (HQ * KC * 2);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int t0 = qt * 32 + 8 * k + 2 * c;              // token inside the tile
-                            const bool v0 = tile * TILE + t0 < len, v1 = tile * TILE + t0 + 1 < len;
-                            const __nv_bfloat162 pr = __floats2bfloat162_rn(v0 ? exp2f(sc[k][0] - mref) : 0.f,
-                                                                            v1 ? exp2f(sc[k][1] - mref) : 0.f);
-                            lsum += __low2float(pr) + __high2float(pr);
-                            const int tc = t0 & 63;
-                            *reinterpret_cast<__nv_bfloat162*>(chunk_img + h * 128 + ((((tc >> 3) ^ (h & 7)) << 4) | ((tc & 7) << 1))) = pr;
+            for (int qq = 0; qq < NQT; ++qq) {
+                const int qt = half * 2 + (HQ == 32 ? part : qq);        // 32-token quarter of the tile
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    const int h = h0 + r + 8 * hh;
+                    float mxv = -INFINITY, ssum = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float x = sc[qq][k][2 * hh + e];
+                            ssum += x;
+                            if (tile * TILE + qt * 32 + 8 * k + 2 * c + e < len) mxv = fmaxf(mxv, x);
                         }
-                        lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
-                        lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
-                        if (c == 0) {
-                            m_out[qt * HQ + h] = mref;
-                            l_out[qt * HQ + h] = lsum;
-                            if (mxv > -INFINITY) atomicMax(p.rowmax + (long long)s * HQ + h, lorc_float_key(mref));
-                        }
+                    // a NaN among the scores means non-finite numbers in the cache, the factors or the query
+                    if (ssum != ssum) lorc_set_status(p.status, LORC_ERR_ARG);
+                    mxv = fmaxf(mxv, __shfl_xor_sync(0xffffffffu, mxv, 1));
+                    mxv = fmaxf(mxv, __shfl_xor_sync(0xffffffffu, mxv, 2));
+                    const float mref = ceilf(mxv);            // -inf: no token of the sequence in this quarter
+                    float lsum = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int t0 = qt * 32 + 8 * k + 2 * c;              // token inside the tile
+                        const bool v0 = tile * TILE + t0 < len, v1 = tile * TILE + t0 + 1 < len;
+                        const __nv_bfloat162 pr = __floats2bfloat162_rn(v0 ? exp2f(sc[qq][k][2 * hh] - mref) : 0.f,
+                                                                        v1 ? exp2f(sc[qq][k][2 * hh + 1] - mref) : 0.f);
+                        lsum += __low2float(pr) + __high2float(pr);
+                        const int tc = t0 & 63;
+                        *reinterpret_cast<__nv_bfloat162*>(chunk_img + h * 128 + ((((tc >> 3) ^ (h & 7)) << 4) | ((tc & 7) << 1))) = pr;
+                    }
+                    lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
+                    lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
+                    if (c == 0) {
+                        m_out[qt * HQ + h] = mref;
+                        l_out[qt * HQ + h] = lsum;
+                        if (mxv > -INFINITY) atomicMax(p.rowmax + (long long)s * HQ + h, lorc_float_key(mref));
                     }
                 }
             }
-            if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
         }
+        if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
     }
     tc_fence_before_sync();
     __syncthreads();
