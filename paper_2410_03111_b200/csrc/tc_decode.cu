@@ -21,8 +21,8 @@ constexpr int KC = 64;               // latent columns per TMA box
 // ------------------------------------------------------------------------------------------------
 struct LorcTcLayer {
     bool has_bkt = false;
-    CUtensorMap mapBKT, mapBVT;         // B_K^T in 64 x 128 swizzled boxes; B_V^T in 64 x 32 swizzled boxes
-    CUtensorMap mapBVT128;              // B_V^T in 64 x 128 boxes (reconstruction of values for prompt processing)
+    CUtensorMap mapBVT;                 // B_V^T in 64 x 32 swizzled boxes
+    CUtensorMap mapBKT[2], mapBVTr[2];  // B_K^T, and B_V^T for the reconstruction of values, in 64 x 128 boxes [0] and 64 x 64 [1]
     // cache maps are rebuilt only when the cache geometry or pointers change
     const void* k_ptr = nullptr;
     const void* v_ptr = nullptr;
@@ -164,13 +164,14 @@ static cudaError_t tc_prepare(lorc_ctx* ctx, LorcTcState* T, LorcTcLayer& TL, co
     }
     if (!TL.has_bkt) {
         uint64_t dims[2] = {(uint64_t)L.r_k, (uint64_t)ctx->n}, str[1] = {(uint64_t)L.r_k * 2};
-        uint32_t box[2] = {KC, 128};
-        if (!lorc_make_tmap_bf16(&TL.mapBKT, L.B_kT, 2, dims, str, box)) return cudaErrorInvalidValue;
         uint64_t d2[2] = {(uint64_t)L.r_v, (uint64_t)ctx->n}, s2[1] = {(uint64_t)L.r_v * 2};
         uint32_t b2[2] = {KC, 32};          // the up-projection takes a quarter of a head's columns per CTA
         if (!lorc_make_tmap_bf16(&TL.mapBVT, L.B_vT, 2, d2, s2, b2)) return cudaErrorInvalidValue;
-        uint32_t b3[2] = {KC, 128};
-        if (!lorc_make_tmap_bf16(&TL.mapBVT128, L.B_vT, 2, d2, s2, b3)) return cudaErrorInvalidValue;
+        for (int i = 0; i < 2; ++i) {
+            uint32_t box[2] = {KC, i ? 64u : 128u};
+            if (!lorc_make_tmap_bf16(&TL.mapBKT[i], L.B_kT, 2, dims, str, box)) return cudaErrorInvalidValue;
+            if (!lorc_make_tmap_bf16(&TL.mapBVTr[i], L.B_vT, 2, d2, s2, box)) return cudaErrorInvalidValue;
+        }
         TL.has_bkt = true;
     }
     if (!build_cache_maps(TL, L, cv, cv.page_table ? cv.page_size : TILE)) return cudaErrorInvalidValue;
@@ -223,7 +224,7 @@ cudaError_t lorc_tc_decode(lorc_ctx* ctx, int layer, const LorcLayer& L, const C
             // no rotation between the key up-projection and the dot product: the up-projection moves to the query
             e = lorc_tc_score_absorbed_launch(ctx, L, cv, TL.mapCK, q, qabs, pimg, T->rowmax, tiles, st, launches);
         else
-            e = lorc_tc_score_launch(ctx, L, cv, TL.mapCK, TL.mapBKT, q, pimg, T->rowmax,
+            e = lorc_tc_score_launch(ctx, L, cv, TL.mapCK, TL.mapBKT[0], q, pimg, T->rowmax,
                                      reinterpret_cast<const float4*>(T->rope_tile), tiles, pos0, q_pos, st, launches);
         if (e != cudaSuccess) return e;
     }
@@ -245,5 +246,5 @@ cudaError_t lorc_tc_prefill(lorc_ctx* ctx, int layer, const LorcLayer& L, const 
     cudaError_t e = tc_prepare(ctx, T, TL, L, cv, st);
     if (e != cudaSuccess) return e;
     if (lorc_tc_prefill_scratch_bytes(ctx, cv.batch, cv.max_seq_len, T_new) > ws_bytes) return cudaErrorMemoryAllocation;
-    return lorc_tc_prefill_launch(ctx, L, cv, TL.mapCK, TL.mapCV, TL.mapBKT, TL.mapBVT128, q, out, T_new, ws, st, launches);
+    return lorc_tc_prefill_launch(ctx, L, cv, TL.mapCK, TL.mapCV, TL.mapBKT, TL.mapBVTr, q, out, T_new, ws, st, launches);
 }

@@ -48,9 +48,12 @@ constexpr float LOG2E = 1.4426950408889634f;
 // conflict-free word, and the finished 128 x 64 boxes leave by TMA.  (With four warps, thread = token row, the row-wise
 // 16-byte stores and table reads touched 32 lines per access and the epilogue took three times as long as the MMAs:
 // 284 us for the keys and values of 16 x 4096 tokens at rank 672, 162 us now.)
+// Where units of two heads would leave half of the pairs idle a unit is one head (N = 128): two thirds of the operand bytes and
+// half of the epilogue in the chain of a launch that is one unit long.  (One prompt of 777 tokens, r 928 and 416, cache write and
+// attention of two layers: 104.1 -> 99.0 us.)
 constexpr int R_STAGES = 5;
 constexpr int R_THREADS = 384;       // warp 0 TMA, warp 1 MMA (leader CTA issues), warps 4..11 epilogue
-constexpr int R_N = 256;             // features per unit: two KV heads
+constexpr int R_N = 256;             // features per unit of two KV heads
 
 struct RecSmem {
     bf16 A[R_STAGES][TILE * KC];          // latent slice of this CTA's tile [128 tokens][64]
@@ -65,7 +68,8 @@ struct RecParams {
     const int32_t* page_table;
     const float2* rope_table;      // [max_pos][64]
     int* status;
-    int r_k, r_v, n_rows, max_pos, batch, tile_pairs, n_hp;
+    int r_k, r_v, n_rows, max_pos, batch, tile_pairs;
+    int n_cols, cols;              // units per pair of tiles and their features: R_N, or 128 (factor boxes of cols / 2 rows)
     int page_size, max_pages_per_seq, n_pages;
 };
 
@@ -78,14 +82,14 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int rank = (int)cluster_ctarank();           // 0 = leader (issues the MMAs, owns the full / acc_empty barriers)
     const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-    const int per_kind = p.batch * p.tile_pairs * p.n_hp, total = 2 * per_kind;
+    const int per_kind = p.batch * p.tile_pairs * p.n_cols, total = 2 * per_kind;
     // unit -> (values?, sequence, tile pair, head pair); a unit whose first tile lies past the sequence's cached tokens is
     // skipped by both CTAs and every role alike (sequences beyond the buffer are reported by the attention kernel)
     auto decode = [&](int u, bool& val, int& s, int& tp, int& hp, int& len) -> bool {
         val = u >= per_kind;
         if (val) u -= per_kind;
-        hp = u % p.n_hp;
-        const int st = u / p.n_hp;
+        hp = u % p.n_cols;
+        const int st = u / p.n_cols;
         tp = st % p.tile_pairs;
         s = st / p.tile_pairs;
         len = p.seq_lens[s];
@@ -148,7 +152,7 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_
                 const uint32_t lead_bar = lead_full0 + st * 8;
                 const uint32_t a_dst = a_base + st * (TILE * KC * 2);
                 if (elect_one()) {
-                    if (rank == 0) mbar_arrive_expect_tx_addr(full0 + st * 8, 2 * 2 * TILE * KC * 2);
+                    if (rank == 0) mbar_arrive_expect_tx_addr(full0 + st * 8, (2 * TILE + p.cols) * KC * 2);
                     if (p.page_table == nullptr) {
                         // (a tile past the buffer's rows reads as zero)
                         tma_load_3d_pair_addr(a_dst, mapC, lead_bar, kc * KC, tile * TILE, s);
@@ -159,7 +163,7 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_
                             if (pg < ppt)
                                 tma_load_3d_pair_addr(a_dst + pg * p.page_size * KC * 2, mapC, lead_bar, kc * KC, 0, pages[pg]);
                     }
-                    tma_load_2d_pair_addr(b_base + st * (TILE * KC * 2), mapBT, lead_bar, kc * KC, hp * R_N + rank * 128);
+                    tma_load_2d_pair_addr(b_base + st * (TILE * KC * 2), mapBT, lead_bar, kc * KC, hp * p.cols + rank * (p.cols / 2));
                 }
                 __syncwarp();
                 if (++st == R_STAGES) { st = 0; par ^= 1; }
@@ -169,7 +173,7 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
         if (rank == 0) {
-            const uint32_t idesc = make_idesc_bf16(256, R_N, 0, 0);
+            const uint32_t idesc = make_idesc_bf16(256, p.cols, 0, 0);
             const uint64_t da0 = make_smem_desc_sw128(smem_u32(sm.A[0]), 0, 1024);
             const uint64_t db0 = make_smem_desc_sw128(smem_u32(sm.B[0]), 0, 1024);
             const uint32_t a_lo0 = (uint32_t)da0, a_hi = (uint32_t)(da0 >> 32);
@@ -213,17 +217,23 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_
         }
     } else if (warp >= 4) {
         // ------------------------------------------------------------------ epilogue (both CTAs): this CTA's 128 tokens
-        const int hd = (warp - 4) >> 2, quarter = warp % 4;          // head of the pair, TMEM lane quarter
+        // (units of one head: the eight warps share it, steps 0..3 and 4..7)
+        const bool one = p.cols == 128;
+        const int grp = (warp - 4) >> 2, hd = one ? 0 : grp, quarter = warp % 4;     // head of the unit, TMEM lane quarter
+        const int kk0 = one ? 4 * grp : 0, n_kk = one ? 4 : 8;
         const int r = lane >> 2, c = lane & 3;                       // tokens 32 quarter + r + 8 m, rotary pairs 8 kk + 2 c, + 1
-        const bool issuer = tid == 128 + hd * 128;                   // the thread that stores this head's boxes
+        const bool issuer = tid == 128 + grp * 128 && !(one && grp);                   // the thread that stores this head's boxes
         const uint32_t lead_acc_empty[2] = {mapa_shared(smem_u32(&sm.acc_empty[0]), 0),
                                             mapa_shared(smem_u32(&sm.acc_empty[1]), 0)};
         // the lane's word of row 32 quarter + r (+ 8 m: 1 KiB further on), 16-byte piece kk, in both boxes
         uint8_t* o0 = sm.O[hd][0] + (quarter * 32 + r) * 128 + c * 4;
         uint8_t* o1 = sm.O[hd][1] + (quarter * 32 + r) * 128 + c * 4;
-        auto head_sync = [&]() {                                     // the four warps of a head
+        auto head_sync = [&]() {                                     // the warps of a head
             __syncwarp();
-            asm volatile("bar.sync %0, 128;" ::"r"(1 + hd) : "memory");
+            if (one)
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+            else
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
         };
         uint32_t uc = 0;
         for (int u = pair_id; u < total; u += n_pairs) {
@@ -271,10 +281,10 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_
             };
             if (val) {
 #pragma unroll 4
-                for (int kk = 0; kk < 8; ++kk) step(kk, false);
+                for (int kk = kk0; kk < kk0 + n_kk; ++kk) step(kk, false);
             } else {
 #pragma unroll 4
-                for (int kk = 0; kk < 8; ++kk) step(kk, true);
+                for (int kk = kk0; kk < kk0 + n_kk; ++kk) step(kk, true);
             }
             // this warp has read its part of the accumulator
             tc_fence_before_sync();
@@ -284,8 +294,8 @@ lorc_reconstruct_kernel(const __grid_constant__ CUtensorMap mapCK, const __grid_
             head_sync();
             if (issuer && ok && tile * TILE < p.n_rows) {
                 const CUtensorMap* mapO = val ? &mapVO : &mapKO;
-                tma_store_3d(mapO, sm.O[hd][0], (hp * 2 + hd) * 128, tile * TILE, s);
-                tma_store_3d(mapO, sm.O[hd][1], (hp * 2 + hd) * 128 + 64, tile * TILE, s);
+                tma_store_3d(mapO, sm.O[hd][0], hp * p.cols + hd * 128, tile * TILE, s);
+                tma_store_3d(mapO, sm.O[hd][1], hp * p.cols + hd * 128 + 64, tile * TILE, s);
                 bulk_commit();
             }
             ++uc;
@@ -682,7 +692,7 @@ cudaError_t lorc_tc_prefill_set_attrs() {
 }
 
 cudaError_t lorc_tc_prefill_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCK,
-                                   const CUtensorMap& mapCV, const CUtensorMap& mapBKT, const CUtensorMap& mapBVT128,
+                                   const CUtensorMap& mapCV, const CUtensorMap* mapBKT, const CUtensorMap* mapBVT,
                                    const bf16* q, bf16* out, int T, void* scratch, cudaStream_t st, int* launches) {
     const lorc_model_desc& d = ctx->desc;
     const size_t rows = prefill_rows(cv.max_seq_len);
@@ -710,11 +720,15 @@ cudaError_t lorc_tc_prefill_launch(lorc_ctx* ctx, const LorcLayer& L, const Cach
     rp.seq_lens = cv.seq_lens; rp.page_table = cv.page_table; rp.rope_table = ctx->rope_table; rp.status = ctx->status_dev;
     rp.r_k = L.r_k; rp.r_v = L.r_v; rp.n_rows = (int)rows; rp.max_pos = d.max_pos;
     rp.page_size = cv.page_size; rp.max_pages_per_seq = cv.max_pages_per_seq; rp.n_pages = cv.n_pages;
-    rp.batch = cv.batch; rp.tile_pairs = (tiles + 1) / 2; rp.n_hp = d.n_kv_heads / 2;
-    const int units = 2 * cv.batch * rp.tile_pairs * rp.n_hp;
-    const int pairs = units < ctx->sm_count / 2 ? units : ctx->sm_count / 2;
+    rp.batch = cv.batch; rp.tile_pairs = (tiles + 1) / 2;
+    const long long head_units = 2ll * cv.batch * rp.tile_pairs * d.n_kv_heads;      // keys and values
+    const bool one = head_units <= ctx->sm_count / 2;                                // a unit is one head
+    rp.n_cols = one ? d.n_kv_heads : d.n_kv_heads / 2;
+    rp.cols = one ? 128 : R_N;
+    const long long units = one ? head_units : head_units / 2;
+    const int pairs = units < ctx->sm_count / 2 ? (int)units : ctx->sm_count / 2;
     e = lorc_launch_dependent(lorc_reconstruct_kernel, dim3(2 * pairs), dim3(R_THREADS), sizeof(RecSmem) + 1024, st, mapCK, mapCV,
-                              mapBKT, mapBVT128, mapK, mapV, rp);
+                              mapBKT[one], mapBVT[one], mapK, mapV, rp);
     *launches += 1;
     if (e != cudaSuccess) return e;
 
