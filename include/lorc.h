@@ -175,15 +175,20 @@ int lorc_append(lorc_ctx* ctx, int layer, const lorc_cache* cache, const void* x
  *   k_n = B_K[:, g]^T C_K[n], rotated at n;  q^ = RoPE(q, seq_lens[s]-1);
  *   p = softmax_n(q^ . k_n / sqrt(d_head)),  out = (sum_n p_n C_V[n]) B_V[:, g]
  * over n in [0, seq_lens[s]).  Keys and values are never written to memory.
- * n_splits = 0 lets the library choose how many CTAs share one sequence's context
- * (in the uncompressed mode with 128-wide heads by the lengths of all sequences);
- * a positive value asks for that many shares (context splits of the plain kernels
- * and of the uncompressed mode; context shares per latent column block of the
- * tensor-core path, at most 16), clamped to what the workspace holds.  Uses the workspace.
+ * n_splits = 0 lets the library choose how many CTAs share one sequence's context,
+ * from the sizes of the call and the GPU's number of SMs (in the uncompressed mode
+ * with 128-wide heads also by the lengths of all sequences); a positive value asks
+ * for that many shares (context splits of the plain kernels and of the uncompressed
+ * mode, clamped to what the workspace holds; context shares per latent column block
+ * of the tensor-core path, at most 64 and one per 128 tokens: those that form one
+ * cluster of up to 16 need no workspace, for others the count is clamped to what
+ * the workspace holds).  The number of shares decides the order of sums, and so
+ * the last bits of a result.  Uses the workspace.
  * A sequence with seq_lens[s] <= 0 gets a row of zeros and sets status EMPTY.
  * The first call on a context, and the first call with a larger batch than any
  * before, sets up small library-owned tables (an in-tile rotation table, one word
- * per sequence and head for the softmax row maxima) with cudaMalloc: make those
+ * per sequence and head for the softmax row maxima, 16 per sequence and KV head for
+ * the context shares) with cudaMalloc: make those
  * calls outside any stream capture.  A table handed to earlier calls is kept until
  * lorc_destroy, so CUDA graphs captured before a larger batch showed up stay valid.
  * Calls on one context must not overlap on the GPU (they share the workspace and

@@ -320,7 +320,7 @@ static int decode_attn_impl(lorc_ctx* ctx, int layer, const lorc_cache* cache, c
     int launches = 0;
     cudaError_t e;
 
-    const size_t tc = lorc_tc_workspace_bytes(ctx, cv.batch, cv.max_seq_len);
+    const size_t tc = lorc_tc_workspace_least(ctx, cv.batch, cv.max_seq_len);
     bool tensor = !(ctx->desc.flags & LORC_FLAG_DEBUG_FP32) && lorc_tc_decode_supported(ctx, *L, cv);
     // interleaved pairs: the plain kernels serve what the tensor-core path cannot take (they need less scratch and no
     // tables of their own).  With 32 heads, b 4, 2049 tokens, r 512 a step takes 34 us here and 3360 us there.

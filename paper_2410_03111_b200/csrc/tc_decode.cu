@@ -32,7 +32,7 @@ struct LorcTcLayer {
 
 struct LorcTcState {
     float2* rope_tile = nullptr;
-    unsigned* rowmax = nullptr;         // [rowmax_cap] row maxima of the softmax, see lorc_tc_decode
+    unsigned* rowmax = nullptr;         // [rowmax_cap] row maxima of the softmax, then the PV kernel's counters, see lorc_tc_decode
     std::vector<unsigned*> retired;     // smaller tables of earlier calls, freed with the context
     size_t rowmax_cap = 0;
     bool rowmax_dirty = true;
@@ -106,7 +106,12 @@ static size_t tc_absorbed_bytes(const lorc_ctx* ctx, int batch) {
 size_t lorc_tc_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_len) {
     if (!tc_shape_ok(ctx)) return 0;
     return tc_image_area_bytes(ctx, batch, max_seq_len) + tc_absorbed_bytes(ctx, batch) +
-           lorc_tc_pv_scratch_bytes(ctx, batch);
+           lorc_tc_pv_scratch_bytes(ctx, batch, max_seq_len);
+}
+
+size_t lorc_tc_workspace_least(const lorc_ctx* ctx, int batch, int max_seq_len) {
+    if (!tc_shape_ok(ctx)) return 0;
+    return tc_image_area_bytes(ctx, batch, max_seq_len) + tc_absorbed_bytes(ctx, batch) + lorc_tc_pv_scratch_least(ctx, batch);
 }
 
 static bool build_cache_maps(LorcTcLayer& T, const LorcLayer& L, const CacheView& cv, int box_rows) {
@@ -156,7 +161,7 @@ static cudaError_t tc_prepare(lorc_ctx* ctx, LorcTcState* T, LorcTcLayer& TL, co
     if (!T->attrs_set) {
         // per context, hence per device: the attribute belongs to the device's copy of the kernel
         cudaError_t e = lorc_tc_score_set_attrs();
-        if (e == cudaSuccess) e = lorc_tc_pv_set_attrs();
+        if (e == cudaSuccess) e = lorc_tc_pv_set_attrs(ctx);
         if (e == cudaSuccess) e = lorc_tc_absorbed_set_attrs();
         if (e == cudaSuccess) e = lorc_tc_prefill_set_attrs();
         if (e != cudaSuccess) return e;
@@ -199,13 +204,15 @@ cudaError_t lorc_tc_decode(lorc_ctx* ctx, int layer, const LorcLayer& L, const C
     LorcPvPlan plan;
     lorc_tc_pv_plan(ctx, L, cv, n_splits, ws_bytes - img_area - abs_area, &plan);
     if (!plan.fits) return cudaErrorMemoryAllocation;
-    // Row maxima [batch, H_q]: all zero between calls (the up-projection kernel clears what the score kernel raised).
+    // Row maxima [batch, H_q]: all zero between calls (the up-projection kernel clears what the score kernel raised), and behind
+    // them the counters of context shares in several clusters, which the PV kernel leaves at zero.
     // Owned by the library because that invariant must hold from the first call on.  The table only ever grows, and a
     // block that was handed to earlier launches is kept until the context dies (a captured graph may still name it).
     const size_t rm_need = (size_t)cv.batch * d.n_q_heads;
+    auto table_words = [&](size_t cap) { return cap + cap / d.n_q_heads * ((ctx->n + 127) / 128) * LORC_PV_MAX_CLUSTER; };
     if (rm_need > T->rowmax_cap) {
         unsigned* fresh = nullptr;
-        cudaError_t e = cudaMalloc(&fresh, rm_need * sizeof(unsigned));
+        cudaError_t e = cudaMalloc(&fresh, table_words(rm_need) * sizeof(unsigned));
         if (e != cudaSuccess) return e;
         if (T->rowmax) T->retired.push_back(T->rowmax);
         T->rowmax = fresh;
@@ -213,7 +220,7 @@ cudaError_t lorc_tc_decode(lorc_ctx* ctx, int layer, const LorcLayer& L, const C
         T->rowmax_dirty = true;
     }
     if (T->rowmax_dirty) {
-        cudaError_t e = cudaMemsetAsync(T->rowmax, 0, T->rowmax_cap * sizeof(unsigned), st);
+        cudaError_t e = cudaMemsetAsync(T->rowmax, 0, table_words(T->rowmax_cap) * sizeof(unsigned), st);
         if (e != cudaSuccess) return e;
     }
     T->rowmax_dirty = true;
@@ -229,8 +236,8 @@ cudaError_t lorc_tc_decode(lorc_ctx* ctx, int layer, const LorcLayer& L, const C
         if (e != cudaSuccess) return e;
     }
     if (d.rope_style == LORC_ROPE_NONE) pos0 = q_pos = nullptr;       // positions play no part
-    const cudaError_t e2 = lorc_tc_pv_launch(ctx, L, cv, TL.mapCV, TL.mapBVT, pimg, T->rowmax, tiles, plan, pv_scratch,
-                                             out, latent_out, pos0, q_pos, ml_out, st, launches);
+    const cudaError_t e2 = lorc_tc_pv_launch(ctx, L, cv, TL.mapCV, TL.mapBVT, pimg, T->rowmax, T->rowmax + T->rowmax_cap, tiles, plan,
+                                             pv_scratch, out, latent_out, pos0, q_pos, ml_out, st, launches);
     if (e2 == cudaSuccess) T->rowmax_dirty = false;
     return e2;
 }

@@ -9,8 +9,10 @@
 bool lorc_tc_decode_supported(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv);
 bool lorc_tc_append_supported(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int T);
 
-// Scratch bytes the tensor-core decode path needs for (batch, max_seq_len), any layer.
+// Scratch bytes the tensor-core decode path wants for (batch, max_seq_len), any layer; with less than that, down to the least it
+// works with, the context shares are limited to those of one cluster.
 size_t lorc_tc_workspace_bytes(const lorc_ctx* ctx, int batch, int max_seq_len);
+size_t lorc_tc_workspace_least(const lorc_ctx* ctx, int batch, int max_seq_len);
 
 // latent_out: `out` receives the normalised latent output [b, H_q, r_v] instead of the up-projected one.
 // pos0, q_pos / ml_out: context shards (see lorc_decode_attn_shard): per sequence the position of the first cached row
@@ -67,16 +69,20 @@ cudaError_t lorc_tc_score_absorbed_launch(lorc_ctx* ctx, const LorcLayer& L, con
 // P.C_V and value up-projection (tc_pv.cu).  mapCV: C_V cache in 64-column x 128-row (or page-sized) swizzled boxes;
 // mapBVT: B_V^T [n, r_v] in swizzled boxes of 64 latent columns x 32 rows.  The plan says how a launch splits the
 // work: column blocks and context shares of each.  The up-projection kernel writes `out` and leaves the row maxima empty again.
+// `arrived` (LORC_PV_MAX_CLUSTER words per sequence and column block) is zero before a launch and after it.
+#define LORC_PV_MAX_CLUSTER 16       // the largest cluster that a GPU may take
 struct LorcPvPlan {
-    int n_blk, n_csplit;
+    int n_blk, n_csplit, cluster, n_clusters;        // n_csplit shares of a block in n_clusters clusters of `cluster` blocks
+    size_t off_part;
     bool fits;
 };
-size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch);
-cudaError_t lorc_tc_pv_set_attrs();
-void lorc_tc_pv_plan(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
+size_t lorc_tc_pv_scratch_least(const lorc_ctx* ctx, int batch);      // without room for shares in several clusters
+size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq_len);
+cudaError_t lorc_tc_pv_set_attrs(lorc_ctx* ctx);
+void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
                      LorcPvPlan* plan);
 cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCV,
-                              const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, int tiles,
+                              const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, unsigned* arrived, int tiles,
                               const LorcPvPlan& plan, void* scratch, bf16* out, bool latent_out, const int32_t* pos0,
                               const int32_t* q_pos, float* ml_out, cudaStream_t st, int* launches);
 

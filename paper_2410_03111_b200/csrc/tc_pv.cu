@@ -9,7 +9,9 @@
 // and add up the denominator; then
 //       O_lat^T += C_V[tile, block]^T . P^T                    tcgen05, MN-major A
 // and at the end the CTA writes its 128 x H_q piece of the latent output, normalised, as bf16.  Several context shares of a
-// block form a cluster: each leaves its piece in shared memory, and each adds up and writes its part of the heads and columns.
+// block form one cluster or several: each leaves its piece in shared memory (several: in memory), and each adds up and writes its
+// part of the heads and columns.  The pieces are always added in the order of the shares, so the result depends on their number,
+// which follows from the sizes and the number of SMs, and not on the clusters, which follow from how a GPU's SMs are grouped.
 //
 // Up-projection.  One CTA per (KV head g, 64 output rows = 64 / G sequences, quarter of the head's columns)
 // multiplies those rows by B_V[:, g] (TMA-staged from a transposed copy): out = o . B_V[:, g] in TMEM, then bf16.
@@ -30,6 +32,7 @@ constexpr int KC = 64;
 template <int NR>
 struct PvStages { static constexpr int value = NR <= 32 ? 5 : NR <= 64 ? 4 : 3; };
 constexpr int P_THREADS = 192;       // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
+constexpr int PV_MAX_CLUSTER = LORC_PV_MAX_CLUSTER, PV_MAX_SHARES = 64;
 
 // ------------------------------------------------------------------------------------------------
 // PV kernel
@@ -53,6 +56,7 @@ struct Pv2Smem {
     float l_inv[HQ];
     uint64_t vfull[P_STAGES], pfull[P_STAGES], fixed[P_STAGES], empty[P_STAGES], o_full;
     uint32_t tmem_base;
+    int last;
 };
 
 struct Pv2Params {
@@ -60,20 +64,27 @@ struct Pv2Params {
     unsigned* rowmax;              // [b, H_q]   row maxima of the softmax (order-preserving keys of integers)
     bf16* o_norm;                  // [b, H_q, r_pad]      normalised latent output; SPLIT: [b, H_q, 2, r_pad], remainders second
     float* ml_out;                 // NULL, or [b, H_q, 2]: reference M (log2 units) and denominator sum_n 2^(s_n - M)
+    float* o_part;                 // several clusters: [b, n_blk, n_csplit, H_q * 128 + H_q]   every share's piece and denominators
+    unsigned* arrived;             // several clusters: [b * n_blk, PV_MAX_CLUSTER]   clusters whose pieces are there; zero between calls
     const int32_t* seq_lens;
     const int32_t* page_table;
     int* status;
     int batch, H_q, n_kv, r_v, tiles, n_blk, n_csplit, max_pos;
+    int cluster, n_clusters;       // shares per cluster, clusters per column block: at least n_csplit together
     int max_rows;                  // SPLIT: rows of a sequence that exist
     const int32_t* pos0;           // as in the score kernel
     const int32_t* q_pos;
     int page_size, max_pages_per_seq, n_pages;
 };
 
+// A share's piece in memory: [H_q][128] outputs, then [H_q] denominators.
+__host__ __device__ constexpr int share_floats(int n_q_heads) { return n_q_heads * 128 + n_q_heads; }
+
 // Biased exponent of 2^d for an integer-valued d <= 0 (0, i.e. the number zero, below 2^-126 and for d = -inf).
 __device__ __forceinline__ uint32_t pow2_exponent(float d) { return d >= -126.f ? (uint32_t)(127 + (int)d) : 0u; }
 
-template <int HQ, bool SPLIT>
+// MANY: the shares of a column block in several clusters
+template <int HQ, bool SPLIT, bool MANY>
 __global__ void __launch_bounds__(P_THREADS, 1)
 lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
     extern __shared__ uint8_t raw[];
@@ -90,7 +101,7 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
     if (SPLIT) len = min(len, p.max_rows);
     if (len > p.tiles * TILE || (len > 0 && !lorc_query_ok(p.pos0, p.q_pos, s, p.seq_lens[s], p.max_pos))) len = 0;
     if (len < 0) len = 0;
-    // this CTA's share of the context: whole 128-token tiles, dealt evenly over the context shares
+    // this CTA's share of the context: whole 128-token tiles, dealt evenly over the context shares (a CTA past them: none)
     const int tiles_s = (len + TILE - 1) / TILE;
     const int per = (tiles_s + p.n_csplit - 1) / p.n_csplit;
     const int tile_lo = min(tiles_s, cs * per), tile_hi = min(tiles_s, tile_lo + per);
@@ -118,6 +129,7 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
     const uint32_t tmem = sm.tmem_base;
     bool ok = true;
     constexpr int XLD = 132;                              // floats per row of the exchanges (16-byte rows, spread over the banks)
+    constexpr int SHARE_FLOATS = share_floats(HQ);
     const int r_pad = p.n_blk * 128;
     const int r_ld = SPLIT ? 2 * r_pad : r_pad;           // row of o_norm
 
@@ -368,7 +380,7 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                 }
             }
         };
-        if (p.n_csplit == 1) {
+        if (!MANY && p.n_csplit == 1) {
             if (t < HQ) {
                 sm.l_inv[t] = l_share > 0.f ? 1.f / l_share : 0.f;
                 if (!(l_share > 0.f) && blk == 0 && !p.ml_out) lorc_set_status(p.status, LORC_ERR_EMPTY);
@@ -406,43 +418,52 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                 }
             }
         } else {
-            // this share's piece, for the CTAs of the cluster
-            float* share = xch + (SPLIT ? HQ * XLD : 0);
+            // this share's piece, for the CTAs of the cluster, or in memory for those of all clusters
+            float* share = MANY ? p.o_part + (((long long)s * p.n_blk + blk) * p.n_csplit + cs) * SHARE_FLOATS
+                                     : xch + (SPLIT ? HQ * XLD : 0);
+            constexpr int ld = MANY ? 128 : XLD;
 #pragma unroll
             for (int c0 = 0; c0 < 128; c0 += 32) {
                 uint32_t r[32];
                 take(c0, r);
-                if (has_row) {
+                if (has_row && (!MANY || cs < p.n_csplit)) {
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4)
-                        *reinterpret_cast<uint4*>(share + hrow * XLD + c0 + q4 * 4) =
+                        *reinterpret_cast<uint4*>(share + hrow * ld + c0 + q4 * 4) =
                             make_uint4(r[q4 * 4], r[q4 * 4 + 1], r[q4 * 4 + 2], r[q4 * 4 + 3]);
                 }
             }
-            if (t < HQ) sm.l_inv[t] = l_share;
+            if (t < HQ && (!MANY || cs < p.n_csplit)) (MANY ? share + HQ * 128 : sm.l_inv)[t] = l_share;
         }
         if (!ok && lane == 0) lorc_set_status(p.status, LORC_ERR_TIMEOUT);
     }
-    if (p.n_csplit > 1) {
-        // The pieces of all shares are there; each CTA takes every n_csplit-th group of 128 x four columns and adds the shares up in
-        // their order.  (Through memory, with the last share to arrive adding all of them, this took 5 us for two shares and 9 for
-        // eighteen.  Interleaved pairs, b 4, 2049 tokens, six shares: step 33.6 -> 31.1 us; 70B shape, b 8, 8201 tokens, two to five
-        // shares: 364 -> 353 us for three layers; b 4, 32777 tokens, r 256: 216 -> 212 us for two.)
+    if (MANY || p.n_csplit > 1) {
+        // One cluster: behind its barrier the pieces of all shares are there.  Several: those of this cluster are, and of the CTAs
+        // of one rank the last to arrive goes on, when those of the others are there too.  Each rank takes every cluster-th group of
+        // 128 x four columns and adds the shares up in their order.  (Through memory, with the last share to arrive adding all of
+        // them, this took 5 us for two shares and 9 for eighteen.  Interleaved pairs, b 4, 2049 tokens, six shares: step 33.6 ->
+        // 31.1 us.)
         __syncwarp();
         cluster_arrive_release();
         cluster_wait_acquire();
-        if (warp >= 2) {
+        const int rank = MANY ? cs % p.cluster : cs;
+        bool mine = warp >= 2;
+        if (MANY && mine) {
+            if (tid == 64) {
+                __threadfence();
+                // (counts up to the number of clusters and wraps, so the word is zero again for the next call)
+                const unsigned before = atomicInc(p.arrived + ((long long)s * p.n_blk + blk) * PV_MAX_CLUSTER + rank, p.n_clusters - 1);
+                sm.last = before == (unsigned)p.n_clusters - 1;
+                __threadfence();
+            }
+            __syncwarp();   // a named barrier counts a warp once only if the warp arrives converged
+            asm volatile("bar.sync 2, 128;" ::: "memory");
+            mine = sm.last != 0;
+        }
+        if (mine) {
             const uint32_t share0 = smem_u32(&sm.V[0][0][0]) + (SPLIT ? HQ * XLD * 4 : 0), l0 = smem_u32(sm.l_inv);
-            for (int i = cs * 128 + tid - 64; i < HQ * 32; i += p.n_csplit * 128) {
+            auto finish = [&](int i, float4 x, float l) {         // element group i: head i / 32, columns 4 (i % 32) ..
                 const int h = i >> 5, c = (i & 31) * 4;
-                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-                float l = 0.f;
-#pragma unroll 4
-                for (int j = 0; j < p.n_csplit; ++j) {
-                    const float4 v = ld_cluster_f4(mapa_shared(share0 + (h * XLD + c) * 4, j));
-                    l += ld_cluster_f1(mapa_shared(l0 + h * 4, j));
-                    x.x += v.x; x.y += v.y; x.z += v.z; x.w += v.w;
-                }
                 if (blk == 0 && c == 0) {
                     if (p.ml_out) {
                         p.ml_out[((long long)s * p.H_q + h) * 2] = sm.m_row[h];
@@ -465,9 +486,66 @@ lorc_pv2_kernel(const __grid_constant__ CUtensorMap mapCV, const Pv2Params p) {
                 }
                 *reinterpret_cast<uint2*>(on) = make_uint2(w[0], w[1]);
                 if (SPLIT) *reinterpret_cast<uint2*>(on + r_pad) = make_uint2(wl[0], wl[1]);
+            };
+            const int t = tid - 64;
+            if (!MANY) {
+                for (int i = rank * 128 + t; i < HQ * 32; i += p.n_csplit * 128) {
+                    const int h = i >> 5, c = (i & 31) * 4;
+                    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float l = 0.f;
+#pragma unroll 4
+                    for (int j = 0; j < p.n_csplit; ++j) {
+                        const float4 v = ld_cluster_f4(mapa_shared(share0 + (h * XLD + c) * 4, j));
+                        l += ld_cluster_f1(mapa_shared(l0 + h * 4, j));
+                        x.x += v.x; x.y += v.y; x.z += v.z; x.w += v.w;
+                    }
+                    finish(i, x, l);
+                }
+            } else {
+                // (up to E x U loads of a thread are in flight at once; with bulk copies into the C_V stages instead a call took
+                // 2 us more)
+                constexpr int E = 4, U = 8;
+                const int step = p.cluster * 128;
+                const float* part = p.o_part + ((long long)s * p.n_blk + blk) * p.n_csplit * SHARE_FLOATS;
+                for (int i0 = rank * 128 + t; i0 < HQ * 32; i0 += E * step) {
+                    float4 x[E];
+                    float l[E];
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        l[e] = 0.f;
+                    }
+                    for (int j0 = 0; j0 < p.n_csplit; j0 += U) {
+                        float4 v[U][E];
+                        float lv[U][E];
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+#pragma unroll
+                            for (int e = 0; e < E; ++e) {
+                                const int i = i0 + e * step;
+                                v[u][e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                lv[u][e] = 0.f;
+                                if (j0 + u < p.n_csplit && i < HQ * 32) {
+                                    const float* piece = part + (long long)(j0 + u) * SHARE_FLOATS;
+                                    v[u][e] = __ldcg(reinterpret_cast<const float4*>(piece) + i);
+                                    lv[u][e] = __ldcg(piece + HQ * 128 + (i >> 5));
+                                }
+                            }
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+#pragma unroll
+                            for (int e = 0; e < E; ++e) {
+                                x[e].x += v[u][e].x; x[e].y += v[u][e].y; x[e].z += v[u][e].z; x[e].w += v[u][e].w;
+                                l[e] += lv[u][e];
+                            }
+                    }
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (i0 + e * step < HQ * 32) finish(i0 + e * step, x[e], l[e]);
+                }
             }
-            __syncwarp();
         }
+        __syncwarp();
         cluster_arrive_release();                        // no CTA leaves while another may still read its piece
         cluster_wait_acquire();
     }
@@ -660,45 +738,43 @@ size_t on_bytes(const lorc_ctx* ctx, int batch, int n_blk) {
     return lorc_align_up((size_t)batch * ctx->desc.n_q_heads * (lorc_tc_split(ctx) ? 2 : 1) * n_blk * 128 * sizeof(bf16), 256);
 }
 
-template <class Fn>
+template <bool MANY, class Fn>
 cudaError_t with_pv_kernel(const lorc_ctx* ctx, Fn fn) {
     const bool split = lorc_tc_split(ctx);
     if (ctx->desc.n_q_heads == 32)
-        return split ? fn(lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>) + 1024)
-                     : fn(lorc_pv2_kernel<32, false>, sizeof(Pv2Smem<32, false>) + 1024);
-    return split ? fn(lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>) + 1024)
-                 : fn(lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>) + 1024);
+        return split ? fn(lorc_pv2_kernel<32, true, MANY>, sizeof(Pv2Smem<32, true>) + 1024)
+                     : fn(lorc_pv2_kernel<32, false, MANY>, sizeof(Pv2Smem<32, false>) + 1024);
+    return split ? fn(lorc_pv2_kernel<64, true, MANY>, sizeof(Pv2Smem<64, true>) + 1024)
+                 : fn(lorc_pv2_kernel<64, false, MANY>, sizeof(Pv2Smem<64, false>) + 1024);
 }
 
-constexpr int PV_MAX_SHARES = 16;    // the largest cluster
+// Scratch of `shares` shares whose pieces go through memory.
+size_t part_bytes(const lorc_ctx* ctx, long long blocks, int shares) {
+    return (size_t)blocks * shares * share_floats(ctx->desc.n_q_heads) * sizeof(float);
+}
 
-// Clusters of `shares` blocks that are resident at once (asked for once per context; 0: no such launch).
-int pv_clusters(lorc_ctx* ctx, int shares) {
-    if (shares == 1) return ctx->sm_count;
-    int& known = ctx->pv_clusters[shares];
-    if (known == 0) {
-        int n = 0;
-        const cudaError_t e = with_pv_kernel(ctx, [&](auto kernel, size_t smem) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(1, shares, 1);
-            cfg.blockDim = dim3(P_THREADS);
-            cfg.dynamicSmemBytes = smem;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 1;
-            attr[0].val.clusterDim.y = (unsigned)shares;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
-        });
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            n = 0;
-        }
-        known = n > 0 ? n : -1;
+// Clusters of `blocks` blocks that are resident at once (0: no such launch).
+int pv_clusters(const lorc_ctx* ctx, int blocks) {
+    int n = 0;
+    const cudaError_t e = with_pv_kernel<false>(ctx, [&](auto kernel, size_t smem) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, blocks, 1);
+        cfg.blockDim = dim3(P_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = (unsigned)blocks;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+    });
+    if (e != cudaSuccess) {
+        cudaGetLastError();      // (a size that the GPU does not take)
+        return 0;
     }
-    return known > 0 ? known : 0;
+    return n;
 }
 
 }  // namespace
@@ -706,57 +782,88 @@ int pv_clusters(lorc_ctx* ctx, int shares) {
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch) { return on_bytes(ctx, batch, (ctx->n + 127) / 128); }
+size_t lorc_tc_pv_scratch_least(const lorc_ctx* ctx, int batch) { return on_bytes(ctx, batch, (ctx->n + 127) / 128); }
 
-cudaError_t lorc_tc_pv_set_attrs() {
-    auto attr = [](const void* kernel, size_t bytes, bool wide_clusters) {
-        cudaError_t e = wide_clusters ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes + 1024);
+// The pieces of as many shares as the plan takes by itself, for any rank.
+size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq_len) {
+    const int tiles = (max_seq_len + TILE - 1) / TILE;
+    size_t most = 0;
+    for (int n_blk = 1; n_blk <= (ctx->n + 127) / 128; ++n_blk) {
+        const long long blocks = (long long)batch * n_blk;
+        int shares = (int)(ctx->sm_count / blocks);
+        if (shares > tiles) shares = tiles;
+        if (shares > PV_MAX_SHARES) shares = PV_MAX_SHARES;
+        if (shares > 1 && part_bytes(ctx, blocks, shares) > most) most = part_bytes(ctx, blocks, shares);
+    }
+    return lorc_tc_pv_scratch_least(ctx, batch) + most;
+}
+
+cudaError_t lorc_tc_pv_set_attrs(lorc_ctx* ctx) {
+    // (one context's kernels; the attributes are the device's, and another context sets those of its own)
+    auto attr = [](auto kernel, size_t bytes) {
+        return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    cudaError_t e = attr((const void*)lorc_pv2_kernel<32, false>, sizeof(Pv2Smem<32, false>), true);
-    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, false>, sizeof(Pv2Smem<64, false>), true);
-    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<32, true>, sizeof(Pv2Smem<32, true>), true);
-    if (e == cudaSuccess) e = attr((const void*)lorc_pv2_kernel<64, true>, sizeof(Pv2Smem<64, true>), true);
-    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel<false>, sizeof(UpSmem<false>), false);
-    if (e == cudaSuccess) e = attr((const void*)lorc_upproj_kernel<true>, sizeof(UpSmem<true>), false);
+    auto pv_attr = [&](auto kernel, size_t bytes) {
+        const cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        return e == cudaSuccess ? attr(kernel, bytes) : e;
+    };
+    cudaError_t e = with_pv_kernel<false>(ctx, pv_attr);
+    if (e == cudaSuccess) e = with_pv_kernel<true>(ctx, pv_attr);
+    if (e == cudaSuccess) e = attr(lorc_upproj_kernel<false>, sizeof(UpSmem<false>) + 1024);
+    if (e == cudaSuccess) e = attr(lorc_upproj_kernel<true>, sizeof(UpSmem<true>) + 1024);
+    ctx->pv_clusters[1] = ctx->sm_count;
+    for (int c = 2; c <= PV_MAX_CLUSTER && e == cudaSuccess; ++c) ctx->pv_clusters[c] = pv_clusters(ctx, c);
     return e;
 }
 
-// One CTA per SM at most, as many clusters as are resident at once, and the number of shares whose chain is shortest.  In units
-// of one tile (about 0.45 us of a CTA's stream): the tiles of a share, and with more than one share 8 and 0.8 per share.  So up to
-// 15 tiles one CTA takes a block.  (That is what merging through memory cost; the exchange in the cluster takes about 2 us less.
-// But the number of shares decides in which order a block's sums are taken, and calls that leave it to the library keep their
-// results to the bit.)
-void lorc_tc_pv_plan(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
+// One CTA per SM at most, and the number of shares whose chain is shortest.  In units of one tile (about 0.45 us of a CTA's
+// stream): the tiles of a share, and with more than one share 8 and 0.8 per share.  So up to 15 tiles one CTA takes a block.
+// (The constants were measured with shares that met in memory, where the last to arrive added all of them; inside one cluster the
+// exchange takes about 2 us less.)  The shares of a block are dealt to as few clusters of equal size as are resident at once.
+void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
                      LorcPvPlan* plan) {
-    const int tiles = (cv.max_seq_len + TILE - 1) / TILE, most = tiles < PV_MAX_SHARES ? tiles : PV_MAX_SHARES;
+    const int tiles = (cv.max_seq_len + TILE - 1) / TILE;
     plan->n_blk = (L.r_v + 127) / 128;
-    plan->n_csplit = 1;
-    plan->fits = on_bytes(ctx, cv.batch, plan->n_blk) <= scratch_bytes;
+    plan->off_part = on_bytes(ctx, cv.batch, plan->n_blk);
+    plan->fits = plan->off_part <= scratch_bytes;
     const long long blocks = (long long)cv.batch * plan->n_blk;
-    if (n_splits_hint > 0) {
-        plan->n_csplit = n_splits_hint < most ? n_splits_hint : most;
-        while (plan->n_csplit > 1 && pv_clusters(ctx, plan->n_csplit) == 0) --plan->n_csplit;
-        return;
-    }
-    int best = 5 * tiles;                                     // five times the cost, in tiles
-    for (int cs = 2; cs <= most && blocks * cs <= ctx->sm_count; ++cs) {
-        const int cost = 5 * ((tiles + cs - 1) / cs + 8) + 4 * cs;
-        if (cost < best && blocks <= pv_clusters(ctx, cs)) {
-            best = cost;
-            plan->n_csplit = cs;
+    long long most = n_splits_hint > 0 ? n_splits_hint : ctx->sm_count / blocks;
+    if (most > tiles) most = tiles;
+    if (most > PV_MAX_SHARES) most = PV_MAX_SHARES;
+    int shares = n_splits_hint > 0 ? (int)most : 1;
+    if (n_splits_hint <= 0) {
+        int best = 5 * tiles;                                 // five times the cost, in tiles
+        for (int cs = 2; cs <= most; ++cs) {
+            const int cost = 5 * ((tiles + cs - 1) / cs + 8) + 4 * cs;
+            if (cost < best) {
+                best = cost;
+                shares = cs;
+            }
         }
     }
+    for (; shares > 1; --shares) {
+        const int fewest = (shares + PV_MAX_CLUSTER - 1) / PV_MAX_CLUSTER;
+        const bool room = plan->off_part + part_bytes(ctx, blocks, shares) <= scratch_bytes;       // for several clusters
+        for (int k = fewest; k <= (room ? shares : 1); ++k) {
+            const int c = (shares + k - 1) / k;
+            // (a share count that was asked for may take more blocks than there are SMs)
+            if (ctx->pv_clusters[c] < (n_splits_hint > 0 ? 1 : blocks * k)) continue;
+            plan->n_csplit = shares;
+            plan->cluster = c;
+            plan->n_clusters = k;
+            return;
+        }
+    }
+    plan->n_csplit = plan->cluster = plan->n_clusters = 1;
 }
 
-// scratch: the normalised latent output
+// scratch: the normalised latent output, then the pieces of shares in several clusters
 cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCV,
-                              const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, int tiles,
+                              const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, unsigned* arrived, int tiles,
                               const LorcPvPlan& plan, void* scratch, bf16* out, bool latent_out, const int32_t* pos0,
                               const int32_t* q_pos, float* ml_out, cudaStream_t st, int* launches) {
     const lorc_model_desc& d = ctx->desc;
-    const int n_blk = plan.n_blk, n_csplit = plan.n_csplit;
+    const int n_blk = plan.n_blk;
     const int r_pad = n_blk * 128;
     const bool split = lorc_tc_split(ctx);
     const int r_ld = split ? 2 * r_pad : r_pad;        // row of o_norm
@@ -768,13 +875,15 @@ cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView
         p.pimg = pimg; p.rowmax = rowmax; p.o_norm = o_norm; p.ml_out = ml_out;
         p.seq_lens = cv.seq_lens; p.page_table = cv.page_table; p.status = ctx->status_dev;
         p.batch = cv.batch; p.H_q = d.n_q_heads; p.n_kv = d.n_kv_heads; p.r_v = L.r_v; p.tiles = tiles;
-        p.n_blk = n_blk; p.n_csplit = n_csplit; p.max_pos = d.max_pos; p.max_rows = lorc_tc_max_rows(cv);
+        p.o_part = (float*)((char*)scratch + plan.off_part); p.arrived = arrived;
+        p.n_blk = n_blk; p.n_csplit = plan.n_csplit; p.cluster = plan.cluster; p.n_clusters = plan.n_clusters; p.max_pos = d.max_pos; p.max_rows = lorc_tc_max_rows(cv);
         p.pos0 = pos0; p.q_pos = q_pos;
         p.page_size = cv.page_size; p.max_pages_per_seq = cv.max_pages_per_seq; p.n_pages = cv.n_pages;
-        dim3 grid(n_blk, n_csplit, cv.batch);
-        e = with_pv_kernel(ctx, [&](auto kernel, size_t smem) {
-            return lorc_launch_dependent_cluster(kernel, grid, dim3(P_THREADS), smem, dim3(1, n_csplit, 1), st, mapCV, p);
-        });
+        dim3 grid(n_blk, plan.cluster * plan.n_clusters, cv.batch);
+        auto launch = [&](auto kernel, size_t smem) {
+            return lorc_launch_dependent_cluster(kernel, grid, dim3(P_THREADS), smem, dim3(1, plan.cluster, 1), st, mapCV, p);
+        };
+        e = plan.n_clusters > 1 ? with_pv_kernel<true>(ctx, launch) : with_pv_kernel<false>(ctx, launch);
         *launches += 1;
         if (e != cudaSuccess) return e;
     }

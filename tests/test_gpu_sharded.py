@@ -28,12 +28,24 @@ def _shard_caches(sess, lens, pos0, cnt, ck, cv, n_max):
 ])
 @pytest.mark.parametrize("world", [2, 3])
 def test_sharded_decode_equals_unsharded_and_oracle(geom, flags, path, world):
+    _check(geom, flags, path, world, [700, 130, 300, 17], 0)       # the last two leave ranks with few or no rows
+
+
+@pytest.mark.parametrize("H_q,r_v,lens,n_splits", [
+    (32, 136, [4200, 300, 17], 0),       # 17 tiles a rank: six context shares of P.C_V by the plan
+    (64, 72, [4200, 17], 3),
+    (32, 136, [4200, 300], 17),          # several clusters
+])
+def test_sharded_decode_with_several_context_shares(H_q, r_v, lens, n_splits):
+    _check(dict(D=1024, H_q=H_q, H_kv=8, d_h=128, r_k=64, r_v=r_v), 0, 2, 2, lens, n_splits)
+
+
+def _check(geom, flags, path, world, lens, n_splits):
     import torch
     from paper_2410_03111_b200 import sharded
     L = H.lib()
-    lens = [700, 130, 300, 17]           # the last two leave ranks with few or no rows
     prob = H.Problem(geom["D"], geom["H_q"], geom["H_kv"], geom["d_h"], geom["r_k"], geom["r_v"], theta=500000.0, layer=7)
-    b, n_max = len(lens), 768
+    b, n_max = len(lens), max(lens) + 68
     sess = H.Session(prob, max_pos=n_max, batch=b, flags=flags)
     xs = [synth.hidden_states(n, prob.D, 7, chunk=50 + s).astype(np.float64) for s, n in enumerate(lens)]
     ck, cv = H.oracle_latents(prob, xs)
@@ -46,7 +58,7 @@ def test_sharded_decode_equals_unsharded_and_oracle(geom, flags, path, world):
     mls = torch.zeros(world, b, prob.H_q, 2, dtype=torch.float32, device="cuda")
     for r in range(world):
         p0 = torch.tensor(pos0[r], dtype=torch.int32, device="cuda")
-        L.lorc_decode_attn_shard(sess.ctx, 0, held[r][0], qd, p0, q_pos, outs[r], mls[r])
+        L.lorc_decode_attn_shard(sess.ctx, 0, held[r][0], qd, p0, q_pos, outs[r], mls[r], n_splits)
         assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
         assert L.lorc_last_path(sess.ctx) == path
         ml = H.host_f64(mls[r])
