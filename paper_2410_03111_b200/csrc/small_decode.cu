@@ -9,13 +9,11 @@
 //   rotation and q.k in registers (the accumulator columns of a rotary pair belong to one thread), softmax over the 64
 //   tokens, then O_lat += P . C_V with fp32 FMAs, thread = (8 latent columns, group of tokens).
 // Such calls are small: the kernel is bound by its chain of dependent loads, so shares are short (64 tokens when that
-// fills the chip).  Where a call has at most eight shares and the rank is low they form a cluster that merges them through
+// fills the chip).  Where a call is small in every way (see SD_MERGE_SHARES) its shares form a cluster that merges them through
 // distributed shared memory and up-projects the result: one launch less.  At 129 tokens, rank 32, 4 heads of 64 the kernel takes
 // 11 us where the scalar kernel took 99 us; the step with cache write and merge took 72 us with that one, then 19; one step among
 // many, launched from Python: 11.8 us with the merge kernel, 9.5 with the merge inside.
 #include <math.h>
-
-#include <type_traits>
 
 #include "common.cuh"
 #include "sm100_pair.cuh"
@@ -29,8 +27,17 @@ namespace {
 constexpr int SD_THREADS = 128;
 constexpr int SD_TILE = LORC_SMALL_TILE;             // tokens per step: 16 per warp
 // Merge inside: as many shares as every GPU takes in a cluster, and r_v * d_h at most this, so that a thread holds its 64 or
-// fewer elements of B_V in registers before the shares meet.  (Larger ranks: a block per head of the merge kernel is faster.)
-constexpr int SD_MERGE_SHARES = 8, SD_MERGE_WORK = 64 * SD_THREADS;
+// fewer elements of B_V in registers before the shares meet.  Its blocks hold more registers and shared memory, and one of them
+// takes the heads of a KV head in series, so the line lies where this was faster than the merge kernel throughout a sweep of
+// heads, ranks, lengths and batches (one call among many, graph replay, merge kernel -> inside; where the rule keeps that kernel
+// the second figure is what merging inside took):
+//   up to two query heads per KV head: d_h 64, r 32, 129 tokens 9.2 -> 7.1 us; r 128, 500 tokens 17.0 -> 11.1.
+//   more: d_h 64, r 32, 40 tokens, four heads 7.9 -> 10.8, eight 9.8 -> 16.1; with as many shares as heads 0.93 to 1.06.
+//   blocks that all run at once (8 / 3 per SM): 320 blocks 18.1 -> 14.8, 384 13.1 -> 11.3, 432 17.5 -> 22.9, 512 14.8 -> 22.5;
+//   clusters of more than five do not pack as well: 256 blocks 10.8 -> 11.3.
+//   d_h 128, where a thread holds a pair's whole row: r 64, 129 tokens 11.0 -> 9.4, r 16 7.8 -> 8.1; one share of two heads
+//   10.0 -> 10.1; 240 blocks 12.7 -> 13.4.
+constexpr int SD_MERGE_SHARES = 8, SD_MERGE_WORK = 64 * SD_THREADS, SD_MERGE_HEADS = 2;
 
 struct SdParams {
     const bf16* q;
@@ -263,7 +270,7 @@ small_decode_kernel(const SdParams p) {
             p.part_ml[unit * 2 + 1] = l_s[tid];
         }
     } else {
-        // The arithmetic and the order of the sums are those of the merge kernel.  A share's CTA takes every n_splits-th head;
+        // The arithmetic is that of the merge kernel, and so is the order of the sums, but for the denominator's (in double).  A share's CTA takes every n_splits-th head;
         // thread = (output column j, slices sl and sl + SL of the rank), its elements of B_V on their way while the shares meet.
         constexpr int SL = SD_THREADS / DH, SLICES = 256 / DH, NW = 64 / 2;
         __shared__ float ml[GM][2];
@@ -357,15 +364,15 @@ cudaError_t lorc_small_decode(const lorc_ctx* ctx, const LorcLayer& L, const Cac
     p.r_k = L.r_k; p.r_v = L.r_v; p.G = ctx->group; p.n_splits = n_splits; p.rope_style = ctx->pair_style;
     p.max_pos = d.max_pos; p.out = out; p.B_v = L.B_v; p.n = ctx->n;
     const bool wide = d.d_head == 128;
-    *merged = may_merge && n_splits <= SD_MERGE_SHARES && L.r_v * d.d_head <= SD_MERGE_WORK;
-    auto pick = [&](auto merge) {
-        constexpr bool M = decltype(merge)::value;
-        return ctx->group <= 2 ? (wide ? small_decode_kernel<128, 2, M> : small_decode_kernel<64, 2, M>)
-               : ctx->group <= 4 ? (wide ? small_decode_kernel<128, 4, M> : small_decode_kernel<64, 4, M>)
-                                 : (wide ? small_decode_kernel<128, 8, M> : small_decode_kernel<64, 8, M>);
-    };
+    const long long blocks = (long long)n_splits * d.n_kv_heads * cv.batch;
+    const bool one_round = wide || n_splits > 5 ? blocks <= ctx->sm_count : 3 * blocks <= 8ll * ctx->sm_count;
+    *merged = may_merge && ctx->group <= SD_MERGE_HEADS && n_splits <= SD_MERGE_SHARES && L.r_v * d.d_head <= SD_MERGE_WORK &&
+              one_round && (!wide || (L.r_v >= 32 && n_splits >= ctx->group));
+    auto kernel = ctx->group <= 2 ? (*merged ? (wide ? small_decode_kernel<128, 2, true> : small_decode_kernel<64, 2, true>)
+                                             : (wide ? small_decode_kernel<128, 2, false> : small_decode_kernel<64, 2, false>))
+                  : ctx->group <= 4 ? (wide ? small_decode_kernel<128, 4, false> : small_decode_kernel<64, 4, false>)
+                                    : (wide ? small_decode_kernel<128, 8, false> : small_decode_kernel<64, 8, false>);
     *launches += 1;
     const dim3 grid(n_splits, d.n_kv_heads, cv.batch), block(SD_THREADS);
-    return *merged ? lorc_launch_dependent_cluster(pick(std::true_type()), grid, block, 0, dim3(n_splits), st, p)
-                   : lorc_launch_dependent(pick(std::false_type()), grid, block, 0, st, p);
+    return lorc_launch_dependent_cluster(kernel, grid, block, 0, dim3(*merged ? n_splits : 1), st, p);
 }
