@@ -277,23 +277,20 @@ def test_shards_that_are_empty_or_end_behind_the_query(style):
 
 
 @pytest.mark.parametrize("geom,lens,page,n_splits", [
-    (G8B, [2049, 1990, 17, 128], 0, 0),             # the default plan: six shares at 17 tiles, one batch of the merge
+    (G8B, [2049, 1990, 17, 128], 0, 0),             # the default plan: six shares at 17 tiles
     (G8B, [2100, 600], 64, 2),
-    (G8B, [2049, 40], 0, 7),                        # one full batch of the merge
-    (G8B, [2049, 1500], 16, 8),                     # a full batch and one share
+    (G8B, [2049, 40], 0, 7),                        
+    (G8B, [2049, 1500], 16, 8),                     
     (G_N512, [1700, 900, 1], 0, 12),
-    (G70B, [1300, 130], 0, 3),                      # two parts of 64 heads: two shares per batch
+    (G70B, [1300, 130], 0, 3),                      # two parts of 64 heads
     (G70B, [1100, 700], 128, 5),
 ])
 def test_interleaved_several_context_shares(geom, lens, page, n_splits):
-    """Shares publish both parts and the last one adds them, batch by batch, in the memory that the parts' exchange used."""
+    """Each share leaves the sum of both parts behind the memory that the parts' exchange used, and adds up its columns of all."""
     import torch
     prob = H.Problem(r_k=64, r_v=136, theta=500000.0, layer=31, style=INTERLEAVED, **geom)
     L, b = H.lib(), len(lens)
     sess = H.Session(prob, max_pos=max(lens) + 3, batch=b)
-    # room for the shares that are asked for: 16 KB (32 heads) or 33 KB a share, sequence and column block
-    ws = torch.zeros(sess.ws.numel() + b * 2 * 12 * 129 * 64 * 4, dtype=torch.uint8, device="cuda")
-    L.lorc_set_workspace(sess.ctx, ws)
     rng = np.random.default_rng(n_splits)
     ck, cv = ([synth.to_bf16_exact(rng.standard_normal((n, r)) * np.arange(1, r + 1) ** -0.8) for n in lens] for r in (64, 136))
     if page:
@@ -303,7 +300,7 @@ def test_interleaved_several_context_shares(geom, lens, page, n_splits):
     q = synth.queries(b, prob.H_q, 128, 31, 10, 8.0).astype(np.float64)
     out = torch.zeros(b, prob.H_q, 128, dtype=torch.bfloat16, device="cuda")
     lat = torch.zeros(b, prob.H_q, 136, dtype=torch.bfloat16, device="cuda")
-    for _ in range(2):                               # the counters of the shares are left empty
+    for _ in range(2):                               # (the row maxima are left empty)
         out.fill_(3.0)
         L.lorc_decode_attn(sess.ctx, 0, held[0], H.dev_bf16(q), out, n_splits=n_splits)
         L.lorc_decode_attn_latent_out(sess.ctx, 0, held[0], H.dev_bf16(q), lat, n_splits=n_splits)

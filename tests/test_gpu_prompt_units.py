@@ -1,5 +1,5 @@
 """Prompt kernels whose units shrink for short launches: reconstruction by single heads (up to four pairs of 128-token tiles with eight
-KV heads) against units of two heads; rank tails, odd tile counts, pages.  Bound as in the other prompt tests."""
+KV heads, nine with four) against units of two heads; rank tails, odd tile counts, pages.  Bound as in the other prompt tests."""
 import numpy as np
 import pytest
 
@@ -11,14 +11,19 @@ import helpers as H
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("H_q,r_k,r_v,lens,T,page", [
-    (32, 200, 72, [450, 130], 60, 16),         # four pairs of tiles: single heads; rank tails below a slice
-    (64, 72, 200, [385], 385, 0),              # odd number of tiles; eight heads per KV head
-    (32, 72, 200, [300, 200, 129], 40, 128),   # six pairs: two heads per unit
+@pytest.mark.parametrize("H_q,H_kv,r_k,r_v,lens,T,page", [
+    (32, 8, 200, 72, [450, 130], 60, 16),         # four pairs of tiles: single heads; rank tails below a slice
+    (64, 8, 72, 200, [385], 385, 0),              # eight heads per KV head
+    (32, 8, 72, 200, [300, 200, 129], 40, 128),   # six pairs: two heads per unit
+    (64, 8, 72, 72, [257], 257, 0),               # single heads, an odd number of tiles: the pair's second tile lies past the end
+    (32, 8, 136, 64, [384, 129], 50, 64),
+    (32, 8, 64, 72, [1100], 33, 0),               # five pairs, nine tiles: two heads per unit
+    (32, 4, 72, 64, [130] * 9, 20, 0),            # nine pairs with four KV heads: single heads, 72 units for 74 pairs of SMs
+    (32, 4, 72, 64, [130] * 10, 20, 32),          # ten: two heads
 ])
-def test_reconstruction_units(H_q, r_k, r_v, lens, T, page):
+def test_reconstruction_units(H_q, H_kv, r_k, r_v, lens, T, page):
     import torch
-    prob = H.Problem(1024, H_q, 8, 128, r_k, r_v, theta=500000.0, layer=24)
+    prob = H.Problem(1024, H_q, H_kv, 128, r_k, r_v, theta=500000.0, layer=24)
     b, n_max = len(lens), max(lens)
     sess = H.Session(prob, max_pos=n_max, batch=b)
     ck, cv = H.oracle_latents(prob, [synth.hidden_states(n, prob.D, 24, chunk=s).astype(np.float64) for s, n in enumerate(lens)])
