@@ -180,10 +180,10 @@ int lorc_append(lorc_ctx* ctx, int layer, const lorc_cache* cache, const void* x
  * with 128-wide heads also by the lengths of all sequences); a positive value asks
  * for that many shares (context splits of the plain kernels and of the uncompressed
  * mode, clamped to what the workspace holds; context shares per latent column block
- * of the tensor-core path, at most 64 and one per 128 tokens: those that form one
- * cluster of up to 16 need no workspace, for others the count is clamped to what
- * the workspace holds).  The number of shares decides the order of sums, and so
- * the last bits of a result.  Uses the workspace.
+ * of the tensor-core path, at most 64 and one per 128 tokens, clamped to what the
+ * workspace holds unless those of all sequences run at once in clusters of up to
+ * 16).  The number of shares decides the order of sums, and so the last bits of a
+ * result.  Uses the workspace.
  * A sequence with seq_lens[s] <= 0 gets a row of zeros and sets status EMPTY.
  * The first call on a context, and the first call with a larger batch than any
  * before, sets up small library-owned tables (an in-tile rotation table, one word

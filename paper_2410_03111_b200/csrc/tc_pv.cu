@@ -842,17 +842,17 @@ void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& c
         }
     }
     for (; shares > 1; --shares) {
-        const int fewest = (shares + PV_MAX_CLUSTER - 1) / PV_MAX_CLUSTER;
-        const bool room = plan->off_part + part_bytes(ctx, blocks, shares) <= scratch_bytes;       // for several clusters
-        for (int k = fewest; k <= (room ? shares : 1); ++k) {
-            const int c = (shares + k - 1) / k;
-            // (a share count that was asked for may take more blocks than there are SMs)
-            if (ctx->pv_clusters[c] < (n_splits_hint > 0 ? 1 : blocks * k)) continue;
-            plan->n_csplit = shares;
-            plan->cluster = c;
-            plan->n_clusters = k;
-            return;
-        }
+        int clusters = (shares + PV_MAX_CLUSTER - 1) / PV_MAX_CLUSTER;
+        while (clusters <= shares && ctx->pv_clusters[(shares + clusters - 1) / clusters] < blocks * clusters) ++clusters;
+        // (a count that was asked for, of more blocks than run at once: pairs, which leave no SM idle.  b 4, r 256, 32777 tokens, 24
+        // and 64 shares: 94 and 113 us before clusters, 103 and 123 in clusters of 12 and 16, 95 and 109 in pairs; b 16, r 512, 4129
+        // tokens, as many as the workspace holds: 83, 114 and 90)
+        if (clusters > shares) clusters = ctx->pv_clusters[2] > 0 ? (shares + 1) / 2 : shares;
+        if (clusters > 1 && plan->off_part + part_bytes(ctx, blocks, shares) > scratch_bytes) continue;
+        plan->n_csplit = shares;
+        plan->n_clusters = clusters;
+        plan->cluster = (shares + clusters - 1) / clusters;
+        return;
     }
     plan->n_csplit = plan->cluster = plan->n_clusters = 1;
 }
