@@ -48,7 +48,7 @@ constexpr float LOG2E = 1.4426950408889634f;
 // conflict-free word, and the finished 128 x 64 boxes leave by TMA.  (With four warps, thread = token row, the row-wise
 // 16-byte stores and table reads touched 32 lines per access and the epilogue took three times as long as the MMAs:
 // 284 us for the keys and values of 16 x 4096 tokens at rank 672, 162 us now.)
-// Where units of two heads would leave half of the pairs idle a unit is one head (N = 128): two thirds of the operand bytes and
+// Where units of two heads would leave half of the pairs idle a unit is one head (N = 128): three quarters of the operand bytes and
 // half of the epilogue in the chain of a launch that is one unit long.  (One prompt of 777 tokens, r 928 and 416, cache write and
 // attention of two layers: 104.1 -> 99.0 us.)
 constexpr int R_STAGES = 5;
