@@ -64,7 +64,7 @@ struct lorc_ctx {
     bool host_out = false;         // the call in progress writes its result to mapped host memory
     int64_t launches = 0;
     LorcTcState* tc = nullptr;
-    int pv_clusters[17] = {0};     // [c]: clusters of c blocks of the PV kernel that are resident at once, see lorc_tc_pv_set_attrs
+    int pv_clusters[17] = {0};     // [c]: clusters of c blocks of the PV kernel that are resident at once (0: not asked yet, -1: none), see lorc_tc_pv_plan
     LorcProfile* prof = nullptr;   // event bookkeeping, created on first use
     bool prof_on = false;          // LORC_FLAG_PROFILE or lorc_profile_enable
 };

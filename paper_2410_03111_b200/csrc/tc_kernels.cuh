@@ -78,8 +78,8 @@ struct LorcPvPlan {
 };
 size_t lorc_tc_pv_scratch_least(const lorc_ctx* ctx, int batch);      // without room for shares in several clusters
 size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq_len);
-cudaError_t lorc_tc_pv_set_attrs(lorc_ctx* ctx);
-void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
+cudaError_t lorc_tc_pv_set_attrs(const lorc_ctx* ctx);
+void lorc_tc_pv_plan(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
                      LorcPvPlan* plan);
 cudaError_t lorc_tc_pv_launch(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, const CUtensorMap& mapCV,
                               const CUtensorMap& mapBVT, const uint8_t* pimg, unsigned* rowmax, unsigned* arrived, int tiles,

@@ -753,28 +753,34 @@ size_t part_bytes(const lorc_ctx* ctx, long long blocks, int shares) {
     return (size_t)blocks * shares * share_floats(ctx->desc.n_q_heads) * sizeof(float);
 }
 
-// Clusters of `blocks` blocks that are resident at once (0: no such launch).
-int pv_clusters(const lorc_ctx* ctx, int blocks) {
-    int n = 0;
-    const cudaError_t e = with_pv_kernel<false>(ctx, [&](auto kernel, size_t smem) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1, blocks, 1);
-        cfg.blockDim = dim3(P_THREADS);
-        cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1;
-        attr[0].val.clusterDim.y = (unsigned)blocks;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
-    });
-    if (e != cudaSuccess) {
-        cudaGetLastError();      // (a size that the GPU does not take)
-        return 0;
+// Clusters of `blocks` blocks that are resident at once (0: no such launch).  Asked for once per context, when a plan first wants
+// to know: the fifteen sizes together take as long as a small layer.
+int pv_clusters(lorc_ctx* ctx, int blocks) {
+    if (blocks == 1) return ctx->sm_count;
+    int& known = ctx->pv_clusters[blocks];
+    if (known == 0) {
+        int n = 0;
+        const cudaError_t e = with_pv_kernel<false>(ctx, [&](auto kernel, size_t smem) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(1, blocks, 1);
+            cfg.blockDim = dim3(P_THREADS);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 1;
+            attr[0].val.clusterDim.y = (unsigned)blocks;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+        });
+        if (e != cudaSuccess) {
+            cudaGetLastError();      // (a size that the GPU does not take)
+            n = 0;
+        }
+        known = n > 0 ? n : -1;
     }
-    return n;
+    return known > 0 ? known : 0;
 }
 
 }  // namespace
@@ -798,7 +804,7 @@ size_t lorc_tc_pv_scratch_bytes(const lorc_ctx* ctx, int batch, int max_seq_len)
     return lorc_tc_pv_scratch_least(ctx, batch) + most;
 }
 
-cudaError_t lorc_tc_pv_set_attrs(lorc_ctx* ctx) {
+cudaError_t lorc_tc_pv_set_attrs(const lorc_ctx* ctx) {
     // (one context's kernels; the attributes are the device's, and another context sets those of its own)
     auto attr = [](auto kernel, size_t bytes) {
         return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -811,8 +817,6 @@ cudaError_t lorc_tc_pv_set_attrs(lorc_ctx* ctx) {
     if (e == cudaSuccess) e = with_pv_kernel<true>(ctx, pv_attr);
     if (e == cudaSuccess) e = attr(lorc_upproj_kernel<false>, sizeof(UpSmem<false>) + 1024);
     if (e == cudaSuccess) e = attr(lorc_upproj_kernel<true>, sizeof(UpSmem<true>) + 1024);
-    ctx->pv_clusters[1] = ctx->sm_count;
-    for (int c = 2; c <= PV_MAX_CLUSTER && e == cudaSuccess; ++c) ctx->pv_clusters[c] = pv_clusters(ctx, c);
     return e;
 }
 
@@ -820,7 +824,7 @@ cudaError_t lorc_tc_pv_set_attrs(lorc_ctx* ctx) {
 // stream): the tiles of a share, and with more than one share 8 and 0.8 per share.  So up to 15 tiles one CTA takes a block.
 // (The constants were measured with shares that met in memory, where the last to arrive added all of them; inside one cluster the
 // exchange takes about 2 us less.)  The shares of a block are dealt to as few clusters of equal size as are resident at once.
-void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
+void lorc_tc_pv_plan(lorc_ctx* ctx, const LorcLayer& L, const CacheView& cv, int n_splits_hint, size_t scratch_bytes,
                      LorcPvPlan* plan) {
     const int tiles = (cv.max_seq_len + TILE - 1) / TILE;
     plan->n_blk = (L.r_v + 127) / 128;
@@ -843,11 +847,11 @@ void lorc_tc_pv_plan(const lorc_ctx* ctx, const LorcLayer& L, const CacheView& c
     }
     for (; shares > 1; --shares) {
         int clusters = (shares + PV_MAX_CLUSTER - 1) / PV_MAX_CLUSTER;
-        while (clusters <= shares && ctx->pv_clusters[(shares + clusters - 1) / clusters] < blocks * clusters) ++clusters;
+        while (clusters <= shares && pv_clusters(ctx, (shares + clusters - 1) / clusters) < blocks * clusters) ++clusters;
         // (a count that was asked for, of more blocks than run at once: pairs, which leave no SM idle.  b 4, r 256, 32777 tokens, 24
         // and 64 shares: 94 and 113 us before clusters, 103 and 123 in clusters of 12 and 16, 95 and 109 in pairs; b 16, r 512, 4129
         // tokens, as many as the workspace holds: 83, 114 and 90)
-        if (clusters > shares) clusters = ctx->pv_clusters[2] > 0 ? (shares + 1) / 2 : shares;
+        if (clusters > shares) clusters = pv_clusters(ctx, 2) > 0 ? (shares + 1) / 2 : shares;
         if (clusters > 1 && plan->off_part + part_bytes(ctx, blocks, shares) > scratch_bytes) continue;
         plan->n_csplit = shares;
         plan->n_clusters = clusters;

@@ -99,3 +99,25 @@ def test_share_count_does_not_depend_on_the_clusters(H_q, r_v, lens, shares, few
     H.assert_rows_close(H.host_f64(outs[0][0]), H.oracle_decode(sess.prob, ck, cv, q), TOL)
     assert _same(outs[0], outs[1]) and not _same(outs[0], outs[2])
     sess.close()
+
+
+def test_share_counts_first_seen_under_stream_capture():
+    """A plan may ask for cluster sizes that no call before has asked for while the stream is being captured."""
+    import torch
+    sess, held, q, ck, cv = _case(32, 136, [4096], 1)
+    L, qd, stream = sess.L, H.dev_bf16(q), torch.cuda.Stream()
+    _run(sess, held, q, [4096], 1)                       # sets the context's tables up
+    outs = {S: torch.zeros(q.shape, dtype=torch.bfloat16, device="cuda") for S in (7, 17)}
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        for S, out in outs.items():
+            L.lorc_decode_attn(sess.ctx, 0, held[0], qd, out, n_splits=S)
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert L.lorc_sync_status(sess.ctx) == 0, L.lorc_last_error(sess.ctx)
+    for S, out in outs.items():
+        assert torch.equal(out, _run(sess, held, q, [4096], S)[0]), S
+    del graph
+    sess.close()
